@@ -91,7 +91,8 @@ enum {
                                samples per thread unless GM_F_SPT1) */
     GM_F_WIDE_BVH = 16,     /* traverse the 4-wide collapse of the tree instead of the binary tree */
     GM_F_REGCAP64 = 32,     /* cap the accumulation kernel at 64 registers (4 blocks per SM; the
-                               one-sample ray-queue kernel, the default, always fits 64) */
+                               default kernel, which traces each tile's rays as one shaft, always
+                               has 64) */
     GM_F_TILE_CONSECUTIVE = 64, /* multi-sample warp tiles of consecutive samples (else runs of 32 spread
                                over 8 tiles' span); a one-sample tile is one run of 32 either way */
     GM_F_STATIC_TILES = 128, /* one warp tile per warp of a full grid (else warps pull tiles from a counter) */
@@ -102,15 +103,16 @@ enum {
     GM_F_EYE_GRID = 1024,   /* occlusion through per-fixation eye grids instead of the BVH (ray-queue
                                kernel only: with NO_COMPACT, WIDE_BVH or REGCAP64 the BVH is kept) */
     GM_F_GRID64 = 2048,     /* with GM_F_EYE_GRID: 64 x 64 cells per fixation instead of 128 x 128 */
-    GM_F_SPT1 = 4096,       /* warp tiles of 32 samples (1 per thread); the default of the ray-queue
-                               binary-tree kernel (the eye grid's default is 4 per thread); with
+    GM_F_SPT1 = 4096,       /* warp tiles of 32 samples (1 per thread): the default (shafts over the 4-wide
+                               tree; the eye grid's default is 4 per thread); with
                                GM_F_NO_COMPACT: one-sample tiles traced in place */
     GM_F_SPT2 = 8192,       /* warp tiles of 64 samples (2 per thread): ray-queue binary tree and eye grid */
     GM_F_BLOCK512 = 16384,  /* blocks of 512 threads: eye grid (1 or 2 samples per thread) and the
                                one-sample ray-queue binary-tree kernel */
     GM_F_FIX_L1 = 32768,    /* ray-queue binary-tree kernel: read the fixations one by one through L1
                                (warp-wide broadcasts) instead of staging them 32 at a time in each
-                               warp's shared memory */
+                               warp's shared memory; one sample per thread: each ray walks the
+                               binary tree on its own instead of as part of a shaft */
     GM_F_SPT4 = 65536       /* warp tiles of 128 samples (4 per thread): the ray-queue binary-tree kernel
                                (the in-place and 4-wide kernels always take 4) */
 };
@@ -125,7 +127,8 @@ typedef struct {
     float accumulate_ms;      /* cone + occlusion + Gaussian + store + max kernel */
     float normalize_ms;
     uint32_t launches;        /* kernels this call launched */
-    uint64_t nodes_visited;   /* BVH nodes fetched by all occlusion rays (eye grid: cell entries read) */
+    uint64_t nodes_visited;   /* BVH nodes fetched by all occlusion rays (shafts: 4-wide nodes, one fetch for the
+                                 rays of a shaft; eye grid: cell entries read) */
     uint64_t tris_tested;     /* ray/triangle tests performed by all occlusion rays */
     uint64_t pairs_tested;    /* sample x fixation cone tests evaluated (pairs of warp tiles whose bounding
                                  sphere the cone misses are skipped without a per-sample test) */
@@ -182,8 +185,7 @@ gm_status gm_scene_info(const gm_scene* scene, uint32_t* n_tris, uint32_t* bvh_d
  * 4 x 4 transform (`transforms`: n_meshes x 16 FP64, host memory): the world triangles are
  * recomputed from the kept mesh-local ones exactly as at build time (a pose equal to the build's
  * transforms reproduces them bit for bit), the BVH boxes are refit bottom-up over the unchanged
- * hierarchy (same depth, looser boxes as meshes move apart), the export's local frames follow,
- * and the 4-wide collapse is dropped. Requires a scene built with gm_build_opts.dynamic;
+ * hierarchy (same depth, looser boxes as meshes move apart), and the export's local frames follow. Requires a scene built with gm_build_opts.dynamic;
  * GM_ERR_INVALID_ARG otherwise or on a non-finite transform. Synchronises `stream` once. Sample
  * sets of the scene keep stale positions until gm_samples_follow. */
 gm_status gm_scene_pose(gm_scene* scene, const double* transforms, gm_stream stream);

@@ -5,16 +5,17 @@
 // rest are stably sorted by window (radix sort on the window id), so every window is one
 // contiguous run of the fixation list.
 //
-// Accumulation (one fused kernel, sample-stationary): every thread owns SPT samples taken in
-// spatial (Morton) work order and keeps their compensated FP32 sums in registers. The block
-// streams the fixation list through shared memory in tiles; for each fixation every thread
-// runs the 4-sigma cone test on its samples (p = s - e, d1 = p.r^, c = p x r^,
-// in-cone <=> d1 > 0 and |c|^2 <= (cutoff tan theta)^2 d1^2, about 20 FP32 instructions per
-// pair) and, for in-cone pairs only, traces the occlusion segment e -> e + (1 - eps) p (any-hit,
-// early exit, the sample's own triangle skipped) with the watertight ray/triangle test of Woop,
-// Benthin and Wald (JCGT 2013), through the BVH or, with GM_F_EYE_GRID, over the triangles of the
-// segment's cell in the fixation's eye grid (gm_eyegrid.cu). With more fixations than one eye-grid
-// chunk holds, the kernel runs once per chunk and the compensated sums carry over. A visible pair adds
+// Accumulation (one fused kernel, sample-stationary): a block keeps a tile of 32 samples, taken in
+// spatial (Morton) work order, and their compensated FP32 sums through the whole fixation list. For
+// each fixation whose cone reaches the tile's bounding sphere the 32 samples run the 4-sigma cone test
+// (p = s - e, d1 = p.r^, c = p x r^, in-cone <=> d1 > 0 and |c|^2 <= (cutoff tan theta)^2 d1^2, about
+// 20 FP32 instructions per pair), and the segments e -> e + (1 - eps) p of the in-cone pairs are traced
+// together as one shaft (any hit, the sample's own triangle skipped; gm_shaft.cuh) with the watertight
+// ray/triangle test of Woop, Benthin and Wald (JCGT 2013). Other forms, picked by flags: each ray on
+// its own through the binary or 4-wide tree, in place or from a per-warp queue, or, with
+// GM_F_EYE_GRID, over the triangles of the segment's cell in the fixation's eye grid (gm_eyegrid.cu;
+// with more fixations than one chunk holds, the kernel runs once per chunk and the compensated sums
+// carry over). A visible pair adds
 // g = w exp(-(|c|/d1)^2 / (2 tan^2 theta)), i.e. the paper's t/(sigma sqrt(2 pi)) *
 // exp(-sigma_k^2 / (2 sigma^2)) with sigma_k = d2 / d1, d2 = |c|, in fixation order (Kahan).
 // When the window id of the next fixation changes (block-uniform), the block stores its sums
@@ -31,7 +32,7 @@
 
 #include "gm_internal.cuh"
 
-#include "gm_trace.cuh"
+#include "gm_shaft.cuh"
 
 namespace {
 
@@ -122,6 +123,35 @@ __global__ void __launch_bounds__(NT, MINB) k_accumulate(
         warp_tile<DEBUG, COMPACT, WIDE, GRID, S, FSM>(tile, spos, sidx, fix, nf, nodes, tris, P, out, max_bits,
                                                           wsmp + wb, wacc + wb, qslot + wb, qg + wb, wbox + warp,
                                                           &counters[2], dbg, err, st, FSM ? wfix + warp * 64 : nullptr);
+    }
+    warp_stats_commit(st, counters);
+}
+
+// The default: the rays of a (32-sample tile, fixation) pair traced as one shaft (gm_shaft.cuh). Blocks pull
+// tiles from a device counter (or, static, take their own).
+template <bool DEBUG>
+__global__ void __launch_bounds__(ACC_THREADS, 4) k_accumulate_shaft(
+    const float4* __restrict__ spos, const uint32_t* __restrict__ sidx, const float4* __restrict__ fix,
+    const uint32_t* __restrict__ n_fix_dev, const float4* __restrict__ nodes, const float4* __restrict__ nodes4,
+    const float4* __restrict__ tris, AccParams P, uint32_t n_tiles, int persistent, float* __restrict__ out,
+    unsigned int* __restrict__ max_bits, unsigned long long* __restrict__ counters, int* __restrict__ err,
+    DebugOut dbg) {
+    __shared__ ShaftBlock B;
+    __shared__ uint32_t s_tile;
+    const uint32_t nf = *n_fix_dev;
+    unsigned int* next = reinterpret_cast<unsigned int*>(&counters[6]);
+    TileStats st;
+    uint32_t tile = blockIdx.x;
+    for (;;) {
+        if (persistent) {
+            __syncthreads();
+            if (threadIdx.x == 0) s_tile = atomicAdd(next, 1u);
+            __syncthreads();
+            tile = s_tile;
+        }
+        if (tile >= n_tiles) break;
+        shaft_tile<DEBUG>(tile, spos, sidx, fix, nf, nodes, nodes4, tris, P, out, max_bits, B, &counters[2], dbg, err, st);
+        if (!persistent) break;
     }
     warp_stats_commit(st, counters);
 }
@@ -397,6 +427,9 @@ gm_status accumulate_impl(gm_scene* sc, gm_samples* sm, const gm_fixations* fx, 
         const bool grid = (prm->flags & GM_F_EYE_GRID) && compact && !wide && !occ4 && nf > 0;
         const float4* tree = wide ? sc->nodes4 : sc->nodes;
         const int code = (compact ? 1 : 0) | (wide ? 2 : 0) | (occ4 ? 4 : 0);
+        // the default shape: ray queue, one sample per thread, 256-thread blocks
+        const bool shaft = !grid && (code == 1 || code == 5) &&
+                           !(prm->flags & (GM_F_SPT4 | GM_F_SPT2 | GM_F_BLOCK128 | GM_F_BLOCK512 | GM_F_FIX_L1));
         // persistent grid: every resident block slot once, never more blocks than tiles need
 #define GM_LAUNCH_ACC_F(D, Cm, Wd, Mb, NT, Gr, S_, Fs)                                                           \
     do {                                                                                                          \
@@ -497,7 +530,19 @@ gm_status accumulate_impl(gm_scene* sc, gm_samples* sm, const gm_fixations* fx, 
                 cudaEventRecord(mp->ev[4], s);
                 cudaEventRecord(mp->ev[5], s);
             }
-            if (debug) {
+            if (shaft) {
+                static const int per_sm = [] {
+                    int b = 0;
+                    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_accumulate_shaft<false>, ACC_THREADS, 0);
+                    return b > 0 ? b : 1;
+                }();
+                const uint32_t tiles = gm_div_up(ns, 32);
+                const uint32_t grd = persistent ? std::min<uint32_t>((uint32_t)(ctx->n_sm * per_sm), tiles) : tiles;
+                auto kern = debug ? k_accumulate_shaft<true> : k_accumulate_shaft<false>;
+                kern<<<grd, ACC_THREADS, 0, s>>>(spos, sidx, packed, n_valid, sc->nodes, sc->nodes4, sc->bvh_tris, P,
+                                                 tiles, persistent, mp->values, mp->max_bits, mp->counters,
+                                                 ctx->dev_err, dbg);
+            } else if (debug) {
                 switch (code & 3) {
                     case 0: GM_LAUNCH_ACC(true, false, false, 3); break;
                     case 1: GM_LAUNCH_ACC(true, true, false, 3); break;
@@ -513,8 +558,7 @@ gm_status accumulate_impl(gm_scene* sc, gm_samples* sm, const gm_fixations* fx, 
                 if ((code == 1 || code == 5) && qspt == 1) {
                     if (b128) GM_LAUNCH_ACC_F(false, true, false, 8, 128, false, 1, true);
                     else if (b512) GM_LAUNCH_ACC_F(false, true, false, 2, 512, false, 1, true);
-                    else if (prm->flags & GM_F_FIX_L1) GM_LAUNCH_ACC_F(false, true, false, 4, 256, false, 1, false);
-                    else GM_LAUNCH_ACC_F(false, true, false, 4, 256, false, 1, true);
+                    else GM_LAUNCH_ACC_F(false, true, false, 4, 256, false, 1, false);   // GM_F_FIX_L1
                 } else if ((code == 0 || code == 4) && (prm->flags & GM_F_SPT1)) {
                     // one-sample tiles traced in place: a lane traces its own sample's ray
                     GM_LAUNCH_ACC_F(false, false, false, 4, 256, false, 1, true);
@@ -532,11 +576,7 @@ gm_status accumulate_impl(gm_scene* sc, gm_samples* sm, const gm_fixations* fx, 
                     case 2: GM_LAUNCH_ACC(false, false, true, 3); break;
                     case 3: GM_LAUNCH_ACC(false, true, true, 3); break;
                     case 4: GM_LAUNCH_ACC(false, false, false, 4); break;
-                    case 5:
-                        if (prm->flags & GM_F_SPT1) GM_LAUNCH_ACC_F(false, true, false, 4, 256, false, 1, true);
-                        else if (prm->flags & GM_F_SPT2) GM_LAUNCH_ACC_F(false, true, false, 4, 256, false, 2, true);
-                        else GM_LAUNCH_ACC(false, true, false, 4);
-                        break;
+                    case 5: GM_LAUNCH_ACC(false, true, false, 4); break;
                     case 6: GM_LAUNCH_ACC(false, false, true, 4); break;
                     default: GM_LAUNCH_ACC(false, true, true, 4); break;
                 }

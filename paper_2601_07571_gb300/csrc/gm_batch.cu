@@ -13,7 +13,7 @@
 // batched normalisation. gm_batch_run replays the graph: no
 // host work and one graph launch per call.
 //
-// Autotuning: the candidates are the accumulation variants (per-warp ray queue on/off, binary
+// Autotuning: the candidates are the accumulation variants (shafts; per-warp ray queue on/off, binary
 // or 4-wide tree, 80- or 64-register cap). Each is timed on every bucket's own launch and each
 // bucket keeps its fastest; results are cached per bucket and size (log2 of samples, fixations,
 // triangles) in memory and in the JSON file named by GM_TUNE_CACHE, if set.
@@ -30,7 +30,7 @@
 #include <string>
 #include <vector>
 
-#include "gm_trace.cuh"
+#include "gm_shaft.cuh"
 
 namespace {
 
@@ -39,7 +39,8 @@ struct SessionDev {
     const uint32_t* sidx;
     const float4* fix;        // this session's packed fixations (sorted by window)
     const uint32_t* n_fix;    // number of valid fixations (device)
-    const float4* nodes;
+    const float4* nodes;      // the tree of the bucket's variant (shafts: the binary one)
+    const float4* nodes4;
     const float4* tris;
     float* out;
     unsigned int* max_bits;
@@ -147,6 +148,45 @@ __global__ void __launch_bounds__(ACC_THREADS, MINB) k_accumulate_batch(const Se
     }
 }
 
+// The default: shafts (gm_shaft.cuh), a block per work item (a 32-sample tile of one session).
+__global__ void __launch_bounds__(ACC_THREADS, 4) k_accumulate_batch_shaft(const SessionDev* __restrict__ sess,
+                                                                           const uint2* __restrict__ items,
+                                                                           uint32_t n_items,
+                                                                           unsigned int* __restrict__ work, AccConst C,
+                                                                           int* __restrict__ err) {
+    __shared__ ShaftBlock B;
+    __shared__ uint32_t s_item;
+    const DebugOut dbg{nullptr, nullptr, nullptr, nullptr, nullptr};
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_item = atomicAdd(work, 1u);
+        __syncthreads();
+        const uint32_t it = s_item;
+        if (it >= n_items) break;
+        const uint2 wi = items[it];
+        const SessionDev Sd = sess[wi.x];
+        AccParams P;
+        P.C2 = C.C2;
+        P.K = C.K;
+        P.tmax = C.tmax;
+        P.ns = Sd.ns;
+        P.W = Sd.W;
+        P.nt = Sd.nt;
+        P.dbg_cap = 0;
+        P.tanphi = sqrtf(C.K) * 1.00001f;
+        TileStats st;
+        shaft_tile<false>(wi.y, Sd.spos, Sd.sidx, Sd.fix, *Sd.n_fix, Sd.nodes, Sd.nodes4, Sd.tris, P, Sd.out, Sd.max_bits,
+                          B, nullptr, dbg, err, st);
+        warp_stats_commit(st, Sd.counters);
+    }
+}
+
+int batch_shaft_blocks() {   // resident blocks per SM
+    int b = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_accumulate_batch_shaft, ACC_THREADS, 0);
+    return std::max(b, 1);
+}
+
 __global__ void k_bnormalize(const SessionDev* __restrict__ sess) {
     const SessionDev S = sess[blockIdx.y];
     const uint64_t total = (uint64_t)S.ns * S.W;
@@ -170,14 +210,14 @@ int occupancy_of() {
 }
 
 // Variant codes: bits 0-2 the kernel (ray queue, 4-wide tree, 64-register cap), 8 x the tile index
-// (ray-queue binary tree only: 2 samples per thread with fixations staged in shared memory, or 1,
-// which also takes 64 registers).
+// (ray-queue binary tree only: 2 samples per thread with fixations staged in shared memory; with 1,
+// the rays are traced as shafts).
 void launch_batch(int code, int grid, cudaStream_t s, const SessionDev* sess, const uint2* items, uint32_t n_items,
                   unsigned int* work, AccConst C, int* err) {
 #define GM_B(Cm, Wd, Mb, S_, Fs) \
     k_accumulate_batch<Cm, Wd, Mb, S_, Fs><<<grid, ACC_THREADS, 0, s>>>(sess, items, n_items, work, C, err)
     const int t = code >> 3;
-    if (t == 2) GM_B(true, false, 4, 1, true);
+    if (t == 2) k_accumulate_batch_shaft<<<grid, ACC_THREADS, 0, s>>>(sess, items, n_items, work, C, err);
     else if (t == 1 && (code & 7) == 5) GM_B(true, false, 4, 2, true);
     else if (t == 1) GM_B(true, false, 3, 2, true);
     else switch (code & 7) {
@@ -195,7 +235,7 @@ void launch_batch(int code, int grid, cudaStream_t s, const SessionDev* sess, co
 
 int batch_occupancy(int code) {
     const int t = code >> 3;
-    if (t == 2) return occupancy_of<true, false, 4, 1, true>();
+    if (t == 2) return batch_shaft_blocks();
     if (t == 1) return (code & 7) == 5 ? occupancy_of<true, false, 4, 2, true>() : occupancy_of<true, false, 3, 2, true>();
     switch (code & 7) {
         case 0: return occupancy_of<false, false, 3>();
@@ -326,8 +366,9 @@ static gm_status batch_capture(gm_batch* b, bool concurrent = true) {
     // the session table points at the tree its bucket's variant traverses
     for (uint32_t i = 0; i < b->n; ++i) {
         const gm_scene* sc = b->scenes[i];
-        const int f = b->bflags[bucket_of_tris(sc->n_tris)];
-        b->host_sess[i].nodes = (f & GM_F_WIDE_BVH) && sc->nodes4 ? sc->nodes4 : sc->nodes;
+        const int code = code_of_flags(b->bflags[bucket_of_tris(sc->n_tris)]);
+        b->host_sess[i].nodes = (code & 2) && sc->nodes4 ? sc->nodes4 : sc->nodes;
+        b->host_sess[i].nodes4 = sc->nodes4;
     }
     GM_TRY_CUDA(cudaMemcpy(b->sess, b->host_sess.data(), sizeof(SessionDev) * b->n, cudaMemcpyHostToDevice));
     cudaStream_t cs;
@@ -376,7 +417,7 @@ static gm_status batch_capture(gm_batch* b, bool concurrent = true) {
                 cudaStream_t ks = concurrent ? b->bs[k] : cs;
                 if (i1 > i0) {
                     const int grid = (int)std::min<uint64_t>((uint64_t)b->ctx->n_sm * batch_occupancy(code),
-                                                             gm_div_up(i1 - i0, ACC_THREADS / 32));
+                                                             tk == 2 ? i1 - i0 : gm_div_up(i1 - i0, ACC_THREADS / 32));
                     // external event records: the graph records them when it runs (a plain record in
                     // a capture only orders the work)
                     cudaEventRecordWithFlags(b->bev[k][0], ks, cudaEventRecordExternal);
@@ -538,7 +579,8 @@ extern "C" gm_status gm_batch_create(gm_ctx* ctx, const gm_session_desc* ss, uin
         d.sidx = sm->work_idx;
         d.fix = b->packed + 2 * (size_t)b->fix_off[i];
         d.n_fix = b->n_valid + i;
-        d.nodes = (b->flags & GM_F_WIDE_BVH) && sc->nodes4 ? sc->nodes4 : sc->nodes;
+        d.nodes = sc->nodes;   // the capture points it at the tree of the bucket's variant
+        d.nodes4 = sc->nodes4;
         d.tris = sc->bvh_tris;
         d.out = b->maps[i]->values;
         d.max_bits = b->maps[i]->max_bits;
@@ -565,7 +607,8 @@ extern "C" gm_status gm_batch_create(gm_ctx* ctx, const gm_session_desc* ss, uin
         const uint64_t per_tile = 32ull * BATCH_TILE_SPT[tk] * BATCH_GROUP;
         for (uint32_t i : order) {
             const int k = bucket_of_tris(ss[i].scene->n_tris);
-            const uint32_t tiles = (uint32_t)(gm_div_up(ss[i].samples->n, per_tile) * BATCH_GROUP);
+            const uint32_t tiles = tk == 2 ? gm_div_up(ss[i].samples->n, 32)
+                                           : (uint32_t)(gm_div_up(ss[i].samples->n, per_tile) * BATCH_GROUP);
             for (uint32_t t = 0; t < tiles; ++t) items[tk].push_back(make_uint2(i, t));
             for (int q = k + 1; q <= BATCH_BUCKETS; ++q) b->bucket_begin[tk][q] = (uint32_t)items[tk].size();
         }

@@ -32,8 +32,6 @@
 
 namespace {
 
-// Store internal nodes in depth-first order (see k_dfs_index).
-constexpr bool kDfsLayout = true;
 // Clustering radius of the PLOC builder: 8 neighbours on each side traced the paper scene in
 // 244 ms against 257 ms for 16 (34.2 vs 34.1 nodes per ray; the depth-first layout of the
 // smaller-radius tree caches better), and builds faster.
@@ -248,18 +246,6 @@ __global__ void k_depth(const int* __restrict__ parent_node, const int* __restri
     atomicMax(depth, d);
 }
 
-// Depth of every internal node (root 0); even-depth nodes become 4-wide nodes.
-__global__ void k_node_depth(const int* __restrict__ parent_node, int n_int, int64_t* __restrict__ flag) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_int) return;
-    int d = 0, p = i;
-    while (p > 0 && d < 4096) {
-        p = parent_node[p];
-        ++d;
-    }
-    flag[i] = (d & 1) == 0 ? 1 : 0;
-}
-
 constexpr int LINK_EMPTY = (int)0x80000000;
 
 __device__ __forceinline__ void child_box(const float* node, int side, float lo[3], float hi[3]) {
@@ -298,15 +284,11 @@ __global__ void k_collapse4(const float4* __restrict__ nodes, int n_int, const i
         link[m] = LINK_EMPTY;
     }
     float4* o = nodes4 + 8 * (size_t)j;
-    o[0] = make_float4(lo[0][0], lo[1][0], lo[2][0], lo[3][0]);
-    o[1] = make_float4(hi[0][0], hi[1][0], hi[2][0], hi[3][0]);
-    o[2] = make_float4(lo[0][1], lo[1][1], lo[2][1], lo[3][1]);
-    o[3] = make_float4(hi[0][1], hi[1][1], hi[2][1], hi[3][1]);
-    o[4] = make_float4(lo[0][2], lo[1][2], lo[2][2], lo[3][2]);
-    o[5] = make_float4(hi[0][2], hi[1][2], hi[2][2], hi[3][2]);
-    o[6] = make_float4(__int_as_float(link[0]), __int_as_float(link[1]), __int_as_float(link[2]),
-                       __int_as_float(link[3]));
-    o[7] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        o[2 * k] = make_float4(lo[k][0], lo[k][1], lo[k][2], __int_as_float(link[k]));
+        o[2 * k + 1] = make_float4(hi[k][0], hi[k][1], hi[k][2], 0.f);
+    }
 }
 
 // ---- PLOC: parallel locally-ordered clustering (Meister & Bittner, TVCG 2018) ----------------
@@ -448,8 +430,10 @@ __global__ void k_leaf_counts(const int* __restrict__ parent_leaf, const int* __
     }
 }
 
+// even[index] = 1 where the node's depth is even (root 0): those become 4-wide nodes.
 __global__ void k_dfs_index(const float4* __restrict__ nodes, const int* __restrict__ parent_node,
-                            const unsigned int* __restrict__ leaves, int n_int, int* __restrict__ dfs) {
+                            const unsigned int* __restrict__ leaves, int n_int, int* __restrict__ dfs,
+                            int64_t* __restrict__ even) {
     int v = blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= n_int) return;
     int idx = 0, u = v, guard = 0;
@@ -462,6 +446,7 @@ __global__ void k_dfs_index(const float4* __restrict__ nodes, const int* __restr
         u = p;
     }
     dfs[v] = idx;
+    even[idx] = (guard & 1) == 0 ? 1 : 0;
 }
 
 __global__ void k_dfs_remap(const float4* __restrict__ nodes, const int* __restrict__ dfs, int n_int,
@@ -796,43 +781,38 @@ static gm_status build_scene(gm_ctx* ctx, const gm_mesh_desc* meshes, uint32_t n
         return fail(gm_set_error(GM_ERR_UNSUPPORTED, "gm_build_scene: BVH deeper than 64 levels (" +
                                                          std::to_string(sc->depth) + ")"));
     if (nt > 1) {
-        const uint32_t n_int = nt - 1;
-        int64_t* incl = nullptr;
-        TMP_ALLOC(incl, sizeof(int64_t) * n_int);
-        k_node_depth<<<gm_div_up(n_int, 256), 256, 0, s>>>(parent_node_keep, (int)n_int, incl);
-        launches = 1;
-        if ((st = gm_inclusive_scan_i64(incl, n_int, s, &launches)) != GM_OK) return fail(st);
-        int64_t n4 = 0;
-        if ((e = cudaMemcpyAsync(&n4, incl + (n_int - 1), sizeof(int64_t), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
-            (e = cudaStreamSynchronize(s)) != cudaSuccess)
-            return fail(gm_cuda_error(e, "gm_build_scene (4-wide count)"));
-        sc->n4 = (uint32_t)n4;
-        SC_ALLOC(sc->nodes4, sizeof(float4) * 8 * (size_t)sc->n4);
-        k_collapse4<<<gm_div_up(n_int, 256), 256, 0, s>>>(sc->nodes, (int)n_int, incl, sc->nodes4);
-        ++launches;
-        ctx->launches += launches;
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return fail(gm_cuda_error(e, "gm_build_scene collapse"));
-    }
-    if (kDfsLayout && nt > 2) {
         const int n_int = (int)nt - 1;
         unsigned int* leaves = nullptr;
         int* dfs = nullptr;
         unsigned int* arrived = nullptr;
         float4* reordered = nullptr;
+        int64_t* incl = nullptr;
         TMP_ALLOC(leaves, sizeof(unsigned int) * n_int);
         TMP_ALLOC(dfs, sizeof(int) * n_int);
         TMP_ALLOC(arrived, sizeof(unsigned int) * n_int);
+        if (dynamic) {
+            SC_ALLOC(sc->incl4, sizeof(int64_t) * n_int);
+            incl = sc->incl4;
+        } else {
+            TMP_ALLOC(incl, sizeof(int64_t) * n_int);
+        }
         GM_TRY_CUDA(cudaMemsetAsync(leaves, 0, sizeof(unsigned int) * n_int, s));
         GM_TRY_CUDA(cudaMemsetAsync(arrived, 0, sizeof(unsigned int) * n_int, s));
         if ((st = gm_alloc((void**)&reordered, sizeof(float4) * 4 * (size_t)n_int, s)) != GM_OK) return fail(st);
         k_leaf_counts<<<gm_div_up(nt, 256), 256, 0, s>>>(parent_leaf, parent_node_keep, sc->nodes, (int)nt, leaves,
                                                          arrived);
-        k_dfs_index<<<gm_div_up(n_int, 256), 256, 0, s>>>(sc->nodes, parent_node_keep, leaves, n_int, dfs);
+        k_dfs_index<<<gm_div_up(n_int, 256), 256, 0, s>>>(sc->nodes, parent_node_keep, leaves, n_int, dfs, incl);
         k_dfs_remap<<<gm_div_up(n_int, 256), 256, 0, s>>>(sc->nodes, dfs, n_int, reordered);
-        ctx->launches += 3;
+        launches = 3;
         cudaFreeAsync(sc->nodes, s);
         sc->nodes = reordered;
+        // the 4-wide nodes follow the depth-first order. Every even-depth node but the root is a child of
+        // an odd-depth one, so at most (2 n_int + 1) / 3 of the nodes are of even depth.
+        if ((st = gm_inclusive_scan_i64(incl, (uint32_t)n_int, s, &launches)) != GM_OK) return fail(st);
+        SC_ALLOC(sc->nodes4, sizeof(float4) * 8 * ((2 * (size_t)n_int + 1) / 3));
+        k_collapse4<<<gm_div_up(n_int, 256), 256, 0, s>>>(sc->nodes, n_int, incl, sc->nodes4);
+        ++launches;
+        ctx->launches += launches;
         e = cudaGetLastError();
         if (e != cudaSuccess) return fail(gm_cuda_error(e, "gm_build_scene layout"));
     }
@@ -919,6 +899,10 @@ extern "C" gm_status gm_scene_pose(gm_scene* sc, const double* transforms, gm_st
     k_refit<<<gm_div_up(nt, 256), 256, 0, s>>>(sc->tri_canon, order, (int)nt, sc->nodes, parent_node, parent_leaf,
                                                 flags, bounds, sc->bvh_tris);
     ++launches;
+    if (nt > 1) {   // the 4-wide nodes take the new boxes
+        k_collapse4<<<gm_div_up(nt - 1, 256), 256, 0, s>>>(sc->nodes, (int)(nt - 1), sc->incl4, sc->nodes4);
+        ++launches;
+    }
     unsigned int hb[12] = {0};
     if ((e = cudaGetLastError()) != cudaSuccess ||
         (e = cudaMemcpyAsync(hb, bounds, sizeof(hb), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
@@ -936,12 +920,6 @@ extern "C" gm_status gm_scene_pose(gm_scene* sc, const double* transforms, gm_st
         sc->box_hi[k] = dec(hb[9 + k]);
     }
     sc->mesh_inv_ok = inv_ok;
-    // the 4-wide collapse holds the old boxes: drop it (the binary tree serves every variant)
-    if (sc->nodes4) {
-        cudaFreeAsync(sc->nodes4, s);
-        sc->nodes4 = nullptr;
-        sc->n4 = 0;
-    }
     for (int k = 0; k < 3; ++k)
         if (!std::isfinite(sc->box_lo[k]) || !std::isfinite(sc->box_hi[k]))
             return done(gm_set_error(GM_ERR_INVALID_ARG, "gm_scene_pose: non-finite vertex"));
@@ -995,6 +973,7 @@ extern "C" void gm_scene_free(gm_scene* sc) {
     cudaFree(sc->mesh_inv);
     cudaFree(sc->nodes);
     cudaFree(sc->nodes4);
+    cudaFree(sc->incl4);
     cudaFree(sc->bvh_tris);
     cudaFree(sc->tri_local);
     delete sc;

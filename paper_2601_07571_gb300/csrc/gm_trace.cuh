@@ -118,25 +118,31 @@ __device__ __forceinline__ float slab(const Ray& R, float lx, float ly, float lz
 // Woop, Benthin, Wald, "Watertight ray/triangle intersection", JCGT 2(1), 2013. Edge functions
 // are evaluated without fused multiply-add so that a shared edge gives exactly opposite values
 // in its two triangles (no ray slips between them).
-__device__ __forceinline__ bool tri_hit(const Ray& R, float4 a, float4 b, float4 c) {
-    float3 A = make_float3(a.x - R.o.x, a.y - R.o.y, a.z - R.o.z);
-    float3 B = make_float3(b.x - R.o.x, b.y - R.o.y, b.z - R.o.z);
-    float3 C = make_float3(c.x - R.o.x, c.y - R.o.y, c.z - R.o.z);
-    float Akz = comp(A, R.kz), Bkz = comp(B, R.kz), Ckz = comp(C, R.kz);
-    float Ax = __fsub_rn(comp(A, R.kx), __fmul_rn(R.Sx, Akz));
-    float Ay = __fsub_rn(comp(A, R.ky), __fmul_rn(R.Sy, Akz));
-    float Bx = __fsub_rn(comp(B, R.kx), __fmul_rn(R.Sx, Bkz));
-    float By = __fsub_rn(comp(B, R.ky), __fmul_rn(R.Sy, Bkz));
-    float Cx = __fsub_rn(comp(C, R.kx), __fmul_rn(R.Sx, Ckz));
-    float Cy = __fsub_rn(comp(C, R.ky), __fmul_rn(R.Sy, Ckz));
+// (Akx, Aky, Akz) and so on: the vertices relative to the ray's origin in the ray's axes.
+__device__ __forceinline__ bool tri_core(float Akx, float Aky, float Akz, float Bkx, float Bky, float Bkz, float Ckx,
+                                         float Cky, float Ckz, float Sx, float Sy, float Sz, float tmax) {
+    float Ax = __fsub_rn(Akx, __fmul_rn(Sx, Akz));
+    float Ay = __fsub_rn(Aky, __fmul_rn(Sy, Akz));
+    float Bx = __fsub_rn(Bkx, __fmul_rn(Sx, Bkz));
+    float By = __fsub_rn(Bky, __fmul_rn(Sy, Bkz));
+    float Cx = __fsub_rn(Ckx, __fmul_rn(Sx, Ckz));
+    float Cy = __fsub_rn(Cky, __fmul_rn(Sy, Ckz));
     float U = __fsub_rn(__fmul_rn(Cx, By), __fmul_rn(Cy, Bx));
     float V = __fsub_rn(__fmul_rn(Ax, Cy), __fmul_rn(Ay, Cx));
     float W = __fsub_rn(__fmul_rn(Bx, Ay), __fmul_rn(By, Ax));
     if ((U < 0.f || V < 0.f || W < 0.f) && (U > 0.f || V > 0.f || W > 0.f)) return false;
     float det = U + V + W;
     if (det == 0.f) return false;
-    float T = U * (R.Sz * Akz) + V * (R.Sz * Bkz) + W * (R.Sz * Ckz);
-    return det > 0.f ? (T > 0.f && T < R.tmax * det) : (T < 0.f && T > R.tmax * det);
+    float T = U * (Sz * Akz) + V * (Sz * Bkz) + W * (Sz * Ckz);
+    return det > 0.f ? (T > 0.f && T < tmax * det) : (T < 0.f && T > tmax * det);
+}
+
+__device__ __forceinline__ bool tri_hit(const Ray& R, float4 a, float4 b, float4 c) {
+    float3 A = make_float3(a.x - R.o.x, a.y - R.o.y, a.z - R.o.z);
+    float3 B = make_float3(b.x - R.o.x, b.y - R.o.y, b.z - R.o.z);
+    float3 C = make_float3(c.x - R.o.x, c.y - R.o.y, c.z - R.o.z);
+    return tri_core(comp(A, R.kx), comp(A, R.ky), comp(A, R.kz), comp(B, R.kx), comp(B, R.ky), comp(B, R.kz),
+                    comp(C, R.kx), comp(C, R.ky), comp(C, R.kz), R.Sx, R.Sy, R.Sz, R.tmax);
 }
 
 __device__ __forceinline__ bool leaf_hit(const Ray& R, const float4* __restrict__ tris, int slot, uint32_t own,
@@ -224,13 +230,13 @@ __device__ bool occluded4(const Ray& R, uint32_t own, const float4* __restrict__
     for (;;) {
         ++n_node;
         const float4* N = nodes4 + 8 * node;
-        const float4 lx = __ldg(N + 0), hx = __ldg(N + 1), ly = __ldg(N + 2), hy = __ldg(N + 3);
-        const float4 lz = __ldg(N + 4), hz = __ldg(N + 5), L = __ldg(N + 6);
-        float t0 = slab(R, lx.x, ly.x, lz.x, hx.x, hy.x, hz.x);
-        float t1 = slab(R, lx.y, ly.y, lz.y, hx.y, hy.y, hz.y);
-        float t2 = slab(R, lx.z, ly.z, lz.z, hx.z, hy.z, hz.z);
-        float t3 = slab(R, lx.w, ly.w, lz.w, hx.w, hy.w, hz.w);
-        int c0 = __float_as_int(L.x), c1 = __float_as_int(L.y), c2 = __float_as_int(L.z), c3 = __float_as_int(L.w);
+        const float4 l0 = __ldg(N + 0), h0 = __ldg(N + 1), l1 = __ldg(N + 2), h1 = __ldg(N + 3);
+        const float4 l2 = __ldg(N + 4), h2 = __ldg(N + 5), l3 = __ldg(N + 6), h3 = __ldg(N + 7);
+        float t0 = slab(R, l0.x, l0.y, l0.z, h0.x, h0.y, h0.z);
+        float t1 = slab(R, l1.x, l1.y, l1.z, h1.x, h1.y, h1.z);
+        float t2 = slab(R, l2.x, l2.y, l2.z, h2.x, h2.y, h2.z);
+        float t3 = slab(R, l3.x, l3.y, l3.z, h3.x, h3.y, h3.z);
+        int c0 = __float_as_int(l0.w), c1 = __float_as_int(l1.w), c2 = __float_as_int(l2.w), c3 = __float_as_int(l3.w);
         if (t0 < INFINITY && c0 < 0) { if (c0 != LINK_EMPTY && leaf_hit(R, tris, ~c0, own, n_tri)) { hit_slot = ~c0; return true; } t0 = INFINITY; }
         if (t1 < INFINITY && c1 < 0) { if (c1 != LINK_EMPTY && leaf_hit(R, tris, ~c1, own, n_tri)) { hit_slot = ~c1; return true; } t1 = INFINITY; }
         if (t2 < INFINITY && c2 < 0) { if (c2 != LINK_EMPTY && leaf_hit(R, tris, ~c2, own, n_tri)) { hit_slot = ~c2; return true; } t2 = INFINITY; }

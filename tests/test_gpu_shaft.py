@@ -1,0 +1,85 @@
+"""The shaft walk (the default accumulation kernel) against the per-ray walk (GM_F_FIX_L1) on the same
+scenes: both decide every ray with the same arithmetic and add the weights in the same order, so the
+maps are equal bit for bit. Sizes at the edges of a warp tile, of a fill step (512 fixations) and of a
+batch; trees of one and two triangles; triangles far smaller than the sample spacing (a shaft over its
+budget); an eye close to the surface, whose rays differ in their dominant axis and cross the planes
+through the eye."""
+import math
+
+import numpy as np
+import pytest
+
+from synth import meshes as M
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_2601_07571_gb300 import build
+    build.build()
+    import paper_2601_07571_gb300 as G
+    ctx = G.gm_create(0)
+    yield G, ctx
+    G.gm_destroy(ctx)
+
+
+def _scene(kind):
+    """(vertices, indices) of one mesh."""
+    tri = np.array([[0.0, 0.0, 1.0], [0.6, 0.0, 1.0], [0.0, 0.6, 1.0]], np.float32)
+    if kind == "one":
+        return tri, np.array([[0, 1, 2]], np.uint32)
+    if kind == "two":
+        return np.concatenate([tri, tri + np.float32([0.1, 0.1, -0.3])]), np.array([[0, 1, 2], [3, 4, 5]], np.uint32)
+    if kind == "fine":      # 80k triangles of about 1 mm on a 6 cm sphere, before a coarse one
+        v, f = M.uv_sphere(12, 24, 0.5)
+        return M.merge([M.uv_sphere(142, 284, 0.06, 0.05, 30.0, seed=3), (M.translate(v, (0.0, 0.0, 0.9)), f)])
+    return M.uv_sphere(40, 80, 1.0, 0.1, 4.0, seed=5)
+
+
+def _points(v, f, n, rng):
+    t = v[f.astype(np.int64)].astype(np.float64)
+    tri = rng.integers(0, len(f), n)
+    s, u = np.sqrt(rng.random((n, 1))), rng.random((n, 1))
+    p = (1 - s) * t[tri, 0] + s * (1 - u) * t[tri, 1] + s * u * t[tri, 2]
+    return np.ascontiguousarray(p, np.float32), tri.astype(np.uint32)
+
+
+@pytest.mark.parametrize("kind,n,nf,theta,near,windows", [
+    ("one", 1, 3, 4.0, False, 1), ("two", 33, 40, 4.0, False, 1),
+    ("sphere", 31, 511, 2.0, False, 1), ("sphere", 32, 512, 2.0, False, 3), ("sphere", 1000, 1300, 6.0, False, 5),
+    ("fine", 2048, 600, 1.0, False, 1), ("sphere", 3000, 200, 15.0, True, 1), ("sphere", 257, 0, 1.0, False, 2)])
+def test_shaft_walk_equals_per_ray_walk(env, kind, n, nf, theta, near, windows):
+    G, ctx = env
+    rng = np.random.default_rng(n + nf)
+    v, f = _scene(kind)
+    scene = G.gm_build_scene(ctx, [(v, f, np.eye(4), 0)])
+    xyz, tri = _points(v, f, n, rng)
+    samples = G.gm_samples_from_points(scene, xyz, tri)
+    at = xyz[rng.integers(0, n, nf)].astype(np.float64)
+    if near:      # a few centimetres off the surface, looking along it or at it
+        eye = at * (1.0 + 0.03 * rng.random((nf, 1)))
+        gaze = rng.normal(size=(nf, 3))
+    else:
+        eye = rng.normal(size=(nf, 3))
+        eye *= 2.5 / np.maximum(np.linalg.norm(eye, axis=1, keepdims=True), 1e-9)
+        gaze = at - eye
+    fix = [np.ascontiguousarray(eye, np.float32), np.ascontiguousarray(gaze, np.float32),
+           rng.uniform(0.1, 0.6, nf).astype(np.float32), np.sort(rng.uniform(0.0, windows, nf))]
+    out = []
+    for flags in (0, G.GM_F_FIX_L1):
+        kw = dict(t_begin=0.0, t_end=float(windows), window_s=1.0) if windows > 1 else {}
+        m = G.gm_accumulate_fixations(scene, samples, *fix, G.make_params(math.radians(theta), normalize=False, flags=flags, **kw))
+        W, ns, st, _ = G.gm_map_info(m)
+        maps = np.empty((W, ns), np.float32)
+        top = [G.gm_map_copy(m, w, maps[w]) for w in range(W)]
+        G.gm_map_free(m)
+        out.append((maps, top, {k: st[k] for k in ("pairs", "in_cone", "visible", "pairs_tested")}))
+    G.gm_samples_free(samples)
+    G.gm_scene_free(scene)
+    assert W == windows and out[0][2] == out[1][2] and out[0][1] == out[1][1]
+    assert np.array_equal(out[0][0], out[1][0])
+    if nf > 10:
+        assert out[0][2]["visible"] > 0
