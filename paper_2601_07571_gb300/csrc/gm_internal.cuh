@@ -135,4 +135,16 @@ __device__ __forceinline__ unsigned int gm_lanemask_lt() {
     return m;
 }
 
+// Minimum and maximum over the warp (all lanes); NaNs are ignored unless every lane holds one.
+__device__ __forceinline__ float redux_min(float v) {
+    float r;
+    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float redux_max(float v) {
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+
 static inline uint32_t gm_div_up(uint64_t a, uint64_t b) { return (uint32_t)((a + b - 1) / b); }

@@ -29,6 +29,7 @@
 #include <vector>
 
 #include "gm_internal.cuh"
+#include "gm_scan.cuh"
 
 namespace {
 
@@ -69,6 +70,32 @@ __global__ void k_bounds_init(unsigned int* b) {
     if (i < 12) b[i] = ((i / 3) % 2 == 0) ? 0xffffffffu : 0u;
 }
 
+// Fold the block's centroid (0..2) and vertex (3..5) boxes into the scene's: one atomic per block and
+// bound (one per warp and bound, all on the same 12 words, took 150 of k_gather's 197 us at 800k
+// triangles). All 256 threads call it.
+__device__ __forceinline__ void fold_bounds(const float lo[6], const float hi[6], unsigned int* __restrict__ bounds) {
+    __shared__ unsigned int slo[6], shi[6];
+    if (threadIdx.x < 6) {
+        slo[threadIdx.x] = 0xffffffffu;
+        shi[threadIdx.x] = 0u;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        const unsigned int l = f2ord(redux_min(lo[c])), h = f2ord(redux_max(hi[c]));
+        if ((threadIdx.x & 31) == 0) {
+            atomicMin(&slo[c], l);
+            atomicMax(&shi[c], h);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        const int at = threadIdx.x < 3 ? threadIdx.x : threadIdx.x + 3;
+        atomicMin(&bounds[at], slo[threadIdx.x]);
+        atomicMax(&bounds[at + 3], shi[threadIdx.x]);
+    }
+}
+
 __global__ void k_gather(const float* __restrict__ wv, const uint32_t* __restrict__ idx, uint32_t nt,
                          uint32_t nv, uint32_t tri_base, uint32_t mesh, float4* __restrict__ tri_canon,
                          uint32_t* __restrict__ tri_mesh, unsigned int* __restrict__ bounds,
@@ -102,22 +129,7 @@ __global__ void k_gather(const float* __restrict__ wv, const uint32_t* __restric
             hi[3 + a] = fmaxf(fmaxf(vf[a], vf[3 + a]), vf[6 + a]);
         }
     }
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-        for (int o = 16; o > 0; o >>= 1) {
-            lo[c] = fminf(lo[c], __shfl_xor_sync(0xffffffffu, lo[c], o));
-            hi[c] = fmaxf(hi[c], __shfl_xor_sync(0xffffffffu, hi[c], o));
-        }
-    }
-    if ((threadIdx.x & 31) == 0 && blockIdx.x * blockDim.x + (threadIdx.x & ~31u) < nt) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            atomicMin(&bounds[a], f2ord(lo[a]));
-            atomicMax(&bounds[3 + a], f2ord(hi[a]));
-            atomicMin(&bounds[6 + a], f2ord(lo[3 + a]));
-            atomicMax(&bounds[9 + a], f2ord(hi[3 + a]));
-        }
-    }
+    fold_bounds(lo, hi, bounds);
 }
 
 __device__ __forceinline__ uint64_t spread3_21(uint32_t v) {
@@ -233,19 +245,6 @@ __global__ void k_refit(const float4* __restrict__ tri_canon, const uint32_t* __
     }
 }
 
-__global__ void k_depth(const int* __restrict__ parent_node, const int* __restrict__ parent_leaf, int n,
-                        unsigned int* __restrict__ depth) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || n < 2) return;
-    unsigned int d = 1;
-    int p = parent_leaf[i];
-    while (p > 0 && d < 4096u) {
-        p = parent_node[p];
-        ++d;
-    }
-    atomicMax(depth, d);
-}
-
 constexpr int LINK_EMPTY = (int)0x80000000;
 
 __device__ __forceinline__ void child_box(const float* node, int side, float lo[3], float hi[3]) {
@@ -295,11 +294,19 @@ __global__ void k_collapse4(const float4* __restrict__ nodes, int n_int, const i
 // Clusters start as the Morton-ordered leaves. Each round, every cluster finds the cluster within
 // +-R positions whose union box has the smallest surface area; mutual nearest neighbours merge
 // into a new node (the lower position keeps the merged cluster), and the array is compacted.
-// Node indices are handed out downwards from n - 2, so the last merge -- the root -- is node 0.
-
-struct Box6 {
-    float lo[3], hi[3];
-};
+// Node indices are handed out downwards from n - 2, in position order, so the last merge -- the root --
+// is node 0. A cluster is two float4: (lo, id) and (hi, leaves below).
+//
+// A round is two kernels: k_ploc_pair (neighbours, with a halo so that a block decides its own pairs, and
+// the number of clusters that leave each block) and k_ploc_apply (nodes and compaction; a block sums the
+// counts of the blocks before it). The cluster count stays on the device: the host launches PLOC_BATCH
+// rounds at a time with the grid of the last count it read, rounds that find PLOC_TAIL clusters or
+// fewer do nothing, and one block runs all remaining rounds in shared memory. At 800k triangles 100
+// rounds of six kernels and a host read each took 3.4 ms of a 4.9 ms build; these take 0.7 ms.
+constexpr int PLOC_T = 256;
+constexpr int PLOC_P = 512;        // positions per block
+constexpr int PLOC_TAIL = 1024;
+constexpr int PLOC_BATCH = 12;
 
 __device__ __forceinline__ float union_area(const float4 al, const float4 ah, const float4 bl, const float4 bh) {
     const float dx = fmaxf(ah.x, bh.x) - fminf(al.x, bl.x);
@@ -309,10 +316,11 @@ __device__ __forceinline__ float union_area(const float4 al, const float4 ah, co
 }
 
 __global__ void k_ploc_init(const float4* __restrict__ tri_canon, const uint32_t* __restrict__ order, int n,
-                            const unsigned int* __restrict__ bounds, int* __restrict__ cid, float4* __restrict__ blo,
-                            float4* __restrict__ bhi, float4* __restrict__ bvh_tris) {
+                            const unsigned int* __restrict__ bounds, float4* __restrict__ blo,
+                            float4* __restrict__ bhi, float4* __restrict__ bvh_tris, int* __restrict__ m_of) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
+    if (i == 0) m_of[0] = n;
     uint32_t t = order[i];
     float4 a = tri_canon[3 * t], b = tri_canon[3 * t + 1], c = tri_canon[3 * t + 2];
     bvh_tris[3 * i + 0] = make_float4(a.x, a.y, a.z, __uint_as_float(t));
@@ -323,83 +331,213 @@ __global__ void k_ploc_init(const float4* __restrict__ tri_canon, const uint32_t
     for (int k = 0; k < 3; ++k) big = fmaxf(big, fmaxf(fabsf(ord2f(bounds[6 + k])), fabsf(ord2f(bounds[9 + k]))));
     const float margin = big * (1.0f / 524288.0f) + 1e-30f;
     blo[i] = make_float4(fminf(fminf(a.x, b.x), c.x) - margin, fminf(fminf(a.y, b.y), c.y) - margin,
-                         fminf(fminf(a.z, b.z), c.z) - margin, 0.f);
+                         fminf(fminf(a.z, b.z), c.z) - margin, __int_as_float(~i));
     bhi[i] = make_float4(fmaxf(fmaxf(a.x, b.x), c.x) + margin, fmaxf(fmaxf(a.y, b.y), c.y) + margin,
-                         fmaxf(fmaxf(a.z, b.z), c.z) + margin, 0.f);
-    cid[i] = ~i;
+                         fmaxf(fmaxf(a.z, b.z), c.z) + margin, __int_as_float(1));
 }
 
+// Nearest neighbour of cluster i (shared-memory position p) among positions i - R .. i + R of [0, m); the
+// lowest position wins a tie. -1: none.
 template <int R>
-__global__ void __launch_bounds__(256) k_ploc_nn(const float4* __restrict__ blo, const float4* __restrict__ bhi,
-                                                 int m, int* __restrict__ nn) {
-    __shared__ float4 sl[256 + 2 * R], sh[256 + 2 * R];
-    const int b0 = blockIdx.x * 256;
-    for (int k = threadIdx.x; k < 256 + 2 * R; k += 256) {
-        const int g = b0 - R + k;
+__device__ __forceinline__ int ploc_nearest(const float4* sl, const float4* sh, int p, int i, int m) {
+    const float4 al = sl[p], ah = sh[p];
+    float best = INFINITY;
+    int bj = -1;
+#pragma unroll 4
+    for (int d = -R; d <= R; ++d) {
+        const int j = i + d;
+        if (d == 0 || j < 0 || j >= m) continue;
+        const float a = union_area(al, ah, sl[p + d], sh[p + d]);
+        if (a < best) {
+            best = a;
+            bj = j;
+        }
+    }
+    return bj;
+}
+
+// Node k from the clusters at positions i < j; returns the merged cluster in (al, ah).
+__device__ __forceinline__ void ploc_node(int k, float4& al, float4& ah, const float4 bl, const float4 bh,
+                                          float4* __restrict__ nodes, int* __restrict__ parent_node,
+                                          int* __restrict__ parent_leaf, unsigned int* __restrict__ leaves) {
+    const int ci = __float_as_int(al.w), cj = __float_as_int(bl.w);
+    const int n = __float_as_int(ah.w) + __float_as_int(bh.w);
+    nodes[4 * (size_t)k + 0] = make_float4(al.x, al.y, al.z, ah.x);
+    nodes[4 * (size_t)k + 1] = make_float4(ah.y, ah.z, bl.x, bl.y);
+    nodes[4 * (size_t)k + 2] = make_float4(bl.z, bh.x, bh.y, bh.z);
+    nodes[4 * (size_t)k + 3] = make_float4(al.w, bl.w, 0.f, 0.f);
+    if (ci < 0) parent_leaf[~ci] = k; else parent_node[ci] = k;
+    if (cj < 0) parent_leaf[~cj] = k; else parent_node[cj] = k;
+    leaves[k] = (unsigned int)n;
+    al = make_float4(fminf(al.x, bl.x), fminf(al.y, bl.y), fminf(al.z, bl.z), __int_as_float(k));
+    ah = make_float4(fmaxf(ah.x, bh.x), fmaxf(ah.y, bh.y), fmaxf(ah.z, bh.z), __int_as_float(n));
+}
+
+// pair[i]: the position that i merges with, or -1; gone[block]: clusters of the block that leave (the
+// upper ones of their pairs).
+template <int R>
+__global__ void __launch_bounds__(PLOC_T) k_ploc_pair(const int* __restrict__ m_of, const float4* __restrict__ blo,
+                                                      const float4* __restrict__ bhi, int* __restrict__ pair,
+                                                      int* __restrict__ gone) {
+    __shared__ float4 sl[PLOC_P + 4 * R], sh[PLOC_P + 4 * R];
+    __shared__ int snn[PLOC_P + 2 * R];
+    __shared__ int count;
+    const int m = *m_of, b0 = blockIdx.x * PLOC_P;
+    if (m <= PLOC_TAIL || b0 >= m) return;
+    if (threadIdx.x == 0) count = 0;
+    for (int k = threadIdx.x; k < PLOC_P + 4 * R; k += PLOC_T) {
+        const int g = b0 - 2 * R + k;
         if (g >= 0 && g < m) {
             sl[k] = blo[g];
             sh[k] = bhi[g];
         }
     }
     __syncthreads();
-    const int i = b0 + threadIdx.x;
-    if (i >= m) return;
-    const float4 al = sl[threadIdx.x + R], ah = sh[threadIdx.x + R];
-    float best = INFINITY;
-    int bj = -1;
-    for (int d = -R; d <= R; ++d) {
-        const int j = i + d;
-        if (d == 0 || j < 0 || j >= m) continue;
-        const float a = union_area(al, ah, sl[threadIdx.x + R + d], sh[threadIdx.x + R + d]);
-        if (a < best || (a == best && j < bj)) {
-            best = a;
-            bj = j;
+    for (int q = threadIdx.x; q < PLOC_P + 2 * R; q += PLOC_T) {
+        const int i = b0 - R + q;
+        snn[q] = i >= 0 && i < m ? ploc_nearest<R>(sl, sh, q + R, i, m) : -1;
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < PLOC_P; q += PLOC_T) {   // whole warps
+        const int i = b0 + q;
+        int p = -1;
+        if (i < m) {
+            const int j = snn[q + R];
+            if (j >= 0 && snn[j - b0 + R] == i) p = j;
+            pair[i] = p;
         }
+        const unsigned up = __ballot_sync(0xffffffffu, p >= 0 && p < i);
+        if ((threadIdx.x & 31) == 0 && up) atomicAdd(&count, __popc(up));
     }
-    nn[i] = bj;
+    __syncthreads();
+    if (threadIdx.x == 0) gone[blockIdx.x] = count;
 }
 
-__global__ void k_ploc_merge(int m, const int* __restrict__ nn, int* __restrict__ cid, float4* __restrict__ blo,
-                             float4* __restrict__ bhi, int64_t* __restrict__ keep, int* __restrict__ counter,
-                             float4* __restrict__ nodes, int* __restrict__ parent_node, int* __restrict__ parent_leaf) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= m) return;
-    const int j = nn[i];
-    const bool mutual = j >= 0 && nn[j] == i;
-    if (!mutual) {
-        keep[i] = 1;
+__global__ void __launch_bounds__(PLOC_T) k_ploc_apply(const int* __restrict__ m_of, int* __restrict__ m_next,
+                                                       const float4* __restrict__ blo, const float4* __restrict__ bhi,
+                                                       const int* __restrict__ pair, const int* __restrict__ gone,
+                                                       float4* __restrict__ blo2, float4* __restrict__ bhi2,
+                                                       float4* __restrict__ nodes, int* __restrict__ parent_node,
+                                                       int* __restrict__ parent_leaf, unsigned int* __restrict__ leaves) {
+    const int m = *m_of, b0 = blockIdx.x * PLOC_P;
+    if (m <= PLOC_TAIL) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) *m_next = m;
         return;
     }
-    if (i > j) {   // the lower position builds the node and keeps the merged cluster
-        keep[i] = 0;
-        return;
+    if (b0 >= m) return;
+    constexpr int PER = PLOC_P / PLOC_T;
+    int s = 0, p[PER];
+    for (int b = threadIdx.x; b < (int)blockIdx.x; b += PLOC_T) s += gone[b];
+    int mine = 0;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const int i = b0 + threadIdx.x * PER + k;
+        p[k] = i < m ? pair[i] : -1;
+        mine += p[k] >= 0 && p[k] < i;
     }
-    const int k = atomicSub(counter, 1) - 1;
-    const float4 al = blo[i], ah = bhi[i], bl = blo[j], bh = bhi[j];
-    const int ci = cid[i], cj = cid[j];
-    float* node = reinterpret_cast<float*>(nodes + 4 * k);
-    node[0] = al.x; node[1] = al.y; node[2] = al.z; node[3] = ah.x; node[4] = ah.y; node[5] = ah.z;
-    node[6] = bl.x; node[7] = bl.y; node[8] = bl.z; node[9] = bh.x; node[10] = bh.y; node[11] = bh.z;
-    nodes[4 * k + 3] = make_float4(__int_as_float(ci), __int_as_float(cj), 0.f, 0.f);
-    if (ci < 0) parent_leaf[~ci] = k; else parent_node[ci] = k;
-    if (cj < 0) parent_leaf[~cj] = k; else parent_node[cj] = k;
-    // position j is only read by its own thread (which returns above), so i may be rewritten here
-    cid[i] = k;
-    blo[i] = make_float4(fminf(al.x, bl.x), fminf(al.y, bl.y), fminf(al.z, bl.z), 0.f);
-    bhi[i] = make_float4(fmaxf(ah.x, bh.x), fmaxf(ah.y, bh.y), fmaxf(ah.z, bh.z), 0.f);
-    keep[i] = 1;
+    int before, in_block;
+    block_excl_scan<int, PLOC_T>(s, &before);
+    int r = before + block_excl_scan<int, PLOC_T>(mine, &in_block);   // clusters gone before this thread's first
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const int i = b0 + threadIdx.x * PER + k;
+        if (i >= m) break;
+        const bool up = p[k] >= 0 && p[k] < i;
+        if (p[k] < 0) {
+            blo2[i - r] = blo[i];
+            bhi2[i - r] = bhi[i];
+        } else if (up) {
+            int between = 0;   // gone in [p, i)
+            for (int y = p[k]; y < i; ++y) {
+                const int py = pair[y];
+                between += py >= 0 && py < y;
+            }
+            float4 al = blo[p[k]], ah = bhi[p[k]];
+            ploc_node(m - 2 - r, al, ah, blo[i], bhi[i], nodes, parent_node, parent_leaf, leaves);
+            const int to = p[k] - (r - between);
+            blo2[to] = al;
+            bhi2[to] = ah;
+        }
+        r += up;
+        if (i == m - 1) *m_next = m - r;
+    }
 }
 
-__global__ void k_ploc_compact(int m, const int64_t* __restrict__ incl, const int* __restrict__ cid,
-                               const float4* __restrict__ blo, const float4* __restrict__ bhi, int* __restrict__ cid2,
-                               float4* __restrict__ blo2, float4* __restrict__ bhi2) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= m) return;
-    const int64_t before = i > 0 ? incl[i - 1] : 0;
-    if (incl[i] == before) return;
-    cid2[before] = cid[i];
-    blo2[before] = blo[i];
-    bhi2[before] = bhi[i];
+// The remaining rounds, PLOC_TAIL clusters or fewer, one block. m_of: the counts before each round
+// launched so far; rounds alternate between the two cluster arrays until the first count of at most
+// PLOC_TAIL. left: 1 when one cluster is left, more when no pair was mutual (non-finite boxes).
+template <int R>
+__global__ void __launch_bounds__(PLOC_TAIL) k_ploc_tail(const int* __restrict__ m_of, int rounds,
+                                                         const float4* __restrict__ blo_a, const float4* __restrict__ bhi_a,
+                                                         const float4* __restrict__ blo_b, const float4* __restrict__ bhi_b,
+                                                         float4* __restrict__ nodes, int* __restrict__ parent_node,
+                                                         int* __restrict__ parent_leaf, unsigned int* __restrict__ leaves,
+                                                         int* __restrict__ left) {
+    __shared__ float4 sl[PLOC_TAIL], sh[PLOC_TAIL];
+    __shared__ int snn[PLOC_TAIL];
+    __shared__ unsigned up_of[PLOC_TAIL / 32];
+    __shared__ int gone_of[PLOC_TAIL / 32];
+    int r0 = 0;
+    while (r0 < rounds && m_of[r0] > PLOC_TAIL) ++r0;
+    int m = m_of[r0];
+    const int i = threadIdx.x, lane = i & 31, warp = i >> 5;
+    if (m > PLOC_TAIL) {
+        if (i == 0) *left = m;
+        return;
+    }
+    float4 al = make_float4(0.f, 0.f, 0.f, 0.f), ah = al;
+    if (i < m) {
+        al = (r0 & 1 ? blo_b : blo_a)[i];
+        ah = (r0 & 1 ? bhi_b : bhi_a)[i];
+    }
+    while (m > 1) {
+        sl[i] = al;
+        sh[i] = ah;
+        __syncthreads();
+        const int j = i < m ? ploc_nearest<R>(sl, sh, i, i, m) : -1;
+        snn[i] = j;
+        __syncthreads();
+        const int p = j >= 0 && snn[j] == i ? j : -1;
+        const bool up = p >= 0 && p < i;
+        const unsigned mask = __ballot_sync(0xffffffffu, up);
+        if (lane == 0) up_of[warp] = mask;
+        __syncthreads();
+        // clusters gone before each warp's first, and in all
+        const int c = __popc(up_of[lane]);
+        int incl = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += u;
+        }
+        if (warp == 0) gone_of[lane] = incl - c;
+        const int all = __shfl_sync(0xffffffffu, incl, 31);
+        const int mine = __shfl_sync(0xffffffffu, incl - c, warp);
+        __syncthreads();
+        if (all == 0) break;
+        const int r = mine + __popc(mask & ((1u << lane) - 1u));
+        int to = -1;
+        float4 nl = al, nh = ah;
+        if (i < m && p < 0) {
+            to = i - r;
+        } else if (up) {
+            nl = sl[p];
+            nh = sh[p];
+            ploc_node(m - 2 - r, nl, nh, al, ah, nodes, parent_node, parent_leaf, leaves);
+            to = p - (gone_of[p >> 5] + __popc(up_of[p >> 5] & ((1u << (p & 31)) - 1u)));
+        }
+        __syncthreads();   // every cluster has been read
+        if (to >= 0) {
+            sl[to] = nl;
+            sh[to] = nh;
+        }
+        m -= all;
+        __syncthreads();
+        al = sl[i];
+        ah = sh[i];
+        __syncthreads();
+    }
+    if (i == 0) *left = m;
 }
 
 // ---- depth-first node layout ------------------------------------------------------------------
@@ -430,11 +568,13 @@ __global__ void k_leaf_counts(const int* __restrict__ parent_leaf, const int* __
     }
 }
 
-// even[index] = 1 where the node's depth is even (root 0): those become 4-wide nodes.
+// even[index] = 1 where the node's depth is even (root 0): those become 4-wide nodes. *depth: the
+// deepest leaf (one level below the deepest node).
 __global__ void k_dfs_index(const float4* __restrict__ nodes, const int* __restrict__ parent_node,
                             const unsigned int* __restrict__ leaves, int n_int, int* __restrict__ dfs,
-                            int64_t* __restrict__ even) {
+                            int64_t* __restrict__ even, unsigned int* __restrict__ depth) {
     int v = blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned live = __ballot_sync(0xffffffffu, v < n_int);
     if (v >= n_int) return;
     int idx = 0, u = v, guard = 0;
     while (u > 0 && guard++ < 4096) {
@@ -447,6 +587,8 @@ __global__ void k_dfs_index(const float4* __restrict__ nodes, const int* __restr
     }
     dfs[v] = idx;
     even[idx] = (guard & 1) == 0 ? 1 : 0;
+    const unsigned deep = __reduce_max_sync(live, (unsigned)guard + 1u);
+    if ((threadIdx.x & 31) == 0) atomicMax(depth, deep);
 }
 
 __global__ void k_dfs_remap(const float4* __restrict__ nodes, const int* __restrict__ dfs, int n_int,
@@ -509,22 +651,7 @@ __global__ void k_pose(const float4* __restrict__ tri_local, const uint32_t* __r
             hi[3 + a] = fmaxf(fmaxf(w[a], w[3 + a]), w[6 + a]);
         }
     }
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-        for (int o = 16; o > 0; o >>= 1) {
-            lo[c] = fminf(lo[c], __shfl_xor_sync(0xffffffffu, lo[c], o));
-            hi[c] = fmaxf(hi[c], __shfl_xor_sync(0xffffffffu, hi[c], o));
-        }
-    }
-    if ((threadIdx.x & 31) == 0 && blockIdx.x * blockDim.x + (threadIdx.x & ~31u) < nt) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            atomicMin(&bounds[a], f2ord(lo[a]));
-            atomicMax(&bounds[3 + a], f2ord(hi[a]));
-            atomicMin(&bounds[6 + a], f2ord(lo[3 + a]));
-            atomicMax(&bounds[9 + a], f2ord(hi[3 + a]));
-        }
-    }
+    fold_bounds(lo, hi, bounds);
 }
 
 // Triangle id of every leaf slot (v0.w of the leaf-order copy).
@@ -656,114 +783,119 @@ static gm_status build_scene(gm_ctx* ctx, const gm_mesh_desc* meshes, uint32_t n
         }
         base += d.n_tris;
     }
-    GM_TRY_CUDA(cudaMemcpyAsync(sc->mesh_object, objs.data(), sizeof(uint32_t) * n_meshes, cudaMemcpyHostToDevice, s));
-    // world -> mesh-local maps for the export format (affine inverse in FP64)
-    {
-        std::vector<double> xf(16 * (size_t)n_meshes);
-        for (uint32_t m = 0; m < n_meshes; ++m) memcpy(&xf[16 * m], meshes[m].transform, sizeof(double) * 16);
-        std::vector<double> inv;
-        sc->mesh_inv_ok = mesh_inverses(xf.data(), n_meshes, inv);
-        SC_ALLOC(sc->mesh_inv, sizeof(double) * 12 * n_meshes);
-        GM_TRY_CUDA(cudaMemcpyAsync(sc->mesh_inv, inv.data(), sizeof(double) * 12 * n_meshes, cudaMemcpyHostToDevice, s));
-        GM_TRY_CUDA(cudaStreamSynchronize(s));   // inv is a host temporary
-    }
+    cudaError_t ce = cudaMemcpyAsync(sc->mesh_object, objs.data(), sizeof(uint32_t) * n_meshes, cudaMemcpyHostToDevice, s);
+    auto wait_fail = [&](gm_status st_) {   // host temporaries may still be read
+        cudaStreamSynchronize(s);
+        return fail(st_);
+    };
+    if (ce != cudaSuccess) return wait_fail(gm_cuda_error(ce, "gm_build_scene"));
+    // world -> mesh-local maps for the export format (affine inverse in FP64); the host copies live until
+    // the stream is waited for below
+    std::vector<double> xf(16 * (size_t)n_meshes), inv;
+    for (uint32_t m = 0; m < n_meshes; ++m) memcpy(&xf[16 * m], meshes[m].transform, sizeof(double) * 16);
+    sc->mesh_inv_ok = mesh_inverses(xf.data(), n_meshes, inv);
+    SC_ALLOC(sc->mesh_inv, sizeof(double) * 12 * n_meshes);
+    if ((ce = cudaMemcpyAsync(sc->mesh_inv, inv.data(), sizeof(double) * 12 * n_meshes, cudaMemcpyHostToDevice, s)) !=
+        cudaSuccess)
+        return wait_fail(gm_cuda_error(ce, "gm_build_scene"));
 
     uint64_t* keys = nullptr;
     uint32_t* order = nullptr;
     int *parent_node = nullptr, *parent_leaf = nullptr;
-    unsigned int *flags = nullptr, *depth = nullptr;
+    unsigned int *leaves = nullptr, *depth = nullptr;
+    const uint32_t n_in = nt > 1 ? nt - 1 : 1;
     TMP_ALLOC(keys, sizeof(uint64_t) * nt);
     TMP_ALLOC(order, sizeof(uint32_t) * nt);
     TMP_ALLOC(parent_leaf, sizeof(int) * nt);
-    TMP_ALLOC(parent_node, sizeof(int) * (nt > 1 ? nt - 1 : 1));
-    TMP_ALLOC(flags, sizeof(unsigned int) * (nt > 1 ? nt - 1 : 1));
-    TMP_ALLOC(depth, sizeof(unsigned int));
-    GM_TRY_CUDA(cudaMemsetAsync(flags, 0, sizeof(unsigned int) * (nt > 1 ? nt - 1 : 1), s));
+    TMP_ALLOC(parent_node, sizeof(int) * n_in);
+    TMP_ALLOC(leaves, sizeof(unsigned int) * n_in);
+    TMP_ALLOC(depth, sizeof(unsigned int) * 2);   // [0] depth, [1] clusters left
     // -1 everywhere: a link the hierarchy step did not write stops the refit instead of escaping
-    GM_TRY_CUDA(cudaMemsetAsync(parent_leaf, 0xff, sizeof(int) * nt, s));
-    GM_TRY_CUDA(cudaMemsetAsync(parent_node, 0xff, sizeof(int) * (nt > 1 ? nt - 1 : 1), s));
-    GM_TRY_CUDA(cudaMemsetAsync(depth, 0, sizeof(unsigned int), s));
+    if ((ce = cudaMemsetAsync(parent_leaf, 0xff, sizeof(int) * nt, s)) != cudaSuccess ||
+        (ce = cudaMemsetAsync(parent_node, 0xff, sizeof(int) * n_in, s)) != cudaSuccess ||
+        (ce = cudaMemsetAsync(depth, 0, sizeof(unsigned int) * 2, s)) != cudaSuccess)
+        return wait_fail(gm_cuda_error(ce, "gm_build_scene"));
     k_morton<<<gm_div_up(nt, 256), 256, 0, s>>>(sc->tri_canon, nt, bounds, keys, order);
-    if ((st = gm_radix_sort_u64(keys, order, nt, 63, s, &launches)) != GM_OK) return fail(st);
-    if (builder == GM_BUILD_PLOC && nt > 1) {
-        int *cid = nullptr, *cid2 = nullptr, *nn = nullptr, *counter = nullptr;
-        float4 *blo = nullptr, *bhi = nullptr, *blo2 = nullptr, *bhi2 = nullptr;
-        int64_t* keep = nullptr;
-        TMP_ALLOC(cid, sizeof(int) * nt);
-        TMP_ALLOC(cid2, sizeof(int) * nt);
-        TMP_ALLOC(nn, sizeof(int) * nt);
-        TMP_ALLOC(counter, sizeof(int));
-        TMP_ALLOC(blo, sizeof(float4) * nt);
-        TMP_ALLOC(bhi, sizeof(float4) * nt);
-        TMP_ALLOC(blo2, sizeof(float4) * nt);
-        TMP_ALLOC(bhi2, sizeof(float4) * nt);
-        TMP_ALLOC(keep, sizeof(int64_t) * nt);
-        k_ploc_init<<<gm_div_up(nt, 256), 256, 0, s>>>(sc->tri_canon, order, (int)nt, bounds, cid, blo, bhi,
-                                                       sc->bvh_tris);
-        const int first = (int)nt - 1;
-        GM_TRY_CUDA(cudaMemcpyAsync(counter, &first, sizeof(int), cudaMemcpyHostToDevice, s));
-        launches += 1;
-        int m = (int)nt;
-        int64_t* m_host = nullptr;
-        GM_TRY_CUDA(cudaMallocHost(&m_host, sizeof(int64_t)));
-        int rounds = 0;
-        while (m > 1 && rounds < 4096) {
-            ++rounds;
-            switch (ploc_radius) {
-                case 4: k_ploc_nn<4><<<gm_div_up(m, 256), 256, 0, s>>>(blo, bhi, m, nn); break;
-                case 16: k_ploc_nn<16><<<gm_div_up(m, 256), 256, 0, s>>>(blo, bhi, m, nn); break;
-                case 32: k_ploc_nn<32><<<gm_div_up(m, 256), 256, 0, s>>>(blo, bhi, m, nn); break;
-                case 64: k_ploc_nn<64><<<gm_div_up(m, 256), 256, 0, s>>>(blo, bhi, m, nn); break;
-                default: k_ploc_nn<8><<<gm_div_up(m, 256), 256, 0, s>>>(blo, bhi, m, nn); break;
-            }
-            k_ploc_merge<<<gm_div_up(m, 256), 256, 0, s>>>(m, nn, cid, blo, bhi, keep, counter, sc->nodes, parent_node,
-                                                           parent_leaf);
-            if ((st = gm_inclusive_scan_i64(keep, (uint32_t)m, s, &launches)) != GM_OK) {
-                cudaFreeHost(m_host);
-                return fail(st);
-            }
-            k_ploc_compact<<<gm_div_up(m, 256), 256, 0, s>>>(m, keep, cid, blo, bhi, cid2, blo2, bhi2);
-            launches += 3;
-            std::swap(cid, cid2);
-            std::swap(blo, blo2);
-            std::swap(bhi, bhi2);
-            cudaError_t ce = cudaMemcpyAsync(m_host, keep + (m - 1), sizeof(int64_t), cudaMemcpyDeviceToHost, s);
-            if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
-            if (ce != cudaSuccess) {
-                cudaFreeHost(m_host);
-                return fail(gm_cuda_error(ce, "gm_build_scene (clustering)"));
-            }
-            if (*m_host >= m) {   // no mutual pair: cannot happen with consistent tie-breaking
-                cudaFreeHost(m_host);
-                return fail(gm_set_error(GM_ERR_INTERNAL, "gm_build_scene: clustering made no progress"));
-            }
-            m = (int)*m_host;
+    ++launches;
+    if ((st = gm_radix_sort_u64(keys, order, nt, 63, s, &launches)) != GM_OK) return wait_fail(st);
+    const bool ploc = builder == GM_BUILD_PLOC && nt > 1;
+    if (ploc) {
+        constexpr int kRounds = 4096;
+        int *m_of = nullptr, *pair = nullptr, *gone = nullptr;
+        float4 *lo[2] = {}, *hi[2] = {};
+        const uint32_t nblk = gm_div_up(nt, PLOC_P);
+        TMP_ALLOC(m_of, sizeof(int) * (kRounds + PLOC_BATCH + 1));
+        for (int k = 0; k < 2; ++k) {
+            TMP_ALLOC(lo[k], sizeof(float4) * nt);
+            TMP_ALLOC(hi[k], sizeof(float4) * nt);
         }
-        cudaFreeHost(m_host);
+        TMP_ALLOC(pair, sizeof(int) * nt);
+        TMP_ALLOC(gone, sizeof(int) * nblk);
+        k_ploc_init<<<gm_div_up(nt, 256), 256, 0, s>>>(sc->tri_canon, order, (int)nt, bounds, lo[0], hi[0], sc->bvh_tris,
+                                                       m_of);
+        ++launches;
+        int m = (int)nt, rounds = 0;
+        while (m > PLOC_TAIL && rounds < kRounds) {
+            const uint32_t grid = gm_div_up((uint32_t)m, PLOC_P);
+            for (int k = 0; k < PLOC_BATCH; ++k, ++rounds) {
+                const int a = rounds & 1;
+                switch (ploc_radius) {
+                    case 4: k_ploc_pair<4><<<grid, PLOC_T, 0, s>>>(m_of + rounds, lo[a], hi[a], pair, gone); break;
+                    case 16: k_ploc_pair<16><<<grid, PLOC_T, 0, s>>>(m_of + rounds, lo[a], hi[a], pair, gone); break;
+                    case 32: k_ploc_pair<32><<<grid, PLOC_T, 0, s>>>(m_of + rounds, lo[a], hi[a], pair, gone); break;
+                    case 64: k_ploc_pair<64><<<grid, PLOC_T, 0, s>>>(m_of + rounds, lo[a], hi[a], pair, gone); break;
+                    default: k_ploc_pair<8><<<grid, PLOC_T, 0, s>>>(m_of + rounds, lo[a], hi[a], pair, gone); break;
+                }
+                k_ploc_apply<<<grid, PLOC_T, 0, s>>>(m_of + rounds, m_of + rounds + 1, lo[a], hi[a], pair, gone,
+                                                     lo[a ^ 1], hi[a ^ 1], sc->nodes, parent_node, parent_leaf, leaves);
+            }
+            launches += 2 * PLOC_BATCH;
+            int now = 0;
+            if ((ce = cudaMemcpyAsync(&now, m_of + rounds, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+                (ce = cudaStreamSynchronize(s)) != cudaSuccess)
+                return wait_fail(gm_cuda_error(ce, "gm_build_scene (clustering)"));
+            if (now >= m) break;   // no mutual pair: reported below
+            m = now;
+        }
+        auto tail = [&](auto kern) {
+            kern<<<1, PLOC_TAIL, 0, s>>>(m_of, rounds, lo[0], hi[0], lo[1], hi[1], sc->nodes, parent_node, parent_leaf,
+                                         leaves, (int*)depth + 1);
+        };
+        switch (ploc_radius) {
+            case 4: tail(k_ploc_tail<4>); break;
+            case 16: tail(k_ploc_tail<16>); break;
+            case 32: tail(k_ploc_tail<32>); break;
+            case 64: tail(k_ploc_tail<64>); break;
+            default: tail(k_ploc_tail<8>); break;
+        }
+        ++launches;
     } else {
+        unsigned int* flags = nullptr;
+        TMP_ALLOC(flags, sizeof(unsigned int) * n_in);
+        if ((ce = cudaMemsetAsync(flags, 0, sizeof(unsigned int) * n_in, s)) != cudaSuccess)
+            return wait_fail(gm_cuda_error(ce, "gm_build_scene"));
         if (nt > 1) k_hierarchy<<<gm_div_up(nt - 1, 256), 256, 0, s>>>(keys, (int)nt, sc->nodes, parent_node, parent_leaf);
         k_refit<<<gm_div_up(nt, 256), 256, 0, s>>>(sc->tri_canon, order, (int)nt, sc->nodes, parent_node, parent_leaf,
                                                     flags, bounds, sc->bvh_tris);
         launches += (nt > 1 ? 2 : 1);
     }
-    k_depth<<<gm_div_up(nt, 256), 256, 0, s>>>(parent_node, parent_leaf, (int)nt, depth);
-    launches += 2;
     ctx->launches += launches;
     cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return fail(gm_cuda_error(e, "gm_build_scene launch"));
+    if (e != cudaSuccess) return wait_fail(gm_cuda_error(e, "gm_build_scene launch"));
     unsigned int hb[16] = {0};
-    unsigned int hdepth = 0;
+    unsigned int hdepth[2] = {0, 0};
     int herr = 0;
     if ((e = cudaMemcpyAsync(hb, bounds, sizeof(unsigned int) * 12, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(&hdepth, depth, sizeof(unsigned int), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+        (e = cudaMemcpyAsync(hdepth, depth, sizeof(hdepth), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
         (e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
         (e = cudaStreamSynchronize(s)) != cudaSuccess)
-        return fail(gm_cuda_error(e, "gm_build_scene"));
-    int* parent_node_keep = parent_node;
+        return wait_fail(gm_cuda_error(e, "gm_build_scene"));
     if (herr == GM_DEV_BAD_INDEX) {
         cudaMemsetAsync(ctx->dev_err, 0, sizeof(int), s);
         return fail(gm_set_error(GM_ERR_INVALID_ARG, "gm_build_scene: a vertex index is out of range"));
     }
+    if (ploc && hdepth[1] != 1)   // no mutual pair: cannot happen with consistent tie-breaking and finite boxes
+        return fail(gm_set_error(GM_ERR_INTERNAL, "gm_build_scene: clustering made no progress"));
     auto dec = [](unsigned int o) {
         unsigned int b = (o & 0x80000000u) ? (o & 0x7fffffffu) : ~o;
         float f;
@@ -776,34 +908,32 @@ static gm_status build_scene(gm_ctx* ctx, const gm_mesh_desc* meshes, uint32_t n
         if (!std::isfinite(sc->box_lo[k]) || !std::isfinite(sc->box_hi[k]))
             return fail(gm_set_error(GM_ERR_INVALID_ARG, "gm_build_scene: non-finite vertex"));
     }
-    sc->depth = nt > 1 ? hdepth : 0;
-    if (sc->depth > 64)
-        return fail(gm_set_error(GM_ERR_UNSUPPORTED, "gm_build_scene: BVH deeper than 64 levels (" +
-                                                         std::to_string(sc->depth) + ")"));
+    sc->depth = 0;
     if (nt > 1) {
         const int n_int = (int)nt - 1;
-        unsigned int* leaves = nullptr;
         int* dfs = nullptr;
-        unsigned int* arrived = nullptr;
         float4* reordered = nullptr;
         int64_t* incl = nullptr;
-        TMP_ALLOC(leaves, sizeof(unsigned int) * n_int);
         TMP_ALLOC(dfs, sizeof(int) * n_int);
-        TMP_ALLOC(arrived, sizeof(unsigned int) * n_int);
         if (dynamic) {
             SC_ALLOC(sc->incl4, sizeof(int64_t) * n_int);
             incl = sc->incl4;
         } else {
             TMP_ALLOC(incl, sizeof(int64_t) * n_int);
         }
-        GM_TRY_CUDA(cudaMemsetAsync(leaves, 0, sizeof(unsigned int) * n_int, s));
-        GM_TRY_CUDA(cudaMemsetAsync(arrived, 0, sizeof(unsigned int) * n_int, s));
+        launches = 2;
+        if (!ploc) {   // the clustering counted the leaves as it merged
+            unsigned int* arrived = nullptr;
+            TMP_ALLOC(arrived, sizeof(unsigned int) * n_int);
+            if ((e = cudaMemsetAsync(leaves, 0, sizeof(unsigned int) * n_int, s)) != cudaSuccess ||
+                (e = cudaMemsetAsync(arrived, 0, sizeof(unsigned int) * n_int, s)) != cudaSuccess)
+                return fail(gm_cuda_error(e, "gm_build_scene"));
+            k_leaf_counts<<<gm_div_up(nt, 256), 256, 0, s>>>(parent_leaf, parent_node, sc->nodes, (int)nt, leaves, arrived);
+            ++launches;
+        }
         if ((st = gm_alloc((void**)&reordered, sizeof(float4) * 4 * (size_t)n_int, s)) != GM_OK) return fail(st);
-        k_leaf_counts<<<gm_div_up(nt, 256), 256, 0, s>>>(parent_leaf, parent_node_keep, sc->nodes, (int)nt, leaves,
-                                                         arrived);
-        k_dfs_index<<<gm_div_up(n_int, 256), 256, 0, s>>>(sc->nodes, parent_node_keep, leaves, n_int, dfs, incl);
+        k_dfs_index<<<gm_div_up(n_int, 256), 256, 0, s>>>(sc->nodes, parent_node, leaves, n_int, dfs, incl, depth);
         k_dfs_remap<<<gm_div_up(n_int, 256), 256, 0, s>>>(sc->nodes, dfs, n_int, reordered);
-        launches = 3;
         cudaFreeAsync(sc->nodes, s);
         sc->nodes = reordered;
         // the 4-wide nodes follow the depth-first order. Every even-depth node but the root is a child of
@@ -813,8 +943,14 @@ static gm_status build_scene(gm_ctx* ctx, const gm_mesh_desc* meshes, uint32_t n
         k_collapse4<<<gm_div_up(n_int, 256), 256, 0, s>>>(sc->nodes, n_int, incl, sc->nodes4);
         ++launches;
         ctx->launches += launches;
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return fail(gm_cuda_error(e, "gm_build_scene layout"));
+        if ((e = cudaGetLastError()) != cudaSuccess ||
+            (e = cudaMemcpyAsync(hdepth, depth, sizeof(unsigned int), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+            (e = cudaStreamSynchronize(s)) != cudaSuccess)
+            return wait_fail(gm_cuda_error(e, "gm_build_scene layout"));
+        sc->depth = hdepth[0];
+        if (sc->depth > 64)
+            return fail(gm_set_error(GM_ERR_UNSUPPORTED, "gm_build_scene: BVH deeper than 64 levels (" +
+                                                             std::to_string(sc->depth) + ")"));
     }
     for (void* p : tmp) cudaFreeAsync(p, s);
     tmp.clear();
