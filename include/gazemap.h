@@ -329,7 +329,7 @@ gm_status gm_accumulate_dynamic(gm_scene* scene, gm_samples* samples, const gm_f
  * whose cone reaches behind their camera have no crop window and are skipped (counted). With
  * `compare` the exact ray test also runs on every in-cone pair and the disagreements are counted
  * (gm_zbuffer_stats). Z-buffers are built for chunks of fixations of at most `zbuffer_bytes`
- * (0: 2 GiB). Synchronises `stream` a few times per chunk. */
+ * (0: 2 GiB). Synchronises `stream` once, and once more when the fixations need several chunks. */
 typedef struct {
     uint32_t res;            /* z-buffer pixels per side (a generation parameter, Section 3.3.4) */
     float near_m, far_m;     /* clip planes, metres, 0 < near < far */

@@ -7,16 +7,15 @@
 //                  hints, the gaze in camera space, the exact crop window (tangent planes through
 //                  the eye; Appendix A centres its window on the gaze point E, which is not the
 //                  centre of an oblique conic section) and the pixel mapping
-//   k_zb_cull      one thread per triangle, frusta staged in shared memory: a triangle is kept for
-//                  a fixation unless all three vertices lie outside one frustum plane; survivors
-//                  are appended as (fixation, triangle) pairs with one atomic per warp
-//   k_zb_raster    one thread per pair: near-plane clipping, projection, point sampling at pixel
-//                  centres with edge functions evaluated in a canonical vertex order (a shared
-//                  edge gives exactly opposite values, no cracks), perspective-correct 1/w, and
-//                  atomicMin of the linear depth w (positive floats order as their bits); pairs
-//                  covering more than RASTER_THREAD_PIXELS pixels go to k_zb_raster_warp (one warp
-//                  each, lanes over pixels), more than RASTER_WARP_PIXELS to k_zb_raster_big (one
-//                  block each): lanes of a warp no longer wait for one lane's large triangle
+//   k_zb_draw      one thread per triangle, frusta staged in shared memory: a triangle is kept for a
+//                  fixation unless all three vertices lie outside one frustum plane. A warp queues its
+//                  surviving (fixation, triangle) pairs and draws them 32 at a time: each lane sets one
+//                  pair up (near-plane test, projection, pixel box, edges in a canonical vertex order, so
+//                  that a shared edge gives exactly opposite values and leaves no cracks), then the lanes
+//                  share the pixels of all 32 boxes evenly: point sampling at pixel centres,
+//                  perspective-correct 1/w, atomicMin of the linear depth w (positive floats order as
+//                  their bits)
+//   k_zb_draw_big  pairs whose box holds more than ZB_BIG_PIXELS pixels, one block each
 //   k_zb_accumulate one thread per work-order sample over the chunk's fixations: the exact cone
 //                  test and Gaussian of the ray path, visibility |w - zbuf| <= eps, compensated
 //                  sums carried across chunks, per-window writes and maxima; optionally the exact
@@ -31,12 +30,12 @@ namespace {
 
 constexpr int ZB_THREADS = 256;
 constexpr int ZB_SMEM_FRUSTA = 64;            // frusta staged per pass of the cull kernel
-constexpr int RASTER_THREAD_PIXELS = 64;      // larger pixel boxes go to the warp rasteriser,
-constexpr int RASTER_WARP_PIXELS = 1024;      // and larger ones still to the block rasteriser
+constexpr int ZB_BIG_PIXELS = 1024;           // larger pixel boxes go to the block rasteriser
+constexpr uint64_t ZB_BIG_CAP = 1u << 20;     // ... through a list of this many pairs (a full list: drawn in place)
 constexpr uint32_t ZB_EMPTY = 0xffffffffu;    // cleared z-buffer word (above every finite depth)
 constexpr uint32_t NO_WINDOW = 0xffffffffu;
 
-struct ZbFrustum {
+struct alignas(16) ZbFrustum {
     float e[3], rgt[3], up[3], fwd[3];
     float n, f;
     float sx, ox, sy, oy;   // pixel coordinates: u = sx x / w + ox, v = sy y / w + oy
@@ -208,122 +207,6 @@ __device__ __forceinline__ bool sphere_outside(const ZbFrustum& F, float cx, flo
            fmaf(-F.sy, yc, b1 * wc) < -slack * sqrtf(fmaf(F.sy, F.sy, b1 * b1));
 }
 
-__global__ void __launch_bounds__(ZB_THREADS) k_zb_cull(const float4* __restrict__ tris, uint32_t nt,
-                                                        const ZbFrustum* __restrict__ frusta, uint32_t nfix,
-                                                        uint32_t res, PairFT* __restrict__ pairs, uint64_t cap,
-                                                        unsigned long long* __restrict__ count) {
-    __shared__ ZbFrustum sF[ZB_SMEM_FRUSTA];
-    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool valid = t < nt;
-    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a, c = a;
-    if (valid) {   // leaf order: a warp's 32 triangles are neighbours in space; v0.w = triangle id
-        a = tris[3 * t];
-        b = tris[3 * t + 1];
-        c = tris[3 * t + 2];
-    }
-    const uint32_t id = __float_as_uint(a.w);
-    const int lane = threadIdx.x & 31;
-    const float R = (float)res;
-    // the warp's triangles in one sphere (box centre, half diagonal), tested against each frustum
-    // before the per-triangle tests
-    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-    if (valid) {
-        lo[0] = fminf(fminf(a.x, b.x), c.x);
-        lo[1] = fminf(fminf(a.y, b.y), c.y);
-        lo[2] = fminf(fminf(a.z, b.z), c.z);
-        hi[0] = fmaxf(fmaxf(a.x, b.x), c.x);
-        hi[1] = fmaxf(fmaxf(a.y, b.y), c.y);
-        hi[2] = fmaxf(fmaxf(a.z, b.z), c.z);
-    }
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        for (int o = 16; o > 0; o >>= 1) {
-            lo[q] = fminf(lo[q], __shfl_xor_sync(0xffffffffu, lo[q], o));
-            hi[q] = fmaxf(hi[q], __shfl_xor_sync(0xffffffffu, hi[q], o));
-        }
-    }
-    const bool wbox = lo[0] <= hi[0];
-    const float wx = 0.5f * (lo[0] + hi[0]), wy = 0.5f * (lo[1] + hi[1]), wz = 0.5f * (lo[2] + hi[2]);
-    const float wR = wbox ? 0.5f * sqrtf((hi[0] - lo[0]) * (hi[0] - lo[0]) + (hi[1] - lo[1]) * (hi[1] - lo[1]) +
-                                         (hi[2] - lo[2]) * (hi[2] - lo[2])) * 1.0001f
-                          : 0.f;
-    // the block's 256 triangles (also neighbours in leaf order) in one sphere: a frustum that
-    // misses it is skipped by every warp of the block without its own sphere test
-    __shared__ float sBox[ZB_THREADS / 32][6];
-    __shared__ float4 sBlk;
-    __shared__ unsigned sMask[ZB_SMEM_FRUSTA / 32];
-    const int warp = threadIdx.x >> 5;
-    if (lane == 0) {
-        sBox[warp][0] = lo[0], sBox[warp][1] = lo[1], sBox[warp][2] = lo[2];
-        sBox[warp][3] = hi[0], sBox[warp][4] = hi[1], sBox[warp][5] = hi[2];
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float bl[3] = {INFINITY, INFINITY, INFINITY}, bh[3] = {-INFINITY, -INFINITY, -INFINITY};
-        for (int w = 0; w < ZB_THREADS / 32; ++w)
-            for (int q = 0; q < 3; ++q) {
-                bl[q] = fminf(bl[q], sBox[w][q]);
-                bh[q] = fmaxf(bh[q], sBox[w][3 + q]);
-            }
-        sBlk = bl[0] <= bh[0]
-                   ? make_float4(0.5f * (bl[0] + bh[0]), 0.5f * (bl[1] + bh[1]), 0.5f * (bl[2] + bh[2]),
-                                 0.5f * sqrtf((bh[0] - bl[0]) * (bh[0] - bl[0]) + (bh[1] - bl[1]) * (bh[1] - bl[1]) +
-                                              (bh[2] - bl[2]) * (bh[2] - bl[2])) * 1.0001f)
-                   : make_float4(0.f, 0.f, 0.f, -1.f);
-    }
-    // blockIdx.y picks a group of fixations (one shared-memory load of their frusta); the blocks of
-    // one group run together, so the pairs they emit -- and the raster's atomics -- stay on a few
-    // z-buffers that fit in L2
-    for (uint32_t f0 = blockIdx.y * ZB_SMEM_FRUSTA; f0 < nfix; f0 += gridDim.y * ZB_SMEM_FRUSTA) {
-        const uint32_t m = min((uint32_t)ZB_SMEM_FRUSTA, nfix - f0);
-        __syncthreads();
-        for (uint32_t k = threadIdx.x; k < m; k += blockDim.x) sF[k] = frusta[f0 + k];
-        __syncthreads();
-        if (threadIdx.x < ZB_SMEM_FRUSTA) {   // whole warps: ZB_SMEM_FRUSTA is a multiple of 32
-            const uint32_t k = threadIdx.x;
-            const float4 bs = sBlk;
-            const bool reach = k < m && sF[k].ok && bs.w >= 0.f && !sphere_outside(sF[k], bs.x, bs.y, bs.z, bs.w, R);
-            const unsigned bits = __ballot_sync(0xffffffffu, reach);
-            if (lane == 0) sMask[k >> 5] = bits;
-        }
-        __syncthreads();
-        for (uint32_t k = 0; k < m; ++k) {
-            if (!((sMask[k >> 5] >> (k & 31)) & 1u)) continue;
-            const ZbFrustum& F = sF[k];
-            if (!wbox || sphere_outside(F, wx, wy, wz, wR, R)) continue;
-            bool keep = false;
-            if (valid) {
-                float x[3], y[3], w[3];
-                to_camera(F, a.x, a.y, a.z, x[0], y[0], w[0]);
-                to_camera(F, b.x, b.y, b.z, x[1], y[1], w[1]);
-                to_camera(F, c.x, c.y, c.z, x[2], y[2], w[2]);
-                int o0 = 0, o1 = 0, o2 = 0, o3 = 0, o4 = 0, o5 = 0;
-#pragma unroll
-                for (int v = 0; v < 3; ++v) {
-                    const float U = fmaf(F.sx, x[v], F.ox * w[v]), V = fmaf(F.sy, y[v], F.oy * w[v]);
-                    o0 += U < -w[v];
-                    o1 += U > (R + 1.f) * w[v];
-                    o2 += V < -w[v];
-                    o3 += V > (R + 1.f) * w[v];
-                    o4 += w[v] < F.n * (1.f - 1e-5f);
-                    o5 += w[v] > F.f * (1.f + 1e-5f);
-                }
-                keep = o0 < 3 && o1 < 3 && o2 < 3 && o3 < 3 && o4 < 3 && o5 < 3;
-            }
-            const unsigned msk = __ballot_sync(0xffffffffu, keep);
-            if (msk) {
-                unsigned long long base = 0;
-                if (lane == __ffs(msk) - 1) base = atomicAdd(count, (unsigned long long)__popc(msk));
-                base = __shfl_sync(0xffffffffu, base, __ffs(msk) - 1);
-                if (keep) {
-                    const unsigned long long q = base + __popc(msk & gm_lanemask_lt());
-                    if (q < cap) pairs[q] = PairFT{f0 + k, id};
-                }
-            }
-        }
-    }
-}
-
 // ---- raster --------------------------------------------------------------------------------
 struct ClipPoly {
     float u[4], v[4], iw[4];
@@ -376,6 +259,17 @@ __device__ __forceinline__ float edge_fn(float ax, float ay, float bx, float by,
     return swap ? -e : e;
 }
 
+// The pixels whose centres px + 1/2 lie within [umin, umax] x [vmin, vmax], widened by 1/100 pixel for the
+// rounding of the edge functions (an FP32 error of a few 1e-4 pixels at these coordinates).
+__device__ __forceinline__ void pixel_box(float umin, float umax, float vmin, float vmax, int res, int& x0, int& x1,
+                                          int& y0, int& y1) {
+    constexpr float e = 0.01f;
+    x0 = max(0, (int)ceilf(fmaxf(umin, -2.f) - 0.5f - e));
+    x1 = min(res - 1, (int)floorf(fminf(umax, (float)res + 2.f) - 0.5f + e));
+    y0 = max(0, (int)ceilf(fmaxf(vmin, -2.f) - 0.5f - e));
+    y1 = min(res - 1, (int)floorf(fminf(vmax, (float)res + 2.f) - 0.5f + e));
+}
+
 __device__ __forceinline__ void poly_bbox(const ClipPoly& P, int res, int& x0, int& x1, int& y0, int& y1) {
     float umin = P.u[0], umax = P.u[0], vmin = P.v[0], vmax = P.v[0];
     for (int k = 1; k < P.n; ++k) {
@@ -384,13 +278,7 @@ __device__ __forceinline__ void poly_bbox(const ClipPoly& P, int res, int& x0, i
         vmin = fminf(vmin, P.v[k]);
         vmax = fmaxf(vmax, P.v[k]);
     }
-    // pixel centres px + 1/2 within [umin, umax], widened by 1/100 pixel for the rounding of the
-    // edge functions (an FP32 error of a few 1e-4 pixels at these coordinates)
-    constexpr float e = 0.01f;
-    x0 = max(0, (int)ceilf(fmaxf(umin, -2.f) - 0.5f - e));
-    x1 = min(res - 1, (int)floorf(fminf(umax, (float)res + 2.f) - 0.5f + e));
-    y0 = max(0, (int)ceilf(fmaxf(vmin, -2.f) - 0.5f - e));
-    y1 = min(res - 1, (int)floorf(fminf(vmax, (float)res + 2.f) - 0.5f + e));
+    pixel_box(umin, umax, vmin, vmax, res, x0, x1, y0, y1);
 }
 
 // Depth test of one pixel against the fan triangles of the polygon.
@@ -411,88 +299,293 @@ __device__ __forceinline__ void shade_pixel(const ClipPoly& P, int px, int py, f
     }
 }
 
-// Append `value` to a list for every lane that wants to, with one atomic per warp. All 32 lanes call it.
-__device__ __forceinline__ void warp_push(bool want, uint32_t value, uint32_t* __restrict__ list, uint64_t cap,
-                                          unsigned long long* __restrict__ counter) {
-    const unsigned m = __ballot_sync(0xffffffffu, want);
-    if (!m) return;
-    const int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
-    unsigned long long base = 0;
-    if (lane == leader) base = atomicAdd(counter, (unsigned long long)__popc(m));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    if (want) {
-        const unsigned long long q = base + __popc(m & gm_lanemask_lt());
-        if (q < cap) list[q] = value;
-    }
-}
-
-__global__ void __launch_bounds__(ZB_THREADS) k_zb_raster(const PairFT* __restrict__ pairs, uint64_t n_pairs,
-                                                          const ZbFrustum* __restrict__ frusta,
-                                                          const float4* __restrict__ tris, uint32_t res,
-                                                          uint32_t* __restrict__ zbuf, uint32_t* __restrict__ big,
-                                                          uint32_t* __restrict__ mid, uint64_t list_cap,
-                                                          unsigned long long* __restrict__ n_lists) {
-    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    PairFT pr{0u, 0u};
-    ZbFrustum F;
+// One thread draws one pair, clipped to the near plane (out of line: few triangles reach it).
+__device__ __noinline__ void draw_clipped(const ZbFrustum& F, float4 a, float4 b, float4 c, uint32_t res,
+                                          uint32_t* __restrict__ zb) {
     ClipPoly P;
-    P.n = 0;
-    int x0 = 0, x1 = -1, y0 = 0, y1 = -1;
-    if (i < n_pairs) {
-        pr = pairs[i];
-        F = frusta[pr.fix];
-        clip_project(F, tris[3 * pr.tri], tris[3 * pr.tri + 1], tris[3 * pr.tri + 2], P);
-        if (P.n >= 3) poly_bbox(P, (int)res, x0, x1, y0, y1);
-    }
-    const int npx = (P.n >= 3 && x1 >= x0 && y1 >= y0) ? (x1 - x0 + 1) * (y1 - y0 + 1) : 0;
-    const bool to_big = npx > RASTER_WARP_PIXELS, to_mid = npx > RASTER_THREAD_PIXELS && !to_big;
-    warp_push(to_big, (uint32_t)i, big, list_cap, &n_lists[0]);
-    warp_push(to_mid, (uint32_t)i, mid, list_cap, &n_lists[1]);
-    if (npx == 0 || to_big || to_mid) return;
-    uint32_t* zb = zbuf + (size_t)pr.fix * res * res;
+    clip_project(F, a, b, c, P);
+    if (P.n < 3) return;
+    int x0, x1, y0, y1;
+    poly_bbox(P, (int)res, x0, x1, y0, y1);
     for (int py = y0; py <= y1; ++py)
         for (int px = x0; px <= x1; ++px) shade_pixel(P, px, py, F.n, F.f, zb, (int)res);
 }
 
-__global__ void __launch_bounds__(ZB_THREADS) k_zb_raster_warp(const uint32_t* __restrict__ mid, uint64_t n_mid,
-                                                               const PairFT* __restrict__ pairs,
-                                                               const ZbFrustum* __restrict__ frusta,
-                                                               const float4* __restrict__ tris, uint32_t res,
-                                                               uint32_t* __restrict__ zbuf) {
-    const uint64_t warp0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    for (uint64_t q = warp0; q < n_mid; q += nwarps) {
-        const PairFT pr = pairs[mid[q]];
-        const ZbFrustum F = frusta[pr.fix];
-        ClipPoly P;
-        clip_project(F, tris[3 * pr.tri], tris[3 * pr.tri + 1], tris[3 * pr.tri + 2], P);
-        if (P.n < 3) continue;
-        int x0, x1, y0, y1;
-        poly_bbox(P, (int)res, x0, x1, y0, y1);
-        if (x1 < x0 || y1 < y0) continue;
-        const int wdt = x1 - x0 + 1, cnt = wdt * (y1 - y0 + 1);
-        uint32_t* zb = zbuf + (size_t)pr.fix * res * res;
-        for (int k = lane; k < cnt; k += 32) shade_pixel(P, x0 + k % wdt, y0 + k / wdt, F.n, F.f, zb, (int)res);
-    }
+// One pair set up for drawing: edges b -> c, c -> a, a -> b as (x0, y0, dx, dy) with the endpoints in
+// canonical order and the sign in dx and dy (negating both negates the edge function exactly).
+struct alignas(16) ZbTri {
+    float4 e0, e1, e2;
+    float4 iw;      // 1/w of a, b, c; box width | first pixel's index among the warp's << 16 (bits)
+    float2 centre;  // of the box's first pixel
+    uint32_t* z;    // that pixel's word
+};
+
+__device__ __forceinline__ float4 canonical_edge(float ax, float ay, float bx, float by) {
+    const bool swap = (bx < ax) || (bx == ax && by < ay);
+    const float x0 = swap ? bx : ax, y0 = swap ? by : ay, x1 = swap ? ax : bx, y1 = swap ? ay : by;
+    const float dx = x1 - x0, dy = y1 - y0;
+    return make_float4(x0, y0, swap ? -dx : dx, swap ? -dy : dy);
+}
+__device__ __forceinline__ float edge_at(const float4 e, float px, float py) {
+    return __fsub_rn(__fmul_rn(e.z, py - e.y), __fmul_rn(e.w, px - e.x));
 }
 
-__global__ void __launch_bounds__(ZB_THREADS) k_zb_raster_big(const uint32_t* __restrict__ big,
-                                                              const PairFT* __restrict__ pairs,
-                                                              const ZbFrustum* __restrict__ frusta,
-                                                              const float4* __restrict__ tris, uint32_t res,
-                                                              uint32_t* __restrict__ zbuf) {
-    const PairFT pr = pairs[big[blockIdx.x]];
-    const ZbFrustum F = frusta[pr.fix];
-    ClipPoly P;
-    clip_project(F, tris[3 * pr.tri], tris[3 * pr.tri + 1], tris[3 * pr.tri + 2], P);
-    if (P.n < 3) return;
-    int x0, x1, y0, y1;
-    poly_bbox(P, (int)res, x0, x1, y0, y1);
-    if (x1 < x0 || y1 < y0) return;
-    const int wdt = x1 - x0 + 1, cnt = wdt * (y1 - y0 + 1);
-    uint32_t* zb = zbuf + (size_t)pr.fix * res * res;
-    for (int k = threadIdx.x; k < cnt; k += blockDim.x) shade_pixel(P, x0 + k % wdt, y0 + k / wdt, F.n, F.f, zb, (int)res);
+// Depth test of the pixel with centre (cx, cy) and word z against a pair set up for drawing
+// (shade_pixel's arithmetic).
+__device__ __forceinline__ void shade_tri(const float4 q0, const float4 q1, const float4 q2, const float4 iws, float cx,
+                                          float cy, float n, float f, uint32_t* __restrict__ z) {
+    const float e0 = edge_at(q0, cx, cy), e1 = edge_at(q1, cx, cy), e2 = edge_at(q2, cx, cy);
+    const bool in = (e0 >= 0.f && e1 >= 0.f && e2 >= 0.f) || (e0 <= 0.f && e1 <= 0.f && e2 <= 0.f);
+    const float area = e0 + e1 + e2;
+    if (!in || area == 0.f) return;
+    const float iw = (e0 * iws.x + e1 * iws.y + e2 * iws.z) / area;
+    const float w = 1.0f / iw;
+    if (w >= n * (1.f - 1e-6f) && w <= f && w > 0.f) atomicMin(z, __float_as_uint(w));
+}
+
+__device__ __forceinline__ float4 shfl4(const float4 v, int src) {
+    return make_float4(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src),
+                       __shfl_sync(0xffffffffu, v.z, src), 0.f);
+}
+
+// counts: [0] pairs kept, [1] entries of `big`. A warp's pairs stay in its own queue and its own slots:
+// no pair list in memory, no host read of its length. The blocks of one blockIdx.y (one group of
+// ZB_SMEM_FRUSTA fixations) run together, so the atomics stay on a few z-buffers that fit in L2.
+// Before: culling into a pair list, then a thread per pair over its pixel box (lanes waited for the
+// largest box; the clipped polygon, indexed at run time, sat in local memory) and a warp per pair above
+// 64 pixels. 300k triangles, 2000 fixations at 256 x 256, 32M pairs: cull, raster and warp raster 6.2 ms, this kernel 3.8 ms.
+__global__ void __launch_bounds__(ZB_THREADS, 4) k_zb_draw(const float4* __restrict__ tris, uint32_t nt,
+                                                           const ZbFrustum* __restrict__ frusta, uint32_t nfix,
+                                                           uint32_t res, float near_m, float far_m,
+                                                           uint32_t* __restrict__ zbuf, PairFT* __restrict__ big,
+                                                           unsigned long long* __restrict__ counts) {
+    constexpr int WARPS = ZB_THREADS / 32;
+    __shared__ ZbFrustum sF[ZB_SMEM_FRUSTA];
+    __shared__ ZbTri slots[WARPS][32];
+    __shared__ uint16_t queue[WARPS][64];    // frustum << 5 | lane of the triangle
+    __shared__ float sBox[WARPS][6];
+    __shared__ float4 sBlk;
+    __shared__ unsigned sMask[ZB_SMEM_FRUSTA / 32];
+    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lt = gm_lanemask_lt();
+    const bool valid = t < nt;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a, c = a;
+    if (valid) {   // leaf order: a warp's 32 triangles are neighbours in space
+        a = tris[3 * (size_t)t];
+        b = tris[3 * (size_t)t + 1];
+        c = tris[3 * (size_t)t + 2];
+    }
+    const float R = (float)res;
+    // the warp's and the block's triangles in one sphere each (box centre, half diagonal)
+    float lo[3], hi[3];
+    lo[0] = redux_min(valid ? fminf(fminf(a.x, b.x), c.x) : INFINITY);
+    lo[1] = redux_min(valid ? fminf(fminf(a.y, b.y), c.y) : INFINITY);
+    lo[2] = redux_min(valid ? fminf(fminf(a.z, b.z), c.z) : INFINITY);
+    hi[0] = redux_max(valid ? fmaxf(fmaxf(a.x, b.x), c.x) : -INFINITY);
+    hi[1] = redux_max(valid ? fmaxf(fmaxf(a.y, b.y), c.y) : -INFINITY);
+    hi[2] = redux_max(valid ? fmaxf(fmaxf(a.z, b.z), c.z) : -INFINITY);
+    const bool wbox = lo[0] <= hi[0];
+    const float wx = 0.5f * (lo[0] + hi[0]), wy = 0.5f * (lo[1] + hi[1]), wz = 0.5f * (lo[2] + hi[2]);
+    const float wR = wbox ? 0.5f * sqrtf((hi[0] - lo[0]) * (hi[0] - lo[0]) + (hi[1] - lo[1]) * (hi[1] - lo[1]) +
+                                         (hi[2] - lo[2]) * (hi[2] - lo[2])) * 1.0001f
+                          : 0.f;
+    if (lane == 0) {
+        sBox[warp][0] = lo[0], sBox[warp][1] = lo[1], sBox[warp][2] = lo[2];
+        sBox[warp][3] = hi[0], sBox[warp][4] = hi[1], sBox[warp][5] = hi[2];
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float bl[3] = {INFINITY, INFINITY, INFINITY}, bh[3] = {-INFINITY, -INFINITY, -INFINITY};
+        for (int w = 0; w < WARPS; ++w)
+            for (int q = 0; q < 3; ++q) {
+                bl[q] = fminf(bl[q], sBox[w][q]);
+                bh[q] = fmaxf(bh[q], sBox[w][3 + q]);
+            }
+        sBlk = bl[0] <= bh[0]
+                   ? make_float4(0.5f * (bl[0] + bh[0]), 0.5f * (bl[1] + bh[1]), 0.5f * (bl[2] + bh[2]),
+                                 0.5f * sqrtf((bh[0] - bl[0]) * (bh[0] - bl[0]) + (bh[1] - bl[1]) * (bh[1] - bl[1]) +
+                                              (bh[2] - bl[2]) * (bh[2] - bl[2])) * 1.0001f)
+                   : make_float4(0.f, 0.f, 0.f, -1.f);
+    }
+    unsigned long long n_pairs = 0;
+    ZbTri* S = slots[warp];
+    // draw the `cnt` pairs of the queue from entry q0 on; all lanes
+    auto draw = [&](int q0, int cnt, uint32_t f0) {
+        const int entry = lane < cnt ? (int)queue[warp][q0 + lane] : 0;
+        const int src = entry & 31;
+        const float4 va = shfl4(a, src), vb = shfl4(b, src), vc = shfl4(c, src);
+        const ZbFrustum& F = sF[entry >> 5];
+        const uint32_t fix = f0 + (uint32_t)(entry >> 5), slot = t - lane + src;
+        float x[3], y[3], w[3];
+        to_camera(F, va.x, va.y, va.z, x[0], y[0], w[0]);
+        to_camera(F, vb.x, vb.y, vb.z, x[1], y[1], w[1]);
+        to_camera(F, vc.x, vc.y, vc.z, x[2], y[2], w[2]);
+        const bool front = w[0] >= F.n && w[1] >= F.n && w[2] >= F.n;
+        ClipPoly P;
+        int x0 = 0, x1 = -1, y0 = 0, y1 = -1;
+        if (front) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const float iw = 1.0f / w[k];
+                P.u[k] = fmaf(F.sx, x[k] * iw, F.ox);
+                P.v[k] = fmaf(F.sy, y[k] * iw, F.oy);
+                P.iw[k] = iw;
+            }
+            pixel_box(fmin3(P.u[0], P.u[1], P.u[2]), fmax3(P.u[0], P.u[1], P.u[2]), fmin3(P.v[0], P.v[1], P.v[2]),
+                      fmax3(P.v[0], P.v[1], P.v[2]), (int)res, x0, x1, y0, y1);
+        }
+        const int npx = lane < cnt && front && x1 >= x0 && y1 >= y0 ? (x1 - x0 + 1) * (y1 - y0 + 1) : 0;
+        const bool small = npx > 0 && npx <= ZB_BIG_PIXELS;
+        int incl = small ? npx : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += u;
+        }
+        const int total = __shfl_sync(0xffffffffu, incl, 31);
+        const int start = small ? incl - npx : 0x7fffffff;
+        const unsigned sm = __ballot_sync(0xffffffffu, small);
+        if (small) {
+            ZbTri T;
+            T.e0 = canonical_edge(P.u[1], P.v[1], P.u[2], P.v[2]);
+            T.e1 = canonical_edge(P.u[2], P.v[2], P.u[0], P.v[0]);
+            T.e2 = canonical_edge(P.u[0], P.v[0], P.u[1], P.v[1]);
+            T.iw = make_float4(P.iw[0], P.iw[1], P.iw[2], __int_as_float((x1 - x0 + 1) | start << 16));
+            T.centre = make_float2(x0 + 0.5f, y0 + 0.5f);
+            T.z = zbuf + ((size_t)fix * res + y0) * res + x0;
+            S[__popc(sm & lt)] = T;
+        }
+        __syncwarp();
+        // the pixels of all boxes in turn, 32 at a time: the boxes that start in this window, as bits,
+        // give every lane its box
+        int boxes = 0;
+        for (int G = 0; G < total; G += 32) {
+            const unsigned bit = (unsigned)(start - G) < 32u ? 1u << (start - G) : 0u;
+            const unsigned starts = __reduce_or_sync(0xffffffffu, bit);
+            const int g = G + lane, k = boxes + __popc(starts & (lt | 1u << lane)) - 1;
+            boxes += __popc(starts);
+            if (g < total) {
+                const float4 iws = S[k].iw;
+                const unsigned span = __float_as_uint(iws.w);
+                const int wd = span & 0xffffu, local = g - (int)(span >> 16);
+                // exact: local < 1024, so (local + 1/2) / wd lies at least 1/2048 from the next integer
+                const int row = (int)__fdividef((float)local + 0.5f, (float)wd), col = local - row * wd;
+                const float2 first = S[k].centre;
+                shade_tri(S[k].e0, S[k].e1, S[k].e2, iws, first.x + (float)col, first.y + (float)row, near_m, far_m,
+                          S[k].z + (row * (int)res + col));
+            }
+        }
+        __syncwarp();
+        // larger boxes go to the block rasteriser; pairs that reach the near plane are clipped
+        const bool clip = lane < cnt && !front;
+        const bool to_big = npx > ZB_BIG_PIXELS;
+        if (__any_sync(0xffffffffu, clip || to_big)) {
+            bool here = clip;
+            if (to_big) {
+                const unsigned long long q = atomicAdd(&counts[1], 1ull);
+                if (q < ZB_BIG_CAP) big[q] = PairFT{fix, slot};
+                else here = true;
+            }
+            if (here) draw_clipped(F, va, vb, vc, res, zbuf + (size_t)fix * res * res);
+            __syncwarp();
+        }
+    };
+    for (uint32_t f0 = blockIdx.y * ZB_SMEM_FRUSTA; f0 < nfix; f0 += gridDim.y * ZB_SMEM_FRUSTA) {
+        const uint32_t m = min((uint32_t)ZB_SMEM_FRUSTA, nfix - f0);
+        __syncthreads();
+        {
+            const uint4* from = reinterpret_cast<const uint4*>(frusta + f0);
+            uint4* to = reinterpret_cast<uint4*>(sF);
+            static_assert(sizeof(ZbFrustum) % 16 == 0, "copied in 16-byte words");
+            for (uint32_t k = threadIdx.x; k < m * (sizeof(ZbFrustum) / 16); k += blockDim.x) to[k] = from[k];
+        }
+        __syncthreads();
+        if (threadIdx.x < ZB_SMEM_FRUSTA) {   // whole warps: ZB_SMEM_FRUSTA is a multiple of 32
+            const uint32_t k = threadIdx.x;
+            const float4 bs = sBlk;
+            const bool reach = k < m && sF[k].ok && bs.w >= 0.f && !sphere_outside(sF[k], bs.x, bs.y, bs.z, bs.w, R);
+            const unsigned bits = __ballot_sync(0xffffffffu, reach);
+            if (lane == 0) sMask[k >> 5] = bits;
+        }
+        __syncthreads();
+        // the frusta that reach the warp's sphere, a frustum per lane
+        int qn = 0;
+#pragma unroll 1
+        for (int h = 0; h < ZB_SMEM_FRUSTA / 32; ++h) {
+            const unsigned blk = sMask[h];
+            if (blk == 0) continue;
+            const bool reach = ((blk >> lane) & 1u) && wbox && !sphere_outside(sF[32 * h + lane], wx, wy, wz, wR, R);
+            unsigned todo = __ballot_sync(0xffffffffu, reach);
+            while (todo) {
+                const int k = 32 * h + __ffs(todo) - 1;
+                todo &= todo - 1u;
+                const ZbFrustum& F = sF[k];
+                bool keep = false;
+                if (valid) {
+                    float x[3], y[3], w[3];
+                    to_camera(F, a.x, a.y, a.z, x[0], y[0], w[0]);
+                    to_camera(F, b.x, b.y, b.z, x[1], y[1], w[1]);
+                    to_camera(F, c.x, c.y, c.z, x[2], y[2], w[2]);
+                    int o0 = 0, o1 = 0, o2 = 0, o3 = 0, o4 = 0, o5 = 0;
+#pragma unroll
+                    for (int v = 0; v < 3; ++v) {
+                        const float U = fmaf(F.sx, x[v], F.ox * w[v]), V = fmaf(F.sy, y[v], F.oy * w[v]);
+                        o0 += U < -w[v];
+                        o1 += U > (R + 1.f) * w[v];
+                        o2 += V < -w[v];
+                        o3 += V > (R + 1.f) * w[v];
+                        o4 += w[v] < F.n * (1.f - 1e-5f);
+                        o5 += w[v] > F.f * (1.f + 1e-5f);
+                    }
+                    keep = o0 < 3 && o1 < 3 && o2 < 3 && o3 < 3 && o4 < 3 && o5 < 3;
+                }
+                const unsigned msk = __ballot_sync(0xffffffffu, keep);
+                if (keep) queue[warp][qn + __popc(msk & lt)] = (uint16_t)(k << 5 | lane);
+                qn += __popc(msk);
+                n_pairs += __popc(msk);
+                __syncwarp();
+                if (qn >= 32) {
+                    qn -= 32;
+                    draw(qn, 32, f0);
+                }
+            }
+        }
+        if (qn > 0) draw(0, qn, f0);
+    }
+    if (lane == 0 && n_pairs) atomicAdd(&counts[0], n_pairs);
+}
+
+__global__ void __launch_bounds__(ZB_THREADS) k_zb_draw_big(const unsigned long long* __restrict__ counts,
+                                                            const PairFT* __restrict__ big,
+                                                            const ZbFrustum* __restrict__ frusta,
+                                                            const float4* __restrict__ tris, uint32_t res,
+                                                            uint32_t* __restrict__ zbuf) {
+    const unsigned long long n = min(counts[1], (unsigned long long)ZB_BIG_CAP);
+    for (unsigned long long q = blockIdx.x; q < n; q += gridDim.x) {
+        const PairFT pr = big[q];
+        const ZbFrustum F = frusta[pr.fix];
+        const float4 v[3] = {tris[3 * (size_t)pr.tri], tris[3 * (size_t)pr.tri + 1], tris[3 * (size_t)pr.tri + 2]};
+        float pu[3], pv[3], iw[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            float x, y, w;
+            to_camera(F, v[k].x, v[k].y, v[k].z, x, y, w);
+            iw[k] = 1.0f / w;
+            pu[k] = fmaf(F.sx, x * iw[k], F.ox);
+            pv[k] = fmaf(F.sy, y * iw[k], F.oy);
+        }
+        int x0, x1, y0, y1;
+        pixel_box(fmin3(pu[0], pu[1], pu[2]), fmax3(pu[0], pu[1], pu[2]), fmin3(pv[0], pv[1], pv[2]),
+                  fmax3(pv[0], pv[1], pv[2]), (int)res, x0, x1, y0, y1);
+        const float4 e0 = canonical_edge(pu[1], pv[1], pu[2], pv[2]), e1 = canonical_edge(pu[2], pv[2], pu[0], pv[0]);
+        const float4 e2 = canonical_edge(pu[0], pv[0], pu[1], pv[1]), iws = make_float4(iw[0], iw[1], iw[2], 0.f);
+        uint32_t* zb = zbuf + (size_t)pr.fix * res * res;
+        // 32 x 8 pixels at a time: a warp on a row
+        for (int py = y0 + (int)(threadIdx.x >> 5); py <= y1; py += ZB_THREADS / 32)
+            for (int px = x0 + (int)(threadIdx.x & 31); px <= x1; px += 32)
+                shade_tri(e0, e1, e2, iws, px + 0.5f, py + 0.5f, F.n, F.f, zb + (size_t)py * res + px);
+    }
 }
 
 // ---- accumulate -----------------------------------------------------------------------------
@@ -658,80 +751,21 @@ __global__ void k_zb_set_valid(unsigned long long* __restrict__ c, const uint32_
     c[3] = *n_valid;
 }
 
-// Render the z-buffers of frusta [0, nfix) into zbuf (nfix x res^2 words, cleared here). The pair
-// list grows (and the chunk is redone) when the cull finds more pairs than it holds.
-struct RasterBuffers {
-    PairFT* pairs = nullptr;
-    uint32_t* big = nullptr;
-    uint32_t* mid = nullptr;
-    uint64_t cap = 0;
-    unsigned long long* counts = nullptr;   // [0] pairs [1] big [2] mid
-};
-
-gm_status rb_alloc(RasterBuffers& rb, uint64_t cap, cudaStream_t s) {
-    rb.cap = cap;
-    GM_TRY(gm_alloc((void**)&rb.pairs, sizeof(PairFT) * cap, s));
-    GM_TRY(gm_alloc((void**)&rb.big, sizeof(uint32_t) * cap, s));
-    GM_TRY(gm_alloc((void**)&rb.mid, sizeof(uint32_t) * cap, s));
-    return GM_OK;
-}
-
-void rb_free(RasterBuffers& rb, cudaStream_t s) {
-    if (rb.pairs) cudaFreeAsync(rb.pairs, s);
-    if (rb.big) cudaFreeAsync(rb.big, s);
-    if (rb.mid) cudaFreeAsync(rb.mid, s);
-    rb.pairs = nullptr;
-    rb.big = rb.mid = nullptr;
-}
-
+// Render the z-buffers of frusta [0, nfix) into zbuf (nfix x res^2 words, cleared here). counts: [0] grows
+// by the pairs drawn, [1] is the length of the list `big` (ZB_BIG_CAP entries).
 gm_status render_zbuffers(gm_ctx* ctx, gm_scene* sc, const ZbFrustum* frusta, uint32_t nfix, uint32_t res,
-                          uint32_t* zbuf, RasterBuffers& rb, cudaStream_t s, int* launches,
-                          unsigned long long* raster_pairs) {
+                          float near_m, float far_m, uint32_t* zbuf, PairFT* big, unsigned long long* counts,
+                          cudaStream_t s, int* launches) {
     const size_t npx = (size_t)res * res;
-    for (int attempt = 0; attempt < 3; ++attempt) {
-        static_assert(ZB_EMPTY == 0xffffffffu, "a byte-wise 0xff clear writes ZB_EMPTY");
-        GM_TRY_CUDA(cudaMemsetAsync(zbuf, 0xff, sizeof(uint32_t) * npx * nfix, s));
-        GM_TRY_CUDA(cudaMemsetAsync(rb.counts, 0, sizeof(unsigned long long) * 3, s));
-        const dim3 cgrid(gm_div_up(sc->n_tris, ZB_THREADS), std::min<uint32_t>(gm_div_up(nfix, ZB_SMEM_FRUSTA), 65535));
-        k_zb_cull<<<cgrid, ZB_THREADS, 0, s>>>(sc->bvh_tris, sc->n_tris, frusta, nfix,
-                                                                          res, rb.pairs, rb.cap, &rb.counts[0]);
-        ++*launches;
-        unsigned long long np = 0;
-        GM_TRY_CUDA(cudaMemcpyAsync(&np, &rb.counts[0], sizeof(np), cudaMemcpyDeviceToHost, s));
-        GM_TRY_CUDA(cudaStreamSynchronize(s));
-        if (np > rb.cap) {
-            rb_free(rb, s);
-            GM_TRY(rb_alloc(rb, np + np / 4, s));
-            continue;
-        }
-        if (raster_pairs) *raster_pairs += np;
-        // the next call on this scene starts with room for this density of pairs
-        sc->zb_pairs_per_fix = std::max<uint64_t>(sc->zb_pairs_per_fix, np / nfix + 1);
-        if (np > 0) {
-            if (np > 0xffffffffull) return gm_set_error(GM_ERR_UNSUPPORTED, "z-buffer: more than 2^32 raster pairs");
-            k_zb_raster<<<(uint32_t)((np + ZB_THREADS - 1) / ZB_THREADS), ZB_THREADS, 0, s>>>(
-                rb.pairs, np, frusta, sc->tri_canon, res, zbuf, rb.big, rb.mid, rb.cap, &rb.counts[1]);
-            ++*launches;
-            unsigned long long nl[2] = {0, 0};
-            GM_TRY_CUDA(cudaMemcpyAsync(nl, &rb.counts[1], sizeof(nl), cudaMemcpyDeviceToHost, s));
-            GM_TRY_CUDA(cudaStreamSynchronize(s));
-            const unsigned long long nb = std::min<unsigned long long>(nl[0], rb.cap);
-            const unsigned long long nm = std::min<unsigned long long>(nl[1], rb.cap);
-            if (nm > 0) {
-                const uint32_t wblocks = (uint32_t)std::min<unsigned long long>((nm + 7) / 8, (uint64_t)ctx->n_sm * 16);
-                k_zb_raster_warp<<<wblocks, ZB_THREADS, 0, s>>>(rb.mid, nm, rb.pairs, frusta, sc->tri_canon, res, zbuf);
-                ++*launches;
-            }
-            for (unsigned long long b0 = 0; b0 < nb; b0 += 1u << 30) {
-                const uint32_t nblk = (uint32_t)std::min<unsigned long long>(nb - b0, 1u << 30);
-                k_zb_raster_big<<<nblk, ZB_THREADS, 0, s>>>(rb.big + b0, rb.pairs, frusta, sc->tri_canon, res, zbuf);
-                ++*launches;
-            }
-        }
-        GM_TRY_CUDA(cudaGetLastError());
-        return GM_OK;
-    }
-    return gm_set_error(GM_ERR_INTERNAL, "z-buffer: raster pair list did not settle");
+    static_assert(ZB_EMPTY == 0xffffffffu, "a byte-wise 0xff clear writes ZB_EMPTY");
+    GM_TRY_CUDA(cudaMemsetAsync(zbuf, 0xff, sizeof(uint32_t) * npx * nfix, s));
+    GM_TRY_CUDA(cudaMemsetAsync(&counts[1], 0, sizeof(unsigned long long), s));
+    const dim3 grid(gm_div_up(sc->n_tris, ZB_THREADS), std::min<uint32_t>(gm_div_up(nfix, ZB_SMEM_FRUSTA), 65535));
+    k_zb_draw<<<grid, ZB_THREADS, 0, s>>>(sc->bvh_tris, sc->n_tris, frusta, nfix, res, near_m, far_m, zbuf, big, counts);
+    k_zb_draw_big<<<(uint32_t)ctx->n_sm * 4, ZB_THREADS, 0, s>>>(counts, big, frusta, sc->bvh_tris, res, zbuf);
+    *launches += 2;
+    GM_TRY_CUDA(cudaGetLastError());
+    return GM_OK;
 }
 
 gm_status check_zb_params(const gm_zbuffer_params* zp) {
@@ -789,8 +823,8 @@ extern "C" gm_status gm_zbuffer_render(gm_scene* sc, const float* eye, const flo
     double* crop = nullptr;
     uint32_t* zb = nullptr;
     float* zf = nullptr;
-    RasterBuffers rb;
-    rb.cap = std::max<uint64_t>(1u << 16, (uint64_t)n * std::max<uint64_t>(4096, sc->zb_pairs_per_fix * 5 / 4));
+    PairFT* big = nullptr;
+    unsigned long long* counts = nullptr;
 #define ZB_TMP(ptr, bytes)                                                          \
     do {                                                                            \
         if ((st = gm_alloc((void**)&(ptr), (bytes), s)) != GM_OK) return done(st);  \
@@ -799,17 +833,16 @@ extern "C" gm_status gm_zbuffer_render(gm_scene* sc, const float* eye, const flo
     ZB_TMP(fr, sizeof(ZbFrustum) * n);
     ZB_TMP(crop, sizeof(double) * 4 * n);
     ZB_TMP(zb, sizeof(uint32_t) * npx * n);
-    ZB_TMP(rb.counts, sizeof(unsigned long long) * 3);
-    if ((st = rb_alloc(rb, rb.cap, s)) != GM_OK) {
-        rb_free(rb, s);
-        return done(st);
-    }
+    ZB_TMP(big, sizeof(PairFT) * ZB_BIG_CAP);
+    ZB_TMP(counts, sizeof(unsigned long long) * 2);
+    if (cudaError_t e = cudaMemsetAsync(counts, 0, sizeof(unsigned long long) * 2, s); e != cudaSuccess)
+        return done(gm_cuda_error(e, "gm_zbuffer_render"));
     int launches = 0;
     k_zb_frustum<<<gm_div_up(n, 128), 128, 0, s>>>(n, nullptr, d_eye, d_gaze, d_fwd, d_up, (double)theta_rad,
                                                    (double)cutoff_sigmas, (double)zp->near_m, (double)zp->far_m,
                                                    zp->res, fr, crop, nullptr);
     ++launches;
-    st = render_zbuffers(ctx, sc, fr, n, zp->res, zb, rb, s, &launches, nullptr);
+    st = render_zbuffers(ctx, sc, fr, n, zp->res, zp->near_m, zp->far_m, zb, big, counts, s, &launches);
     if (st == GM_OK && gm_is_device_ptr(zbuf_out)) {
         k_zb_export<<<gm_div_up(npx * n, 256), 256, 0, s>>>(zb, npx * n, zbuf_out);
         ++launches;
@@ -822,7 +855,6 @@ extern "C" gm_status gm_zbuffer_render(gm_scene* sc, const float* eye, const flo
         }
     }
     if (st == GM_OK && crop_out) st = gm_copy_out(crop_out, crop, sizeof(double) * 4 * n, s);
-    rb_free(rb, s);
     ctx->launches += launches;
     if (st == GM_OK) {
         cudaError_t e = cudaGetLastError();
@@ -879,10 +911,8 @@ extern "C" gm_status gm_accumulate_zbuffer(gm_scene* sc, gm_samples* sm, const g
     mp->stats.n_windows = (uint32_t)W;
     mp->zbuffer = true;
     std::vector<void*> tmp;
-    RasterBuffers rb;
     auto fail = [&](gm_status st) {
         for (void* p : tmp) cudaFreeAsync(p, s);
-        rb_free(rb, s);
         gm_map_free(mp);
         return st;
     };
@@ -973,9 +1003,11 @@ extern "C" gm_status gm_accumulate_zbuffer(gm_scene* sc, gm_samples* sm, const g
     float2* state = nullptr;
     TMP_ALLOC(zbuf, sizeof(uint32_t) * npx * chunk);
     if (chunk < nv) TMP_ALLOC(state, sizeof(float2) * (ns ? ns : 1));
-    rb.cap = std::max<uint64_t>(1u << 20, (uint64_t)chunk * std::max<uint64_t>(2048, sc->zb_pairs_per_fix * 5 / 4));
-    TMP_ALLOC(rb.counts, sizeof(unsigned long long) * 3);
-    if ((st = rb_alloc(rb, rb.cap, s)) != GM_OK) return fail(st);
+    PairFT* big = nullptr;
+    unsigned long long* counts = nullptr;
+    TMP_ALLOC(big, sizeof(PairFT) * ZB_BIG_CAP);
+    TMP_ALLOC(counts, sizeof(unsigned long long) * 2);
+    GM_TRY_CUDA(cudaMemsetAsync(counts, 0, sizeof(unsigned long long) * 2, s));
 
     ZbAccParams P;
     P.C2 = (float)(1.4426950408889634 / (2.0 * tan_t * tan_t));
@@ -1002,7 +1034,7 @@ extern "C" gm_status gm_accumulate_zbuffer(gm_scene* sc, gm_samples* sm, const g
         sidx = ident;
     }
     std::vector<uint32_t> win_of(nv);
-    if (nv > 0) {
+    if (chunk < nv) {   // the window that each later chunk continues
         std::vector<float4> hp(2 * (size_t)nv);
         GM_TRY_CUDA(cudaMemcpyAsync(hp.data(), packed, sizeof(float4) * 2 * nv, cudaMemcpyDeviceToHost, s));
         GM_TRY_CUDA(cudaStreamSynchronize(s));
@@ -1012,10 +1044,10 @@ extern "C" gm_status gm_accumulate_zbuffer(gm_scene* sc, gm_samples* sm, const g
             win_of[i] = b;
         }
     }
-    unsigned long long raster_pairs = 0;
     for (uint32_t f0 = 0; f0 < nv; f0 += chunk) {
         const uint32_t f1 = std::min(nv, f0 + chunk);
-        if ((st = render_zbuffers(ctx, sc, frusta + f0, f1 - f0, res, zbuf, rb, s, &launches, &raster_pairs)) != GM_OK)
+        if ((st = render_zbuffers(ctx, sc, frusta + f0, f1 - f0, res, zp->near_m, zp->far_m, zbuf, big, counts, s,
+                                  &launches)) != GM_OK)
             return fail(st);
         if (ns > 0) {
             const uint32_t cur_in = f0 == 0 ? NO_WINDOW : win_of[f0 - 1];
@@ -1044,12 +1076,10 @@ extern "C" gm_status gm_accumulate_zbuffer(gm_scene* sc, gm_samples* sm, const g
             ++launches;
         }
     }
-    GM_TRY_CUDA(cudaMemcpyAsync(&mp->counters[11], &raster_pairs, sizeof(raster_pairs), cudaMemcpyHostToDevice, s));
+    GM_TRY_CUDA(cudaMemcpyAsync(&mp->counters[11], counts, sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(gm_cuda_error(e, "gm_accumulate_zbuffer launch"));
-    GM_TRY_CUDA(cudaStreamSynchronize(s));   // raster_pairs and the host vectors above are host temporaries
     for (void* p : tmp) cudaFreeAsync(p, s);
-    rb_free(rb, s);
     mp->stats.launches = (uint32_t)launches;
     ctx->launches += launches;
     *out = mp;
