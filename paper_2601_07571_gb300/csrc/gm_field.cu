@@ -259,36 +259,46 @@ __global__ void __launch_bounds__(256) k_field_query(const float* __restrict__ x
 
 
 // ---- inference on the 5th-generation tensor cores ---------------------------------------------
-// Blocks of 256 threads, persistent; each half (128 threads, its own named barrier) runs its own
-// pipeline over tiles of 128 points (the MMA's M), so two tiles per block -- and those of the other
-// resident blocks -- overlap one tile's tensor-core products with another's epilogue, while the
-// weights are staged once per block. Per tile: the point coordinates arrive by a bulk asynchronous
-// copy (double-buffered, the next tile's copy in flight while this one computes; plain loads when
-// the input is not 16-byte aligned or the tile is the ragged tail); thread t of the half encodes
-// point t's 64 features into row t of its A tile (bf16, K-major core-matrix layout: 8 x 8 blocks
-// of 128 bytes); per layer one thread issues four tcgen05.mma (M 128, N 64, K 16, bf16 x bf16 ->
-// FP32 in tensor memory, columns 64 h .. 64 h + 63 for half h) and commits them to the half's
-// mbarrier; every thread then reads its row of the accumulator with tcgen05.ld, adds the bias,
-// applies ReLU, rounds to bf16 and writes the next A row. The output layer is
-// a fifth product with N = 16 whose B rows are the three bf16 parts of w5. Waits are bounded: on a
-// timeout the block records GM_DEV_WAIT_TIMEOUT, drains its own copies, frees its tensor memory and
-// returns.
-constexpr int TQ = 128;                       // points per tile (threads per half)
-constexpr int TQ_THREADS = 2 * TQ;
-constexpr uint32_t TQ_TMEM_COLS = 128;        // two FP32 accumulators of N = 64
+// One persistent block of TQ_H groups of 128 threads per SM; each group (its own named barrier and
+// mbarriers, 96 tensor-memory columns) runs its own pipeline over tiles of 128 points (the MMA's M),
+// so one tile's tensor-core products overlap the others' epilogues, while the weights are staged once
+// per SM. Per tile: the point coordinates arrive by a bulk asynchronous copy (double-buffered, the
+// next tile's copy in flight while this one computes; plain loads when the input is not 16-byte
+// aligned or the tile is the ragged tail); thread t of the group encodes point t's 64 features as
+// packed bf16 pairs into row t of the A operand in tensor memory (32 columns); per layer one thread
+// issues five tcgen05.mma (M 128, N 64, K 16, A in tensor memory, B in shared memory, FP32 accumulator
+// in tensor memory) and commits them to the group's mbarrier: the first puts the bias into the
+// accumulator (A = ones, B = the three bf16 parts of every bias, which sum to it exactly), the others
+// add the layer's products; every thread then reads its row of the accumulator with tcgen05.ld, applies
+// ReLU while rounding to bf16 and writes the next A row with tcgen05.st. The output layer is a fifth
+// product with N = 16 whose B rows are the three bf16 parts of w5. Waits are bounded: on a timeout the
+// group records GM_DEV_WAIT_TIMEOUT, drains its own copies and stops; the block frees its tensor memory
+// and returns.
+//
+// Bound by the latency of a tile's five rounds of product and epilogue, five tiles at a time (a tile: 700
+// cycles of products, 4 x 828 warp instructions). With A in shared memory the products (6 KB a K step, 48 cycles at 128 bytes a cycle
+// against 32 of arithmetic) and the A rows' stores filled the shared-memory pipe: 10M points 603 us with
+// three blocks of two groups and the bias added by the threads, 547 us with eight groups and the bias as
+// a product; 437 us as it is (ncu: issue 50 %, tensor pipe 40 %, 828 instructions a warp and tile).
+constexpr int TQ = 128;                       // points per tile (threads per group)
+constexpr int TQ_H = 5;                       // groups per block: 96 of 512 tensor-memory columns each
+constexpr int TQ_THREADS = TQ_H * TQ;
+constexpr uint32_t TQ_TMEM_COLS = 512;
+constexpr uint32_t TQ_COL_D = 0;              // accumulators: 64 columns per group
+constexpr uint32_t TQ_COL_A = 64 * TQ_H;      // A operands: 32 columns per group (two bf16 a column)
+constexpr uint32_t TQ_COL_ONE = 96 * TQ_H;    // the biases' A (K = 16): ones in k = 0..2, 8 columns
 constexpr int TQ_WAIT_ITERS = 1 << 22;
 
 struct QuerySmem {
-    alignas(1024) __nv_bfloat16 A[2][TQ * FW];    // 2 x 16 KB
-    alignas(1024) __nv_bfloat16 W[FD][FW * FW];   // 32 KB
-    alignas(1024) __nv_bfloat16 W5[16 * FW];      // output layer as B (N = 16): w5 = hi + mid + lo in rows 0..2
-    alignas(16) float bias[FD * FW];
-    float w5[FW + 1];
-    alignas(16) float xyz[2][2][TQ * 3];          // [half][buffer]
-    alignas(8) uint64_t mbar_mma[2];
-    uint64_t mbar_ld[2][2];
+    alignas(1024) __nv_bfloat16 W[FD][FW * FW];     // 32 KB
+    alignas(1024) __nv_bfloat16 WB[FD][FW * 16];    // biases as B (K = 16): bias = hi + mid + lo in k = 0..2
+    alignas(1024) __nv_bfloat16 W5[16 * FW];        // output layer as B (N = 16): w5 = hi + mid + lo in rows 0..2
+    alignas(16) float xyz[TQ_H][2][TQ * 3];         // [group][buffer]
+    alignas(8) uint64_t mbar_mma[TQ_H];
+    uint64_t mbar_ld[TQ_H][2];
+    float b5;
     uint32_t tmem;
-    int abort;
+    int abort[TQ_H];
 };
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -349,22 +359,8 @@ __device__ __forceinline__ void bulk_load(float* dst, const float* src, uint32_t
         : "memory");
 }
 
-__device__ __forceinline__ void half_sync(int h) {
-    if (h == 0) asm volatile("bar.sync 1, 128;" ::: "memory");
-    else asm volatile("bar.sync 2, 128;" ::: "memory");
-}
-
-// Row t of an A tile: 64 values as bf16, eight 16-byte stores into the core-matrix layout.
-__device__ __forceinline__ void store_a_row(__nv_bfloat16* A, int t, const float* v) {
-#pragma unroll
-    for (int kg = 0; kg < 8; ++kg) {
-        uint4 q;
-        q.x = pack_bf16(v[8 * kg + 0], v[8 * kg + 1]);
-        q.y = pack_bf16(v[8 * kg + 2], v[8 * kg + 3]);
-        q.z = pack_bf16(v[8 * kg + 4], v[8 * kg + 5]);
-        q.w = pack_bf16(v[8 * kg + 6], v[8 * kg + 7]);
-        *reinterpret_cast<uint4*>(reinterpret_cast<char*>(A) + kg * 2048 + (t >> 3) * 128 + (t & 7) * 16) = q;
-    }
+__device__ __forceinline__ void group_sync(int h) {   // the 128 threads of group h
+    asm volatile("bar.sync %0, 128;" ::"r"(h + 1) : "memory");
 }
 
 // The 64 features of one point for the tensor-core kernel: sine and cosine of 2^k pi x~ from an
@@ -408,19 +404,72 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
     for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
 }
 
-__global__ void __launch_bounds__(TQ_THREADS, 3) k_field_query_tc(const float* __restrict__ xyz, uint64_t n,
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* w) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(w[0]), "r"(w[1]),
+                 "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]));
+}
+
+// The same 64 features as packed bf16 pairs into this thread's row of an A operand in tensor memory, 8
+// columns at a time as their values come up (few of them live at once).
+__device__ __forceinline__ void encode_row(const float xt[3], uint32_t a_row) {
+    float held = 0.f;
+    uint32_t w[8];
+    auto put = [&](int j, float v) {   // feature j, in order; j is known at compile time
+        if (j & 1) w[(j >> 1) & 7] = pack_bf16(held, v);
+        else held = v;
+        if ((j & 15) == 15) tmem_st8(a_row + (j >> 4) * 8, w);
+    };
+    put(0, xt[0]);
+    put(1, xt[1]);
+    put(2, xt[2]);
+    float sn[3], cs[3];
+#pragma unroll
+    for (int k = 0; k < FOCT; ++k) {
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            if (k % 3 == 0) {
+                float y = ldexpf(xt[r], k);
+                y = y - 2.f * rintf(0.5f * y);
+                __sincosf(3.14159265358979f * y, &sn[r], &cs[r]);
+            } else {
+                const float s2 = 2.f * (sn[r] * cs[r]);
+                const float c2 = fmaf(cs[r], cs[r], -(sn[r] * sn[r]));
+                sn[r] = s2;
+                cs[r] = c2;
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 3; ++r) put(3 + 6 * k + r, sn[r]);
+#pragma unroll
+        for (int r = 0; r < 3; ++r) put(6 + 6 * k + r, cs[r]);
+    }
+    put(63, 0.f);
+}
+
+__global__ void __launch_bounds__(TQ_THREADS, 1) k_field_query_tc(const float* __restrict__ xyz, uint64_t n,
                                                               const __nv_bfloat16* __restrict__ wbf,
                                                               const float* __restrict__ theta, FieldBox B, int bulk,
                                                               float* __restrict__ out, int* __restrict__ err) {
     extern __shared__ __align__(1024) unsigned char q_smem_raw[];
     QuerySmem& S = *reinterpret_cast<QuerySmem*>(q_smem_raw);
     const int tid = threadIdx.x, warp = tid >> 5;
-    const int h = tid / TQ, t = tid % TQ;   // half and row within the half's tile
+    const int h = tid / TQ, t = tid % TQ;   // group and row within the group's tile
     // weights in the core-matrix layout: (n, k) at (k / 8) * 1024 + (n / 8) * 128 + (n % 8) * 16 + (k % 8) * 2
     for (int i = tid; i < FD * FW * 8; i += TQ_THREADS) {
         const int l = i / (FW * 8), nn = (i / 8) % FW, kg = i % 8;
         const uint4 q = reinterpret_cast<const uint4*>(wbf + (size_t)l * FW * FW + nn * FW)[kg];
         *reinterpret_cast<uint4*>(reinterpret_cast<char*>(S.W[l]) + kg * 1024 + (nn >> 3) * 128 + (nn & 7) * 16) = q;
+    }
+    // the biases, K = 16: parts in k = 0..2, zeros above
+    for (int i = tid; i < FD * FW; i += TQ_THREADS) {
+        const int l = i / FW, nn = i % FW;
+        __nv_bfloat16 part[3];
+        split3_bf16(theta[b_off(l) + nn], part);
+        char* row = reinterpret_cast<char*>(S.WB[l]) + (nn >> 3) * 128 + (nn & 7) * 16;
+        *reinterpret_cast<uint4*>(row) =
+            make_uint4(__bfloat16_as_ushort(part[0]) | (uint32_t)__bfloat16_as_ushort(part[1]) << 16,
+                       __bfloat16_as_ushort(part[2]), 0u, 0u);
+        *reinterpret_cast<uint4*>(row + 1024) = make_uint4(0u, 0u, 0u, 0u);
     }
     // the output layer as a 16 x 64 B operand: rows 0..2 the three bf16 parts of w5, the rest zero;
     // (n, k) at (k / 8) * 256 + (n / 8) * 128 + (n % 8) * 16 + (k % 8) * 2
@@ -432,11 +481,10 @@ __global__ void __launch_bounds__(TQ_THREADS, 3) k_field_query_tc(const float* _
         *reinterpret_cast<__nv_bfloat16*>(reinterpret_cast<char*>(S.W5) + (k >> 3) * 256 + (nn >> 3) * 128 +
                                           (nn & 7) * 16 + (k & 7) * 2) = v;
     }
-    for (int i = tid; i < FD * FW; i += TQ_THREADS) S.bias[i] = theta[b_off(i / FW) + i % FW];
-    for (int i = tid; i <= FW; i += TQ_THREADS) S.w5[i] = theta[W5_OFF + i];
     if (tid == 0) {
-        S.abort = 0;
-        for (int k = 0; k < 2; ++k) {
+        S.b5 = theta[B5_OFF];
+        for (int k = 0; k < TQ_H; ++k) {
+            S.abort[k] = 0;
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&S.mbar_mma[k])));
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&S.mbar_ld[k][0])));
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&S.mbar_ld[k][1])));
@@ -452,124 +500,116 @@ __global__ void __launch_bounds__(TQ_THREADS, 3) k_field_query_tc(const float* _
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
-    const uint32_t tmem_h = S.tmem + (uint32_t)(h * FW);         // this half's accumulator columns
-    const uint32_t row_addr = tmem_h + ((uint32_t)((warp & 3) * 32) << 16);
-    __nv_bfloat16* A = S.A[h];
-    const uint32_t a_addr = smem_addr(A);
+    const uint32_t lanes = (uint32_t)((warp & 3) * 32) << 16;    // this warp's rows of the tile
+    const uint32_t d_cols = S.tmem + TQ_COL_D + 64 * h, a_cols = S.tmem + TQ_COL_A + 32 * h, one_cols = S.tmem + TQ_COL_ONE;
+    const uint32_t d_row = d_cols + lanes, a_row = a_cols + lanes, mbar = smem_addr(&S.mbar_mma[h]);
+    if (h == 0) {
+        const uint32_t one[8] = {0x3F803F80u, 0x3F80u, 0u, 0u, 0u, 0u, 0u, 0u};   // bf16 1, 1, 1, 0, ...
+        tmem_st8(one_cols + lanes, one);
+        asm volatile("tcgen05.wait::st.sync.aligned;");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
     const uint64_t ntiles = (n + TQ - 1) / TQ;
-    const uint64_t pipes = 2ull * gridDim.x, pipe = 2ull * blockIdx.x + h;
-    uint32_t pm = 0, pl[2] = {0, 0};
-    bool pending[2] = {false, false};   // row 0 of the half: a bulk copy into this buffer is in flight
+    // few tiles go to as many SMs as there are
+    const uint64_t pipes = (uint64_t)TQ_H * gridDim.x;
+    uint32_t pm = 0, pl = 0;            // phases: products; copies (bit per buffer)
+    uint32_t pending = 0;               // row 0 of the group: bulk copies in flight (bit per buffer)
     auto full_tile = [&](uint64_t tile) { return (tile + 1) * TQ <= n; };
-    uint64_t tile = pipe;
+    uint64_t tile = blockIdx.x + (uint64_t)h * gridDim.x;
     if (t == 0 && bulk && tile < ntiles && full_tile(tile)) {
         bulk_load(S.xyz[h][0], xyz + tile * TQ * 3, TQ * 12, &S.mbar_ld[h][0]);
-        pending[0] = true;
+        pending = 1;
     }
-    bool stop = false;
-    for (int it = 0; tile < ntiles && !stop; ++it, tile += pipes) {
-        const int buf = it & 1;
+    for (int buf = 0; tile < ntiles; buf ^= 1, tile += pipes) {
         const uint64_t next = tile + pipes;
         if (t == 0 && bulk && next < ntiles && full_tile(next)) {
             bulk_load(S.xyz[h][buf ^ 1], xyz + next * TQ * 3, TQ * 12, &S.mbar_ld[h][buf ^ 1]);
-            pending[buf ^ 1] = true;
+            pending |= 2u >> buf;
         }
         const uint64_t i = tile * TQ + t;
-        float x[3] = {0.f, 0.f, 0.f};
+        float xt[3] = {0.f, 0.f, 0.f};
         if (bulk && full_tile(tile)) {
-            if (!mbar_wait(smem_addr(&S.mbar_ld[h][buf]), pl[buf])) S.abort = 1;
-            pl[buf] ^= 1;
-            if (t == 0) pending[buf] = false;
-            x[0] = S.xyz[h][buf][3 * t];
-            x[1] = S.xyz[h][buf][3 * t + 1];
-            x[2] = S.xyz[h][buf][3 * t + 2];
+            if (!mbar_wait(smem_addr(&S.mbar_ld[h][buf]), (pl >> buf) & 1u)) S.abort[h] = 1;
+            pl ^= 1u << buf;
+            pending &= ~(1u << buf);
+            xt[0] = S.xyz[h][buf][3 * t];
+            xt[1] = S.xyz[h][buf][3 * t + 1];
+            xt[2] = S.xyz[h][buf][3 * t + 2];
         } else if (i < n) {
-            x[0] = xyz[3 * i];
-            x[1] = xyz[3 * i + 1];
-            x[2] = xyz[3 * i + 2];
+            xt[0] = xyz[3 * i];
+            xt[1] = xyz[3 * i + 1];
+            xt[2] = xyz[3 * i + 2];
         }
-        float xt[3] = {(x[0] - B.cx) * B.inv_h, (x[1] - B.cy) * B.inv_h, (x[2] - B.cz) * B.inv_h};
-        float v[FW];
-        features_fast(xt, v);
-        store_a_row(A, t, v);
+        xt[0] = (xt[0] - B.cx) * B.inv_h;
+        xt[1] = (xt[1] - B.cy) * B.inv_h;
+        xt[2] = (xt[2] - B.cz) * B.inv_h;
+        encode_row(xt, a_row);
         // four hidden layers, then the output layer (l == FD) as one more product: A = h4, B = the
         // three parts of w5, so z5 - b5 is the sum of the first three accumulator columns. Each
-        // product starts a fresh accumulator (the previous tile's last read is complete); the bias
-        // is added to the 64 sums as they are read back.
+        // product starts a fresh accumulator (the previous tile's last read is complete).
+        bool stop = false;
+#pragma unroll 1
         for (int l = 0; l <= FD; ++l) {
-            asm volatile("fence.proxy.async.shared::cta;");   // this thread's A row, visible to the MMA
+            asm volatile("tcgen05.wait::st.sync.aligned;");   // this thread's A row
             asm volatile("tcgen05.fence::before_thread_sync;");
-            half_sync(h);
+            group_sync(h);
             asm volatile("tcgen05.fence::after_thread_sync;");
-            if (S.abort) {
+            if (S.abort[h]) {   // set before the barrier by a thread of this group: all 128 see it
                 stop = true;
                 break;
             }
             if (t == 0) {
+                auto mma = [&](uint32_t a_tmem, uint64_t db, uint32_t idesc, uint32_t acc) {
+                    asm volatile(
+                        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                        " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_cols),
+                        "r"(a_tmem), "l"(db), "r"(idesc), "r"(acc));
+                };
                 if (l < FD) {
+                    mma(one_cols, umma_desc(smem_addr(S.WB[l]), 1024, 128), kQueryIdesc, 0u);
                     const uint32_t w_addr = smem_addr(S.W[l]);
 #pragma unroll
-                    for (int s = 0; s < 4; ++s) {
-                        const uint64_t da = umma_desc(a_addr + s * 4096, 2048, 128);
-                        const uint64_t db = umma_desc(w_addr + s * 2048, 1024, 128);
-                        asm volatile(
-                            "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_h),
-                            "l"(da), "l"(db), "r"(kQueryIdesc), "r"(s > 0 ? 1u : 0u));
-                    }
+                    for (int s = 0; s < 4; ++s) mma(a_cols + 8 * s, umma_desc(w_addr + s * 2048, 1024, 128), kQueryIdesc, 1u);
                 } else {
                     const uint32_t w5_addr = smem_addr(S.W5);
 #pragma unroll
-                    for (int s = 0; s < 4; ++s) {
-                        const uint64_t da = umma_desc(a_addr + s * 4096, 2048, 128);
-                        const uint64_t db = umma_desc(w5_addr + s * 512, 256, 128);
-                        asm volatile(
-                            "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_h),
-                            "l"(da), "l"(db), "r"(kQueryIdescN16), "r"(s > 0 ? 1u : 0u));
-                    }
+                    for (int s = 0; s < 4; ++s)
+                        mma(a_cols + 8 * s, umma_desc(w5_addr + s * 512, 256, 128), kQueryIdescN16, s > 0 ? 1u : 0u);
                 }
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                    smem_addr(&S.mbar_mma[h])));
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar));
             }
-            if (!mbar_wait(smem_addr(&S.mbar_mma[h]), pm)) S.abort = 1;
+            if (!mbar_wait(mbar, pm)) S.abort[h] = 1;
             pm ^= 1;
             asm volatile("tcgen05.fence::after_thread_sync;");
             if (l == FD) {
                 float v[16];
-                tmem_ld16(row_addr, v);
+                tmem_ld16(d_row, v);
                 asm volatile("tcgen05.wait::ld.sync.aligned;");
-                if (i < n) out[i] = softplusf(((v[0] + v[1]) + v[2]) + S.w5[FW]);
+                if (i < n) out[i] = softplusf(((v[0] + v[1]) + v[2]) + S.b5);
                 break;
             }
-            // 32 columns at a time: read, add the bias, ReLU and round to bf16, write the next A row
-            const float* bl = S.bias + l * FW;
+            // 32 columns at a time: read, ReLU and round to bf16, write the next A row
 #pragma unroll
             for (int c0 = 0; c0 < FW; c0 += 32) {
                 float va[32];
-                tmem_ld16(row_addr + c0, va);
-                tmem_ld16(row_addr + c0 + 16, va + 16);
+                tmem_ld16(d_row + c0, va);
+                tmem_ld16(d_row + c0 + 16, va + 16);
                 asm volatile("tcgen05.wait::ld.sync.aligned;");
-                uint32_t pk[16];
+                uint32_t w[16];
 #pragma unroll
-                for (int c = 0; c < 32; c += 4) {
-                    const float4 b4 = *reinterpret_cast<const float4*>(bl + c0 + c);   // one 16-byte broadcast
-                    pk[c / 2] = pack_bf16_relu(va[c] + b4.x, va[c + 1] + b4.y);
-                    pk[c / 2 + 1] = pack_bf16_relu(va[c + 2] + b4.z, va[c + 3] + b4.w);
-                }
-#pragma unroll
-                for (int g = 0; g < 4; ++g) {
-                    const int kg = c0 / 8 + g;
-                    *reinterpret_cast<uint4*>(reinterpret_cast<char*>(A) + kg * 2048 + (t >> 3) * 128 + (t & 7) * 16) =
-                        make_uint4(pk[4 * g], pk[4 * g + 1], pk[4 * g + 2], pk[4 * g + 3]);
-                }
+                for (int c = 0; c < 16; ++c) w[c] = pack_bf16_relu(va[2 * c], va[2 * c + 1]);
+                tmem_st8(a_row + c0 / 2, w);
+                tmem_st8(a_row + c0 / 2 + 8, w + 8);
             }
         }
+        if (stop) break;
     }
-    if (S.abort && t == 0) {
+    if (S.abort[h] && t == 0) {
         atomicCAS(err, 0, GM_DEV_WAIT_TIMEOUT);
         for (int b = 0; b < 2; ++b)
-            if (pending[b]) mbar_wait(smem_addr(&S.mbar_ld[h][b]), pl[b]);   // drain this half's own copies
+            if ((pending >> b) & 1u) mbar_wait(smem_addr(&S.mbar_ld[h][b]), (pl >> b) & 1u);   // drain this group's own copies
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
@@ -1446,20 +1486,9 @@ extern "C" gm_status gm_field_query(const gm_field* f, const float* xyz, uint64_
             if (e != cudaSuccess) st = gm_cuda_error(e, "gm_field_query (shared memory)");
             else configured_device = f->ctx->device;
         }
-        // blocks per SM from the shared memory each one holds (the occupancy query reports one block
-        // for this kernel; the hardware runs as many as their shared memory and tensor-memory
-        // columns allow, here 3 x 128 of 512 columns)
-        int per_sm = 1;
-        if (st == GM_OK) {
-            int smem_sm = 0;
-            cudaError_t e = cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, f->ctx->device);
-            if (e != cudaSuccess) st = gm_cuda_error(e, "gm_field_query (shared memory per SM)");
-            else per_sm = std::max(1, std::min(8, smem_sm / (smem + 1024)));
-        }
         if (st == GM_OK) {
             const uint64_t ntiles = (n + TQ - 1) / TQ;
-            const uint32_t grid = (uint32_t)std::min<uint64_t>(
-                (ntiles + 1) / 2, (uint64_t)f->ctx->n_sm * (uint64_t)std::max(1, per_sm));
+            const uint32_t grid = (uint32_t)std::min<uint64_t>(ntiles, (uint64_t)std::max(1, f->ctx->n_sm));
             const int bulk = (reinterpret_cast<uintptr_t>(dx) % 16) == 0;
             k_field_query_tc<<<grid, TQ_THREADS, smem, s>>>((const float*)dx, n, f->wbf, f->theta, f->box, bulk,
                                                             dout, f->ctx->dev_err);
