@@ -851,60 +851,63 @@ __global__ void __launch_bounds__(256, 1) k_field_train(const float* __restrict_
 }
 
 // ---- training on the 5th-generation tensor cores ----------------------------------------------
-// Persistent blocks of 256 threads, one per SM; two threads per point (accumulator row): thread
-// (quarter q, half c) owns point 32 q + lane and the columns [32 c, 32 c + 32). Per tile of 128
-// batch points, every product of the hidden layers is a tcgen05.mma (bf16 x bf16, FP32 in tensor
-// memory):
-//   forward   Z_l = H_l W_l^T + b_l        A = H_l rows (K = inputs),   B = W_l   (N = outputs)
-//   backward  dH_l = dZ_l W_l              A = dZ_l rows (K = outputs), B = W_l^T (N = inputs)
-//             gW_l += dZ_l^T H_l           A = dZ_l^T (K = points),     B = H_l^T (N = inputs)
-//             gb_l += dZ_l^T 1             A = dZ_l^T,                  B = a 16 x 128 block whose row 0 is ones
-// The weight and bias gradients accumulate in tensor memory over all tiles of the block and leave
-// it once, into the block's own slice of a partial-sum buffer that the update kernel reduces in a
-// fixed order (deterministic, no atomics on the gradient). The point-major operands (dZ^T, H^T)
-// are written one 2-byte element per (row, point) into a no-swizzle K-major layout whose core
-// matrices sit 144 bytes apart along the points, so that the 32 lanes of a warp (32 consecutive
-// points) store into 32 different banks. The gradient products have 64 real rows (outputs); the
-// MMA runs with M = 128 and rows 64..127 read the next buffer and are never read back. The output
-// layer (w5, b5) and the loss stay in FP32 on the CUDA cores: w5's gradient is a warp transpose-sum.
-// Waits are bounded; on a timeout the block records GM_DEV_WAIT_TIMEOUT, frees its tensor memory
-// and returns.
+// One persistent block per SM: two pipelines of 256 threads, each a tile of 128 batch points in flight,
+// and a warp whose one thread issues every product of both. Two threads per point (accumulator row):
+// thread (quarter q, half c) of a pipeline owns point 32 q + lane and the columns [32 c, 32 c + 32). Per
+// tile, every product of the hidden layers is a tcgen05.mma (bf16 x bf16, FP32 in tensor memory):
+//   forward   Z_l = H_l W_l^T + b_l        A = H_l rows (K = inputs),   B = W_l   (N = outputs); the bias
+//                                          first, as ones (in tensor memory) times its three bf16 parts
+//   backward  dH_l = dZ_l W_l              A = dZ_l rows (K = outputs), B = W_l   (N = inputs, N contiguous)
+//             gW_l += dZ_l^T H_l           A = dZ_l (M contiguous),     B = H_l   (N contiguous), K = points
+//             gb_l += dZ_l^T 1             A = dZ_l (M contiguous),     B = a 16 x 128 block whose row 0 is ones
+// The same copies of H_l, dZ_l and W_l serve as operands contiguous in K and in M or N: their core
+// matrices of 8 x 16 bytes read either way. The weight and bias gradients of both pipelines accumulate in
+// tensor memory over all tiles of the block and leave it once, into the block's own slice of a
+// partial-sum buffer that the update kernel reduces in a fixed order; the issuing thread serves the
+// pipelines in strict turns, so the order of every sum is fixed (deterministic, no atomics on the
+// gradient). The gradient products have 64 real rows (outputs); the MMA runs with M = 128 and rows
+// 64..127 read the next buffer and are never read back. The output layer (w5, b5) and the loss stay in
+// FP32 on the CUDA cores: w5's gradient is a warp transpose-sum, taken while the products run.
+// Threads signal their stores to the issuer on an mbarrier and wait for its products on another; waits
+// are bounded: on a timeout the block records GM_DEV_WAIT_TIMEOUT, frees its tensor memory and returns.
+//
+// Bound by latency: a tile is eight rounds of product and epilogue, one after another. One tile per SM
+// at a time, with copies of every H, dZ and W transposed by 2-byte stores, took 47.9 us for 65536 points
+// (issue 21 %, tensor pipe 10 %); without the copies (102 KB a tile and 32 KB of W^T) two tiles fit.
 constexpr int TT = 128;                        // points per tile
-constexpr int TT_CW = 32;                      // accumulator columns per thread (16: 53.9 vs 49.8 us a step)
+constexpr int TT_CW = 32;                      // accumulator columns per thread
 constexpr int TT_GROUPS = FW / TT_CW;          // threads per point
-constexpr int TT_THREADS = TT * TT_GROUPS;
+constexpr int TT_PIPE = TT * TT_GROUPS;        // threads per pipeline
+constexpr int TT_PIPES = 2;
+constexpr int TT_WARPS = TT_PIPES * TT_PIPE / 32;
+constexpr int TT_THREADS = TT_PIPES * TT_PIPE + 32;
 constexpr uint32_t TT_TMEM_COLS = 512;
-constexpr uint32_t TT_COL_ACC = 0;             // forward / dH accumulator (64 columns)
-constexpr uint32_t TT_COL_GW = 64;             // weight gradients, 64 columns per layer
-constexpr uint32_t TT_COL_GB = 320;            // bias gradients, 16 columns per layer (column 0 used)
-constexpr int T_LBO = 144;                     // point-major operands: core matrices along the points
-constexpr int T_SBO = 16 * T_LBO;              // ... and along the rows
-constexpr int T_BYTES = 8 * T_SBO;             // 64 rows x 128 points
+constexpr uint32_t TT_COL_ACC = 0;             // forward / dH accumulators, 64 columns per pipeline
+constexpr uint32_t TT_COL_GW = 128;            // weight gradients, 64 columns per layer
+constexpr uint32_t TT_COL_GB = 384;            // bias gradients, 16 columns per layer (column 0 used)
+constexpr uint32_t TT_COL_ONE = 448;           // A of the biases (K = 16): ones in k = 0..2
 
 struct TrainTcSmem {
-    alignas(1024) __nv_bfloat16 A[TT * FW];        // rows = points: H_l (forward) or dZ_l (backward)
-    alignas(1024) __nv_bfloat16 W[FD][FW * FW];    // W_l, rows = outputs
-    alignas(1024) __nv_bfloat16 WT[FD][FW * FW];   // W_l^T, rows = inputs
-    alignas(1024) unsigned char DZT[T_BYTES];      // dZ_l^T; rows 64..127 of its M = 128 read HT[0]
-    alignas(1024) unsigned char HT[FD][T_BYTES];   // H_l^T, l = 0..3
-    alignas(1024) unsigned char ONES[2 * T_SBO];   // 16 rows x 128 points, row 0 = 1
-    alignas(16) float bias[FD * FW];
+    // element (point, feature) of a tile: (f / 8) * 2048 + (p / 8) * 128 + (p % 8) * 16 + (f % 8) * 2
+    alignas(1024) __nv_bfloat16 H[TT_PIPES][FD][TT * FW];   // H_l, l = 0..3
+    alignas(1024) __nv_bfloat16 DZ[TT_PIPES][TT * FW];      // dZ_l; rows 64..127 of its M = 128 read on from here
+    alignas(1024) __nv_bfloat16 W[FD][FW * FW];             // W_l, rows = outputs
+    alignas(1024) __nv_bfloat16 WB[FD][FW * 16];            // biases as B (K = 16): hi + mid + lo in k = 0..2
+    alignas(1024) __nv_bfloat16 ONES[16 * TT];              // 16 rows x 128 points, row 0 = 1
     float w5[FW + 1];
-    float gw5w[TT_THREADS / 32][32];   // per warp: w5-gradient sums of its columns
-    float zpart[TT_GROUPS][TT];
-    float gb5w[4], lossw[4];           // per warp of the first column half
-    alignas(8) uint64_t mbar;
+    float gw5w[TT_WARPS][32];          // per warp: w5-gradient sums of its columns
+    float zpart[TT_PIPES][TT_GROUPS][TT];
+    float gb5w[TT_PIPES][4], lossw[TT_PIPES][4];   // per warp of the first column half
+    alignas(8) uint64_t ready[TT_PIPES];   // a pipeline's operands are stored
+    uint64_t done[TT_PIPES];               // its products are complete
+    uint64_t xch[TT_PIPES];                // both halves of z5 are stored
     uint32_t tmem;
     int abort;
 };
 
-// Byte offset of element (row, point) of a point-major operand.
-__device__ __forceinline__ int tp_off(int row, int k) {
-    return (k >> 3) * T_LBO + (row >> 3) * T_SBO + (row & 7) * 16 + (k & 7) * 2;
-}
-
 constexpr uint32_t kIdescN64 = (1u << 4) | (1u << 7) | (1u << 10) | ((64u >> 3) << 17) | ((128u >> 4) << 24);
 constexpr uint32_t kIdescN16 = (1u << 4) | (1u << 7) | (1u << 10) | ((16u >> 3) << 17) | ((128u >> 4) << 24);
+constexpr uint32_t kIdescAT = 1u << 15, kIdescBT = 1u << 16;   // A contiguous in M, B contiguous in N
 
 __device__ __forceinline__ void umma_bf16(uint32_t d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
     asm volatile(
@@ -912,32 +915,59 @@ __device__ __forceinline__ void umma_bf16(uint32_t d, uint64_t da, uint64_t db, 
         " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
         "l"(da), "l"(db), "r"(idesc), "r"(acc));
 }
-
-__device__ __forceinline__ void tmem_st_cw(uint32_t taddr, const float* v) {
-#pragma unroll
-    for (int c0 = 0; c0 < TT_CW; c0 += 16)
-        asm volatile(
-            "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::
-                "r"(taddr + c0),
-            "f"(v[c0]), "f"(v[c0 + 1]), "f"(v[c0 + 2]), "f"(v[c0 + 3]), "f"(v[c0 + 4]), "f"(v[c0 + 5]),
-            "f"(v[c0 + 6]), "f"(v[c0 + 7]), "f"(v[c0 + 8]), "f"(v[c0 + 9]), "f"(v[c0 + 10]), "f"(v[c0 + 11]),
-            "f"(v[c0 + 12]), "f"(v[c0 + 13]), "f"(v[c0 + 14]), "f"(v[c0 + 15]));
+__device__ __forceinline__ void umma_bf16_ta(uint32_t d, uint32_t a_tmem, uint64_t db, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d),
+        "r"(a_tmem), "l"(db), "r"(idesc), "r"(acc));
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 
-// This thread's part of a row (columns c0 .. c0 + TT_CW - 1 as packed bf16 pairs) into the K-major
-// A tile and into column p of a point-major operand.
-__device__ __forceinline__ void store_part(__nv_bfloat16* A, unsigned char* T, int p, int c0, const uint32_t* pk) {
+// This thread's part of row p of a tile: columns c0 .. c0 + 31 as packed bf16 pairs.
+__device__ __forceinline__ void store_part(__nv_bfloat16* T, int p, int c0, const uint32_t* pk) {
+    char* row = reinterpret_cast<char*>(T) + (c0 / 8) * 2048 + (p >> 3) * 128 + (p & 7) * 16;
 #pragma unroll
-    for (int g = 0; g < TT_CW / 8; ++g) {
-        const int kg = c0 / 8 + g;
-        *reinterpret_cast<uint4*>(reinterpret_cast<char*>(A) + kg * 2048 + (p >> 3) * 128 + (p & 7) * 16) =
-            make_uint4(pk[4 * g], pk[4 * g + 1], pk[4 * g + 2], pk[4 * g + 3]);
-    }
+    for (int g = 0; g < TT_CW / 8; ++g)
+        *reinterpret_cast<uint4*>(row + g * 2048) = make_uint4(pk[4 * g], pk[4 * g + 1], pk[4 * g + 2], pk[4 * g + 3]);
+}
+
+// Features 32 HI .. 32 HI + 31 (features_fast's values) as packed bf16 pairs; the upper half starts at
+// octave 3, whose sine and cosine are evaluated afresh.
+template <int HI>
+__device__ __forceinline__ void encode_half(const float xt[3], uint32_t* pk) {
+    float held = 0.f;
+    auto put = [&](int j, float v) {   // feature j, in order; j is known at compile time
+        if (j < 32 * HI || j >= 32 * HI + 32) return;
+        if (j & 1) pk[(j - 32 * HI) >> 1] = pack_bf16(held, v);
+        else held = v;
+    };
+    put(0, xt[0]);
+    put(1, xt[1]);
+    put(2, xt[2]);
+    float sn[3], cs[3];
 #pragma unroll
-    for (int j = 0; j < TT_CW; j += 2) {
-        *reinterpret_cast<uint16_t*>(T + tp_off(c0 + j, p)) = (uint16_t)(pk[j / 2] & 0xffffu);
-        *reinterpret_cast<uint16_t*>(T + tp_off(c0 + j + 1, p)) = (uint16_t)(pk[j / 2] >> 16);
+    for (int k = HI ? 3 : 0; k < (HI ? FOCT : 5); ++k) {
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            if (k % 3 == 0) {
+                float y = ldexpf(xt[r], k);
+                y = y - 2.f * rintf(0.5f * y);
+                __sincosf(3.14159265358979f * y, &sn[r], &cs[r]);
+            } else {
+                const float s2 = 2.f * (sn[r] * cs[r]);
+                const float c2 = fmaf(cs[r], cs[r], -(sn[r] * sn[r]));
+                sn[r] = s2;
+                cs[r] = c2;
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 3; ++r) put(3 + 6 * k + r, sn[r]);
+#pragma unroll
+        for (int r = 0; r < 3; ++r) put(6 + 6 * k + r, cs[r]);
     }
+    put(63, 0.f);
 }
 
 __device__ __forceinline__ float bf_lo(uint32_t v) { return __uint_as_float(v << 16); }
@@ -967,72 +997,25 @@ __device__ __forceinline__ float warp_transpose_sum(float v[TT_CW]) {
 __global__ void __launch_bounds__(TT_THREADS, 1) k_field_train_tc(
     const float* __restrict__ pts, int stride, const float* __restrict__ target, uint64_t n,
     const uint32_t* __restrict__ idx, uint32_t batch, uint32_t step, uint2 seed, FieldBox B,
-    const __nv_bfloat16* __restrict__ wbf, const __nv_bfloat16* __restrict__ wtbf, const float* __restrict__ theta,
-    float* __restrict__ partial, int* __restrict__ err) {
+    const __nv_bfloat16* __restrict__ wbf, const float* __restrict__ theta, float* __restrict__ partial,
+    int* __restrict__ err) {
     extern __shared__ __align__(1024) unsigned char t_smem_raw[];
     TrainTcSmem& S = *reinterpret_cast<TrainTcSmem*>(t_smem_raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int q = warp & 3, c = warp >> 2;
+    const int pipe = warp / (TT_PIPE / 32);              // TT_PIPES: the issuing warp
+    const int q = warp & 3, c = (warp >> 2) & (TT_GROUPS - 1);
     const int p = 32 * q + lane, c0 = TT_CW * c;
-    // weights in the core-matrix layout: (n, k) at (k / 8) * 1024 + (n / 8) * 128 + (n % 8) * 16 + (k % 8) * 2
-    for (int i = tid; i < FD * FW * 8; i += TT_THREADS) {
-        const int l = i / (FW * 8), nn = (i / 8) % FW, kg = i % 8;
-        const size_t src = (size_t)l * FW * FW + nn * FW;
-        const int dst = kg * 1024 + (nn >> 3) * 128 + (nn & 7) * 16;
-        *reinterpret_cast<uint4*>(reinterpret_cast<char*>(S.W[l]) + dst) = reinterpret_cast<const uint4*>(wbf + src)[kg];
-        *reinterpret_cast<uint4*>(reinterpret_cast<char*>(S.WT[l]) + dst) =
-            reinterpret_cast<const uint4*>(wtbf + src)[kg];
-    }
-    for (int i = tid; i < 2 * T_SBO / 16; i += TT_THREADS) reinterpret_cast<uint4*>(S.ONES)[i] = make_uint4(0, 0, 0, 0);
-    for (int i = tid; i < FD * FW; i += TT_THREADS) S.bias[i] = theta[b_off(i / FW) + i % FW];
-    for (int i = tid; i <= FW; i += TT_THREADS) S.w5[i] = theta[W5_OFF + i];
-    S.gw5w[warp][lane] = 0.f;
-    if (tid == 0) {
-        S.abort = 0;
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&S.mbar)));
-        asm volatile("fence.mbarrier_init.release.cluster;");
-    }
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&S.tmem)),
-                     "r"(TT_TMEM_COLS));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-    }
-    __syncthreads();
-    if (tid < TT) *reinterpret_cast<uint16_t*>(S.ONES + tp_off(0, tid)) = 0x3F80;   // bf16 1.0
-    asm volatile("fence.proxy.async.shared::cta;");
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    const uint32_t tm = S.tmem;
-    const uint32_t row_acc = tm + ((uint32_t)(32 * q) << 16) + TT_COL_ACC + c0;
-    const uint32_t a_addr = smem_addr(S.A), dzt_addr = smem_addr(S.DZT), ones_addr = smem_addr(S.ONES);
     const uint32_t ntiles = (batch + TT - 1) / TT;
-    const float inv_b = 1.f / (float)batch;
-    uint32_t ph = 0;
-    bool first = true, stop = false;
-    float loss_acc = 0.f, gb5_acc = 0.f;
-    // bounded wait on the block's MMA barrier; every thread takes part
-    auto sync_mma = [&]() {
-        if (!mbar_wait(smem_addr(&S.mbar), ph)) S.abort = 1;
-        ph ^= 1;
-        asm volatile("tcgen05.fence::after_thread_sync;");
-    };
-    auto block_sync = [&]() {
-        asm volatile("fence.proxy.async.shared::cta;");
-        asm volatile("tcgen05.fence::before_thread_sync;");
-        __syncthreads();
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        return S.abort != 0;
-    };
-    // the batch entry of this thread's point in a tile, its position and target; issued one tile
-    // ahead so that the random gathers are in flight while the previous tile computes
+    const uint32_t mine = (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x;   // tiles of this block (>= 1)
+    // the batch entry of this thread's point in the block's k-th tile, its position and target; issued a
+    // tile ahead so that the random gathers are in flight while the previous tile computes
     uint32_t ne = 0;
     uint64_t ni = n;
     float nx[3] = {0.f, 0.f, 0.f}, ny = 0.f;
-    auto prefetch = [&](uint32_t t) {
-        ne = t * TT + p;
+    auto prefetch = [&](uint32_t k) {
+        ne = (blockIdx.x + k * gridDim.x) * TT + p;
         ni = n;
-        if (t < ntiles && ne < batch)
+        if (k < mine && ne < batch)
             ni = idx ? (uint64_t)idx[ne] : (uint64_t)(philox_x(step, ne, seed.x, seed.y) % (uint32_t)n);
         if (ni < n) {
             nx[0] = pts[stride * ni];
@@ -1041,132 +1024,211 @@ __global__ void __launch_bounds__(TT_THREADS, 1) k_field_train_tc(
             ny = target[ni];
         }
     };
-    prefetch(blockIdx.x);
-    for (uint32_t tile = blockIdx.x; tile < ntiles && !stop; tile += gridDim.x) {
-        const uint32_t e = ne;
-        const uint64_t i = ni;
-        float xt[3] = {0.f, 0.f, 0.f};
-        if (i < n) {
-            xt[0] = (nx[0] - B.cx) * B.inv_h;
-            xt[1] = (nx[1] - B.cy) * B.inv_h;
-            xt[2] = (nx[2] - B.cz) * B.inv_h;
+    if (pipe < TT_PIPES) prefetch((uint32_t)pipe);
+    // weights in the core-matrix layout: (n, k) at (k / 8) * 1024 + (n / 8) * 128 + (n % 8) * 16 + (k % 8) * 2
+    for (int i = tid; i < FD * FW * 8; i += TT_THREADS) {
+        const int l = i / (FW * 8), nn = (i / 8) % FW, kg = i % 8;
+        const int dst = kg * 1024 + (nn >> 3) * 128 + (nn & 7) * 16;
+        *reinterpret_cast<uint4*>(reinterpret_cast<char*>(S.W[l]) + dst) =
+            reinterpret_cast<const uint4*>(wbf + (size_t)l * FW * FW + nn * FW)[kg];
+    }
+    for (int i = tid; i < FD * FW; i += TT_THREADS) {
+        const int l = i / FW, nn = i % FW;
+        __nv_bfloat16 part[3];
+        split3_bf16(theta[b_off(l) + nn], part);
+        char* row = reinterpret_cast<char*>(S.WB[l]) + (nn >> 3) * 128 + (nn & 7) * 16;
+        *reinterpret_cast<uint4*>(row) =
+            make_uint4(__bfloat16_as_ushort(part[0]) | (uint32_t)__bfloat16_as_ushort(part[1]) << 16,
+                       __bfloat16_as_ushort(part[2]), 0u, 0u);
+        *reinterpret_cast<uint4*>(row + 1024) = make_uint4(0u, 0u, 0u, 0u);
+    }
+    // (n, k) of the ones at (k / 8) * 256 + (n / 8) * 128 + (n % 8) * 16 + (k % 8) * 2: row 0 = 1
+    for (int i = tid; i < 16 * TT / 8; i += TT_THREADS)
+        reinterpret_cast<uint4*>(S.ONES)[i] = i % 16 == 0 ? make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u)
+                                                          : make_uint4(0u, 0u, 0u, 0u);
+    for (int i = tid; i <= FW; i += TT_THREADS) S.w5[i] = theta[W5_OFF + i];
+    if (warp < TT_WARPS) S.gw5w[warp][lane] = 0.f;
+    if (tid == 0) {
+        S.abort = 0;
+        for (int k = 0; k < TT_PIPES; ++k) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&S.ready[k])), "r"(TT_PIPE));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&S.done[k])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&S.xch[k])), "r"(TT_PIPE));
         }
-        const float y = i < n ? ny : 0.f;
-        prefetch(tile + gridDim.x);
-        uint32_t pk[TT_CW / 2];
-        {
-            float v[FW];
-            features_fast(xt, v);
+        asm volatile("fence.mbarrier_init.release.cluster;");
+    }
+    if (pipe == TT_PIPES) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&S.tmem)),
+                     "r"(TT_TMEM_COLS));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    asm volatile("fence.proxy.async.shared::cta;");
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    const uint32_t tm = S.tmem;
+    if (warp < 4) {
+        const uint32_t one[8] = {0x3F803F80u, 0x3F80u, 0u, 0u, 0u, 0u, 0u, 0u};   // bf16 1, 1, 1, 0, ...
+        tmem_st8(tm + TT_COL_ONE + ((uint32_t)(32 * q) << 16), one);
+        asm volatile("tcgen05.wait::st.sync.aligned;");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    const float inv_b = 1.f / (float)batch;
+    float loss_acc = 0.f, gb5_acc = 0.f;
+    bool ok = true;
+    if (pipe == TT_PIPES) {
+        // the issuer: forward l = 0..3, then backward l = 3..0, of the two pipelines in turn
+        uint32_t phase[TT_PIPES] = {0, 0};
+        for (uint32_t k0 = 0; k0 < mine && ok; k0 += TT_PIPES) {
+            for (int st = 0; st < 2 * FD && ok; ++st) {
 #pragma unroll
-            for (int g = 0; g < TT_GROUPS; ++g)   // static indices keep v in registers
-                if (g == c) {
+                for (int w = 0; w < TT_PIPES; ++w) {
+                    if (k0 + w >= mine || !ok) continue;
+                    if (!mbar_wait(smem_addr(&S.ready[w]), phase[w])) {
+                        ok = false;
+                        continue;
+                    }
+                    phase[w] ^= 1;
+                    asm volatile("tcgen05.fence::after_thread_sync;");
+                    if (lane == 0) {
+                        const uint32_t acc = tm + TT_COL_ACC + 64 * w, dz = smem_addr(S.DZ[w]);
+                        if (st < FD) {
+                            const uint32_t h = smem_addr(S.H[w][st]), wl = smem_addr(S.W[st]);
+                            umma_bf16_ta(acc, tm + TT_COL_ONE, umma_desc(smem_addr(S.WB[st]), 1024, 128), kIdescN64, 0u);
 #pragma unroll
-                    for (int j = 0; j < TT_CW; j += 2) pk[j / 2] = pack_bf16(v[g * TT_CW + j], v[g * TT_CW + j + 1]);
+                            for (int s = 0; s < 4; ++s)
+                                umma_bf16(acc, umma_desc(h + s * 4096, 2048, 128), umma_desc(wl + s * 2048, 1024, 128),
+                                          kIdescN64, 1u);
+                        } else {
+                            const int l = 2 * FD - 1 - st;
+                            const uint32_t h = smem_addr(S.H[w][l]), wl = smem_addr(S.W[l]), ones = smem_addr(S.ONES);
+                            if (l > 0) {
+#pragma unroll
+                                for (int s = 0; s < 4; ++s)
+                                    umma_bf16(acc, umma_desc(dz + s * 4096, 2048, 128), umma_desc(wl + s * 256, 128, 1024),
+                                              kIdescN64 | kIdescBT, s > 0 ? 1u : 0u);
+                            }
+                            const bool fresh = k0 == 0 && w == 0;
+#pragma unroll
+                            for (int s = 0; s < 8; ++s) {
+                                const uint32_t add = !fresh || s > 0 ? 1u : 0u;
+                                const uint64_t da = umma_desc(dz + s * 256, 128, 2048);
+                                umma_bf16(tm + TT_COL_GW + 64 * l, da, umma_desc(h + s * 256, 128, 2048),
+                                          kIdescN64 | kIdescAT | kIdescBT, add);
+                                umma_bf16(tm + TT_COL_GB + 16 * l, da, umma_desc(ones + s * 512, 256, 128),
+                                          kIdescN16 | kIdescAT, add);
+                            }
+                        }
+                        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                            smem_addr(&S.done[w])));
+                    }
+                    __syncwarp();
                 }
+            }
         }
-        store_part(S.A, S.HT[0], p, c0, pk);
-        uint32_t mask[FD];
-        float zp = 0.f;
-#pragma unroll
-        for (int l = 0; l < FD; ++l) {
-            tmem_st_cw(row_acc, S.bias + l * FW + c0);
-            asm volatile("tcgen05.wait::st.sync.aligned;");
-            if (block_sync()) {
-                stop = true;
-                break;
+    } else {
+        const uint32_t row_acc = tm + ((uint32_t)(32 * q) << 16) + TT_COL_ACC + 64 * pipe + c0;
+        const uint32_t bar_done = smem_addr(&S.done[pipe]);
+        uint32_t ph = 0, phx = 0;
+        // stores into shared memory, visible to the products; reads of the accumulator, before them
+        auto give = [&]() {
+            asm volatile("fence.proxy.async.shared::cta;");
+            asm volatile("tcgen05.fence::before_thread_sync;");
+            mbar_arrive(&S.ready[pipe]);
+        };
+        auto take = [&]() {
+            ok = mbar_wait(bar_done, ph);
+            ph ^= 1;
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            return ok;
+        };
+        for (uint32_t k = (uint32_t)pipe; k < mine && ok; k += TT_PIPES) {
+            const uint32_t e = ne;
+            const uint64_t i = ni;
+            float xt[3] = {0.f, 0.f, 0.f};
+            if (i < n) {
+                xt[0] = (nx[0] - B.cx) * B.inv_h;
+                xt[1] = (nx[1] - B.cy) * B.inv_h;
+                xt[2] = (nx[2] - B.cz) * B.inv_h;
             }
-            if (tid == 0) {
-                const uint32_t w_addr = smem_addr(S.W[l]);
+            const float y = i < n ? ny : 0.f;
+            prefetch(k + TT_PIPES);
+            uint32_t pk[TT_CW / 2];
+            if (c == 0) encode_half<0>(xt, pk);
+            else encode_half<1>(xt, pk);
+            if (k >= TT_PIPES && !take()) break;   // the last gradients of the pipeline's previous tile
+            store_part(S.H[pipe][0], p, c0, pk);
+            uint32_t mask[FD];
+            float zp = 0.f;
 #pragma unroll
-                for (int s = 0; s < 4; ++s)
-                    umma_bf16(tm + TT_COL_ACC, umma_desc(a_addr + s * 4096, 2048, 128),
-                              umma_desc(w_addr + s * 2048, 1024, 128), kIdescN64, 1u);
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                    smem_addr(&S.mbar)));
-            }
-            sync_mma();
-            float z[TT_CW];
+            for (int l = 0; l < FD; ++l) {
+                give();
+                if (!take()) break;
+                float z[TT_CW];
 #pragma unroll
-            for (int j = 0; j < TT_CW; j += 16) tmem_ld16(row_acc + j, z + j);
-            asm volatile("tcgen05.wait::ld.sync.aligned;");
-            uint32_t m = 0;
-#pragma unroll
-            for (int j = 0; j < TT_CW; j += 2) {
-                pk[j / 2] = pack_bf16_relu(z[j], z[j + 1]);
-                m |= (z[j] > 0.f ? 1u : 0u) << j;
-                m |= (z[j + 1] > 0.f ? 1u : 0u) << (j + 1);
-            }
-            mask[l] = m;
-            if (l + 1 < FD) {
-                store_part(S.A, S.HT[l + 1], p, c0, pk);
-            } else {
+                for (int j = 0; j < TT_CW; j += 16) tmem_ld16(row_acc + j, z + j);
+                asm volatile("tcgen05.wait::ld.sync.aligned;");
+                uint32_t m = 0;
 #pragma unroll
                 for (int j = 0; j < TT_CW; j += 2) {
-                    zp = fmaf(bf_lo(pk[j / 2]), S.w5[c0 + j], zp);
-                    zp = fmaf(bf_hi(pk[j / 2]), S.w5[c0 + j + 1], zp);
+                    pk[j / 2] = pack_bf16_relu(z[j], z[j + 1]);
+                    m |= (z[j] > 0.f ? 1u : 0u) << j;
+                    m |= (z[j + 1] > 0.f ? 1u : 0u) << (j + 1);
+                }
+                mask[l] = m;
+                if (l + 1 < FD) {
+                    store_part(S.H[pipe][l + 1], p, c0, pk);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < TT_CW; j += 2) {
+                        zp = fmaf(bf_lo(pk[j / 2]), S.w5[c0 + j], zp);
+                        zp = fmaf(bf_hi(pk[j / 2]), S.w5[c0 + j + 1], zp);
+                    }
                 }
             }
-        }
-        if (stop) break;
-        // output layer: both halves form z5 in the same order
-        S.zpart[c][p] = zp;
-        __syncthreads();
-        float z5 = S.zpart[0][p];
+            if (!ok) break;
+            // output layer: both halves form z5 in the same order
+            S.zpart[pipe][c][p] = zp;
+            mbar_arrive(&S.xch[pipe]);
+            ok = mbar_wait(smem_addr(&S.xch[pipe]), phx);
+            phx ^= 1;
+            if (!ok) break;
+            float z5 = S.zpart[pipe][0][p];
 #pragma unroll
-        for (int g = 1; g < TT_GROUPS; ++g) z5 += S.zpart[g][p];
-        z5 += S.w5[FW];
-        const float r = e < batch ? softplusf(z5) - y : 0.f;
-        const float dz5 = 2.f * r * inv_b * sigmoidf_(z5);
-        if (c == 0) {
-            loss_acc = fmaf(r, r, loss_acc);
-            gb5_acc += dz5;
-        }
-        {
-            float gv[TT_CW];
+            for (int g = 1; g < TT_GROUPS; ++g) z5 += S.zpart[pipe][g][p];
+            z5 += S.w5[FW];
+            const float r = e < batch ? softplusf(z5) - y : 0.f;
+            const float dz5 = 2.f * r * inv_b * sigmoidf_(z5);
+            // dZ_3 = bf16(dz5 w5 . [z_3 > 0])
+            {
+                uint32_t dz[TT_CW / 2];
 #pragma unroll
-            for (int j = 0; j < TT_CW; j += 2) {
-                gv[j] = dz5 * bf_lo(pk[j / 2]);
-                gv[j + 1] = dz5 * bf_hi(pk[j / 2]);
-            }
-            S.gw5w[warp][lane] += warp_transpose_sum(gv);
-        }
-        // dZ_3 = bf16(dz5 w5 . [z_3 > 0])
-#pragma unroll
-        for (int j = 0; j < TT_CW; j += 2) {
-            const float d0 = (mask[FD - 1] >> j) & 1u ? dz5 * S.w5[c0 + j] : 0.f;
-            const float d1 = (mask[FD - 1] >> (j + 1)) & 1u ? dz5 * S.w5[c0 + j + 1] : 0.f;
-            pk[j / 2] = pack_bf16(d0, d1);
-        }
-        store_part(S.A, S.DZT, p, c0, pk);
-#pragma unroll
-        for (int l = FD - 1; l >= 0; --l) {
-            if (block_sync()) {
-                stop = true;
-                break;
-            }
-            if (tid == 0) {
-                const uint32_t ht_addr = smem_addr(S.HT[l]);
-#pragma unroll
-                for (int s = 0; s < 8; ++s) {
-                    const uint32_t acc = (!first || s > 0) ? 1u : 0u;
-                    const uint64_t da = umma_desc(dzt_addr + s * 2 * T_LBO, T_LBO, T_SBO);
-                    umma_bf16(tm + TT_COL_GW + 64 * l, da, umma_desc(ht_addr + s * 2 * T_LBO, T_LBO, T_SBO),
-                              kIdescN64, acc);
-                    umma_bf16(tm + TT_COL_GB + 16 * l, da, umma_desc(ones_addr + s * 2 * T_LBO, T_LBO, T_SBO),
-                              kIdescN16, acc);
+                for (int j = 0; j < TT_CW; j += 2) {
+                    const float d0 = (mask[FD - 1] >> j) & 1u ? dz5 * S.w5[c0 + j] : 0.f;
+                    const float d1 = (mask[FD - 1] >> (j + 1)) & 1u ? dz5 * S.w5[c0 + j + 1] : 0.f;
+                    dz[j / 2] = pack_bf16(d0, d1);
                 }
-                if (l > 0) {
-                    const uint32_t wt_addr = smem_addr(S.WT[l]);
-#pragma unroll
-                    for (int s = 0; s < 4; ++s)
-                        umma_bf16(tm + TT_COL_ACC, umma_desc(a_addr + s * 4096, 2048, 128),
-                                  umma_desc(wt_addr + s * 2048, 1024, 128), kIdescN64, s > 0 ? 1u : 0u);
-                }
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                    smem_addr(&S.mbar)));
+                store_part(S.DZ[pipe], p, c0, dz);
             }
-            sync_mma();
-            if (l > 0) {
+            give();
+            if (c == 0) {
+                loss_acc = fmaf(r, r, loss_acc);
+                gb5_acc += dz5;
+            }
+            {
+                float gv[TT_CW];
+#pragma unroll
+                for (int j = 0; j < TT_CW; j += 2) {
+                    gv[j] = dz5 * bf_lo(pk[j / 2]);
+                    gv[j + 1] = dz5 * bf_hi(pk[j / 2]);
+                }
+                S.gw5w[warp][lane] += warp_transpose_sum(gv);
+            }
+#pragma unroll
+            for (int l = FD - 1; l > 0; --l) {
+                if (!take()) break;
                 // dZ_{l-1} = bf16(dH_l . [z_{l-1} > 0])
                 float dh[TT_CW];
 #pragma unroll
@@ -1178,68 +1240,76 @@ __global__ void __launch_bounds__(TT_THREADS, 1) k_field_train_tc(
                     const float d1 = (mask[l - 1] >> (j + 1)) & 1u ? dh[j + 1] : 0.f;
                     pk[j / 2] = pack_bf16(d0, d1);
                 }
-                store_part(S.A, S.DZT, p, c0, pk);
+                store_part(S.DZ[pipe], p, c0, pk);
+                give();
             }
         }
-        first = false;
+        if (ok && (uint32_t)pipe < mine) take();   // the last tile's last gradients
+        if (c == 0) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                loss_acc += __shfl_xor_sync(0xffffffffu, loss_acc, o);
+                gb5_acc += __shfl_xor_sync(0xffffffffu, gb5_acc, o);
+            }
+            if (lane == 0) {
+                S.lossw[pipe][q] = loss_acc;
+                S.gb5w[pipe][q] = gb5_acc;
+            }
+        }
     }
+    if (!ok) S.abort = 1;
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
     // the block's sums into its slice of the partial-sum buffer
-    if (c == 0) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            loss_acc += __shfl_xor_sync(0xffffffffu, loss_acc, o);
-            gb5_acc += __shfl_xor_sync(0xffffffffu, gb5_acc, o);
-        }
-        if (lane == 0) {
-            S.lossw[q] = loss_acc;
-            S.gb5w[q] = gb5_acc;
-        }
-    }
-    const bool ok = !block_sync() && !stop;
     float* P = partial + (size_t)blockIdx.x * NPAR_PAD;
-    if (ok && q < 2) {
-        // accumulator rows 0..63 are the outputs of each layer
+    if (!S.abort) {
+        if (pipe < TT_PIPES && q < 2) {
+            // accumulator rows 0..63 are the outputs of each layer; a pipeline's warps read two layers
 #pragma unroll 1
-        for (int l = 0; l < FD; ++l) {
-            float v[TT_CW];
-            const uint32_t ra = tm + ((uint32_t)(32 * q) << 16) + TT_COL_GW + 64 * l + c0;
-            if (first) {
-#pragma unroll
-                for (int j = 0; j < TT_CW; ++j) v[j] = 0.f;
-            } else {
+            for (int l = 2 * pipe; l < 2 * pipe + 2; ++l) {
+                float v[TT_CW];
+                const uint32_t ra = tm + ((uint32_t)(32 * q) << 16) + TT_COL_GW + 64 * l + c0;
 #pragma unroll
                 for (int j = 0; j < TT_CW; j += 16) tmem_ld16(ra + j, v + j);
                 asm volatile("tcgen05.wait::ld.sync.aligned;");
-            }
-            float4* dst = reinterpret_cast<float4*>(P + w_off(l) + p * FW + c0);
+                float4* dst = reinterpret_cast<float4*>(P + w_off(l) + p * FW + c0);
 #pragma unroll
-            for (int j = 0; j < TT_CW / 4; ++j) dst[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-            if (c == 0) {
-                float gb[16];
-                if (first) gb[0] = 0.f;
-                else {
+                for (int j = 0; j < TT_CW / 4; ++j)
+                    dst[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                if (c == 0) {
+                    float gb[16];
                     tmem_ld16(tm + ((uint32_t)(32 * q) << 16) + TT_COL_GB + 16 * l, gb);
                     asm volatile("tcgen05.wait::ld.sync.aligned;");
+                    P[b_off(l) + p] = gb[0];
                 }
-                P[b_off(l) + p] = gb[0];
             }
         }
-    }
-    if (ok) {
-        // warps in a fixed order: the block's sums do not depend on scheduling
+        // pipelines and warps in a fixed order: the block's sums do not depend on scheduling
         if (tid < FW) {
             const int g = tid / TT_CW, j = tid % TT_CW;   // column group and column within it
-            P[W5_OFF + tid] = ((S.gw5w[4 * g][j] + S.gw5w[4 * g + 1][j]) + S.gw5w[4 * g + 2][j]) + S.gw5w[4 * g + 3][j];
+            float v = 0.f;
+            for (int k = 0; k < TT_PIPES; ++k)
+                for (int w = 0; w < 4; ++w) v += S.gw5w[k * (TT_PIPE / 32) + 4 * g + w][j];
+            P[W5_OFF + tid] = v;
         }
         if (tid == 0) {
-            P[B5_OFF] = ((S.gb5w[0] + S.gb5w[1]) + S.gb5w[2]) + S.gb5w[3];
-            P[NPAR] = ((S.lossw[0] + S.lossw[1]) + S.lossw[2]) + S.lossw[3];   // the padding slot
+            float gb = 0.f, ls = 0.f;
+            for (int k = 0; k < TT_PIPES; ++k)
+                for (int w = 0; w < 4; ++w) {
+                    gb += S.gb5w[k][w];
+                    ls += S.lossw[k][w];
+                }
+            P[B5_OFF] = gb;
+            P[NPAR] = ls;   // the padding slot
         }
+    } else if (tid == 0) {
+        atomicCAS(err, 0, GM_DEV_WAIT_TIMEOUT);
     }
-    if (S.abort && tid == 0) atomicCAS(err, 0, GM_DEV_WAIT_TIMEOUT);
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tm), "r"(TT_TMEM_COLS));
+    if (pipe == TT_PIPES)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tm), "r"(TT_TMEM_COLS));
 }
 
 // Gradient = the fixed-order sum of the blocks' partial sums; then either that gradient is
@@ -1368,7 +1438,7 @@ static gm_status field_grad(gm_field* f, const float* pts, int stride, const flo
         const int grid = (int)std::min<uint32_t>((uint32_t)std::max(1, f->ctx->n_sm), ntiles);
         k_field_train_tc<<<grid, TT_THREADS, kTrainTcSmem, s>>>(
             pts, stride, target, n, idx, batch, step, make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)), f->box,
-            f->wbf, f->wtbf, f->theta, f->partial, f->ctx->dev_err);
+            f->wbf, f->theta, f->partial, f->ctx->dev_err);
         f->nblk = grid;
         f->ctx->launches += 1;
         GM_TRY_CUDA(cudaGetLastError());
