@@ -899,7 +899,8 @@ struct TrainTcSmem {
     float zpart[TT_PIPES][TT_GROUPS][TT];
     float gb5w[TT_PIPES][4], lossw[TT_PIPES][4];   // per warp of the first column half
     alignas(8) uint64_t ready[TT_PIPES];   // a pipeline's operands are stored
-    uint64_t done[TT_PIPES];               // its products are complete
+    uint64_t done[TT_PIPES];               // its accumulator is complete
+    uint64_t free_dz[TT_PIPES];            // the gradient products that read its dZ are complete
     uint64_t xch[TT_PIPES];                // both halves of z5 are stored
     uint32_t tmem;
     int abort;
@@ -972,6 +973,12 @@ __device__ __forceinline__ void encode_half(const float xt[3], uint32_t* pk) {
 
 __device__ __forceinline__ float bf_lo(uint32_t v) { return __uint_as_float(v << 16); }
 __device__ __forceinline__ float bf_hi(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
+
+// All ones in each half of a bf16 pair that is > 0.
+__device__ __forceinline__ uint32_t positive2(uint32_t pair) {
+    const __nv_bfloat162 zero = __float2bfloat162_rn(0.f);
+    return __hgt2_mask(*reinterpret_cast<const __nv_bfloat162*>(&pair), zero);
+}
 
 // Lane L ends with the sum over the warp's 32 lanes of v[L mod TT_CW].
 __device__ __forceinline__ float warp_transpose_sum(float v[TT_CW]) {
@@ -1053,6 +1060,7 @@ __global__ void __launch_bounds__(TT_THREADS, 1) k_field_train_tc(
         for (int k = 0; k < TT_PIPES; ++k) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&S.ready[k])), "r"(TT_PIPE));
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&S.done[k])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&S.free_dz[k])));
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&S.xch[k])), "r"(TT_PIPE));
         }
         asm volatile("fence.mbarrier_init.release.cluster;");
@@ -1093,6 +1101,10 @@ __global__ void __launch_bounds__(TT_THREADS, 1) k_field_train_tc(
                     phase[w] ^= 1;
                     asm volatile("tcgen05.fence::after_thread_sync;");
                     if (lane == 0) {
+                        auto commit = [&](uint64_t* bar) {
+                            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                smem_addr(bar)));
+                        };
                         const uint32_t acc = tm + TT_COL_ACC + 64 * w, dz = smem_addr(S.DZ[w]);
                         if (st < FD) {
                             const uint32_t h = smem_addr(S.H[w][st]), wl = smem_addr(S.W[st]);
@@ -1101,6 +1113,7 @@ __global__ void __launch_bounds__(TT_THREADS, 1) k_field_train_tc(
                             for (int s = 0; s < 4; ++s)
                                 umma_bf16(acc, umma_desc(h + s * 4096, 2048, 128), umma_desc(wl + s * 2048, 1024, 128),
                                           kIdescN64, 1u);
+                            commit(&S.done[w]);
                         } else {
                             const int l = 2 * FD - 1 - st;
                             const uint32_t h = smem_addr(S.H[w][l]), wl = smem_addr(S.W[l]), ones = smem_addr(S.ONES);
@@ -1109,6 +1122,7 @@ __global__ void __launch_bounds__(TT_THREADS, 1) k_field_train_tc(
                                 for (int s = 0; s < 4; ++s)
                                     umma_bf16(acc, umma_desc(dz + s * 4096, 2048, 128), umma_desc(wl + s * 256, 128, 1024),
                                               kIdescN64 | kIdescBT, s > 0 ? 1u : 0u);
+                                commit(&S.done[w]);   // the pipeline goes on while its gradients are summed
                             }
                             const bool fresh = k0 == 0 && w == 0;
 #pragma unroll
@@ -1120,9 +1134,8 @@ __global__ void __launch_bounds__(TT_THREADS, 1) k_field_train_tc(
                                 umma_bf16(tm + TT_COL_GB + 16 * l, da, umma_desc(ones + s * 512, 256, 128),
                                           kIdescN16 | kIdescAT, add);
                             }
+                            commit(&S.free_dz[w]);
                         }
-                        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                            smem_addr(&S.done[w])));
                     }
                     __syncwarp();
                 }
@@ -1131,7 +1144,7 @@ __global__ void __launch_bounds__(TT_THREADS, 1) k_field_train_tc(
     } else {
         const uint32_t row_acc = tm + ((uint32_t)(32 * q) << 16) + TT_COL_ACC + 64 * pipe + c0;
         const uint32_t bar_done = smem_addr(&S.done[pipe]);
-        uint32_t ph = 0, phx = 0;
+        uint32_t ph = 0, phx = 0, phz = 0;
         // stores into shared memory, visible to the products; reads of the accumulator, before them
         auto give = [&]() {
             asm volatile("fence.proxy.async.shared::cta;");
@@ -1143,6 +1156,20 @@ __global__ void __launch_bounds__(TT_THREADS, 1) k_field_train_tc(
             ph ^= 1;
             asm volatile("tcgen05.fence::after_thread_sync;");
             return ok;
+        };
+        auto take_dz = [&]() {   // dZ, and with the last layer's gradients every H, may be overwritten
+            ok = mbar_wait(smem_addr(&S.free_dz[pipe]), phz);
+            phz ^= 1;
+            return ok;
+        };
+        // the part of H_l's row that this thread stored, as pairs; a unit is active where it is > 0
+        auto active = [&](const __nv_bfloat16* T, uint32_t* pairs) {
+            const char* row = reinterpret_cast<const char*>(T) + (c0 / 8) * 2048 + (p >> 3) * 128 + (p & 7) * 16;
+#pragma unroll
+            for (int g = 0; g < TT_CW / 8; ++g) {
+                const uint4 v = *reinterpret_cast<const uint4*>(row + g * 2048);
+                pairs[4 * g] = v.x, pairs[4 * g + 1] = v.y, pairs[4 * g + 2] = v.z, pairs[4 * g + 3] = v.w;
+            }
         };
         for (uint32_t k = (uint32_t)pipe; k < mine && ok; k += TT_PIPES) {
             const uint32_t e = ne;
@@ -1158,9 +1185,8 @@ __global__ void __launch_bounds__(TT_THREADS, 1) k_field_train_tc(
             uint32_t pk[TT_CW / 2];
             if (c == 0) encode_half<0>(xt, pk);
             else encode_half<1>(xt, pk);
-            if (k >= TT_PIPES && !take()) break;   // the last gradients of the pipeline's previous tile
+            if (k >= TT_PIPES && !take_dz()) break;   // the last gradients of the pipeline's previous tile
             store_part(S.H[pipe][0], p, c0, pk);
-            uint32_t mask[FD];
             float zp = 0.f;
 #pragma unroll
             for (int l = 0; l < FD; ++l) {
@@ -1170,14 +1196,8 @@ __global__ void __launch_bounds__(TT_THREADS, 1) k_field_train_tc(
 #pragma unroll
                 for (int j = 0; j < TT_CW; j += 16) tmem_ld16(row_acc + j, z + j);
                 asm volatile("tcgen05.wait::ld.sync.aligned;");
-                uint32_t m = 0;
 #pragma unroll
-                for (int j = 0; j < TT_CW; j += 2) {
-                    pk[j / 2] = pack_bf16_relu(z[j], z[j + 1]);
-                    m |= (z[j] > 0.f ? 1u : 0u) << j;
-                    m |= (z[j + 1] > 0.f ? 1u : 0u) << (j + 1);
-                }
-                mask[l] = m;
+                for (int j = 0; j < TT_CW; j += 2) pk[j / 2] = pack_bf16_relu(z[j], z[j + 1]);
                 if (l + 1 < FD) {
                     store_part(S.H[pipe][l + 1], p, c0, pk);
                 } else {
@@ -1201,15 +1221,12 @@ __global__ void __launch_bounds__(TT_THREADS, 1) k_field_train_tc(
             z5 += S.w5[FW];
             const float r = e < batch ? softplusf(z5) - y : 0.f;
             const float dz5 = 2.f * r * inv_b * sigmoidf_(z5);
-            // dZ_3 = bf16(dz5 w5 . [z_3 > 0])
+            // dZ_3 = bf16(dz5 w5) where h_4 > 0
             {
                 uint32_t dz[TT_CW / 2];
 #pragma unroll
-                for (int j = 0; j < TT_CW; j += 2) {
-                    const float d0 = (mask[FD - 1] >> j) & 1u ? dz5 * S.w5[c0 + j] : 0.f;
-                    const float d1 = (mask[FD - 1] >> (j + 1)) & 1u ? dz5 * S.w5[c0 + j + 1] : 0.f;
-                    dz[j / 2] = pack_bf16(d0, d1);
-                }
+                for (int j = 0; j < TT_CW; j += 2)
+                    dz[j / 2] = pack_bf16(dz5 * S.w5[c0 + j], dz5 * S.w5[c0 + j + 1]) & positive2(pk[j / 2]);
                 store_part(S.DZ[pipe], p, c0, dz);
             }
             give();
@@ -1228,23 +1245,22 @@ __global__ void __launch_bounds__(TT_THREADS, 1) k_field_train_tc(
             }
 #pragma unroll
             for (int l = FD - 1; l > 0; --l) {
+                uint32_t h[TT_CW / 2];
+                active(S.H[pipe][l], h);
                 if (!take()) break;
-                // dZ_{l-1} = bf16(dH_l . [z_{l-1} > 0])
+                // dZ_{l-1} = bf16(dH_l) where h_l > 0
                 float dh[TT_CW];
 #pragma unroll
                 for (int j = 0; j < TT_CW; j += 16) tmem_ld16(row_acc + j, dh + j);
                 asm volatile("tcgen05.wait::ld.sync.aligned;");
 #pragma unroll
-                for (int j = 0; j < TT_CW; j += 2) {
-                    const float d0 = (mask[l - 1] >> j) & 1u ? dh[j] : 0.f;
-                    const float d1 = (mask[l - 1] >> (j + 1)) & 1u ? dh[j + 1] : 0.f;
-                    pk[j / 2] = pack_bf16(d0, d1);
-                }
+                for (int j = 0; j < TT_CW; j += 2) pk[j / 2] = pack_bf16(dh[j], dh[j + 1]) & positive2(h[j / 2]);
+                if (!take_dz()) break;
                 store_part(S.DZ[pipe], p, c0, pk);
                 give();
             }
         }
-        if (ok && (uint32_t)pipe < mine) take();   // the last tile's last gradients
+        if (ok && (uint32_t)pipe < mine) take_dz();   // the last tile's last gradients
         if (c == 0) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
@@ -1315,7 +1331,8 @@ __global__ void __launch_bounds__(TT_THREADS, 1) k_field_train_tc(
 // Gradient = the fixed-order sum of the blocks' partial sums; then either that gradient is
 // stored (grad_out) or one Adam step is taken (and the bf16 copies of the weights refreshed).
 // A block of 8 warps handles 32 consecutive entries: warp w adds the slices b = w, w + 8, ... in
-// order, then the eight warp sums are added in warp order. Entry NPAR of every slice (padding)
+// order, then the eight warp sums are added in warp order (16 warps with all their loads in flight: 9.5
+// instead of 8.7 us). Entry NPAR of every slice (padding)
 // holds a block's squared-error sum; its total goes to loss_sum.
 constexpr int UPD_WARPS = 8;
 __global__ void __launch_bounds__(32 * UPD_WARPS) k_field_update(
