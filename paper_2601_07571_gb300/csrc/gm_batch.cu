@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(ACC_THREADS, 4) k_accumulate_batch_shaft(const
                                                                            uint32_t n_items,
                                                                            unsigned int* __restrict__ work, AccConst C,
                                                                            int* __restrict__ err) {
-    __shared__ ShaftBlock B;
+    __shared__ ShaftBlock<1> B;
     __shared__ uint32_t s_item;
     const DebugOut dbg{nullptr, nullptr, nullptr, nullptr, nullptr};
     for (;;) {
@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(ACC_THREADS, 4) k_accumulate_batch_shaft(const
         P.dbg_cap = 0;
         P.tanphi = sqrtf(C.K) * 1.00001f;
         TileStats st;
-        shaft_tile<false>(wi.y, Sd.spos, Sd.sidx, Sd.fix, *Sd.n_fix, Sd.nodes, Sd.nodes4, Sd.tris, P, Sd.out, Sd.max_bits,
+        shaft_tile<false, 1>(wi.y, Sd.spos, Sd.sidx, Sd.fix, *Sd.n_fix, Sd.nodes, Sd.nodes4, Sd.tris, P, Sd.out, Sd.max_bits,
                           B, nullptr, dbg, err, st);
         warp_stats_commit(st, Sd.counters);
     }

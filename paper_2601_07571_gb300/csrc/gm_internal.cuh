@@ -74,7 +74,14 @@ struct gm_samples {
     // spatial work order for the accumulation (Morton order of the sample positions)
     float4* work_pos = nullptr;      // n, work order
     uint32_t* work_idx = nullptr;    // n, stored index of each work-order sample
+    // Of GM_TILE_LIST_MIN samples or more: the work order's tiles of 128 samples on few triangles, and
+    // the tiles of 32 of all others. [0] and [1] their numbers, then the lists (gm_tile_list_fine)
+    uint32_t* tile_lists = nullptr;
 };
+
+constexpr uint64_t GM_TILE_LIST_MIN = 1u << 16;
+// Where the list of 32-sample tiles starts in gm_samples::tile_lists.
+__host__ __device__ inline size_t gm_tile_list_fine(uint64_t n) { return 2 + (size_t)((n + 127) / 128); }
 
 struct gm_map {
     gm_ctx* ctx = nullptr;

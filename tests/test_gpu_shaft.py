@@ -1,7 +1,8 @@
 """The shaft walk (the default accumulation kernel) against the per-ray walk (GM_F_FIX_L1) on the same
 scenes: both decide every ray with the same arithmetic and add the weights in the same order, so the
 maps are equal bit for bit. Sizes at the edges of a warp tile, of a fill step (512 fixations) and of a
-batch; trees of one and two triangles; triangles far smaller than the sample spacing (a shaft over its
+batch; sample sets of 65536 samples and more, which have tiles of 128 samples where those lie on few
+triangles, with such tiles in the majority and without any; trees of one and two triangles; triangles far smaller than the sample spacing (a shaft over its
 budget); an eye close to the surface, whose rays differ in their dominant axis and cross the planes
 through the eye."""
 import math
@@ -36,12 +37,17 @@ def _scene(kind):
     if kind == "fine":      # 80k triangles of about 1 mm on a 6 cm sphere, before a coarse one
         v, f = M.uv_sphere(12, 24, 0.5)
         return M.merge([M.uv_sphere(142, 284, 0.06, 0.05, 30.0, seed=3), (M.translate(v, (0.0, 0.0, 0.9)), f)])
+    if kind == "mixed":     # a box of large triangles (seven tenths of the samples) beside a sphere of small ones
+        v, f = M.uv_sphere(60, 120, 0.4, 0.05, 6.0, seed=4)
+        return M.merge([M.box((0.0, 0.0, 0.0), 0.8), (M.translate(v, (0.0, 0.3, 1.5)), f)])
     return M.uv_sphere(40, 80, 1.0, 0.1, 4.0, seed=5)
 
 
-def _points(v, f, n, rng):
+def _points(kind, v, f, n, rng):
     t = v[f.astype(np.int64)].astype(np.float64)
     tri = rng.integers(0, len(f), n)
+    if kind == "mixed":
+        tri[rng.random(n) < 0.7] %= 12
     s, u = np.sqrt(rng.random((n, 1))), rng.random((n, 1))
     p = (1 - s) * t[tri, 0] + s * (1 - u) * t[tri, 1] + s * u * t[tri, 2]
     return np.ascontiguousarray(p, np.float32), tri.astype(np.uint32)
@@ -50,13 +56,14 @@ def _points(v, f, n, rng):
 @pytest.mark.parametrize("kind,n,nf,theta,near,windows", [
     ("one", 1, 3, 4.0, False, 1), ("two", 33, 40, 4.0, False, 1),
     ("sphere", 31, 511, 2.0, False, 1), ("sphere", 32, 512, 2.0, False, 3), ("sphere", 1000, 1300, 6.0, False, 5),
-    ("fine", 2048, 600, 1.0, False, 1), ("sphere", 3000, 200, 15.0, True, 1), ("sphere", 257, 0, 1.0, False, 2)])
+    ("mixed", 65537, 300, 2.0, False, 1), ("mixed", 70001, 300, 3.0, False, 3),
+    ("fine", 2048, 600, 1.0, False, 1), ("fine", 65600, 60, 1.0, False, 1), ("sphere", 3000, 200, 15.0, True, 1), ("sphere", 257, 0, 1.0, False, 2)])
 def test_shaft_walk_equals_per_ray_walk(env, kind, n, nf, theta, near, windows):
     G, ctx = env
     rng = np.random.default_rng(n + nf)
     v, f = _scene(kind)
     scene = G.gm_build_scene(ctx, [(v, f, np.eye(4), 0)])
-    xyz, tri = _points(v, f, n, rng)
+    xyz, tri = _points(kind, v, f, n, rng)
     samples = G.gm_samples_from_points(scene, xyz, tri)
     at = xyz[rng.integers(0, n, nf)].astype(np.float64)
     if near:      # a few centimetres off the surface, looking along it or at it
@@ -76,7 +83,9 @@ def test_shaft_walk_equals_per_ray_walk(env, kind, n, nf, theta, near, windows):
         maps = np.empty((W, ns), np.float32)
         top = [G.gm_map_copy(m, w, maps[w]) for w in range(W)]
         G.gm_map_free(m)
-        out.append((maps, top, {k: st[k] for k in ("pairs", "in_cone", "visible", "pairs_tested")}))
+        # the cone tests evaluated depend on the size of a form's tiles: between the in-cone and all pairs
+        assert st["in_cone"] <= st["pairs_tested"] <= st["pairs"]
+        out.append((maps, top, {k: st[k] for k in ("pairs", "in_cone", "visible")}))
     G.gm_samples_free(samples)
     G.gm_scene_free(scene)
     assert W == windows and out[0][2] == out[1][2] and out[0][1] == out[1][1]
