@@ -11,6 +11,7 @@
 // Bound by launches and latency at these sizes (800k 63-bit keys: 19 MB a pass).
 #include <algorithm>
 
+#include "gm_blocksort.cuh"
 #include "gm_internal.cuh"
 #include "gm_scan.cuh"
 
@@ -20,7 +21,6 @@ constexpr int RS_THREADS = 256;
 constexpr int RS_ITEMS = 8;
 constexpr int RS_TILE = RS_THREADS * RS_ITEMS;
 constexpr int RS_WARPS = RS_THREADS / 32;
-constexpr int RS_SMALL = 2048;   // keys sorted by one block
 
 template <typename K>
 __global__ void __launch_bounds__(RS_THREADS) rs_hist(const K* __restrict__ keys, uint32_t n, int shift,
@@ -119,68 +119,19 @@ __global__ void __launch_bounds__(RS_THREADS) rs_scatter(const K* __restrict__ k
 // All passes of n <= RS_SMALL keys in one block, in place.
 template <typename K>
 __global__ void __launch_bounds__(1024) rs_small(K* __restrict__ keys, uint32_t* __restrict__ vals, uint32_t n, int bits) {
-    constexpr int PER = RS_SMALL / 1024;
-    __shared__ K sk[RS_SMALL];
-    __shared__ uint32_t sv[RS_SMALL];
-    __shared__ uint16_t count[32][256];
-    __shared__ uint32_t dbase[256];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint32_t base = warp * (32 * PER) + lane;
-    K k[PER];
-    uint32_t v[PER];
+    __shared__ BlockSort<K> B;
+    const uint32_t base = block_sort_base();
+    K k[RS_PER];
+    uint32_t v[RS_PER];
 #pragma unroll
-    for (int i = 0; i < PER; ++i) {
+    for (int i = 0; i < RS_PER; ++i) {
         const uint32_t idx = base + i * 32;
         k[i] = idx < n ? keys[idx] : K(0);
         v[i] = idx < n ? vals[idx] : 0u;
     }
-    for (int shift = 0; shift < bits; shift += 8) {
-        for (int i = tid; i < 32 * 256; i += 1024) (&count[0][0])[i] = 0;
-        __syncthreads();
-        uint32_t rank[PER];
+    block_sort(k, v, n, bits, B);
 #pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            const uint32_t d = base + i * 32 < n ? (uint32_t)((k[i] >> shift) & 255u) : 256u;
-            const unsigned peers = __match_any_sync(0xffffffffu, d);
-            const uint32_t before = d < 256u ? count[warp][d] : 0u;
-            __syncwarp();
-            if (d < 256u && (peers & gm_lanemask_lt()) == 0) count[warp][d] = (uint16_t)(before + __popc(peers));
-            __syncwarp();
-            rank[i] = before + __popc(peers & gm_lanemask_lt());
-        }
-        __syncthreads();
-        uint32_t run = 0;
-        if (tid < 256) {
-            for (int w = 0; w < 32; ++w) {
-                const uint32_t c = count[w][tid];
-                count[w][tid] = (uint16_t)run;
-                run += c;
-            }
-        }
-        uint32_t all;
-        const uint32_t below = block_excl_scan<uint32_t, 1024>(run, &all);
-        if (tid < 256) dbase[tid] = below;
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            if (base + i * 32 >= n) continue;
-            const uint32_t d = (uint32_t)((k[i] >> shift) & 255u);
-            const uint32_t pos = dbase[d] + count[warp][d] + rank[i];
-            sk[pos] = k[i];
-            sv[pos] = v[i];
-        }
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            const uint32_t idx = base + i * 32;
-            if (idx < n) {
-                k[i] = sk[idx];
-                v[i] = sv[idx];
-            }
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
+    for (int i = 0; i < RS_PER; ++i) {
         const uint32_t idx = base + i * 32;
         if (idx < n) {
             keys[idx] = k[i];
