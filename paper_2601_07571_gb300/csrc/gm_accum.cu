@@ -411,14 +411,8 @@ gm_status accumulate_impl(gm_scene* sc, gm_samples* sm, const gm_fixations* fx, 
         // the persistent kernel's tile counter starts from 0 on every launch
         if (!prep) GM_TRY_CUDA(cudaMemsetAsync(&mp->counters[6], 0, sizeof(unsigned long long), s));
     } else {
-        MAP_ALLOC(mp->values, sizeof(float) * W * ns);
-        MAP_ALLOC(mp->max_bits, sizeof(unsigned int) * W);
-        MAP_ALLOC(mp->counters, sizeof(unsigned long long) * 8);
-        if (!prep) {
-            GM_TRY_CUDA(cudaMemsetAsync(mp->max_bits, 0, sizeof(unsigned int) * W, s));
-            GM_TRY_CUDA(cudaMemsetAsync(mp->counters, 0, sizeof(unsigned long long) * 8, s));
-        }
-        if (W > 1) GM_TRY_CUDA(cudaMemsetAsync(mp->values, 0, sizeof(float) * W * ns, s));
+        if ((st = gm_map_alloc(mp, 8, s)) != GM_OK) return fail(st);
+        if (W > 1 || !prep) GM_TRY_CUDA(gm_map_zero(mp, W > 1, s));
     }
     if (debug && !into) {
         mp->dbg_cap = prm->debug_pair_cap;
@@ -866,9 +860,7 @@ extern "C" gm_status gm_map_debug_pairs(const gm_map* mp, uint32_t* sample, uint
 
 extern "C" void gm_map_free(gm_map* mp) {
     if (!mp) return;
-    cudaFree(mp->values);
-    cudaFree(mp->max_bits);
-    cudaFree(mp->counters);
+    cudaFree(mp->block);
     cudaFree(mp->dbg_sample);
     cudaFree(mp->dbg_fix);
     cudaFree(mp->dbg_vis);

@@ -382,9 +382,7 @@ static gm_status batch_capture(gm_batch* b, bool concurrent = true) {
         cudaMemsetAsync(b->n_valid, 0, sizeof(uint32_t) * b->n, cs);
         for (uint32_t i = 0; i < b->n; ++i) {
             gm_map* m = b->maps[i];
-            cudaMemsetAsync(m->max_bits, 0, sizeof(unsigned int) * m->W, cs);
-            cudaMemsetAsync(m->counters, 0, sizeof(unsigned long long) * 8, cs);
-            if (m->W > 1 && m->ns) cudaMemsetAsync(m->values, 0, sizeof(float) * m->W * m->ns, cs);
+            gm_map_zero(m, m->W > 1, cs);
         }
         if (b->nf_total > 0) {
             k_bfix_keys<<<gm_div_up(b->nf_total, 256), 256, 0, cs>>>(
@@ -530,9 +528,7 @@ extern "C" gm_status gm_batch_create(gm_ctx* ctx, const gm_session_desc* ss, uin
         m->stream = s;
         m->stats.n_windows = b->W;
         b->maps.push_back(m);
-        if ((st = gm_alloc((void**)&m->values, sizeof(float) * m->W * (m->ns ? m->ns : 1), s)) != GM_OK) return fail(st);
-        if ((st = gm_alloc((void**)&m->max_bits, sizeof(unsigned int) * m->W, s)) != GM_OK) return fail(st);
-        if ((st = gm_alloc((void**)&m->counters, sizeof(unsigned long long) * 8, s)) != GM_OK) return fail(st);
+        if ((st = gm_map_alloc(m, 8, s)) != GM_OK) return fail(st);
         b->pairs += (uint64_t)ss[i].fix.n * m->ns;
     }
     b->nf_total = b->fix_off[n];

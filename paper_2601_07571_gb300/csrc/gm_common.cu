@@ -40,6 +40,21 @@ gm_status gm_alloc(void** p, size_t bytes, cudaStream_t s) {
     return GM_OK;
 }
 
+gm_status gm_map_alloc(gm_map* mp, int n_counters, cudaStream_t s) {
+    const size_t c = sizeof(unsigned long long) * n_counters;
+    mp->head = (c + sizeof(unsigned int) * (size_t)mp->W + 255) / 256 * 256;
+    GM_TRY(gm_alloc(&mp->block, mp->head + sizeof(float) * (size_t)mp->W * mp->ns, s));
+    char* base = static_cast<char*>(mp->block);
+    mp->counters = reinterpret_cast<unsigned long long*>(base);
+    mp->max_bits = reinterpret_cast<unsigned int*>(base + c);
+    mp->values = reinterpret_cast<float*>(base + mp->head);
+    return GM_OK;
+}
+
+cudaError_t gm_map_zero(gm_map* mp, bool values, cudaStream_t s) {
+    return cudaMemsetAsync(mp->block, 0, mp->head + (values ? sizeof(float) * (size_t)mp->W * mp->ns : 0), s);
+}
+
 gm_status gm_stage_to_device(const void* src, size_t bytes, cudaStream_t s, void** dev, bool* owned) {
     *owned = false;
     *dev = nullptr;

@@ -87,6 +87,9 @@ struct gm_map {
     gm_ctx* ctx = nullptr;
     uint32_t W = 1;
     uint64_t ns = 0;
+    // one allocation: counters, maxima (head bytes together), values
+    void* block = nullptr;
+    size_t head = 0;
     float* values = nullptr;           // W x ns
     unsigned int* max_bits = nullptr;  // W (bit pattern of a non-negative float)
     unsigned long long* counters = nullptr;  // [0] in_cone [1] visible [2] debug cursor [3] fixations used
@@ -114,6 +117,9 @@ bool gm_is_device_ptr(const void* p);
 gm_status gm_stage_to_device(const void* src, size_t bytes, cudaStream_t s, void** dev, bool* owned);
 gm_status gm_copy_out(void* dst, const void* dev_src, size_t bytes, cudaStream_t s);
 gm_status gm_alloc(void** p, size_t bytes, cudaStream_t s);
+// A map's values, maxima and n_counters counters (W and ns are set), and zeroing the latter two or all.
+gm_status gm_map_alloc(gm_map* mp, int n_counters, cudaStream_t s);
+cudaError_t gm_map_zero(gm_map* mp, bool values, cudaStream_t s);
 
 // ------------------------------------------------------------------------------------------
 // sort / scan (gm_sort.cu)

@@ -924,12 +924,8 @@ extern "C" gm_status gm_accumulate_zbuffer(gm_scene* sc, gm_samples* sm, const g
     } while (0)
 #define MAP_ALLOC(ptr, bytes) \
     if ((st = gm_alloc((void**)&(ptr), (bytes), s)) != GM_OK) return fail(st)
-    MAP_ALLOC(mp->values, sizeof(float) * W * (ns ? ns : 1));
-    MAP_ALLOC(mp->max_bits, sizeof(unsigned int) * W);
-    MAP_ALLOC(mp->counters, sizeof(unsigned long long) * 16);
-    GM_TRY_CUDA(cudaMemsetAsync(mp->values, 0, sizeof(float) * W * (ns ? ns : 1), s));
-    GM_TRY_CUDA(cudaMemsetAsync(mp->max_bits, 0, sizeof(unsigned int) * W, s));
-    GM_TRY_CUDA(cudaMemsetAsync(mp->counters, 0, sizeof(unsigned long long) * 16, s));
+    if ((st = gm_map_alloc(mp, 16, s)) != GM_OK) return fail(st);
+    GM_TRY_CUDA(gm_map_zero(mp, true, s));
     if (debug) {
         mp->dbg_cap = prm->debug_pair_cap;
         MAP_ALLOC(mp->dbg_sample, sizeof(uint32_t) * mp->dbg_cap);
