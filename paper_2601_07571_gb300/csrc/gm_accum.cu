@@ -186,15 +186,17 @@ __global__ void __launch_bounds__(NT, MINB) k_accumulate(
 // take 9.4 ms with the cube in wide tiles, 8.0 without.
 __device__ __forceinline__ bool wide_tiles_pay(const uint32_t* lists, uint64_t ns) { return 2ull * 128 * lists[0] >= ns; }
 
-template <bool DEBUG, bool LISTS>
-__global__ void __launch_bounds__(ACC_THREADS, 4) k_accumulate_shaft(
+template <bool DEBUG, bool LISTS, int NT = ACC_THREADS>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_accumulate_shaft(
     const float4* __restrict__ spos, const uint32_t* __restrict__ sidx, const float4* __restrict__ fix,
     const uint32_t* __restrict__ n_fix_dev, const float4* __restrict__ nodes, const float4* __restrict__ nodes4,
     const float4* __restrict__ tris, AccParams P, uint32_t n_tiles, const uint32_t* __restrict__ lists,
     int persistent, float* __restrict__ out, unsigned int* __restrict__ max_bits,
     unsigned long long* __restrict__ counters, int* __restrict__ err, DebugOut dbg) {
     constexpr size_t BYTES = LISTS && sizeof(ShaftBlock<4>) > sizeof(ShaftBlock<1>) ? sizeof(ShaftBlock<4>) : sizeof(ShaftBlock<1>);
-    __shared__ __align__(16) unsigned char smem[BYTES];
+    __shared__ __align__(16) unsigned char fixed[NT == ACC_THREADS ? BYTES : 16];
+    extern __shared__ __align__(16) unsigned char dynamic[];   // above 48 KB
+    unsigned char* smem = NT == ACC_THREADS ? fixed : dynamic;
     __shared__ uint32_t s_tile;
     const uint32_t nf = *n_fix_dev;
     if (lists && wide_tiles_pay(lists, P.ns) != LISTS) return;
@@ -215,8 +217,8 @@ __global__ void __launch_bounds__(ACC_THREADS, 4) k_accumulate_shaft(
             shaft_tile<DEBUG, 4>(__ldg(&lists[2 + k]), spos, sidx, fix, nf, nodes, nodes4, tris, P, out, max_bits,
                                  *reinterpret_cast<ShaftBlock<4>*>(smem), &counters[2], dbg, err, st);
         else
-            shaft_tile<DEBUG, 1>(LISTS ? __ldg(&lists[gm_tile_list_fine(P.ns) + (k - n_wide)]) : k, spos, sidx, fix, nf, nodes,
-                                 nodes4, tris, P, out, max_bits, *reinterpret_cast<ShaftBlock<1>*>(smem), &counters[2],
+            shaft_tile<DEBUG, 1, NT>(LISTS ? __ldg(&lists[gm_tile_list_fine(P.ns) + (k - n_wide)]) : k, spos, sidx, fix, nf, nodes,
+                                 nodes4, tris, P, out, max_bits, *reinterpret_cast<ShaftBlock<1, NT>*>(smem), &counters[2],
                                  dbg, err, st);
         if (!persistent) break;
     }
@@ -336,6 +338,18 @@ gm_status n_windows_of(const gm_params* prm, uint64_t* W_out) {
 // The accumulation of one fixation set. into == nullptr: a new map (returned in *out) over all
 // windows. into != nullptr: adds the fixations of window `only_window` to that existing map
 // (no normalisation, no stage timing), for dynamic scenes posed window by window.
+// Threads of a shaft kernel's blocks for n_fix fixations. A tile is one block's from beginning to end, so
+// where the GPU has few tiles a block and each sees many fixations, the longest tile sets the time and more
+// warps shorten it; where they see few, a large block mostly waits at the end of its batches. With 256 /
+// 512 / 1024 threads, us: 9 tiles x 734 fixations 287 / 219 / 189, 94 x 400: 151 / 123 / 115, 337 x 784:
+// 1676 / 1173 / 1078, 208 x 100: 88 / 80 / 86, 1563 x 1000: 689 / 646, 1875 x 800 (tiles of tiny triangles
+// among others): 2386 / 1618, 3125 x 1000 (the same): 3186 / 2301; but 938 x 120: 225 / 242, 1875 x 200:
+// 438 / 472, 3125 x 400: 654 / 739, and 62500 x 6000: 60.2 / 65.7 / 78.1 ms.
+int shaft_threads(uint64_t tiles, uint64_t n_fix, int n_sm) {
+    if (tiles <= 3ull * n_sm && n_fix >= 256) return 1024;
+    return tiles <= 24ull * n_sm && tiles <= 4 * n_fix ? 512 : ACC_THREADS;
+}
+
 template <typename K>
 int blocks_per_sm(K kern) {
     int b = 0;
@@ -620,17 +634,34 @@ gm_status accumulate_impl(gm_scene* sc, gm_samples* sm, const gm_fixations* fx, 
                 const uint32_t* lists = reorder && persistent ? sm->tile_lists : nullptr;
                 const uint32_t tiles = gm_div_up(ns, 32);
                 auto grid = [&](int b) { return persistent ? std::min<uint32_t>((uint32_t)(ctx->n_sm * b), tiles) : tiles; };
-                auto kern = debug ? k_accumulate_shaft<true, false> : k_accumulate_shaft<false, false>;
-                kern<<<grid(per_sm), ACC_THREADS, 0, s>>>(spos, sidx, packed, n_valid, sc->nodes, sc->nodes4,
-                                                          sc->bvh_tris, P, tiles, lists, persistent, mp->values,
-                                                          mp->max_bits, mp->counters, ctx->dev_err, dbg);
-                if (lists) {
-                    kern = debug ? k_accumulate_shaft<true, true> : k_accumulate_shaft<false, true>;
-                    kern<<<grid(per_sm_lists), ACC_THREADS, 0, s>>>(spos, sidx, packed, n_valid, sc->nodes, sc->nodes4,
-                                                                    sc->bvh_tris, P, tiles, lists, persistent,
-                                                                    mp->values, mp->max_bits, mp->counters,
-                                                                    ctx->dev_err, dbg);
-                    launches++;
+                // (large blocks take tiles of 32 samples alone)
+                auto few = [&](auto kern, int nt, size_t bytes) -> cudaError_t {
+                    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+                    if (e != cudaSuccess) return e;
+                    kern<<<grid(1024 / nt), nt, bytes, s>>>(spos, sidx, packed, n_valid, sc->nodes, sc->nodes4, sc->bvh_tris,
+                                                            P, tiles, nullptr, persistent, mp->values, mp->max_bits,
+                                                            mp->counters, ctx->dev_err, dbg);
+                    return cudaSuccess;
+                };
+                const int nt = debug || !persistent ? ACC_THREADS
+                                                    : shaft_threads(tiles, only_window >= 0 ? nf / W : nf, ctx->n_sm);
+                if (nt == 1024) {
+                    GM_TRY_CUDA(few(k_accumulate_shaft<false, false, 1024>, 1024, sizeof(ShaftBlock<1, 1024>)));
+                } else if (nt == 512) {
+                    GM_TRY_CUDA(few(k_accumulate_shaft<false, false, 512>, 512, sizeof(ShaftBlock<1, 512>)));
+                } else {
+                    auto kern = debug ? k_accumulate_shaft<true, false> : k_accumulate_shaft<false, false>;
+                    kern<<<grid(per_sm), ACC_THREADS, 0, s>>>(spos, sidx, packed, n_valid, sc->nodes, sc->nodes4,
+                                                              sc->bvh_tris, P, tiles, lists, persistent, mp->values,
+                                                              mp->max_bits, mp->counters, ctx->dev_err, dbg);
+                    if (lists) {
+                        kern = debug ? k_accumulate_shaft<true, true> : k_accumulate_shaft<false, true>;
+                        kern<<<grid(per_sm_lists), ACC_THREADS, 0, s>>>(spos, sidx, packed, n_valid, sc->nodes, sc->nodes4,
+                                                                        sc->bvh_tris, P, tiles, lists, persistent,
+                                                                        mp->values, mp->max_bits, mp->counters,
+                                                                        ctx->dev_err, dbg);
+                        launches++;
+                    }
                 }
             } else if (debug) {
                 switch (code & 3) {

@@ -532,23 +532,22 @@ __device__ __forceinline__ unsigned shaft_visible_wide(unsigned in, const float4
 // triangles), sample sets of a few thousand fill the GPU, and the sums stay those of a sequential pass.
 // (A tile per warp with shared lists instead: 126 ms against 68 ms at the 800k-triangle scene, whose
 // patch of 1 mm triangles then falls to few blocks.)
-constexpr int SH_WARPS = ACC_THREADS / 32;
 // Fixations are listed until a batch has shaft_fill of them (or none is left), shaft_per a thread at a
 // step. Smaller batches wait for their last item more often: a wide tile's at 1 instead of 128 takes
 // 33 ms at the city's windows instead of 21, a narrow tile's at 64 or 128 instead of 256 more as well.
 constexpr int SH_FILL1 = 256, SH_FILL4 = 128;
 __host__ __device__ constexpr int shaft_fill(int ns) { return ns == 1 ? SH_FILL1 : SH_FILL4; }
-__host__ __device__ constexpr int shaft_per(int ns) { return ns == 1 ? 2 : 1; }
-__host__ __device__ constexpr int shaft_list(int ns) { return shaft_fill(ns) - 1 + shaft_per(ns) * ACC_THREADS; }
+__host__ __device__ constexpr int shaft_per(int ns, int nt) { return ns == 1 && nt == ACC_THREADS ? 2 : 1; }
+__host__ __device__ constexpr int shaft_list(int ns, int nt) { return shaft_fill(ns) - 1 + shaft_per(ns, nt) * nt; }
 
-template <int NS>
+template <int NS, int NT = ACC_THREADS>
 struct ShaftBlock {
-    ShaftWarp warp[SH_WARPS];
+    ShaftWarp warp[NT / 32];
     ShaftStart start;
     float4 pos[NS == 1 ? 1 : 32 * NS];   // the tile's samples (NS = 1: in registers)
-    uint32_t list[shaft_list(NS)];      // fixation indices
-    uint32_t vis[NS][shaft_list(NS)];   // visible samples of each item
-    uint32_t pass[SH_WARPS];    // passing fixations of each warp's 64 in one fill step
+    uint32_t list[shaft_list(NS, NT)];      // fixation indices
+    uint32_t vis[NS][shaft_list(NS, NT)];   // visible samples of each item
+    uint32_t pass[NT / 32];    // passing fixations of each warp's 64 in one fill step
     int next;                   // next item to trace
 };
 
@@ -578,13 +577,13 @@ __device__ __forceinline__ float4 work_sample(const float4* __restrict__ spos, u
 // One block, all threads: tile `tile` (32 NS consecutive work-order samples) against fixations [0, nf) of
 // `fix` (packed (e, w), (r^, window), sorted by window). A window's sums are written when the next visible
 // fixation opens another one, or at the end.
-template <bool DEBUG, int NS>
+template <bool DEBUG, int NS, int NT = ACC_THREADS>
 __device__ __forceinline__ void shaft_tile(const uint32_t tile, const float4* __restrict__ spos,
                                            const uint32_t* __restrict__ sidx, const float4* __restrict__ fix,
                                            const uint32_t nf, const float4* __restrict__ nodes,
                                            const float4* __restrict__ nodes4, const float4* __restrict__ tris,
                                            const AccParams& P, float* __restrict__ out,
-                                           unsigned int* __restrict__ max_bits, ShaftBlock<NS>& B,
+                                           unsigned int* __restrict__ max_bits, ShaftBlock<NS, NT>& B,
                                            unsigned long long* __restrict__ dbg_cursor, const DebugOut& dbg,
                                            int* __restrict__ err, TileStats& st) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -629,7 +628,7 @@ __device__ __forceinline__ void shaft_tile(const uint32_t tile, const float4* __
     };
     for (uint32_t pos = 0; pos < nf;) {
         // list the fixations that reach the tile: a warp takes 32 PER consecutive ones of each step
-        constexpr int PER = shaft_per(NS);
+        constexpr int PER = shaft_per(NS, NT);
         int cnt = 0;
         while (cnt < shaft_fill(NS) && pos < nf) {
             unsigned reach[PER];
@@ -643,7 +642,7 @@ __device__ __forceinline__ void shaft_tile(const uint32_t tile, const float4* __
             }
             if (lane == 0) B.pass[warp] = mine;
             __syncthreads();
-            const int n = lane < SH_WARPS ? (int)B.pass[lane] : 0;
+            const int n = lane < NT / 32 ? (int)B.pass[lane] : 0;
             int at = cnt + __reduce_add_sync(0xffffffffu, lane < warp ? n : 0);
             cnt += __reduce_add_sync(0xffffffffu, n);
 #pragma unroll
@@ -651,7 +650,7 @@ __device__ __forceinline__ void shaft_tile(const uint32_t tile, const float4* __
                 if ((reach[r] >> lane) & 1u) B.list[at + __popc(reach[r] & lt)] = pos + (warp * PER + r) * 32 + lane;
                 at += __popc(reach[r]);
             }
-            pos += PER * ACC_THREADS;
+            pos += PER * NT;
             if (threadIdx.x == 0) B.next = 0;
             __syncthreads();
         }

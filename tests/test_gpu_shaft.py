@@ -1,10 +1,11 @@
 """The shaft walk (the default accumulation kernel) against the per-ray walk (GM_F_FIX_L1) on the same
 scenes: both decide every ray with the same arithmetic and add the weights in the same order, so the
-maps are equal bit for bit. Sizes at the edges of a warp tile, of a fill step (512 fixations) and of a
-batch; sample sets of 65536 samples and more, which have tiles of 128 samples where those lie on few
-triangles, with such tiles in the majority and without any; trees of one and two triangles; triangles far smaller than the sample spacing (a shaft over its
-budget); an eye close to the surface, whose rays differ in their dominant axis and cross the planes
-through the eye."""
+maps are equal bit for bit. Sizes at the edges of a warp tile, of a fill step (512 fixations), of a batch
+and of the ranges of the block sizes (456 tiles, 256 fixations, a quarter as many fixations as tiles);
+sample sets of 65536 samples and more, which have tiles of 128 samples where those lie on few triangles,
+with such tiles in the majority and without any; trees of one and two triangles; triangles far smaller
+than the sample spacing (a shaft over its budget); an eye close to the surface, whose rays differ in
+their dominant axis and cross the planes through the eye."""
 import math
 
 import numpy as np
@@ -56,6 +57,8 @@ def _points(kind, v, f, n, rng):
 @pytest.mark.parametrize("kind,n,nf,theta,near,windows", [
     ("one", 1, 3, 4.0, False, 1), ("two", 33, 40, 4.0, False, 1),
     ("sphere", 31, 511, 2.0, False, 1), ("sphere", 32, 512, 2.0, False, 3), ("sphere", 1000, 1300, 6.0, False, 5),
+    ("sphere", 14592, 255, 2.0, False, 1), ("sphere", 14592, 256, 2.0, False, 2), ("sphere", 14624, 256, 2.0, False, 1),
+    ("sphere", 32768, 256, 2.0, False, 1), ("sphere", 32769, 256, 2.0, False, 1),
     ("mixed", 65537, 300, 2.0, False, 1), ("mixed", 70001, 300, 3.0, False, 3),
     ("fine", 2048, 600, 1.0, False, 1), ("fine", 65600, 60, 1.0, False, 1), ("sphere", 3000, 200, 15.0, True, 1), ("sphere", 257, 0, 1.0, False, 2)])
 def test_shaft_walk_equals_per_ray_walk(env, kind, n, nf, theta, near, windows):
