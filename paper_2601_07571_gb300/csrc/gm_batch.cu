@@ -192,7 +192,9 @@ __global__ void k_bnormalize(const SessionDev* __restrict__ sess) {
     const uint64_t total = (uint64_t)S.ns * S.W;
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < total; i += (uint64_t)gridDim.x * blockDim.x) {
         const float m = __uint_as_float(S.max_bits[i / S.ns]);
-        S.out[i] = m > 0.f ? __fdiv_rn(S.out[i], m) : 0.f;
+        const float x = S.out[i];
+        if (!(m > 0.f)) S.out[i] = 0.f;
+        else if (x != 0.f) S.out[i] = __fdiv_rn(x, m);   // (0 takes the division's slow path)
     }
 }
 

@@ -738,8 +738,11 @@ __global__ void k_zb_normalize(float* __restrict__ v, uint64_t ns, const unsigne
     const uint32_t w = w0 + blockIdx.y;
     const float m = __uint_as_float(max_bits[w]);
     float* p = v + (size_t)w * ns;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < ns; i += (uint64_t)gridDim.x * blockDim.x)
-        p[i] = m > 0.f ? __fdiv_rn(p[i], m) : 0.f;
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < ns; i += (uint64_t)gridDim.x * blockDim.x) {
+        const float x = p[i];
+        if (!(m > 0.f)) p[i] = 0.f;
+        else if (x != 0.f) p[i] = __fdiv_rn(x, m);   // (0 takes the division's slow path)
+    }
 }
 
 __global__ void k_zb_export(const uint32_t* __restrict__ zb, uint64_t n, float* __restrict__ out) {
