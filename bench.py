@@ -35,19 +35,21 @@ sys.path.insert(0, ROOT)
 METRIC = "sample×fixation pairs/s at ≤1e-4 rel err"
 FP32_INSTR_PER_PAIR = 18          # algorithmic FP32 work of the cone test per pair
 FP32_INSTR_PER_NODE = 28          # two slab tests: 6 FMA + 6 min/max + two 3-input min/max each
+FP32_INSTR_PER_SHAFT_NODE = 100   # shafts, per 4-wide node: 4 boxes x (6 sub, 6 products, 3 FMA, 10 min/max/compare)
 FP32_INSTR_PER_TRI = 25           # watertight test: 3 x 3 sub, 6 products with 3 subtractions, U V W, det, T
 FP32_INSTR_PER_INCONE = 12        # Gaussian (divide, scale, ex2, weight) and the compensated sum (4 adds)
 FP32_INSTR_PER_ENTRY = 1          # eye grid: the depth-bound compare of a list entry
 FP32_LANES_PER_SM = 128
 SM_MAX_MHZ_NOMINAL = 2070.0
 
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one k_accumulate launch, from a
+# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one accumulation launch, from a
 # one-pass ncu capture of the default bench command (paper scene, default flags and builder).
 # The figure stands only while the sources that shape the kernel and its inputs are the ones it
 # was taken on: their SHA-256 is stored beside it and `traffic` is null on any mismatch.
-ACC_TRAFFIC = {"workload": "paper_scene_800ktri_2Msample_6000fix", "bytes": 168.055296e6,
-               "sources_sha256": "23103779d73037ce45bbabf1a5134c689c5acd655942c8dcc03478fa3a1feed0"}
+ACC_TRAFFIC = {"workload": "paper_scene_800ktri_2Msample_6000fix", "bytes": 302.960896e6,
+               "sources_sha256": "c59521bbaaf6497f4b1adecafce564437f0c6675df823863a8315827be39c6ab"}
 ACC_TRAFFIC_SOURCES = ("paper_2601_07571_gb300/csrc/gm_trace.cuh", "paper_2601_07571_gb300/csrc/gm_accum.cu",
+                       "paper_2601_07571_gb300/csrc/gm_shaft.cuh",
                        "paper_2601_07571_gb300/csrc/gm_scene.cu", "paper_2601_07571_gb300/csrc/gm_sampler.cu")
 
 
@@ -900,19 +902,23 @@ def main():
     # tiles whose sphere the cone misses are skipped), the Gaussian and compensated sum of every
     # in-cone pair, and the occlusion tests (BVH: two slab tests per node visit; eye grid: one
     # depth compare per list entry) plus one watertight test per triangle tested
-    per_visit = FP32_INSTR_PER_ENTRY if grid_on else FP32_INSTR_PER_NODE
+    # (the default's shafts: four box tests per node of the 4-wide tree, one visit for all rays of a
+    # shaft; their triangle set-up and image-box tests are not counted)
+    shafts = not grid_on and not args.flags & (G.GM_F_NO_COMPACT | G.GM_F_WIDE_BVH | G.GM_F_SPT4 | G.GM_F_SPT2 |
+                                               G.GM_F_BLOCK128 | G.GM_F_BLOCK512 | G.GM_F_FIX_L1)
+    per_visit = FP32_INSTR_PER_ENTRY if grid_on else FP32_INSTR_PER_SHAFT_NODE if shafts else FP32_INSTR_PER_NODE
     executed = (FP32_INSTR_PER_PAIR * stats["pairs_tested"] + FP32_INSTR_PER_INCONE * stats["in_cone"]
                 + per_visit * stats["nodes_visited"] + FP32_INSTR_PER_TRI * stats["tris_tested"])
     achieved = executed / (acc * 1e-3) / 1e12
     roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tinst/s (FP32)", "frac": achieved / peak,
             "traffic": recorded_traffic(w.name, args.flags, args.builder,
                                         args.ploc_radius in (0, 8) and args.eps_rel is None),
-            "kernel": "k_accumulate" + ("<eye grid>" if grid_on else "<BVH>"),
+            "kernel": "k_accumulate_shaft" if shafts else "k_accumulate" + ("<eye grid>" if grid_on else "<BVH>"),
             "peak_basis": f"{n_sm} SMs x {FP32_LANES_PER_SM} FP32 lanes x {SM_MAX_MHZ_NOMINAL:.0f} MHz (nominal)",
             "work_basis": (f"executed FP32 instructions from the kernel's counters: {FP32_INSTR_PER_PAIR} per cone test "
                            f"evaluated ({stats['pairs_tested']:.4g} of {stats['pairs']:.4g} nominal pairs), "
                            f"{FP32_INSTR_PER_INCONE} per in-cone pair (Gaussian + compensated sum), {per_visit} per "
-                           + ("eye-grid entry read" if grid_on else "BVH node visit")
+                           + ("eye-grid entry read" if grid_on else "4-wide node visit of a shaft" if shafts else "BVH node visit")
                            + f", {FP32_INSTR_PER_TRI} per triangle test"),
             "kernel_ms": acc}
     if clk and clk.get("sm_mhz"):

@@ -363,36 +363,6 @@ __device__ __forceinline__ void group_sync(int h) {   // the 128 threads of grou
     asm volatile("bar.sync %0, 128;" ::"r"(h + 1) : "memory");
 }
 
-// The 64 features of one point for the tensor-core kernel: sine and cosine of 2^k pi x~ from an
-// exact reduction and the hardware sincos at octaves 0, 3, 6 and 9, and by the double-angle
-// formulas (sin 2a = 2 sin a cos a, cos 2a = cos^2 a - sin^2 a) for the two octaves after each;
-// two doublings keep the error within a few 1e-6, far under the bf16 rounding that follows.
-__device__ __forceinline__ void features_fast(const float xt[3], float* v) {
-    v[0] = xt[0];
-    v[1] = xt[1];
-    v[2] = xt[2];
-    v[63] = 0.f;
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        float sn = 0.f, cs = 1.f;
-#pragma unroll
-        for (int k = 0; k < FOCT; ++k) {
-            if (k % 3 == 0) {
-                float y = ldexpf(xt[r], k);
-                y = y - 2.f * rintf(0.5f * y);
-                __sincosf(3.14159265358979f * y, &sn, &cs);
-            } else {
-                const float s2 = 2.f * (sn * cs);
-                const float c2 = fmaf(cs, cs, -(sn * sn));
-                sn = s2;
-                cs = c2;
-            }
-            v[3 + 6 * k + r] = sn;
-            v[6 + 6 * k + r] = cs;
-        }
-    }
-}
-
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
     uint32_t r[16];
     asm volatile(
@@ -934,7 +904,7 @@ __device__ __forceinline__ void store_part(__nv_bfloat16* T, int p, int c0, cons
         *reinterpret_cast<uint4*>(row + g * 2048) = make_uint4(pk[4 * g], pk[4 * g + 1], pk[4 * g + 2], pk[4 * g + 3]);
 }
 
-// Features 32 HI .. 32 HI + 31 (features_fast's values) as packed bf16 pairs; the upper half starts at
+// Features 32 HI .. 32 HI + 31 (the query kernel's values) as packed bf16 pairs; the upper half starts at
 // octave 3, whose sine and cosine are evaluated afresh.
 template <int HI>
 __device__ __forceinline__ void encode_half(const float xt[3], uint32_t* pk) {
