@@ -502,15 +502,16 @@ def dynamic_arm(args):
 
 def normalize_roofline(ns: int, nonempty_windows: int, ms: float):
     """HBM roofline of the map normalisation (Section 3.2.3): every value of a non-empty window
-    read and written once, 8 B per sample and window, over the kernel's CUDA-event time."""
+    read once, 4 B per sample and window (the non-zero ones are written too, which is not counted), over
+    the kernel's CUDA-event time."""
     peak, basis = measured_hbm_peak()
     if ms <= 0:
         return None
-    nbytes = 8.0 * ns * nonempty_windows
+    nbytes = 4.0 * ns * nonempty_windows
     achieved = nbytes / (ms * 1e-3) / 1e9
     return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
             "kernel": "k_normalize", "bytes": nbytes, "kernel_ms": ms, "peak_basis": basis,
-            "work_basis": f"8 B (read + write) per sample of each of {nonempty_windows} non-empty window(s)"}
+            "work_basis": f"4 B (read) per sample of each of {nonempty_windows} non-empty window(s)"}
 
 
 def measured_hbm_peak():
