@@ -3,12 +3,12 @@
 //
 // A session is (scene, samples, fixations); all sessions share the generation parameters. At
 // plan creation every session's fixations are staged into one device buffer and a work list
-// of warp tiles (session, 32*SPT consecutive work-order samples) is built on the host: sessions
+// of tiles (session, 32 samples for shafts, else 32*SPT work-order samples) is built on the host: sessions
 // grouped into three size buckets by triangle count, within a bucket ordered by decreasing cost
 // (fixations per tile, i.e. longest processing time first). The plan then captures into one
 // CUDA graph: the counter resets, the batched fixation prep (window keys per session, one stable
 // radix sort, packing), one persistent accumulation launch per bucket on forked streams (its
-// warps pull the bucket's work items from the bucket's counter; each bucket has its own kernel
+// blocks, or warps in the ray-queue forms, pull the bucket's work items from the bucket's counter; each bucket has its own kernel
 // variant and events around its launch; a bucket's tail overlaps the next one's start), and the
 // batched normalisation. gm_batch_run replays the graph: no
 // host work and one graph launch per call.
