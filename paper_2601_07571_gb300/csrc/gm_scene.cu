@@ -569,15 +569,19 @@ __global__ void k_leaf_counts(const int* __restrict__ parent_leaf, const int* __
 }
 
 // even[index] = 1 where the node's depth is even (root 0): those become 4-wide nodes. *depth: the
-// deepest leaf (one level below the deepest node).
+// deepest leaf (one level below the deepest node), counted up to 4097; a tree above MAX_DEPTH is refused
+// before anything reads dfs or even, which hold nothing for the nodes whose climb was cut off. left: the
+// clusters that the clustering ended with (nullptr: another builder); without one root there is no tree.
+constexpr unsigned MAX_DEPTH = 64;
 __global__ void k_dfs_index(const float4* __restrict__ nodes, const int* __restrict__ parent_node,
-                            const unsigned int* __restrict__ leaves, int n_int, int* __restrict__ dfs,
-                            int64_t* __restrict__ even, unsigned int* __restrict__ depth) {
+                            const unsigned int* __restrict__ leaves, int n_int, const int* __restrict__ left,
+                            int* __restrict__ dfs, int64_t* __restrict__ even, unsigned int* __restrict__ depth) {
     int v = blockIdx.x * blockDim.x + threadIdx.x;
     const unsigned live = __ballot_sync(0xffffffffu, v < n_int);
-    if (v >= n_int) return;
-    int idx = 0, u = v, guard = 0;
-    while (u > 0 && guard++ < 4096) {
+    if (v >= n_int || (left && *left != 1)) return;
+    int idx = 0, u = v, steps = 0;
+    while (u > 0 && steps < 4096) {
+        ++steps;
         const int p = parent_node[u];
         const float4 l = nodes[4 * p + 3];
         const int left = __float_as_int(l.x);
@@ -585,9 +589,11 @@ __global__ void k_dfs_index(const float4* __restrict__ nodes, const int* __restr
         if (left != u) idx += left >= 0 ? (int)leaves[left] - 1 : 0;   // internal nodes of the left subtree
         u = p;
     }
-    dfs[v] = idx;
-    even[idx] = (guard & 1) == 0 ? 1 : 0;
-    const unsigned deep = __reduce_max_sync(live, (unsigned)guard + 1u);
+    if (u <= 0) {
+        dfs[v] = idx;
+        even[idx] = (steps & 1) == 0 ? 1 : 0;
+    }
+    const unsigned deep = __reduce_max_sync(live, (unsigned)steps + 1u);
     if ((threadIdx.x & 31) == 0) atomicMax(depth, deep);
 }
 
@@ -879,6 +885,30 @@ static gm_status build_scene(gm_ctx* ctx, const gm_mesh_desc* meshes, uint32_t n
                                                     flags, bounds, sc->bvh_tris);
         launches += (nt > 1 ? 2 : 1);
     }
+    int* dfs = nullptr;
+    int64_t* incl = nullptr;
+    const int n_int = (int)nt - 1;
+    if (nt > 1) {
+        TMP_ALLOC(dfs, sizeof(int) * n_int);
+        if (dynamic) {
+            SC_ALLOC(sc->incl4, sizeof(int64_t) * n_int);
+            incl = sc->incl4;
+        } else {
+            TMP_ALLOC(incl, sizeof(int64_t) * n_int);
+        }
+        if (!ploc) {   // the clustering counted the leaves as it merged
+            unsigned int* arrived = nullptr;
+            TMP_ALLOC(arrived, sizeof(unsigned int) * n_int);
+            if ((ce = cudaMemsetAsync(leaves, 0, sizeof(unsigned int) * n_int, s)) != cudaSuccess ||
+                (ce = cudaMemsetAsync(arrived, 0, sizeof(unsigned int) * n_int, s)) != cudaSuccess)
+                return wait_fail(gm_cuda_error(ce, "gm_build_scene"));
+            k_leaf_counts<<<gm_div_up(nt, 256), 256, 0, s>>>(parent_leaf, parent_node, sc->nodes, (int)nt, leaves, arrived);
+            ++launches;
+        }
+        k_dfs_index<<<gm_div_up(n_int, 256), 256, 0, s>>>(sc->nodes, parent_node, leaves, n_int,
+                                                          ploc ? (int*)depth + 1 : nullptr, dfs, incl, depth);
+        ++launches;
+    }
     ctx->launches += launches;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return wait_fail(gm_cuda_error(e, "gm_build_scene launch"));
@@ -908,31 +938,15 @@ static gm_status build_scene(gm_ctx* ctx, const gm_mesh_desc* meshes, uint32_t n
         if (!std::isfinite(sc->box_lo[k]) || !std::isfinite(sc->box_hi[k]))
             return fail(gm_set_error(GM_ERR_INVALID_ARG, "gm_build_scene: non-finite vertex"));
     }
-    sc->depth = 0;
+    // the layout below uses the depth: nothing of a deeper tree is laid out
+    sc->depth = nt > 1 ? hdepth[0] : 0;
+    if (sc->depth > MAX_DEPTH)
+        return fail(gm_set_error(GM_ERR_UNSUPPORTED, "gm_build_scene: BVH deeper than 64 levels (" +
+                                                         std::to_string(sc->depth) + ")"));
     if (nt > 1) {
-        const int n_int = (int)nt - 1;
-        int* dfs = nullptr;
         float4* reordered = nullptr;
-        int64_t* incl = nullptr;
-        TMP_ALLOC(dfs, sizeof(int) * n_int);
-        if (dynamic) {
-            SC_ALLOC(sc->incl4, sizeof(int64_t) * n_int);
-            incl = sc->incl4;
-        } else {
-            TMP_ALLOC(incl, sizeof(int64_t) * n_int);
-        }
-        launches = 2;
-        if (!ploc) {   // the clustering counted the leaves as it merged
-            unsigned int* arrived = nullptr;
-            TMP_ALLOC(arrived, sizeof(unsigned int) * n_int);
-            if ((e = cudaMemsetAsync(leaves, 0, sizeof(unsigned int) * n_int, s)) != cudaSuccess ||
-                (e = cudaMemsetAsync(arrived, 0, sizeof(unsigned int) * n_int, s)) != cudaSuccess)
-                return fail(gm_cuda_error(e, "gm_build_scene"));
-            k_leaf_counts<<<gm_div_up(nt, 256), 256, 0, s>>>(parent_leaf, parent_node, sc->nodes, (int)nt, leaves, arrived);
-            ++launches;
-        }
+        launches = 1;
         if ((st = gm_alloc((void**)&reordered, sizeof(float4) * 4 * (size_t)n_int, s)) != GM_OK) return fail(st);
-        k_dfs_index<<<gm_div_up(n_int, 256), 256, 0, s>>>(sc->nodes, parent_node, leaves, n_int, dfs, incl, depth);
         k_dfs_remap<<<gm_div_up(n_int, 256), 256, 0, s>>>(sc->nodes, dfs, n_int, reordered);
         cudaFreeAsync(sc->nodes, s);
         sc->nodes = reordered;
@@ -943,14 +957,8 @@ static gm_status build_scene(gm_ctx* ctx, const gm_mesh_desc* meshes, uint32_t n
         k_collapse4<<<gm_div_up(n_int, 256), 256, 0, s>>>(sc->nodes, n_int, incl, sc->nodes4);
         ++launches;
         ctx->launches += launches;
-        if ((e = cudaGetLastError()) != cudaSuccess ||
-            (e = cudaMemcpyAsync(hdepth, depth, sizeof(unsigned int), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
-            (e = cudaStreamSynchronize(s)) != cudaSuccess)
+        if ((e = cudaGetLastError()) != cudaSuccess || (e = cudaStreamSynchronize(s)) != cudaSuccess)
             return wait_fail(gm_cuda_error(e, "gm_build_scene layout"));
-        sc->depth = hdepth[0];
-        if (sc->depth > 64)
-            return fail(gm_set_error(GM_ERR_UNSUPPORTED, "gm_build_scene: BVH deeper than 64 levels (" +
-                                                             std::to_string(sc->depth) + ")"));
     }
     for (void* p : tmp) cudaFreeAsync(p, s);
     tmp.clear();

@@ -88,3 +88,27 @@ def test_sorted_windows_equal_single_intervals(env, nf, windows):
         assert np.array_equal(out[w], one[0])
     G.gm_samples_free(samples)
     G.gm_scene_free(scene)
+
+
+@pytest.mark.parametrize("copies,others", [(66, 0), (1100, 50), (4096, 0), (5000, 0), (5000, 300)])
+def test_coincident_triangles_are_refused(env, copies, others):
+    """Equal boxes merge one pair a round into a chain: a tree deeper than the traversal's 64 levels (from 4097
+    levels on, deeper than its layout follows) is refused before it is laid out, and the next build works."""
+    G, ctx = env
+    rng = np.random.default_rng(copies + others)
+    v, f = _soup(others + 1, rng)
+    f = np.concatenate([f, np.repeat(f[:1], copies - 1, 0)])
+    with pytest.raises(G.GazeMapError, match="deeper than 64 levels") as e:
+        G.gm_build_scene(ctx, [(v, f, np.eye(4), 0)])
+    assert e.value.status == G.GM_ERR_UNSUPPORTED
+    for n in (2, 40):      # a chain that is not too deep builds, and traces as the other builder's tree does
+        f = np.repeat(f[:1], n, 0)
+        xyz, tri = np.ascontiguousarray(v[:3].mean(0, keepdims=True)), np.zeros(1, np.uint32)
+        fix, got = _look(60, rng), []
+        for b in (G.GM_BUILD_PLOC, G.GM_BUILD_LBVH):
+            scene = G.gm_build_scene(ctx, [(v, f, np.eye(4), 0)], builder=b)
+            samples = G.gm_samples_from_points(scene, xyz, tri)
+            got.append(_map(G, scene, samples, fix, np.arange(60.0))[0])
+            G.gm_samples_free(samples)
+            G.gm_scene_free(scene)
+        assert np.array_equal(got[0], got[1])
