@@ -160,7 +160,7 @@ gm_status gm_ctx_launches(const gm_ctx* ctx, uint64_t* kernel_launches);
  * Karras' HPG 2012 hierarchy, bottom-up boxes, internal nodes stored depth-first. The BVH
  * replaces the per-view z-buffer of Section 3.2.2 as the occlusion structure. Meshes are
  * concatenated in order; global triangle ids follow that order. Synchronises `stream` (to
- * check the tree depth; the clustering reads its cluster count back once per round). */
+ * check the tree depth; the clustering reads its cluster count back every twelve rounds). */
 gm_status gm_build_scene(gm_ctx* ctx, const gm_mesh_desc* meshes, uint32_t n_meshes,
                          gm_stream stream, gm_scene** out);
 /* Builders of the hierarchy (same node layout and traversal either way):

@@ -825,6 +825,7 @@ static gm_status build_scene(gm_ctx* ctx, const gm_mesh_desc* meshes, uint32_t n
     ++launches;
     if ((st = gm_radix_sort_u64(keys, order, nt, 63, s, &launches)) != GM_OK) return wait_fail(st);
     const bool ploc = builder == GM_BUILD_PLOC && nt > 1;
+    bool cut = false;   // the clustering was still merging after its last round
     if (ploc) {
         constexpr int kRounds = 4096;
         int *m_of = nullptr, *pair = nullptr, *gone = nullptr;
@@ -862,6 +863,7 @@ static gm_status build_scene(gm_ctx* ctx, const gm_mesh_desc* meshes, uint32_t n
                 return wait_fail(gm_cuda_error(ce, "gm_build_scene (clustering)"));
             if (now >= m) break;   // no mutual pair: reported below
             m = now;
+            cut = m > PLOC_TAIL && rounds >= kRounds;
         }
         auto tail = [&](auto kern) {
             kern<<<1, PLOC_TAIL, 0, s>>>(m_of, rounds, lo[0], hi[0], lo[1], hi[1], sc->nodes, parent_node, parent_leaf,
@@ -924,6 +926,9 @@ static gm_status build_scene(gm_ctx* ctx, const gm_mesh_desc* meshes, uint32_t n
         cudaMemsetAsync(ctx->dev_err, 0, sizeof(int), s);
         return fail(gm_set_error(GM_ERR_INVALID_ARG, "gm_build_scene: a vertex index is out of range"));
     }
+    if (cut)   // one pair a round, as runs of equal boxes merge: a chain
+        return fail(gm_set_error(GM_ERR_UNSUPPORTED, "gm_build_scene: BVH deeper than 64 levels (" + std::to_string(hdepth[1]) +
+                                                         " clusters left after 4096 rounds)"));
     if (ploc && hdepth[1] != 1)   // no mutual pair: cannot happen with consistent tie-breaking and finite boxes
         return fail(gm_set_error(GM_ERR_INTERNAL, "gm_build_scene: clustering made no progress"));
     auto dec = [](unsigned int o) {

@@ -90,7 +90,7 @@ def test_sorted_windows_equal_single_intervals(env, nf, windows):
     G.gm_scene_free(scene)
 
 
-@pytest.mark.parametrize("copies,others", [(66, 0), (1100, 50), (4096, 0), (5000, 0), (5000, 300)])
+@pytest.mark.parametrize("copies,others", [(66, 0), (1100, 50), (4096, 0), (5000, 0), (5000, 300), (5200, 0), (20000, 100)])
 def test_coincident_triangles_are_refused(env, copies, others):
     """Equal boxes merge one pair a round into a chain: a tree deeper than the traversal's 64 levels (from 4097
     levels on, deeper than its layout follows) is refused before it is laid out, and the next build works."""
