@@ -398,7 +398,7 @@ __device__ __forceinline__ unsigned shaft_visible_wide(unsigned in, const float4
         const float dz = comp(d, rz);
         qx[k] = comp(d, rx) / dz;
         qy[k] = comp(d, ry) / dz;
-        qz[k] = 1.0f / dz;
+        qz[k] = dz == 0.f ? 0.f : 1.0f / dz;   // 0: no image point (never a ray in its own axes)
         own[k] = __float_as_uint(pos[32 * k + lane].w);
         same = same && (!((in >> k) & 1u) || axis_of(d) == ref);
     }

@@ -95,3 +95,45 @@ def test_shaft_walk_equals_per_ray_walk(env, kind, n, nf, theta, near, windows):
     assert np.array_equal(out[0][0], out[1][0])
     if nf > 10:
         assert out[0][2]["visible"] > 0
+
+
+def _floor(n, occluder):
+    """n samples on a grid of a unit floor of two triangles (so that every tile of 128 is wide), the occluder's
+    triangles after it; samples lie on floats, so that an eye can stand exactly above one."""
+    q = np.array([[0.0, 0.0, 0.0], [1.0, 0.0, 0.0], [1.0, 0.0, 1.0], [0.0, 0.0, 1.0]], np.float32)
+    v, f = M.merge([(q, np.array([[0, 2, 1], [0, 3, 2]], np.uint32)), occluder])
+    k = math.ceil(math.sqrt(n))
+    x, z = np.divmod(np.arange(n), k)
+    xyz = np.ascontiguousarray(np.stack([(x + 0.5) / k, np.zeros(n), (z + 0.5) / k], 1), np.float32)
+    return v, f, xyz, (xyz[:, 2] > xyz[:, 0]).astype(np.uint32)
+
+
+def test_wide_tile_with_a_ray_in_a_coordinate_plane(env):
+    """Eyes exactly above samples, 1.5 cm over the floor: the ray straight down has no image point on the side of the
+    tile's first ray (0 / 0 there), and what hides it crosses the plane through the eye."""
+    G, ctx = env
+    rng = np.random.default_rng(5)
+    q = np.array([[0.2, 0.007, 0.2], [0.8, 0.007, 0.2], [0.8, 0.007, 0.8], [0.2, 0.007, 0.8]], np.float32)
+    v, f, xyz, tri = _floor(70000, (q, np.array([[0, 2, 1], [0, 3, 2]], np.uint32)))
+    nf = 400
+    at = rng.integers(0, len(xyz), nf)
+    turn = rng.uniform(0.0, 2.0 * math.pi, nf)
+    tilt = math.radians(24.0)
+    eye = xyz[at] + np.float32([0.0, 0.015, 0.0])
+    gaze = np.stack([math.sin(tilt) * np.cos(turn), np.full(nf, -math.cos(tilt)), math.sin(tilt) * np.sin(turn)], 1)
+    fix = [np.ascontiguousarray(eye, np.float32), np.ascontiguousarray(gaze, np.float32),
+           rng.uniform(0.1, 0.6, nf).astype(np.float32), np.arange(float(nf))]
+    scene = G.gm_build_scene(ctx, [(v, f, np.eye(4), 0)])
+    samples = G.gm_samples_from_points(scene, xyz, tri)
+    out = []
+    for flags in (0, G.GM_F_FIX_L1):
+        m = G.gm_accumulate_fixations(scene, samples, *fix, G.make_params(math.radians(9.0), normalize=False, flags=flags))
+        _, ns, st, _ = G.gm_map_info(m)
+        values = np.empty(ns, np.float32)
+        G.gm_map_copy(m, 0, values)
+        G.gm_map_free(m)
+        out.append((values, st["in_cone"], st["visible"]))
+    G.gm_samples_free(samples)
+    G.gm_scene_free(scene)
+    assert out[0][1:] == out[1][1:] and 0 < out[0][2] < out[0][1]
+    assert np.array_equal(out[0][0], out[1][0])
