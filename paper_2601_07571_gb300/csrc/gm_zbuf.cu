@@ -14,7 +14,8 @@
 //                  that a shared edge gives exactly opposite values and leaves no cracks), then the lanes
 //                  share the pixels of all 32 boxes evenly: point sampling at pixel centres,
 //                  perspective-correct 1/w, atomicMin of the linear depth w (positive floats order as
-//                  their bits)
+//                  their bits). Pairs that reach the near plane are clipped first, and drawn by the
+//                  size of their box: by a lane, by the warp or by k_zb_draw_big (draw_others)
 //   k_zb_draw_big  pairs whose box holds more than ZB_BIG_PIXELS pixels, one block each
 //   k_zb_accumulate one thread per work-order sample over the chunk's fixations: the exact cone
 //                  test and Gaussian of the ray path, visibility |w - zbuf| <= eps, compensated
@@ -31,6 +32,7 @@ namespace {
 constexpr int ZB_THREADS = 256;
 constexpr int ZB_SMEM_FRUSTA = 64;            // frusta staged per pass of the cull kernel
 constexpr int ZB_BIG_PIXELS = 1024;           // larger pixel boxes go to the block rasteriser
+constexpr int ZB_LANE_PIXELS = 32;            // clipped pairs: larger ones go to the warp
 constexpr uint64_t ZB_BIG_CAP = 1u << 20;     // ... through a list of this many pairs (a full list: drawn in place)
 constexpr uint32_t ZB_EMPTY = 0xffffffffu;    // cleared z-buffer word (above every finite depth)
 constexpr uint32_t NO_WINDOW = 0xffffffffu;
@@ -249,16 +251,6 @@ __device__ __forceinline__ void clip_project(const ZbFrustum& F, float4 a, float
     }
 }
 
-// Edge function of p against the directed edge a -> b, evaluated with the endpoints in a
-// canonical (lexicographic) order and the sign restored, so that the two triangles sharing an
-// edge get exactly opposite values.
-__device__ __forceinline__ float edge_fn(float ax, float ay, float bx, float by, float px, float py) {
-    const bool swap = (bx < ax) || (bx == ax && by < ay);
-    const float x0 = swap ? bx : ax, y0 = swap ? by : ay, x1 = swap ? ax : bx, y1 = swap ? ay : by;
-    const float e = __fsub_rn(__fmul_rn(x1 - x0, py - y0), __fmul_rn(y1 - y0, px - x0));
-    return swap ? -e : e;
-}
-
 // The pixels whose centres px + 1/2 lie within [umin, umax] x [vmin, vmax], widened by 1/100 pixel for the
 // rounding of the edge functions (an FP32 error of a few 1e-4 pixels at these coordinates).
 __device__ __forceinline__ void pixel_box(float umin, float umax, float vmin, float vmax, int res, int& x0, int& x1,
@@ -281,38 +273,9 @@ __device__ __forceinline__ void poly_bbox(const ClipPoly& P, int res, int& x0, i
     pixel_box(umin, umax, vmin, vmax, res, x0, x1, y0, y1);
 }
 
-// Depth test of one pixel against the fan triangles of the polygon.
-__device__ __forceinline__ void shade_pixel(const ClipPoly& P, int px, int py, float n, float f,
-                                            uint32_t* __restrict__ zb, int res) {
-    const float cx = px + 0.5f, cy = py + 0.5f;
-    for (int k = 1; k + 1 < P.n; ++k) {
-        const float ax = P.u[0], ay = P.v[0], bx = P.u[k], by = P.v[k], qx = P.u[k + 1], qy = P.v[k + 1];
-        const float e0 = edge_fn(bx, by, qx, qy, cx, cy);
-        const float e1 = edge_fn(qx, qy, ax, ay, cx, cy);
-        const float e2 = edge_fn(ax, ay, bx, by, cx, cy);
-        const bool in = (e0 >= 0.f && e1 >= 0.f && e2 >= 0.f) || (e0 <= 0.f && e1 <= 0.f && e2 <= 0.f);
-        const float area = e0 + e1 + e2;
-        if (!in || area == 0.f) continue;
-        const float iw = (e0 * P.iw[0] + e1 * P.iw[k] + e2 * P.iw[k + 1]) / area;
-        const float w = 1.0f / iw;
-        if (w >= n * (1.f - 1e-6f) && w <= f && w > 0.f) atomicMin(zb + (size_t)py * res + px, __float_as_uint(w));
-    }
-}
-
-// One thread draws one pair, clipped to the near plane (out of line: few triangles reach it).
-__device__ __noinline__ void draw_clipped(const ZbFrustum& F, float4 a, float4 b, float4 c, uint32_t res,
-                                          uint32_t* __restrict__ zb) {
-    ClipPoly P;
-    clip_project(F, a, b, c, P);
-    if (P.n < 3) return;
-    int x0, x1, y0, y1;
-    poly_bbox(P, (int)res, x0, x1, y0, y1);
-    for (int py = y0; py <= y1; ++py)
-        for (int px = x0; px <= x1; ++px) shade_pixel(P, px, py, F.n, F.f, zb, (int)res);
-}
-
 // One pair set up for drawing: edges b -> c, c -> a, a -> b as (x0, y0, dx, dy) with the endpoints in
-// canonical order and the sign in dx and dy (negating both negates the edge function exactly).
+// canonical (lexicographic) order and the sign in dx and dy (negating both negates the edge function
+// exactly), so that the two triangles sharing an edge get exactly opposite values.
 struct alignas(16) ZbTri {
     float4 e0, e1, e2;
     float4 iw;      // 1/w of a, b, c; box width | first pixel's index among the warp's << 16 (bits)
@@ -330,8 +293,7 @@ __device__ __forceinline__ float edge_at(const float4 e, float px, float py) {
     return __fsub_rn(__fmul_rn(e.z, py - e.y), __fmul_rn(e.w, px - e.x));
 }
 
-// Depth test of the pixel with centre (cx, cy) and word z against a pair set up for drawing
-// (shade_pixel's arithmetic).
+// Depth test of the pixel with centre (cx, cy) and word z against a pair set up for drawing.
 __device__ __forceinline__ void shade_tri(const float4 q0, const float4 q1, const float4 q2, const float4 iws, float cx,
                                           float cy, float n, float f, uint32_t* __restrict__ z) {
     const float e0 = edge_at(q0, cx, cy), e1 = edge_at(q1, cx, cy), e2 = edge_at(q2, cx, cy);
@@ -343,9 +305,75 @@ __device__ __forceinline__ void shade_tri(const float4 q0, const float4 q1, cons
     if (w >= n * (1.f - 1e-6f) && w <= f && w > 0.f) atomicMin(z, __float_as_uint(w));
 }
 
+// Triangle k of a polygon's fan around its first vertex, set up for drawing.
+__device__ __forceinline__ void fan_tri(const ClipPoly& P, int k, float4& e0, float4& e1, float4& e2, float4& iw) {
+    e0 = canonical_edge(P.u[k], P.v[k], P.u[k + 1], P.v[k + 1]);
+    e1 = canonical_edge(P.u[k + 1], P.v[k + 1], P.u[0], P.v[0]);
+    e2 = canonical_edge(P.u[0], P.v[0], P.u[k], P.v[k]);
+    iw = make_float4(P.iw[0], P.iw[k], P.iw[k + 1], 0.f);
+}
+
 __device__ __forceinline__ float4 shfl4(const float4 v, int src) {
     return make_float4(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src),
                        __shfl_sync(0xffffffffu, v.z, src), 0.f);
+}
+
+// Draws every step-th pixel of a polygon's box from pixel `first` on.
+__device__ __forceinline__ void draw_poly(const ClipPoly& P, int x0, int y0, int wd, int n, float near_m, float far_m,
+                                          uint32_t res, uint32_t* __restrict__ zb, int first, int step) {
+    for (int t = 1; t + 1 < P.n; ++t) {
+        float4 e0, e1, e2, iw;
+        fan_tri(P, t, e0, e1, e2, iw);
+        for (int k = first; k < n; k += step) {
+            const int px = x0 + k % wd, py = y0 + k / wd;
+            shade_tri(e0, e1, e2, iw, px + 0.5f, py + 0.5f, near_m, far_m, zb + (size_t)py * res + px);
+        }
+    }
+}
+
+// The pairs of a warp's entries that its shared pixels leave out: boxes above ZB_BIG_PIXELS, for the block
+// rasteriser, and pairs that reach the near plane (`clip`). Those are clipped first; a floor or wall that
+// passes the viewer fills the whole window, so they too go to the block rasteriser, to the warp (above
+// ZB_LANE_PIXELS) or to their lane by the size of their box. (Out of line: few warps come here, and its
+// registers are its own.) 12 triangles of a room and 60k of objects in it, 2000 fixations at 256 x 256:
+// 165 ms with every clipped pair drawn by its lane, 1.8 so.
+__device__ __noinline__ void draw_others(const ZbFrustum* sF, const float4* __restrict__ tris, const int entry,
+                                         const bool clip, int npx, const uint32_t f0, const uint32_t slot0,
+                                         const uint32_t res, uint32_t* __restrict__ zbuf, PairFT* __restrict__ big,
+                                         unsigned long long* __restrict__ n_big) {
+    const int lane = threadIdx.x & 31, src = entry & 31, own = entry >> 5;
+    auto project = [&](int k, int from, ClipPoly& P) {
+        const float4* v = tris + 3 * (size_t)(slot0 + from);
+        clip_project(sF[k], v[0], v[1], v[2], P);
+    };
+    ClipPoly P;
+    P.n = 0;
+    int x0 = 0, x1 = -1, y0 = 0, y1 = -1;
+    if (clip || npx > ZB_BIG_PIXELS) {
+        project(own, src, P);
+        if (P.n >= 3) poly_bbox(P, (int)res, x0, x1, y0, y1);
+        npx = x1 >= x0 && y1 >= y0 ? (x1 - x0 + 1) * (y1 - y0 + 1) : 0;
+    } else {
+        npx = 0;   // drawn
+    }
+    bool here = npx > 0 && npx <= ZB_LANE_PIXELS;
+    if (npx > ZB_BIG_PIXELS) {
+        const unsigned long long q = atomicAdd(n_big, 1ull);
+        if (q < ZB_BIG_CAP) big[q] = PairFT{f0 + (uint32_t)own, slot0 + (uint32_t)src};
+        else here = true;
+    }
+    if (here) draw_poly(P, x0, y0, x1 - x0 + 1, npx, sF[own].n, sF[own].f, res, zbuf + (size_t)(f0 + own) * res * res, 0, 1);
+    unsigned todo = __ballot_sync(0xffffffffu, npx > ZB_LANE_PIXELS && npx <= ZB_BIG_PIXELS);
+    while (todo) {
+        const int who = __ffs(todo) - 1;
+        todo &= todo - 1u;
+        const int k = __shfl_sync(0xffffffffu, own, who), from = __shfl_sync(0xffffffffu, src, who);
+        project(k, from, P);
+        poly_bbox(P, (int)res, x0, x1, y0, y1);
+        const int n = __shfl_sync(0xffffffffu, npx, who);
+        draw_poly(P, x0, y0, x1 - x0 + 1, n, sF[k].n, sF[k].f, res, zbuf + (size_t)(f0 + k) * res * res, lane, 32);
+    }
+    __syncwarp();
 }
 
 // counts: [0] pairs kept, [1] entries of `big`. A warp's pairs stay in its own queue and its own slots:
@@ -416,7 +444,7 @@ __global__ void __launch_bounds__(ZB_THREADS, 4) k_zb_draw(const float4* __restr
         const int src = entry & 31;
         const float4 va = shfl4(a, src), vb = shfl4(b, src), vc = shfl4(c, src);
         const ZbFrustum& F = sF[entry >> 5];
-        const uint32_t fix = f0 + (uint32_t)(entry >> 5), slot = t - lane + src;
+        const uint32_t fix = f0 + (uint32_t)(entry >> 5);
         float x[3], y[3], w[3];
         to_camera(F, va.x, va.y, va.z, x[0], y[0], w[0]);
         to_camera(F, vb.x, vb.y, vb.z, x[1], y[1], w[1]);
@@ -477,19 +505,9 @@ __global__ void __launch_bounds__(ZB_THREADS, 4) k_zb_draw(const float4* __restr
             }
         }
         __syncwarp();
-        // larger boxes go to the block rasteriser; pairs that reach the near plane are clipped
         const bool clip = lane < cnt && !front;
-        const bool to_big = npx > ZB_BIG_PIXELS;
-        if (__any_sync(0xffffffffu, clip || to_big)) {
-            bool here = clip;
-            if (to_big) {
-                const unsigned long long q = atomicAdd(&counts[1], 1ull);
-                if (q < ZB_BIG_CAP) big[q] = PairFT{fix, slot};
-                else here = true;
-            }
-            if (here) draw_clipped(F, va, vb, vc, res, zbuf + (size_t)fix * res * res);
-            __syncwarp();
-        }
+        if (__any_sync(0xffffffffu, clip || npx > ZB_BIG_PIXELS))
+            draw_others(sF, tris, entry, clip, npx, f0, t - lane, res, zbuf, big, &counts[1]);
     };
     for (uint32_t f0 = blockIdx.y * ZB_SMEM_FRUSTA; f0 < nfix; f0 += gridDim.y * ZB_SMEM_FRUSTA) {
         const uint32_t m = min((uint32_t)ZB_SMEM_FRUSTA, nfix - f0);
@@ -565,26 +583,19 @@ __global__ void __launch_bounds__(ZB_THREADS) k_zb_draw_big(const unsigned long 
     for (unsigned long long q = blockIdx.x; q < n; q += gridDim.x) {
         const PairFT pr = big[q];
         const ZbFrustum F = frusta[pr.fix];
-        const float4 v[3] = {tris[3 * (size_t)pr.tri], tris[3 * (size_t)pr.tri + 1], tris[3 * (size_t)pr.tri + 2]};
-        float pu[3], pv[3], iw[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            float x, y, w;
-            to_camera(F, v[k].x, v[k].y, v[k].z, x, y, w);
-            iw[k] = 1.0f / w;
-            pu[k] = fmaf(F.sx, x * iw[k], F.ox);
-            pv[k] = fmaf(F.sy, y * iw[k], F.oy);
-        }
-        int x0, x1, y0, y1;
-        pixel_box(fmin3(pu[0], pu[1], pu[2]), fmax3(pu[0], pu[1], pu[2]), fmin3(pv[0], pv[1], pv[2]),
-                  fmax3(pv[0], pv[1], pv[2]), (int)res, x0, x1, y0, y1);
-        const float4 e0 = canonical_edge(pu[1], pv[1], pu[2], pv[2]), e1 = canonical_edge(pu[2], pv[2], pu[0], pv[0]);
-        const float4 e2 = canonical_edge(pu[0], pv[0], pu[1], pv[1]), iws = make_float4(iw[0], iw[1], iw[2], 0.f);
         uint32_t* zb = zbuf + (size_t)pr.fix * res * res;
-        // 32 x 8 pixels at a time: a warp on a row
-        for (int py = y0 + (int)(threadIdx.x >> 5); py <= y1; py += ZB_THREADS / 32)
-            for (int px = x0 + (int)(threadIdx.x & 31); px <= x1; px += 32)
-                shade_tri(e0, e1, e2, iws, px + 0.5f, py + 0.5f, F.n, F.f, zb + (size_t)py * res + px);
+        ClipPoly P;
+        clip_project(F, tris[3 * (size_t)pr.tri], tris[3 * (size_t)pr.tri + 1], tris[3 * (size_t)pr.tri + 2], P);
+        int x0, x1, y0, y1;
+        poly_bbox(P, (int)res, x0, x1, y0, y1);
+        for (int t = 1; t + 1 < P.n; ++t) {
+            float4 e0, e1, e2, iw;
+            fan_tri(P, t, e0, e1, e2, iw);
+            // 32 x 8 pixels at a time: a warp on a row
+            for (int py = y0 + (int)(threadIdx.x >> 5); py <= y1; py += ZB_THREADS / 32)
+                for (int px = x0 + (int)(threadIdx.x & 31); px <= x1; px += 32)
+                    shade_tri(e0, e1, e2, iw, px + 0.5f, py + 0.5f, F.n, F.f, zb + (size_t)py * res + px);
+        }
     }
 }
 

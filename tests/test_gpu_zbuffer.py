@@ -230,3 +230,78 @@ def test_zbuffer_full_scene_sampled(env):
     # triangle edge far more often than in the small scenes: the bookkeeping marks such reads
     # ambiguous whatever the neighbour's depth (measured: 8.6 % of 6334 pairs).
     assert amb.mean() < 0.15 and vis.sum() > 50
+
+
+def _box(lo, hi):
+    """A closed box of 12 triangles."""
+    v = np.array([[x, y, z] for x in (lo[0], hi[0]) for y in (lo[1], hi[1]) for z in (lo[2], hi[2])], np.float32)
+    f = np.array([[0, 1, 3], [0, 3, 2], [4, 6, 7], [4, 7, 5], [0, 4, 5], [0, 5, 1], [2, 3, 7], [2, 7, 6], [0, 2, 6],
+                  [0, 6, 4], [1, 5, 7], [1, 7, 3]], np.uint32)
+    return v, f
+
+
+def test_room_around_the_viewer_against_oracle(env):
+    """Floor and walls pass the viewers (clipped at the near plane, most of them over the whole window), a strip of
+    triangles a few pixels wide reaches it too: depths against the oracle."""
+    G, pipe, ctx = env
+    rng = np.random.default_rng(3)
+    n, theta, zb = 24, f32(math.radians(3.0)), oracle.ZBuffer(res=48, near=f32(0.05), far=100.0)
+    eye = np.stack([rng.uniform(-3, 3, n), np.full(n, 1.7), rng.uniform(-3, 3, n)], 1).astype(np.float32)
+    gaze = rng.normal(size=(n, 3))
+    gaze /= np.linalg.norm(gaze, axis=1, keepdims=True)
+    gaze = gaze.astype(np.float32)
+    fwd, up = gaze.copy(), np.tile(np.float32([0, 1, 0]), (n, 1))
+    v, f = _box((-4, 0, -4), (4, 2.8, 4))
+    parts = [(v, f)]
+    for i in range(0, n, 2):      # slivers from behind the eye to 2 m before it, across the gaze ray
+        g, side = gaze[i].astype(np.float64), np.cross(gaze[i], rng.normal(size=3))
+        side /= np.linalg.norm(side)
+        a, b = eye[i] - 0.3 * g + 0.02 * side, eye[i] + 2.0 * g
+        w = np.cross(g, side) * (0.002 if i % 4 else 0.02)
+        parts.append((np.array([a, b, b + w], np.float32), np.array([[0, 1, 2]], np.uint32)))
+    meshes = [(p, q, np.eye(4), k) for k, (p, q) in enumerate(parts)]
+    sc = G.gm_build_scene(ctx, meshes)
+    z, _ = G.gm_zbuffer_render(sc, eye, gaze, theta, 4.0, G.zbuffer_params(zb.res, zb.near, zb.far), fwd, up)
+    G.gm_scene_free(sc)
+    tri = np.concatenate([p[q.astype(np.int64)] for p, q in parts]).astype(np.float64)
+    sure_px = 0
+    for i in range(n):
+        F = oracle.zb_frustum(eye[i], gaze[i], fwd[i], up[i], theta, 4.0, zb.near, zb.far)
+        zo, amb = oracle.zb_render(tri, F, zb.res, delta_px=DPX)
+        zg, sure = z[i].astype(np.float64), ~amb & np.isfinite(zo)
+        assert np.all(np.isfinite(zg[sure])) and np.all(np.abs(zg[sure] - zo[sure]) <= 1e-4 * zo[sure])
+        sure_px += int(sure.sum())
+    assert sure_px > 0.9 * n * zb.res ** 2
+
+
+def test_walls_that_pass_the_viewer_take_no_longer_than_walls_before_it(env):
+    """A clipped triangle over the whole window is drawn by a block, as an unclipped one is (by one lane it took a
+    thousand times as long): 64 fixations on a tilted plane that goes on behind the eyes, and on one before them."""
+    import time
+
+    import torch
+    G, pipe, ctx = env
+    rng = np.random.default_rng(4)
+    n, res = 64, 512
+    eye = rng.uniform(-0.1, 0.1, (n, 3)).astype(np.float32)
+    gaze = np.float32([0, 0, 1]) + rng.uniform(-0.1, 0.1, (n, 3)).astype(np.float32)
+    up, dur, ts = np.tile(np.float32([0, 1, 0]), (n, 1)), np.ones(n, np.float32), np.arange(float(n))
+    prm, f = G.make_params(math.radians(1.0)), np.array([[0, 1, 2], [0, 2, 3]], np.uint32)
+
+    def best(v):
+        sc = G.gm_build_scene(ctx, [(np.array(v, np.float32), f, np.eye(4), 0)])
+        sm = G.gm_samples_from_points(sc, np.float32([[0, 0, 3]]), np.zeros(1, np.uint32))
+        t = math.inf
+        for _ in range(4):
+            t0 = time.perf_counter()
+            m = G.gm_accumulate_zbuffer(sc, sm, eye, gaze, dur, ts, prm, G.zbuffer_params(res), gaze, up)
+            torch.cuda.synchronize()
+            t = min(t, time.perf_counter() - t0)
+            G.gm_map_free(m)
+        G.gm_samples_free(sm)
+        G.gm_scene_free(sc)
+        return t
+
+    passing = best([[-20, -6.5, -10], [20, -6.5, -10], [20, 3.5, 10], [-20, 3.5, 10]])
+    before = best([[-5, -5, 3], [5, -5, 3], [5, 5, 3], [-5, 5, 3]])
+    assert passing < 10 * before + 2e-3, (passing, before)
