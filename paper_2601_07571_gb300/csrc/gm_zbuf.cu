@@ -33,7 +33,7 @@ constexpr int ZB_THREADS = 256;
 constexpr int ZB_SMEM_FRUSTA = 64;            // frusta staged per pass of the cull kernel
 constexpr int ZB_BIG_PIXELS = 1024;           // larger pixel boxes go to the block rasteriser
 constexpr int ZB_LANE_PIXELS = 32;            // clipped pairs: larger ones go to the warp
-constexpr uint64_t ZB_BIG_CAP = 1u << 20;     // ... through a list of this many pairs (a full list: drawn in place)
+                                              // (through a list of zb_big_cap pairs)
 constexpr uint32_t ZB_EMPTY = 0xffffffffu;    // cleared z-buffer word (above every finite depth)
 constexpr uint32_t NO_WINDOW = 0xffffffffu;
 
@@ -334,13 +334,13 @@ __device__ __forceinline__ void draw_poly(const ClipPoly& P, int x0, int y0, int
 // The pairs of a warp's entries that its shared pixels leave out: boxes above ZB_BIG_PIXELS, for the block
 // rasteriser, and pairs that reach the near plane (`clip`). Those are clipped first; a floor or wall that
 // passes the viewer fills the whole window, so they too go to the block rasteriser, to the warp (above
-// ZB_LANE_PIXELS) or to their lane by the size of their box. (Out of line: few warps come here, and its
+// ZB_LANE_PIXELS, and what finds the list full) or to their lane by the size of their box. (Out of line: few warps come here, and its
 // registers are its own.) 12 triangles of a room and 60k of objects in it, 2000 fixations at 256 x 256:
 // 165 ms with every clipped pair drawn by its lane, 1.8 so.
 __device__ __noinline__ void draw_others(const ZbFrustum* sF, const float4* __restrict__ tris, const int entry,
                                          const bool clip, int npx, const uint32_t f0, const uint32_t slot0,
                                          const uint32_t res, uint32_t* __restrict__ zbuf, PairFT* __restrict__ big,
-                                         unsigned long long* __restrict__ n_big) {
+                                         const uint64_t cap, unsigned long long* __restrict__ n_big) {
     const int lane = threadIdx.x & 31, src = entry & 31, own = entry >> 5;
     auto project = [&](int k, int from, ClipPoly& P) {
         const float4* v = tris + 3 * (size_t)(slot0 + from);
@@ -356,14 +356,15 @@ __device__ __noinline__ void draw_others(const ZbFrustum* sF, const float4* __re
     } else {
         npx = 0;   // drawn
     }
-    bool here = npx > 0 && npx <= ZB_LANE_PIXELS;
+    bool shared = npx > ZB_LANE_PIXELS;
     if (npx > ZB_BIG_PIXELS) {
         const unsigned long long q = atomicAdd(n_big, 1ull);
-        if (q < ZB_BIG_CAP) big[q] = PairFT{f0 + (uint32_t)own, slot0 + (uint32_t)src};
-        else here = true;
+        shared = q >= cap;
+        if (!shared) big[q] = PairFT{f0 + (uint32_t)own, slot0 + (uint32_t)src};
+    } else if (!shared) {
+        draw_poly(P, x0, y0, x1 - x0 + 1, npx, sF[own].n, sF[own].f, res, zbuf + (size_t)(f0 + own) * res * res, 0, 1);
     }
-    if (here) draw_poly(P, x0, y0, x1 - x0 + 1, npx, sF[own].n, sF[own].f, res, zbuf + (size_t)(f0 + own) * res * res, 0, 1);
-    unsigned todo = __ballot_sync(0xffffffffu, npx > ZB_LANE_PIXELS && npx <= ZB_BIG_PIXELS);
+    unsigned todo = __ballot_sync(0xffffffffu, shared);
     while (todo) {
         const int who = __ffs(todo) - 1;
         todo &= todo - 1u;
@@ -386,7 +387,7 @@ __global__ void __launch_bounds__(ZB_THREADS, 4) k_zb_draw(const float4* __restr
                                                            const ZbFrustum* __restrict__ frusta, uint32_t nfix,
                                                            uint32_t res, float near_m, float far_m,
                                                            uint32_t* __restrict__ zbuf, PairFT* __restrict__ big,
-                                                           unsigned long long* __restrict__ counts) {
+                                                           uint64_t cap, unsigned long long* __restrict__ counts) {
     constexpr int WARPS = ZB_THREADS / 32;
     __shared__ ZbFrustum sF[ZB_SMEM_FRUSTA];
     __shared__ ZbTri slots[WARPS][32];
@@ -507,7 +508,7 @@ __global__ void __launch_bounds__(ZB_THREADS, 4) k_zb_draw(const float4* __restr
         __syncwarp();
         const bool clip = lane < cnt && !front;
         if (__any_sync(0xffffffffu, clip || npx > ZB_BIG_PIXELS))
-            draw_others(sF, tris, entry, clip, npx, f0, t - lane, res, zbuf, big, &counts[1]);
+            draw_others(sF, tris, entry, clip, npx, f0, t - lane, res, zbuf, big, cap, &counts[1]);
     };
     for (uint32_t f0 = blockIdx.y * ZB_SMEM_FRUSTA; f0 < nfix; f0 += gridDim.y * ZB_SMEM_FRUSTA) {
         const uint32_t m = min((uint32_t)ZB_SMEM_FRUSTA, nfix - f0);
@@ -575,11 +576,11 @@ __global__ void __launch_bounds__(ZB_THREADS, 4) k_zb_draw(const float4* __restr
 }
 
 __global__ void __launch_bounds__(ZB_THREADS) k_zb_draw_big(const unsigned long long* __restrict__ counts,
-                                                            const PairFT* __restrict__ big,
+                                                            const PairFT* __restrict__ big, uint64_t cap,
                                                             const ZbFrustum* __restrict__ frusta,
                                                             const float4* __restrict__ tris, uint32_t res,
                                                             uint32_t* __restrict__ zbuf) {
-    const unsigned long long n = min(counts[1], (unsigned long long)ZB_BIG_CAP);
+    const unsigned long long n = min(counts[1], (unsigned long long)cap);
     for (unsigned long long q = blockIdx.x; q < n; q += gridDim.x) {
         const PairFT pr = big[q];
         const ZbFrustum F = frusta[pr.fix];
@@ -765,18 +766,26 @@ __global__ void k_zb_set_valid(unsigned long long* __restrict__ c, const uint32_
     c[3] = *n_valid;
 }
 
+// Entries of the list of large pairs of nfix z-buffers: eight layers of pairs of 2 x 1024-pixel boxes that fill
+// every window (1/32 of the z-buffers' bytes), more than which is drawn by the warps that find it. 65000
+// fixations at 64 x 64 before 24 walls (3.1M pairs): 143 ms with 2^20 entries, 59 with all in the list.
+uint64_t zb_big_cap(uint64_t n_tris, uint64_t nfix, uint64_t res) {
+    return std::min(n_tris * nfix, std::max<uint64_t>(1024, nfix * res * res / 64));
+}
+
 // Render the z-buffers of frusta [0, nfix) into zbuf (nfix x res^2 words, cleared here). counts: [0] grows
-// by the pairs drawn, [1] is the length of the list `big` (ZB_BIG_CAP entries).
+// by the pairs drawn, [1] is the length of the list `big` (`cap` entries).
 gm_status render_zbuffers(gm_ctx* ctx, gm_scene* sc, const ZbFrustum* frusta, uint32_t nfix, uint32_t res,
-                          float near_m, float far_m, uint32_t* zbuf, PairFT* big, unsigned long long* counts,
-                          cudaStream_t s, int* launches) {
+                          float near_m, float far_m, uint32_t* zbuf, PairFT* big, uint64_t cap,
+                          unsigned long long* counts, cudaStream_t s, int* launches) {
     const size_t npx = (size_t)res * res;
     static_assert(ZB_EMPTY == 0xffffffffu, "a byte-wise 0xff clear writes ZB_EMPTY");
     GM_TRY_CUDA(cudaMemsetAsync(zbuf, 0xff, sizeof(uint32_t) * npx * nfix, s));
     GM_TRY_CUDA(cudaMemsetAsync(&counts[1], 0, sizeof(unsigned long long), s));
     const dim3 grid(gm_div_up(sc->n_tris, ZB_THREADS), std::min<uint32_t>(gm_div_up(nfix, ZB_SMEM_FRUSTA), 65535));
-    k_zb_draw<<<grid, ZB_THREADS, 0, s>>>(sc->bvh_tris, sc->n_tris, frusta, nfix, res, near_m, far_m, zbuf, big, counts);
-    k_zb_draw_big<<<(uint32_t)ctx->n_sm * 4, ZB_THREADS, 0, s>>>(counts, big, frusta, sc->bvh_tris, res, zbuf);
+    k_zb_draw<<<grid, ZB_THREADS, 0, s>>>(sc->bvh_tris, sc->n_tris, frusta, nfix, res, near_m, far_m, zbuf, big, cap,
+                                          counts);
+    k_zb_draw_big<<<(uint32_t)ctx->n_sm * 4, ZB_THREADS, 0, s>>>(counts, big, cap, frusta, sc->bvh_tris, res, zbuf);
     *launches += 2;
     GM_TRY_CUDA(cudaGetLastError());
     return GM_OK;
@@ -847,7 +856,8 @@ extern "C" gm_status gm_zbuffer_render(gm_scene* sc, const float* eye, const flo
     ZB_TMP(fr, sizeof(ZbFrustum) * n);
     ZB_TMP(crop, sizeof(double) * 4 * n);
     ZB_TMP(zb, sizeof(uint32_t) * npx * n);
-    ZB_TMP(big, sizeof(PairFT) * ZB_BIG_CAP);
+    const uint64_t cap = zb_big_cap(sc->n_tris, n, zp->res);
+    ZB_TMP(big, sizeof(PairFT) * cap);
     ZB_TMP(counts, sizeof(unsigned long long) * 2);
     if (cudaError_t e = cudaMemsetAsync(counts, 0, sizeof(unsigned long long) * 2, s); e != cudaSuccess)
         return done(gm_cuda_error(e, "gm_zbuffer_render"));
@@ -856,7 +866,7 @@ extern "C" gm_status gm_zbuffer_render(gm_scene* sc, const float* eye, const flo
                                                    (double)cutoff_sigmas, (double)zp->near_m, (double)zp->far_m,
                                                    zp->res, fr, crop, nullptr);
     ++launches;
-    st = render_zbuffers(ctx, sc, fr, n, zp->res, zp->near_m, zp->far_m, zb, big, counts, s, &launches);
+    st = render_zbuffers(ctx, sc, fr, n, zp->res, zp->near_m, zp->far_m, zb, big, cap, counts, s, &launches);
     if (st == GM_OK && gm_is_device_ptr(zbuf_out)) {
         k_zb_export<<<gm_div_up(npx * n, 256), 256, 0, s>>>(zb, npx * n, zbuf_out);
         ++launches;
@@ -1015,7 +1025,8 @@ extern "C" gm_status gm_accumulate_zbuffer(gm_scene* sc, gm_samples* sm, const g
     if (chunk < nv) TMP_ALLOC(state, sizeof(float2) * (ns ? ns : 1));
     PairFT* big = nullptr;
     unsigned long long* counts = nullptr;
-    TMP_ALLOC(big, sizeof(PairFT) * ZB_BIG_CAP);
+    const uint64_t cap = zb_big_cap(sc->n_tris, chunk, res);
+    TMP_ALLOC(big, sizeof(PairFT) * cap);
     TMP_ALLOC(counts, sizeof(unsigned long long) * 2);
     GM_TRY_CUDA(cudaMemsetAsync(counts, 0, sizeof(unsigned long long) * 2, s));
 
@@ -1056,7 +1067,7 @@ extern "C" gm_status gm_accumulate_zbuffer(gm_scene* sc, gm_samples* sm, const g
     }
     for (uint32_t f0 = 0; f0 < nv; f0 += chunk) {
         const uint32_t f1 = std::min(nv, f0 + chunk);
-        if ((st = render_zbuffers(ctx, sc, frusta + f0, f1 - f0, res, zp->near_m, zp->far_m, zbuf, big, counts, s,
+        if ((st = render_zbuffers(ctx, sc, frusta + f0, f1 - f0, res, zp->near_m, zp->far_m, zbuf, big, cap, counts, s,
                                   &launches)) != GM_OK)
             return fail(st);
         if (ns > 0) {

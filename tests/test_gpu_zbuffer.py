@@ -305,3 +305,33 @@ def test_walls_that_pass_the_viewer_take_no_longer_than_walls_before_it(env):
     passing = best([[-20, -6.5, -10], [20, -6.5, -10], [20, 3.5, 10], [-20, 3.5, 10]])
     before = best([[-5, -5, 3], [5, -5, 3], [5, 5, 3], [-5, 5, 3]])
     assert passing < 10 * before + 2e-3, (passing, before)
+
+
+def test_full_list_of_large_pairs(env):
+    """30 walls that fill the window: 60 pairs of more than 1024 pixels a fixation, more than the list of large pairs
+    of 64 fixations holds (at most a pair per 64 pixels, or the scene's pairs), and, two fixations at a time, fewer
+    than its smallest size: the same map."""
+    G, pipe, ctx = env
+    rng = np.random.default_rng(6)
+    n, res, layers = 64, 40, 30
+    z = 3.0 - 0.05 * np.arange(layers)
+    v = np.concatenate([np.float32([[-5, -5, d], [5, -5, d], [5, 5, d], [-5, 5, d]]) for d in z])
+    f = np.concatenate([np.array([[0, 1, 2], [0, 2, 3]], np.uint32) + np.uint32(4 * k) for k in range(layers)])
+    eye = rng.uniform(-0.1, 0.1, (n, 3)).astype(np.float32)
+    gaze = np.float32([0, 0, 1]) + rng.uniform(-0.1, 0.1, (n, 3)).astype(np.float32)
+    up = np.tile(np.float32([0, 1, 0]), (n, 1))
+    sc = G.gm_build_scene(ctx, [(v, f, np.eye(4), 0)])
+    sm = G.gm_sample_surface(sc, [30.0], 8)
+    ns, out = G.gm_samples_info(sm), []
+    for per in (n, 2):
+        m = G.gm_accumulate_zbuffer(sc, sm, eye, gaze, np.ones(n, np.float32), np.arange(float(n)),
+                                    G.make_params(math.radians(2.0), normalize=False),
+                                    G.zbuffer_params(res, zbuffer_bytes=per * res * res * 4), gaze, up)
+        out.append((np.empty(ns, np.float32), G.gm_zbuffer_stats(m)["raster_pairs"]))
+        G.gm_map_copy(m, 0, out[-1][0])
+        G.gm_map_free(m)
+    G.gm_samples_free(sm)
+    G.gm_scene_free(sc)
+    assert out[0][1] == out[1][1] > n * res * res // 64
+    # the cones cover about 0.9 m2 of the nearest wall: 27 samples at 30 a m2
+    assert np.array_equal(out[0][0], out[1][0]) and (out[0][0] > 0).sum() > 10
