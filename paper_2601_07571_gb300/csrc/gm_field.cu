@@ -316,10 +316,11 @@ constexpr uint32_t kQueryIdescN16 = (1u << 4) | (1u << 7) | (1u << 10) | ((16u >
 
 // The three bf16 parts of an FP32 value: hi = bf16(w), mid = bf16(w - hi), lo = w - hi - mid. Each
 // difference is exact in FP32 and lo needs at most 8 significant bits, so hi + mid + lo = w exactly;
-// a product with a bf16 activation is then three exact products summed in FP32.
+// a product with a bf16 activation is then three exact products summed in FP32. (An infinity is (w, 0, 0).)
 __device__ __forceinline__ void split3_bf16(float w, __nv_bfloat16 part[3]) {
     part[0] = __float2bfloat16_rn(w);
-    const float r1 = w - __bfloat162float(part[0]);
+    if (__hisinf(part[0])) part[0] = __float2bfloat16_rz(w);   // above the largest bf16 (infinities stay)
+    const float r1 = isinf(w) ? 0.f : w - __bfloat162float(part[0]);
     part[1] = __float2bfloat16_rn(r1);
     part[2] = __float2bfloat16_rn(r1 - __bfloat162float(part[1]));
 }

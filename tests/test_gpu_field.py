@@ -161,6 +161,31 @@ def test_field_gradient_and_adam_step_match_oracle(env, kernel):
     G.gm_field_free(f)
 
 
+@pytest.mark.parametrize("off", [-np.inf, -3.4e38, -3.39e38])
+def test_units_switched_off_by_their_bias(env, off):
+    """A hidden unit of bias -inf, or of one above the largest bf16 (3.3895e38), is 0 for every point, as one of bias
+    -1e30 is: queries, loss and gradient are those of that field bit for bit, and finite."""
+    G, torch, ctx = env
+    n = 700
+    x = torch.from_numpy(_points(n, 3)).cuda()
+    y = torch.from_numpy(np.random.default_rng(4).uniform(0, 1, n).astype(np.float32)).cuda()
+    idx = torch.arange(n, dtype=torch.int32, device="cuda")
+    got = []
+    for bias in (off, -1e30):
+        theta = synth.field_init(12)
+        for layer in range(4):
+            at = layer * (64 * 64 + 64) + 64 * 64
+            theta[at + 3 * layer:at + 64:9] = np.float32(bias)
+        f = G.gm_field_create(ctx, BOX_LO, BOX_HI, theta)
+        out, g = torch.empty(n, device="cuda"), np.empty(G.GM_FIELD_N_PARAMS, np.float32)
+        G.gm_field_query(f, x, n, out)
+        loss = G.gm_field_loss_grad(f, x, y, n, idx, n, g)
+        G.gm_sync(ctx)
+        G.gm_field_free(f)
+        got.append(np.concatenate([out.cpu().numpy(), [np.float32(loss)], g]))
+    assert np.all(np.isfinite(got[0])) and np.array_equal(got[0], got[1])
+
+
 def test_field_tensor_core_gradient_over_many_tiles(env):
     """70 001 batch points: 547 full tiles and a ragged one, several tiles per block, so the weight
     and bias gradients accumulate in tensor memory across tiles. The gradient matches the oracle to
