@@ -430,7 +430,8 @@ gm_status gm_accumulate_batch(gm_ctx* ctx, const gm_session_desc* sessions, uint
  * all of them and the faster is kept. *best_flags gets the GM_F_* variant bits to OR into
  * params->flags. Results are
  * cached per size bucket (log2 of samples, fixations and triangles) for the process and, when the
- * environment variable GM_TUNE_CACHE names a file, in that JSON file across processes. */
+ * environment variable GM_TUNE_CACHE names a file, in that JSON file across processes. Entries of
+ * a library with other kernels behind the flags are kept in the file but not used. */
 gm_status gm_autotune_accumulate(gm_scene* scene, gm_samples* samples, const gm_fixations* fix,
                                  const gm_params* params, gm_stream stream, int32_t* best_flags, float* best_ms);
 

@@ -275,10 +275,14 @@ std::mutex g_tune_mutex;
 std::map<std::string, int> g_tune;
 bool g_tune_loaded = false;
 
+// Raised whenever the kernel behind a flag value becomes another one: entries of other sets (and of files
+// from before the sets were numbered) are kept, but not found, and the candidates are timed again.
+constexpr int kKernelSet = 2;   // 2: the default flags trace shafts
+
 std::string bucket_key(const char* kind, uint64_t ns, uint64_t nf, uint64_t nt) {
     auto lg = [](uint64_t v) { return v ? (int)std::floor(std::log2((double)v)) : -1; };
     std::ostringstream o;
-    o << kind << ":" << lg(ns) << ":" << lg(nf) << ":" << lg(nt);
+    o << "set" << kKernelSet << ":" << kind << ":" << lg(ns) << ":" << lg(nf) << ":" << lg(nt);
     return o.str();
 }
 

@@ -206,3 +206,37 @@ def test_autotune_picks_a_variant_and_keeps_results(env, tmp_path, monkeypatch):
     for sc, sm, *_ in hs:
         G.gm_samples_free(sm)
         G.gm_scene_free(sc)
+
+
+_TUNE = """
+import sys, numpy as np
+import paper_2601_07571_gb300 as G
+ctx = G.gm_create(0)
+v = np.float32([[0, 0, 0], [1, 0, 0], [1, 1, 0], [0, 1, 0]])
+sc = G.gm_build_scene(ctx, [(v, np.uint32([[0, 1, 2], [0, 2, 3]]), np.eye(4), 0)])
+sm = G.gm_samples_from_points(sc, np.float32([[0.2, 0.1, 0], [0.7, 0.5, 0], [0.1, 0.9, 0]]), np.uint32([0, 0, 1]))
+n = 5
+fix = (np.float32([[0.5, 0.5, 2]] * n), np.float32([[0, 0, -1]] * n), np.ones(n, np.float32), np.arange(float(n)))
+print(*G.gm_autotune_accumulate(sc, sm, *fix, G.make_params(0.1)))
+"""
+
+
+def test_tuning_file_of_other_kernels_is_timed_again(env, tmp_path):
+    """An entry written when other kernels stood behind the flags (its key names no kernel set) neither decides nor
+    gets lost; the entry that takes its place is found by the next process."""
+    import os
+    import subprocess
+    import sys
+    G, _, _ = env
+    path = tmp_path / "tune.json"
+    # the size bucket of the program above: 3 samples, 5 fixations, 2 triangles
+    path.write_text('{\n  "plain:1:2:1": %d\n}\n' % G.GM_F_NO_COMPACT)
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    times = []
+    for _ in range(2):
+        r = subprocess.run([sys.executable, "-c", _TUNE], cwd=root, env=dict(os.environ, GM_TUNE_CACHE=str(path)),
+                           capture_output=True, text=True, check=True)
+        times.append(r.stdout.split())
+    assert float(times[0][1]) > 0.0 and float(times[1][1]) == 0.0 and times[0][0] == times[1][0]
+    text = path.read_text()
+    assert '"plain:1:2:1": %d' % G.GM_F_NO_COMPACT in text and ':plain:1:2:1": %s' % times[0][0] in text
