@@ -131,7 +131,10 @@ __global__ void __launch_bounds__(1024) k_fix_prep(FixIn I, int bits, bool into,
         else if (threadIdx.x == 3) counters[3] += n;
         else if (threadIdx.x == 6) counters[6] = 0ull;
     }
-    if (threadIdx.x == 0) *n_valid = (uint32_t)valid;
+    if (threadIdx.x == 0) {
+        n_valid[0] = (uint32_t)valid;
+        n_valid[1] = 0u;   // k_sparse_probe's
+    }
 }
 
 
@@ -177,29 +180,72 @@ __global__ void __launch_bounds__(NT, MINB) k_accumulate(
     warp_stats_commit(st, counters);
 }
 
-// The default: the rays of a (tile, fixation) pair traced as one shaft (gm_shaft.cuh). Blocks pull tiles
-// from a device counter (or, static, take their own): all tiles of 32 samples or, LISTS, the sample set's
-// tiles of 128 samples on few triangles and then its other tiles of 32 (gm_samples::tile_lists). For a set
-// with lists both are launched and the device knows which has the work.
 // From half of the samples on. Below that what stands before the large triangles is mostly fine, and a wide
 // shaft meets more of it: 10 windows of a cube (an eighth of 300k samples) among objects of 1 cm triangles
 // take 9.4 ms with the cube in wide tiles, 8.0 without.
 __device__ __forceinline__ bool wide_tiles_pay(const uint32_t* lists, uint64_t ns) { return 2ull * 128 * lists[0] >= ns; }
 
+// Whether a set with wide tiles takes blocks of 128 threads: where a wide tile is reached by few fixations, most
+// warps of a larger block wait for its slowest shaft, and twice the tiles in flight help more. The measure is
+// the mean, over SPARSE_TILES tiles of 128 samples spread over the work order, of the fixations that reach the
+// tile (64 at most: a few tiles are reached by all). Probed are lists of up to RS_SMALL fixations over
+// SPARSE_MIN samples or more: with more fixations tiles are not sparse, smaller sets end by their longest tile.
+// Walks in cities of 0.1-0.6M triangles, 1000-1500 fixations, us with 256 / 128 threads (per-ray walks): mean
+// 4: 2429 / 2107 (2260), 5: 1186 / 947 (1121), 8: 2920 / 2573 (2874), 9: 815 / 675 (799), but on four objects
+// of 20k triangles, where the longest tile decides: 6: 932 / 818, 10: 1193 / 1275, 12: 1441 / 1498,
+// 19: 1980 / 2191, 37: 3583 / 4126. (A city at 14: 672 / 583 (634): the line is drawn for the objects.) The probe
+// and a kernel that returns at once take 3 to 9 us.
+constexpr int SPARSE_TILES = 256;
+constexpr uint32_t SPARSE_SUM = 19 * SPARSE_TILES / 2;
+constexpr uint64_t SPARSE_MIN = 1u << 19;
+__device__ __forceinline__ bool sparse_tiles(const uint32_t* n_fix) { return n_fix[1] <= SPARSE_SUM; }
+
+// n_fix: [0] their number, [1] grows by the fixations that reach the tile of each block.
+__global__ void __launch_bounds__(256) k_sparse_probe(const float4* __restrict__ spos, uint32_t ns,
+                                                      const float4* __restrict__ fix, uint32_t* __restrict__ n_fix,
+                                                      float tanphi) {
+    __shared__ uint32_t total;
+    const int lane = threadIdx.x & 31;
+    const uint32_t tiles = ns / 128, tile = (uint32_t)((2ull * blockIdx.x + 1) * tiles / (2 * SPARSE_TILES));
+    if (threadIdx.x == 0) total = 0;
+    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float4 p = spos[128ull * tile + 32 * k + lane];
+        lo[0] = fminf(lo[0], p.x), lo[1] = fminf(lo[1], p.y), lo[2] = fminf(lo[2], p.z);
+        hi[0] = fmaxf(hi[0], p.x), hi[1] = fmaxf(hi[1], p.y), hi[2] = fmaxf(hi[2], p.z);
+    }
+    const float4 bs = tile_sphere(lo, hi);
+    __syncthreads();
+    uint32_t n = 0;
+    for (uint32_t i = threadIdx.x; i < n_fix[0]; i += 256)
+        n += cone_reaches_sphere(bs, __ldg(&fix[2 * i]), __ldg(&fix[2 * i + 1]), tanphi);
+    n = __reduce_add_sync(0xffffffffu, n);
+    if (lane == 0) atomicAdd(&total, n);
+    __syncthreads();
+    if (threadIdx.x == 0) atomicAdd(&n_fix[1], min(total, 64u));
+}
+
+// The default: the rays of a (tile, fixation) pair traced as one shaft (gm_shaft.cuh). Blocks pull tiles
+// from a device counter (or, static, take their own): all tiles of 32 samples or, LISTS, the sample set's
+// tiles of 128 samples on few triangles and then its other tiles of 32 (gm_samples::tile_lists). For a set
+// with lists several forms are launched and the device knows which has the work; probed: among them the one
+// of 128 threads.
 template <bool DEBUG, bool LISTS, int NT = ACC_THREADS>
 __global__ void __launch_bounds__(NT, 1024 / NT) k_accumulate_shaft(
     const float4* __restrict__ spos, const uint32_t* __restrict__ sidx, const float4* __restrict__ fix,
     const uint32_t* __restrict__ n_fix_dev, const float4* __restrict__ nodes, const float4* __restrict__ nodes4,
-    const float4* __restrict__ tris, AccParams P, uint32_t n_tiles, const uint32_t* __restrict__ lists,
+    const float4* __restrict__ tris, AccParams P, uint32_t n_tiles, const uint32_t* __restrict__ lists, bool probed,
     int persistent, float* __restrict__ out, unsigned int* __restrict__ max_bits,
     unsigned long long* __restrict__ counters, int* __restrict__ err, DebugOut dbg) {
-    constexpr size_t BYTES = LISTS && sizeof(ShaftBlock<4>) > sizeof(ShaftBlock<1>) ? sizeof(ShaftBlock<4>) : sizeof(ShaftBlock<1>);
-    __shared__ __align__(16) unsigned char fixed[NT == ACC_THREADS ? BYTES : 16];
+    constexpr size_t B1 = sizeof(ShaftBlock<1, NT>), B4 = sizeof(ShaftBlock<4, NT>);
+    __shared__ __align__(16) unsigned char fixed[NT > ACC_THREADS ? 16 : LISTS && B4 > B1 ? B4 : B1];
     extern __shared__ __align__(16) unsigned char dynamic[];   // above 48 KB
-    unsigned char* smem = NT == ACC_THREADS ? fixed : dynamic;
+    unsigned char* smem = NT > ACC_THREADS ? dynamic : fixed;
     __shared__ uint32_t s_tile;
     const uint32_t nf = *n_fix_dev;
     if (lists && wide_tiles_pay(lists, P.ns) != LISTS) return;
+    if (LISTS && probed && sparse_tiles(n_fix_dev) != (NT < ACC_THREADS)) return;
     const uint32_t n_wide = LISTS ? lists[0] : 0u;
     const uint32_t n = LISTS ? n_wide + lists[1] : n_tiles;
     unsigned int* next = reinterpret_cast<unsigned int*>(&counters[6]);
@@ -214,8 +260,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_accumulate_shaft(
         }
         if (k >= n) break;
         if (LISTS && k < n_wide)
-            shaft_tile<DEBUG, 4>(__ldg(&lists[2 + k]), spos, sidx, fix, nf, nodes, nodes4, tris, P, out, max_bits,
-                                 *reinterpret_cast<ShaftBlock<4>*>(smem), &counters[2], dbg, err, st);
+            shaft_tile<DEBUG, 4, NT>(__ldg(&lists[2 + k]), spos, sidx, fix, nf, nodes, nodes4, tris, P, out, max_bits,
+                                 *reinterpret_cast<ShaftBlock<4, NT>*>(smem), &counters[2], dbg, err, st);
         else
             shaft_tile<DEBUG, 1, NT>(LISTS ? __ldg(&lists[gm_tile_list_fine(P.ns) + (k - n_wide)]) : k, spos, sidx, fix, nf, nodes,
                                  nodes4, tris, P, out, max_bits, *reinterpret_cast<ShaftBlock<1, NT>*>(smem), &counters[2],
@@ -354,9 +400,9 @@ int shaft_threads(uint64_t tiles, uint64_t n_fix, int n_sm) {
 }
 
 template <typename K>
-int blocks_per_sm(K kern) {
+int blocks_per_sm(K kern, int nt) {
     int b = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, ACC_THREADS, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, nt, 0);
     return b > 0 ? b : 1;
 }
 
@@ -453,7 +499,7 @@ gm_status accumulate_impl(gm_scene* sc, gm_samples* sm, const gm_fixations* fx, 
     if (o4) tmp.push_back(d_ts);
     uint32_t *n_valid = nullptr, *orig = nullptr;
     float4* packed = nullptr;
-    TMP_ALLOC(packed, (2 * sizeof(float4) + sizeof(uint32_t)) * (size_t)nf + sizeof(uint32_t));
+    TMP_ALLOC(packed, (2 * sizeof(float4) + sizeof(uint32_t)) * (size_t)nf + 2 * sizeof(uint32_t));
     orig = reinterpret_cast<uint32_t*>(packed + 2 * (size_t)nf);
     n_valid = orig + nf;
     const double tan_t = std::tan((double)prm->theta_rad);
@@ -632,8 +678,9 @@ gm_status accumulate_impl(gm_scene* sc, gm_samples* sm, const gm_fixations* fx, 
                 cudaEventRecord(mp->ev[5], s);
             }
             if (shaft) {
-                static const int per_sm = blocks_per_sm(k_accumulate_shaft<false, false>);
-                static const int per_sm_lists = blocks_per_sm(k_accumulate_shaft<false, true>);
+                static const int per_sm = blocks_per_sm(k_accumulate_shaft<false, false>, ACC_THREADS);
+                static const int per_sm_lists = blocks_per_sm(k_accumulate_shaft<false, true>, ACC_THREADS);
+                static const int per_sm_128 = blocks_per_sm(k_accumulate_shaft<false, true, 128>, 128);
                 const uint32_t* lists = reorder && persistent ? sm->tile_lists : nullptr;
                 const uint32_t tiles = gm_div_up(ns, 32);
                 auto grid = [&](int b) { return persistent ? std::min<uint32_t>((uint32_t)(ctx->n_sm * b), tiles) : tiles; };
@@ -642,7 +689,7 @@ gm_status accumulate_impl(gm_scene* sc, gm_samples* sm, const gm_fixations* fx, 
                     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
                     if (e != cudaSuccess) return e;
                     kern<<<grid(1024 / nt), nt, bytes, s>>>(spos, sidx, packed, n_valid, sc->nodes, sc->nodes4, sc->bvh_tris,
-                                                            P, tiles, nullptr, persistent, mp->values, mp->max_bits,
+                                                            P, tiles, nullptr, false, persistent, mp->values, mp->max_bits,
                                                             mp->counters, ctx->dev_err, dbg);
                     return cudaSuccess;
                 };
@@ -653,16 +700,21 @@ gm_status accumulate_impl(gm_scene* sc, gm_samples* sm, const gm_fixations* fx, 
                 } else if (nt == 512) {
                     GM_TRY_CUDA(few(k_accumulate_shaft<false, false, 512>, 512, sizeof(ShaftBlock<1, 512>)));
                 } else {
-                    auto kern = debug ? k_accumulate_shaft<true, false> : k_accumulate_shaft<false, false>;
-                    kern<<<grid(per_sm), ACC_THREADS, 0, s>>>(spos, sidx, packed, n_valid, sc->nodes, sc->nodes4,
-                                                              sc->bvh_tris, P, tiles, lists, persistent, mp->values,
-                                                              mp->max_bits, mp->counters, ctx->dev_err, dbg);
+                    auto run = [&](auto kern, int threads, int blocks, bool probed) {
+                        kern<<<grid(blocks), threads, 0, s>>>(spos, sidx, packed, n_valid, sc->nodes, sc->nodes4,
+                                                              sc->bvh_tris, P, tiles, lists, probed, persistent,
+                                                              mp->values, mp->max_bits, mp->counters, ctx->dev_err, dbg);
+                    };
+                    const bool probed = lists && prep && !debug && P.tile_cull && ns >= SPARSE_MIN;
+                    if (probed) {
+                        k_sparse_probe<<<SPARSE_TILES, 256, 0, s>>>(spos, P.ns, packed, n_valid, P.tanphi);
+                        run(k_accumulate_shaft<false, true, 128>, 128, per_sm_128, true);
+                        launches += 2;
+                    }
+                    run(debug ? k_accumulate_shaft<true, false> : k_accumulate_shaft<false, false>, ACC_THREADS, per_sm, false);
                     if (lists) {
-                        kern = debug ? k_accumulate_shaft<true, true> : k_accumulate_shaft<false, true>;
-                        kern<<<grid(per_sm_lists), ACC_THREADS, 0, s>>>(spos, sidx, packed, n_valid, sc->nodes, sc->nodes4,
-                                                                        sc->bvh_tris, P, tiles, lists, persistent,
-                                                                        mp->values, mp->max_bits, mp->counters,
-                                                                        ctx->dev_err, dbg);
+                        run(debug ? k_accumulate_shaft<true, true> : k_accumulate_shaft<false, true>, ACC_THREADS,
+                            per_sm_lists, probed);
                         launches++;
                     }
                 }

@@ -574,6 +574,18 @@ __device__ __forceinline__ float4 work_sample(const float4* __restrict__ spos, u
     return j < ns ? spos[j] : make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, __uint_as_float(0xffffffffu));
 }
 
+// The box of the warp's samples from each lane's bounds, and the sphere around it.
+__device__ __forceinline__ float4 tile_sphere(float lo[3], float hi[3]) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        lo[c] = redux_min(lo[c]);
+        hi[c] = redux_max(hi[c]);
+    }
+    return make_float4(0.5f * (lo[0] + hi[0]), 0.5f * (lo[1] + hi[1]), 0.5f * (lo[2] + hi[2]),
+                       0.5f * sqrtf((hi[0] - lo[0]) * (hi[0] - lo[0]) + (hi[1] - lo[1]) * (hi[1] - lo[1]) +
+                                    (hi[2] - lo[2]) * (hi[2] - lo[2])) * 1.0001f);
+}
+
 // One block, all threads: tile `tile` (32 NS consecutive work-order samples) against fixations [0, nf) of
 // `fix` (packed (e, w), (r^, window), sorted by window). A window's sums are written when the next visible
 // fixation opens another one, or at the end.
@@ -603,16 +615,9 @@ __device__ __forceinline__ void shaft_tile(const uint32_t tile, const float4* __
             hi[0] = fmaxf(hi[0], p.x), hi[1] = fmaxf(hi[1], p.y), hi[2] = fmaxf(hi[2], p.z);
         }
     }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        lo[c] = redux_min(lo[c]);
-        hi[c] = redux_max(hi[c]);
-    }
+    float4 bs = tile_sphere(lo, hi);
     if (warp == 0) shaft_start(lo, hi, nodes4, tris, P.nt, B.warp[0].tri, B.start);
-    const float4 bs = make_float4(0.5f * (lo[0] + hi[0]), 0.5f * (lo[1] + hi[1]), 0.5f * (lo[2] + hi[2]),
-                                  P.tile_cull ? 0.5f * sqrtf((hi[0] - lo[0]) * (hi[0] - lo[0]) + (hi[1] - lo[1]) * (hi[1] - lo[1]) +
-                                                             (hi[2] - lo[2]) * (hi[2] - lo[2])) * 1.0001f
-                                              : -1.f);
+    if (!P.tile_cull) bs.w = -1.f;
     // warp k < NS keeps the sums of samples 32 k + lane
     const uint32_t j = j0 + 32 * warp;
     const bool live = warp < NS && j < P.ns;

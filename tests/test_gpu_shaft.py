@@ -137,3 +137,36 @@ def test_wide_tile_with_a_ray_in_a_coordinate_plane(env):
     G.gm_scene_free(scene)
     assert out[0][1:] == out[1][1:] and 0 < out[0][2] < out[0][1]
     assert np.array_equal(out[0][0], out[1][0])
+
+
+def _maps(G, scene, samples, fix, theta, flags, **kw):
+    m = G.gm_accumulate_fixations(scene, samples, *fix, G.make_params(theta, normalize=False, flags=flags, **kw))
+    W, ns, st, _ = G.gm_map_info(m)
+    values = np.empty((W, ns), np.float32)
+    for w in range(W):
+        G.gm_map_copy(m, w, values[w])
+    G.gm_map_free(m)
+    return values, st["in_cone"], st["visible"]
+
+
+@pytest.mark.parametrize("n,nf,theta,windows", [
+    (1 << 19, 1, 1.0, 1), (1 << 19, 40, 1.0, 3), ((1 << 19) + 77, 2048, 0.3, 5), (1 << 19, 2048, 2.0, 1),
+    ((1 << 19) - 1, 40, 1.0, 1), (1 << 19, 2049, 0.3, 2)])
+def test_blocks_of_wide_tiles(env, n, nf, theta, windows):
+    """Sets of 2^19 samples and more whose tiles few fixations reach take smaller blocks, by a probe on the device
+    that lists of up to 2048 fixations get: either way the per-ray walk's maps."""
+    G, ctx = env
+    rng = np.random.default_rng(nf)
+    ball = M.uv_sphere(30, 60, 0.1, 0.1, 8.0, seed=2)
+    v, f, xyz, tri = _floor(n, (M.translate(ball[0], (0.5, 0.2, 0.5)), ball[1]))
+    at = xyz[rng.integers(0, n, nf)].astype(np.float64)
+    eye = np.stack([rng.uniform(0, 1, nf), rng.uniform(0.4, 0.8, nf), rng.uniform(0, 1, nf)], 1)
+    fix = [np.ascontiguousarray(eye, np.float32), np.ascontiguousarray(at - eye, np.float32),
+           rng.uniform(0.1, 0.6, nf).astype(np.float32), rng.uniform(0, windows, nf)]
+    kw = dict(t_begin=0.0, t_end=float(windows), window_s=1.0) if windows > 1 else {}
+    scene = G.gm_build_scene(ctx, [(v, f, np.eye(4), 0)])
+    samples = G.gm_samples_from_points(scene, xyz, tri)
+    a, b = (_maps(G, scene, samples, fix, math.radians(theta), flags, **kw) for flags in (0, G.GM_F_FIX_L1))
+    G.gm_samples_free(samples)
+    G.gm_scene_free(scene)
+    assert a[1:] == b[1:] and a[2] > 0 and np.array_equal(a[0], b[0])
