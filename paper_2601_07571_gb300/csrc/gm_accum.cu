@@ -693,12 +693,13 @@ gm_status accumulate_impl(gm_scene* sc, gm_samples* sm, const gm_fixations* fx, 
                                                             mp->counters, ctx->dev_err, dbg);
                     return cudaSuccess;
                 };
-                const int nt = debug || !persistent ? ACC_THREADS
-                                                    : shaft_threads(tiles, only_window >= 0 ? nf / W : nf, ctx->n_sm);
+                const int nt = !persistent ? ACC_THREADS : shaft_threads(tiles, only_window >= 0 ? nf / W : nf, ctx->n_sm);
                 if (nt == 1024) {
-                    GM_TRY_CUDA(few(k_accumulate_shaft<false, false, 1024>, 1024, sizeof(ShaftBlock<1, 1024>)));
+                    GM_TRY_CUDA(few(debug ? k_accumulate_shaft<true, false, 1024> : k_accumulate_shaft<false, false, 1024>,
+                                    1024, sizeof(ShaftBlock<1, 1024>)));
                 } else if (nt == 512) {
-                    GM_TRY_CUDA(few(k_accumulate_shaft<false, false, 512>, 512, sizeof(ShaftBlock<1, 512>)));
+                    GM_TRY_CUDA(few(debug ? k_accumulate_shaft<true, false, 512> : k_accumulate_shaft<false, false, 512>,
+                                    512, sizeof(ShaftBlock<1, 512>)));
                 } else {
                     auto run = [&](auto kern, int threads, int blocks, bool probed) {
                         kern<<<grid(blocks), threads, 0, s>>>(spos, sidx, packed, n_valid, sc->nodes, sc->nodes4,

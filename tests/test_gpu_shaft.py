@@ -170,3 +170,32 @@ def test_blocks_of_wide_tiles(env, n, nf, theta, windows):
     G.gm_samples_free(samples)
     G.gm_scene_free(scene)
     assert a[1:] == b[1:] and a[2] > 0 and np.array_equal(a[0], b[0])
+
+
+@pytest.mark.parametrize("n,nf", [(7000, 100), (7000, 400), (14592, 300), (20000, 6000), (130000, 60), (70000, 200)])
+def test_pair_records_of_every_block_size(env, n, nf):
+    """The recorded pairs (blocks of 512, 1024, 1024, 512 and 256 threads; 256 with wide tiles) are the per-ray walk's:
+    sample, fixation, visibility and weight."""
+    G, ctx = env
+    rng = np.random.default_rng(n)
+    v, f = _scene("mixed" if n == 70000 else "sphere")
+    xyz, tri = _points("mixed" if n == 70000 else "sphere", v, f, n, rng)
+    eye = rng.normal(size=(nf, 3))
+    eye *= 2.5 / np.linalg.norm(eye, axis=1, keepdims=True)
+    at = xyz[rng.integers(0, n, nf)].astype(np.float64)
+    fix = [np.ascontiguousarray(eye, np.float32), np.ascontiguousarray(at - eye, np.float32),
+           rng.uniform(0.1, 0.6, nf).astype(np.float32), np.arange(float(nf))]
+    scene = G.gm_build_scene(ctx, [(v, f, np.eye(4), 0)])
+    samples = G.gm_samples_from_points(scene, xyz, tri)
+    cap, out = 8_000_000, []
+    for flags in (0, G.GM_F_FIX_L1):
+        m = G.gm_accumulate_fixations(scene, samples, *fix, G.make_params(
+            math.radians(0.6), normalize=False, flags=flags | G.GM_F_DEBUG_PAIRS, debug_pair_cap=cap))
+        p = G.gm_map_debug_pairs(m, cap)
+        G.gm_map_free(m)
+        order = np.argsort(p["sample"].astype(np.int64) * (1 << 20) + p["fix"])
+        out.append([p[k][order] for k in ("sample", "fix", "visible", "g")])
+    G.gm_samples_free(samples)
+    G.gm_scene_free(scene)
+    assert 0 < len(out[0][0]) < cap
+    assert all(np.array_equal(a, b) for a, b in zip(*out))
