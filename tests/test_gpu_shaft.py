@@ -3,8 +3,9 @@ scenes: both decide every ray with the same arithmetic and add the weights in th
 maps are equal bit for bit. Sizes at the edges of a warp tile, of a fill step (512 fixations), of a batch
 and of the ranges of the block sizes (456 tiles, 256 fixations, a quarter as many fixations as tiles);
 sample sets of 65536 samples and more, which have tiles of 128 samples where those lie on few triangles,
-with such tiles in the majority and without any; trees of one and two triangles; triangles far smaller
-than the sample spacing (a shaft over its budget); an eye close to the surface, whose rays differ in
+with such tiles in the majority and without any, near a surface, over the budget, reached by few fixations
+and in a posed scene; trees of one and two triangles; triangles far smaller than the sample spacing (a
+shaft over its budget); an eye close to the surface, whose rays differ in
 their dominant axis and cross the planes through the eye."""
 import math
 
@@ -199,3 +200,58 @@ def test_pair_records_of_every_block_size(env, n, nf):
     G.gm_scene_free(scene)
     assert 0 < len(out[0][0]) < cap
     assert all(np.array_equal(a, b) for a, b in zip(*out))
+
+
+def _above(n, rng, lo=0.3, hi=0.6, target=None):
+    """n viewers above the unit floor, gazing at points of it (or at one point)."""
+    eye = np.stack([rng.uniform(0, 1, n), rng.uniform(lo, hi, n), rng.uniform(0, 1, n)], 1)
+    at = np.stack([rng.uniform(0, 1, n), np.zeros(n), rng.uniform(0, 1, n)], 1) if target is None else np.float64(target)
+    return [np.ascontiguousarray(eye, np.float32), np.ascontiguousarray(at - eye, np.float32),
+            rng.uniform(0.1, 0.6, n).astype(np.float32)]
+
+
+def test_wide_tiles_over_the_budget(env):
+    """80k triangles of about 1 mm between the viewers and a floor in wide tiles: shafts run over their budget and
+    their four rays a lane walk the tree one by one."""
+    G, ctx = env
+    rng = np.random.default_rng(8)
+    ball = M.uv_sphere(142, 284, 0.06, 0.05, 30.0, seed=3)
+    v, f, xyz, tri = _floor(70000, (M.translate(ball[0], (0.5, 0.07, 0.5)), ball[1]))
+    fix = [*_above(60, rng, target=(0.52, 0.02, 0.5)), np.arange(60.0)]
+    scene = G.gm_build_scene(ctx, [(v, f, np.eye(4), 0)])
+    samples = G.gm_samples_from_points(scene, xyz, tri)
+    a, b = (_maps(G, scene, samples, fix, math.radians(2.0), flags) for flags in (0, G.GM_F_FIX_L1))
+    G.gm_samples_free(samples)
+    G.gm_scene_free(scene)
+    assert a[1:] == b[1:] and 0 < a[2] < a[1] and np.array_equal(a[0], b[0])
+
+
+def test_wide_tiles_of_a_posed_scene(env):
+    """A floor in wide tiles, turning, below a ball that moves: every window's map is the per-ray walk's."""
+    G, ctx = env
+    rng = np.random.default_rng(9)
+    q = np.array([[0.0, 0.0, 0.0], [1.0, 0.0, 0.0], [1.0, 0.0, 1.0], [0.0, 0.0, 1.0]], np.float32)
+    ball, windows = M.uv_sphere(30, 60, 0.12, 0.1, 8.0, seed=2), 3
+    scene = G.gm_build_scene(ctx, [(q, np.array([[0, 2, 1], [0, 3, 2]], np.uint32), np.eye(4), 0), (*ball, np.eye(4), 1)],
+                             dynamic=True)
+    samples = G.gm_sample_surface(scene, [70000.0, 0.0], 3)
+    poses = np.tile(np.eye(4), (windows, 2, 1, 1))
+    for w in range(windows):
+        a = 0.1 * w
+        poses[w, 0, :3, :3] = [[math.cos(a), 0, math.sin(a)], [0, 1, 0], [-math.sin(a), 0, math.cos(a)]]
+        poses[w, 1, :3, 3] = [0.3 + 0.2 * w, 0.2, 0.5]
+    fix = [*_above(300, rng), np.sort(rng.uniform(0, windows, 300))]
+    prm = dict(t_begin=0.0, t_end=float(windows), window_s=1.0, normalize=False)
+    out = []
+    for flags in (0, G.GM_F_FIX_L1):
+        m = G.gm_accumulate_dynamic(scene, samples, *fix, G.make_params(math.radians(2.0), flags=flags, **prm), poses)
+        W, ns, st, _ = G.gm_map_info(m)
+        values = np.empty((W, ns), np.float32)
+        for w in range(W):
+            G.gm_map_copy(m, w, values[w])
+        G.gm_map_free(m)
+        out.append((values, st["in_cone"], st["visible"]))
+    G.gm_samples_free(samples)
+    G.gm_scene_free(scene)
+    assert out[0][1:] == out[1][1:] and 0 < out[0][2] < out[0][1]
+    assert np.array_equal(out[0][0], out[1][0]) and (out[0][0] > 0).any(1).all()
