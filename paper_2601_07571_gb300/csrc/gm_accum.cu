@@ -180,11 +180,6 @@ __global__ void __launch_bounds__(NT, MINB) k_accumulate(
     warp_stats_commit(st, counters);
 }
 
-// From half of the samples on. Below that what stands before the large triangles is mostly fine, and a wide
-// shaft meets more of it: 10 windows of a cube (an eighth of 300k samples) among objects of 1 cm triangles
-// take 9.4 ms with the cube in wide tiles, 8.0 without.
-__device__ __forceinline__ bool wide_tiles_pay(const uint32_t* lists, uint64_t ns) { return 2ull * 128 * lists[0] >= ns; }
-
 // Whether a set with wide tiles takes blocks of 128 threads: where a wide tile is reached by few fixations, most
 // warps of a larger block wait for its slowest shaft, and twice the tiles in flight help more. The measure is
 // the mean, over SPARSE_TILES tiles of 128 samples spread over the work order, of the fixations that reach the
@@ -244,7 +239,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_accumulate_shaft(
     unsigned char* smem = NT > ACC_THREADS ? dynamic : fixed;
     __shared__ uint32_t s_tile;
     const uint32_t nf = *n_fix_dev;
-    if (lists && wide_tiles_pay(lists, P.ns) != LISTS) return;
+    if (lists && gm_wide_tiles_pay(lists[0], P.ns) != LISTS) return;
     if (LISTS && probed && sparse_tiles(n_fix_dev) != (NT < ACC_THREADS)) return;
     const uint32_t n_wide = LISTS ? lists[0] : 0u;
     const uint32_t n = LISTS ? n_wide + lists[1] : n_tiles;

@@ -3,7 +3,7 @@
 //
 // A session is (scene, samples, fixations); all sessions share the generation parameters. At
 // plan creation every session's fixations are staged into one device buffer and a work list
-// of tiles (session, 32 samples for shafts, else 32*SPT work-order samples) is built on the host: sessions
+// of tiles (session, 32 or 128 samples for shafts, else 32*SPT work-order samples) is built on the host: sessions
 // grouped into three size buckets by triangle count, within a bucket ordered by decreasing cost
 // (fixations per tile, i.e. longest processing time first). The plan then captures into one
 // CUDA graph: the counter resets, the batched fixation prep (window keys per session, one stable
@@ -148,13 +148,21 @@ __global__ void __launch_bounds__(ACC_THREADS, MINB) k_accumulate_batch(const Se
     }
 }
 
-// The default: shafts (gm_shaft.cuh), a block per work item (a 32-sample tile of one session).
+// The default: shafts (gm_shaft.cuh), a block per work item: a 32-sample tile of one session or, with
+// WIDE_ITEM, a tile of 128 samples on few triangles (sessions whose samples lie mostly on such tiles, as in a
+// single call; the plan's host knows them, so a bucket without any keeps the narrow kernel). Four city sessions
+// of 1.7M samples, 5000 fixations of 0.5 degrees: 7.5 ms with per-ray walks, 8.5 with narrow tiles alone,
+// 4.9 so. Blocks of 256 threads throughout: the sessions fill the GPU together (16 of 10k samples: 2.0 ms,
+// 6.5 as single calls, which take larger blocks).
+constexpr uint32_t WIDE_ITEM = 0x80000000u;
+template <bool WIDE>
 __global__ void __launch_bounds__(ACC_THREADS, 4) k_accumulate_batch_shaft(const SessionDev* __restrict__ sess,
                                                                            const uint2* __restrict__ items,
                                                                            uint32_t n_items,
                                                                            unsigned int* __restrict__ work, AccConst C,
                                                                            int* __restrict__ err) {
-    __shared__ ShaftBlock<1> B;
+    constexpr size_t B1 = sizeof(ShaftBlock<1>), B4 = sizeof(ShaftBlock<4>);
+    __shared__ __align__(16) unsigned char smem[WIDE && B4 > B1 ? B4 : B1];
     __shared__ uint32_t s_item;
     const DebugOut dbg{nullptr, nullptr, nullptr, nullptr, nullptr};
     for (;;) {
@@ -175,15 +183,20 @@ __global__ void __launch_bounds__(ACC_THREADS, 4) k_accumulate_batch_shaft(const
         P.dbg_cap = 0;
         P.tanphi = sqrtf(C.K) * 1.00001f;
         TileStats st;
-        shaft_tile<false, 1>(wi.y, Sd.spos, Sd.sidx, Sd.fix, *Sd.n_fix, Sd.nodes, Sd.nodes4, Sd.tris, P, Sd.out, Sd.max_bits,
-                          B, nullptr, dbg, err, st);
+        if (WIDE && (wi.y & WIDE_ITEM))
+            shaft_tile<false, 4>(wi.y & ~WIDE_ITEM, Sd.spos, Sd.sidx, Sd.fix, *Sd.n_fix, Sd.nodes, Sd.nodes4, Sd.tris, P,
+                                 Sd.out, Sd.max_bits, *reinterpret_cast<ShaftBlock<4>*>(smem), nullptr, dbg, err, st);
+        else
+            shaft_tile<false, 1>(wi.y, Sd.spos, Sd.sidx, Sd.fix, *Sd.n_fix, Sd.nodes, Sd.nodes4, Sd.tris, P, Sd.out,
+                                 Sd.max_bits, *reinterpret_cast<ShaftBlock<1>*>(smem), nullptr, dbg, err, st);
         warp_stats_commit(st, Sd.counters);
     }
 }
 
-int batch_shaft_blocks() {   // resident blocks per SM
+int batch_shaft_blocks(bool wide) {   // resident blocks per SM
     int b = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_accumulate_batch_shaft, ACC_THREADS, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, wide ? k_accumulate_batch_shaft<true> : k_accumulate_batch_shaft<false>,
+                                                  ACC_THREADS, 0);
     return std::max(b, 1);
 }
 
@@ -214,12 +227,14 @@ int occupancy_of() {
 // Variant codes: bits 0-2 the kernel (ray queue, 4-wide tree, 64-register cap), 8 x the tile index
 // (ray-queue binary tree only: 2 samples per thread with fixations staged in shared memory; with 1,
 // the rays are traced as shafts).
-void launch_batch(int code, int grid, cudaStream_t s, const SessionDev* sess, const uint2* items, uint32_t n_items,
+// wide: the work items (of shafts) include wide tiles
+void launch_batch(int code, bool wide, int grid, cudaStream_t s, const SessionDev* sess, const uint2* items, uint32_t n_items,
                   unsigned int* work, AccConst C, int* err) {
 #define GM_B(Cm, Wd, Mb, S_, Fs) \
     k_accumulate_batch<Cm, Wd, Mb, S_, Fs><<<grid, ACC_THREADS, 0, s>>>(sess, items, n_items, work, C, err)
     const int t = code >> 3;
-    if (t == 2) k_accumulate_batch_shaft<<<grid, ACC_THREADS, 0, s>>>(sess, items, n_items, work, C, err);
+    if (t == 2 && wide) k_accumulate_batch_shaft<true><<<grid, ACC_THREADS, 0, s>>>(sess, items, n_items, work, C, err);
+    else if (t == 2) k_accumulate_batch_shaft<false><<<grid, ACC_THREADS, 0, s>>>(sess, items, n_items, work, C, err);
     else if (t == 1 && (code & 7) == 5) GM_B(true, false, 4, 2, true);
     else if (t == 1) GM_B(true, false, 3, 2, true);
     else switch (code & 7) {
@@ -235,9 +250,9 @@ void launch_batch(int code, int grid, cudaStream_t s, const SessionDev* sess, co
 #undef GM_B
 }
 
-int batch_occupancy(int code) {
+int batch_occupancy(int code, bool wide) {
     const int t = code >> 3;
-    if (t == 2) return batch_shaft_blocks();
+    if (t == 2) return batch_shaft_blocks(wide);
     if (t == 1) return (code & 7) == 5 ? occupancy_of<true, false, 4, 2, true>() : occupancy_of<true, false, 3, 2, true>();
     switch (code & 7) {
         case 0: return occupancy_of<false, false, 3>();
@@ -343,6 +358,7 @@ struct gm_batch {
     // own kernel variant and its own persistent launch, timed by events recorded in the graph
     uint32_t bucket_begin[BATCH_TILES][BATCH_BUCKETS + 1] = {};
     uint32_t bucket_sessions[BATCH_BUCKETS] = {};
+    bool wide[BATCH_BUCKETS] = {};             // some session's shafts take wide tiles
     int bflags[BATCH_BUCKETS] = {};
     cudaEvent_t bev[BATCH_BUCKETS][2] = {};
     cudaStream_t bs[BATCH_BUCKETS] = {};       // capture-time fork streams of the bucket launches
@@ -420,12 +436,12 @@ static gm_status batch_capture(gm_batch* b, bool concurrent = true) {
                 const uint32_t i0 = b->bucket_begin[tk][k], i1 = b->bucket_begin[tk][k + 1];
                 cudaStream_t ks = concurrent ? b->bs[k] : cs;
                 if (i1 > i0) {
-                    const int grid = (int)std::min<uint64_t>((uint64_t)b->ctx->n_sm * batch_occupancy(code),
+                    const int grid = (int)std::min<uint64_t>((uint64_t)b->ctx->n_sm * batch_occupancy(code, b->wide[k]),
                                                              tk == 2 ? i1 - i0 : gm_div_up(i1 - i0, ACC_THREADS / 32));
                     // external event records: the graph records them when it runs (a plain record in
                     // a capture only orders the work)
                     cudaEventRecordWithFlags(b->bev[k][0], ks, cudaEventRecordExternal);
-                    launch_batch(code, grid, ks, b->sess, b->items[tk] + i0, i1 - i0, b->work + k, C, b->ctx->dev_err);
+                    launch_batch(code, b->wide[k], grid, ks, b->sess, b->items[tk] + i0, i1 - i0, b->work + k, C, b->ctx->dev_err);
                     cudaEventRecordWithFlags(b->bev[k][1], ks, cudaEventRecordExternal);
                     ++launches;
                 }
@@ -604,6 +620,26 @@ extern "C" gm_status gm_batch_create(gm_ctx* ctx, const gm_session_desc* ss, uin
         return ba != bc ? ba < bc : ss[a].fix.n > ss[c].fix.n;
     });
     for (uint32_t i : order) ++b->bucket_sessions[bucket_of_tris(ss[i].scene->n_tris)];
+    // the tile lists of the sessions whose shafts take wide tiles (the others' stay empty)
+    std::vector<std::vector<uint32_t>> lists(n);
+    for (uint32_t i = 0; i < n; ++i) {
+        const gm_samples* sm = ss[i].samples;
+        if (!sm->tile_lists) continue;
+        uint32_t cnt[2] = {0, 0};
+        if ((e = cudaMemcpyAsync(cnt, sm->tile_lists, sizeof(cnt), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+            (e = cudaStreamSynchronize(s)) != cudaSuccess)
+            return fail(gm_cuda_error(e, "gm_batch_create: tile lists"));
+        if (!gm_wide_tiles_pay(cnt[0], sm->n)) continue;
+        lists[i].resize((size_t)cnt[0] + cnt[1]);
+        if ((e = cudaMemcpyAsync(lists[i].data(), sm->tile_lists + 2, sizeof(uint32_t) * cnt[0], cudaMemcpyDeviceToHost, s)) !=
+                cudaSuccess ||
+            (e = cudaMemcpyAsync(lists[i].data() + cnt[0], sm->tile_lists + gm_tile_list_fine(sm->n), sizeof(uint32_t) * cnt[1],
+                                 cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+            (e = cudaStreamSynchronize(s)) != cudaSuccess)
+            return fail(gm_cuda_error(e, "gm_batch_create: tile lists"));
+        for (uint32_t t = 0; t < cnt[0]; ++t) lists[i][t] |= WIDE_ITEM;
+        b->wide[bucket_of_tris(ss[i].scene->n_tris)] = true;
+    }
     std::vector<uint2> items[BATCH_TILES];
     for (int tk = 0; tk < BATCH_TILES; ++tk) {
         const uint64_t per_tile = 32ull * BATCH_TILE_SPT[tk] * BATCH_GROUP;
@@ -611,7 +647,10 @@ extern "C" gm_status gm_batch_create(gm_ctx* ctx, const gm_session_desc* ss, uin
             const int k = bucket_of_tris(ss[i].scene->n_tris);
             const uint32_t tiles = tk == 2 ? gm_div_up(ss[i].samples->n, 32)
                                            : (uint32_t)(gm_div_up(ss[i].samples->n, per_tile) * BATCH_GROUP);
-            for (uint32_t t = 0; t < tiles; ++t) items[tk].push_back(make_uint2(i, t));
+            if (tk == 2 && !lists[i].empty())
+                for (const uint32_t t : lists[i]) items[tk].push_back(make_uint2(i, t));
+            else
+                for (uint32_t t = 0; t < tiles; ++t) items[tk].push_back(make_uint2(i, t));
             for (int q = k + 1; q <= BATCH_BUCKETS; ++q) b->bucket_begin[tk][q] = (uint32_t)items[tk].size();
         }
         b->n_items[tk] = (uint32_t)items[tk].size();

@@ -82,6 +82,11 @@ struct gm_samples {
 constexpr uint64_t GM_TILE_LIST_MIN = 1u << 16;
 // Where the list of 32-sample tiles starts in gm_samples::tile_lists.
 __host__ __device__ inline size_t gm_tile_list_fine(uint64_t n) { return 2 + (size_t)((n + 127) / 128); }
+// Whether n samples of which n_wide tiles of 128 lie on few triangles are traced in wide tiles: from half of
+// the samples on. Below that what stands before the large triangles is mostly fine, and a wide shaft meets
+// more of it: 10 windows of a cube (an eighth of 300k samples) among objects of 1 cm triangles take 9.4 ms
+// with the cube in wide tiles, 8.0 without.
+__host__ __device__ inline bool gm_wide_tiles_pay(uint32_t n_wide, uint64_t n) { return 2ull * 128 * n_wide >= n; }
 
 struct gm_map {
     gm_ctx* ctx = nullptr;

@@ -240,3 +240,48 @@ def test_tuning_file_of_other_kernels_is_timed_again(env, tmp_path):
     assert float(times[0][1]) > 0.0 and float(times[1][1]) == 0.0 and times[0][0] == times[1][0]
     text = path.read_text()
     assert '"plain:1:2:1": %d' % G.GM_F_NO_COMPACT in text and ':plain:1:2:1": %s' % times[0][0] in text
+
+
+def test_sessions_in_wide_tiles(env):
+    """Sessions of 65536 samples and more on few triangles are traced in tiles of 128 samples, as a single call does,
+    beside sessions that are not: each map is its single call's, also after the plan is tuned."""
+    import math
+    G, pipe, ctx = env
+    from synth import meshes as M
+    rng = np.random.default_rng(2)
+    q = np.array([[0.0, 0.0, 0.0], [1.0, 0.0, 0.0], [1.0, 0.0, 1.0], [0.0, 0.0, 1.0]], np.float32)
+    floor, ball = (q, np.array([[0, 2, 1], [0, 3, 2]], np.uint32)), M.uv_sphere(40, 80, 0.15, 0.1, 8.0, seed=2)
+    above = M.translate(ball[0], (0.5, 0.3, 0.5))
+    sess = []
+    for meshes, density in (((floor, (above, ball[1])), [70000.0, 9000.0]), ((ball,), [2000.0]), ((floor,), [66000.0])):
+        sc = G.gm_build_scene(ctx, [(v, f, np.eye(4), i) for i, (v, f) in enumerate(meshes)])
+        sm = G.gm_sample_surface(sc, density, 4)
+        n = 120
+        eye = np.stack([rng.uniform(0, 1, n), rng.uniform(0.5, 0.9, n), rng.uniform(0, 1, n)], 1)
+        gaze = np.stack([rng.uniform(0, 1, n), np.zeros(n), rng.uniform(0, 1, n)], 1) - eye
+        sess.append((sc, sm, np.ascontiguousarray(eye, np.float32), np.ascontiguousarray(gaze, np.float32),
+                     rng.uniform(0.1, 0.6, n).astype(np.float32), np.sort(rng.uniform(0, 3, n))))
+    prm = G.make_params(math.radians(2.0), t_begin=0.0, t_end=3.0, window_s=1.0)
+
+    def maps(m):
+        W, ns, st, _ = G.gm_map_info(m)
+        out = np.empty((W, ns), np.float32)
+        for w in range(W):
+            G.gm_map_copy(m, w, out[w])
+        return out, st["in_cone"], st["visible"]
+
+    plan = G.gm_batch_create(ctx, sess, prm)
+    for tuned in (False, True):
+        if tuned:
+            G.gm_batch_autotune(plan)
+        G.gm_batch_run(plan)
+        G.gm_sync(ctx)
+        for i, s in enumerate(sess):
+            m = G.gm_accumulate_fixations(*s, prm)
+            one, many = maps(m), maps(G.gm_batch_map(plan, i))
+            G.gm_map_free(m)
+            assert one[1:] == many[1:] and one[2] > 0 and np.array_equal(one[0], many[0])
+    G.gm_batch_free(plan)
+    for sc, sm, *_ in sess:
+        G.gm_samples_free(sm)
+        G.gm_scene_free(sc)
