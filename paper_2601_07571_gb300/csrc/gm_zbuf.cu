@@ -31,6 +31,7 @@ namespace {
 
 constexpr int ZB_THREADS = 256;
 constexpr int ZB_SMEM_FRUSTA = 64;            // frusta staged per pass of the cull kernel
+constexpr int ZB_MIXED_PIXELS = 128;          // larger pixel boxes are drawn one at a time by their warp
 constexpr int ZB_BIG_PIXELS = 1024;           // larger pixel boxes go to the block rasteriser
 constexpr int ZB_LANE_PIXELS = 32;            // clipped pairs: larger ones go to the warp
                                               // (through a list of zb_big_cap pairs)
@@ -324,19 +325,48 @@ __device__ __forceinline__ void draw_poly(const ClipPoly& P, int x0, int y0, int
     for (int t = 1; t + 1 < P.n; ++t) {
         float4 e0, e1, e2, iw;
         fan_tri(P, t, e0, e1, e2, iw);
+        int row = first / wd, col = first - row * wd;
+        const int rows = step / wd, cols = step - rows * wd;
         for (int k = first; k < n; k += step) {
-            const int px = x0 + k % wd, py = y0 + k / wd;
+            const int px = x0 + col, py = y0 + row;
             shade_tri(e0, e1, e2, iw, px + 0.5f, py + 0.5f, near_m, far_m, zb + (size_t)py * res + px);
+            row += rows;
+            col += cols;
+            if (col >= wd) col -= wd, ++row;
         }
+    }
+}
+
+// The block draws a box, a warp on a row: 32 x 8 pixels at a time.
+__device__ __forceinline__ void draw_rows(const float4 e0, const float4 e1, const float4 e2, const float4 iw, int x0, int x1,
+                                          int y0, int y1, float near_m, float far_m, uint32_t res,
+                                          uint32_t* __restrict__ zb) {
+    for (int py = y0 + (int)(threadIdx.x >> 5); py <= y1; py += ZB_THREADS / 32)
+        for (int px = x0 + (int)(threadIdx.x & 31); px <= x1; px += 32)
+            shade_tri(e0, e1, e2, iw, px + 0.5f, py + 0.5f, near_m, far_m, zb + (size_t)py * res + px);
+}
+
+// The block draws a pair that reaches the near plane.
+__device__ __noinline__ void draw_rows_clipped(const ZbFrustum& F, const float4* __restrict__ v, uint32_t res,
+                                               uint32_t* __restrict__ zb) {
+    ClipPoly P;
+    clip_project(F, v[0], v[1], v[2], P);
+    if (P.n < 3) return;
+    int x0, x1, y0, y1;
+    poly_bbox(P, (int)res, x0, x1, y0, y1);
+    for (int t = 1; t + 1 < P.n; ++t) {
+        float4 e0, e1, e2, iw;
+        fan_tri(P, t, e0, e1, e2, iw);
+        draw_rows(e0, e1, e2, iw, x0, x1, y0, y1, F.n, F.f, res, zb);
     }
 }
 
 // The pairs of a warp's entries that its shared pixels leave out: boxes above ZB_BIG_PIXELS, for the block
 // rasteriser, and pairs that reach the near plane (`clip`). Those are clipped first; a floor or wall that
 // passes the viewer fills the whole window, so they too go to the block rasteriser, to the warp (above
-// ZB_LANE_PIXELS, and what finds the list full) or to their lane by the size of their box. (Out of line: few warps come here, and its
-// registers are its own.) 12 triangles of a room and 60k of objects in it, 2000 fixations at 256 x 256:
-// 165 ms with every clipped pair drawn by its lane, 1.8 so.
+// ZB_LANE_PIXELS, and what finds the list full) or to their lane by the size of their box. (Out of line: few
+// warps come here, and its registers are its own.) 12 triangles of a room and 60k of objects in it, 2000
+// fixations at 256 x 256: 165 ms with every clipped pair drawn by its lane, 1.8 so.
 __device__ __noinline__ void draw_others(const ZbFrustum* sF, const float4* __restrict__ tris, const int entry,
                                          const bool clip, int npx, const uint32_t f0, const uint32_t slot0,
                                          const uint32_t res, uint32_t* __restrict__ zbuf, PairFT* __restrict__ big,
@@ -380,9 +410,14 @@ __device__ __noinline__ void draw_others(const ZbFrustum* sF, const float4* __re
 // counts: [0] pairs kept, [1] entries of `big`. A warp's pairs stay in its own queue and its own slots:
 // no pair list in memory, no host read of its length. The blocks of one blockIdx.y (one group of
 // ZB_SMEM_FRUSTA fixations) run together, so the atomics stay on a few z-buffers that fit in L2.
-// Before: culling into a pair list, then a thread per pair over its pixel box (lanes waited for the
-// largest box; the clipped polygon, indexed at run time, sat in local memory) and a warp per pair above
-// 64 pixels. 300k triangles, 2000 fixations at 256 x 256, 32M pairs: cull, raster and warp raster 6.2 ms, this kernel 3.8 ms.
+// Small boxes share the warp's lanes evenly; above ZB_MIXED_PIXELS finding each pixel's box costs more than the
+// lanes that a box of its own leaves idle in its last turn.
+// 300k triangles, 2000 fixations at 256 x 256, 32M pairs: 6.2 ms as culling into a pair list, a thread per pair
+// over its pixel box (lanes waited for the largest box; the clipped polygon, indexed at run time, sat in local
+// memory) and a warp per pair above 64 pixels; 3.8 ms with all boxes up to 1024 pixels mixed, 3.4 above 128
+// one at a time. The same calls, ms, with 128 / 256 / 512 / 1024: 4.60 / - / - / 5.01; 1000 fixations on 20k
+// triangles 3.37 / 3.47 / 3.68 / 4.01; 100k triangles, 500 fixations of 0.25 degrees 1.41 / 1.42 / 1.48 / 1.75
+// (1.68 with the three kernels).
 __global__ void __launch_bounds__(ZB_THREADS, 4) k_zb_draw(const float4* __restrict__ tris, uint32_t nt,
                                                            const ZbFrustum* __restrict__ frusta, uint32_t nfix,
                                                            uint32_t res, float near_m, float far_m,
@@ -465,25 +500,25 @@ __global__ void __launch_bounds__(ZB_THREADS, 4) k_zb_draw(const float4* __restr
                       fmax3(P.v[0], P.v[1], P.v[2]), (int)res, x0, x1, y0, y1);
         }
         const int npx = lane < cnt && front && x1 >= x0 && y1 >= y0 ? (x1 - x0 + 1) * (y1 - y0 + 1) : 0;
-        const bool small = npx > 0 && npx <= ZB_BIG_PIXELS;
-        int incl = small ? npx : 0;
+        const bool small = npx > 0 && npx <= ZB_BIG_PIXELS, mixed = npx > 0 && npx <= ZB_MIXED_PIXELS;
+        int incl = mixed ? npx : 0;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int u = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += u;
         }
         const int total = __shfl_sync(0xffffffffu, incl, 31);
-        const int start = small ? incl - npx : 0x7fffffff;
-        const unsigned sm = __ballot_sync(0xffffffffu, small);
+        const int start = mixed ? incl - npx : 0x7fffffff;
+        const unsigned sm = __ballot_sync(0xffffffffu, small), mx = __ballot_sync(0xffffffffu, mixed);
         if (small) {
             ZbTri T;
             T.e0 = canonical_edge(P.u[1], P.v[1], P.u[2], P.v[2]);
             T.e1 = canonical_edge(P.u[2], P.v[2], P.u[0], P.v[0]);
             T.e2 = canonical_edge(P.u[0], P.v[0], P.u[1], P.v[1]);
-            T.iw = make_float4(P.iw[0], P.iw[1], P.iw[2], __int_as_float((x1 - x0 + 1) | start << 16));
+            T.iw = make_float4(P.iw[0], P.iw[1], P.iw[2], __int_as_float((x1 - x0 + 1) | (mixed ? start << 16 : 0)));
             T.centre = make_float2(x0 + 0.5f, y0 + 0.5f);
             T.z = zbuf + ((size_t)fix * res + y0) * res + x0;
-            S[__popc(sm & lt)] = T;
+            S[mixed ? __popc(mx & lt) : __popc(mx) + __popc(sm & ~mx & lt)] = T;
         }
         __syncwarp();
         // the pixels of all boxes in turn, 32 at a time: the boxes that start in this window, as bits,
@@ -503,6 +538,23 @@ __global__ void __launch_bounds__(ZB_THREADS, 4) k_zb_draw(const float4* __restr
                 const float2 first = S[k].centre;
                 shade_tri(S[k].e0, S[k].e1, S[k].e2, iws, first.x + (float)col, first.y + (float)row, near_m, far_m,
                           S[k].z + (row * (int)res + col));
+            }
+        }
+        // boxes of more than ZB_MIXED_PIXELS, one after another
+        unsigned one = __ballot_sync(0xffffffffu, npx > ZB_MIXED_PIXELS && npx <= ZB_BIG_PIXELS);
+        for (int k = boxes; one; ++k) {   // (their slots follow)
+            const int n = __shfl_sync(0xffffffffu, npx, __ffs(one) - 1);
+            one &= one - 1u;
+            const float4 q0 = S[k].e0, q1 = S[k].e1, q2 = S[k].e2, iws = S[k].iw;
+            const int wd = __float_as_int(iws.w), rows = 32 / wd, cols = 32 - rows * wd;
+            const float2 first = S[k].centre;
+            uint32_t* z = S[k].z;
+            int row = lane / wd, col = lane - row * wd;
+            for (int g = lane; g < n; g += 32) {
+                shade_tri(q0, q1, q2, iws, first.x + (float)col, first.y + (float)row, near_m, far_m, z + (row * (int)res + col));
+                row += rows;
+                col += cols;
+                if (col >= wd) col -= wd, ++row;
             }
         }
         __syncwarp();
@@ -528,75 +580,90 @@ __global__ void __launch_bounds__(ZB_THREADS, 4) k_zb_draw(const float4* __restr
             if (lane == 0) sMask[k >> 5] = bits;
         }
         __syncthreads();
-        // the frusta that reach the warp's sphere, a frustum per lane
+        // the frusta that reach the warp's sphere, a frustum per lane; the last turn draws what is queued (one call
+        // of `draw`: twice in line it is slower)
         int qn = 0;
 #pragma unroll 1
-        for (int h = 0; h < ZB_SMEM_FRUSTA / 32; ++h) {
-            const unsigned blk = sMask[h];
-            if (blk == 0) continue;
+        for (int h = 0; h <= ZB_SMEM_FRUSTA / 32; ++h) {
+            const bool last = h == ZB_SMEM_FRUSTA / 32;
+            const unsigned blk = last ? 0u : sMask[h];
             const bool reach = ((blk >> lane) & 1u) && wbox && !sphere_outside(sF[32 * h + lane], wx, wy, wz, wR, R);
-            unsigned todo = __ballot_sync(0xffffffffu, reach);
+            unsigned todo = last ? (unsigned)qn : __ballot_sync(0xffffffffu, reach);
             while (todo) {
-                const int k = 32 * h + __ffs(todo) - 1;
-                todo &= todo - 1u;
-                const ZbFrustum& F = sF[k];
-                bool keep = false;
-                if (valid) {
-                    float x[3], y[3], w[3];
-                    to_camera(F, a.x, a.y, a.z, x[0], y[0], w[0]);
-                    to_camera(F, b.x, b.y, b.z, x[1], y[1], w[1]);
-                    to_camera(F, c.x, c.y, c.z, x[2], y[2], w[2]);
-                    int o0 = 0, o1 = 0, o2 = 0, o3 = 0, o4 = 0, o5 = 0;
+                int cnt = qn;
+                if (last) {
+                    todo = 0;
+                } else {
+                    const int k = 32 * h + __ffs(todo) - 1;
+                    todo &= todo - 1u;
+                    const ZbFrustum& F = sF[k];
+                    bool keep = false;
+                    if (valid) {
+                        float x[3], y[3], w[3];
+                        to_camera(F, a.x, a.y, a.z, x[0], y[0], w[0]);
+                        to_camera(F, b.x, b.y, b.z, x[1], y[1], w[1]);
+                        to_camera(F, c.x, c.y, c.z, x[2], y[2], w[2]);
+                        int o0 = 0, o1 = 0, o2 = 0, o3 = 0, o4 = 0, o5 = 0;
 #pragma unroll
-                    for (int v = 0; v < 3; ++v) {
-                        const float U = fmaf(F.sx, x[v], F.ox * w[v]), V = fmaf(F.sy, y[v], F.oy * w[v]);
-                        o0 += U < -w[v];
-                        o1 += U > (R + 1.f) * w[v];
-                        o2 += V < -w[v];
-                        o3 += V > (R + 1.f) * w[v];
-                        o4 += w[v] < F.n * (1.f - 1e-5f);
-                        o5 += w[v] > F.f * (1.f + 1e-5f);
+                        for (int v = 0; v < 3; ++v) {
+                            const float U = fmaf(F.sx, x[v], F.ox * w[v]), V = fmaf(F.sy, y[v], F.oy * w[v]);
+                            o0 += U < -w[v];
+                            o1 += U > (R + 1.f) * w[v];
+                            o2 += V < -w[v];
+                            o3 += V > (R + 1.f) * w[v];
+                            o4 += w[v] < F.n * (1.f - 1e-5f);
+                            o5 += w[v] > F.f * (1.f + 1e-5f);
+                        }
+                        keep = o0 < 3 && o1 < 3 && o2 < 3 && o3 < 3 && o4 < 3 && o5 < 3;
                     }
-                    keep = o0 < 3 && o1 < 3 && o2 < 3 && o3 < 3 && o4 < 3 && o5 < 3;
+                    const unsigned msk = __ballot_sync(0xffffffffu, keep);
+                    if (keep) queue[warp][qn + __popc(msk & lt)] = (uint16_t)(k << 5 | lane);
+                    qn += __popc(msk);
+                    n_pairs += __popc(msk);
+                    __syncwarp();
+                    if (qn < 32) continue;
+                    cnt = 32;
                 }
-                const unsigned msk = __ballot_sync(0xffffffffu, keep);
-                if (keep) queue[warp][qn + __popc(msk & lt)] = (uint16_t)(k << 5 | lane);
-                qn += __popc(msk);
-                n_pairs += __popc(msk);
-                __syncwarp();
-                if (qn >= 32) {
-                    qn -= 32;
-                    draw(qn, 32, f0);
-                }
+                qn -= cnt;
+                draw(qn, cnt, f0);
             }
         }
-        if (qn > 0) draw(0, qn, f0);
     }
     if (lane == 0 && n_pairs) atomicAdd(&counts[0], n_pairs);
 }
 
-__global__ void __launch_bounds__(ZB_THREADS) k_zb_draw_big(const unsigned long long* __restrict__ counts,
-                                                            const PairFT* __restrict__ big, uint64_t cap,
-                                                            const ZbFrustum* __restrict__ frusta,
-                                                            const float4* __restrict__ tris, uint32_t res,
-                                                            uint32_t* __restrict__ zbuf) {
+__global__ void __launch_bounds__(ZB_THREADS, 6) k_zb_draw_big(const unsigned long long* __restrict__ counts,
+                                                               const PairFT* __restrict__ big, uint64_t cap,
+                                                               const ZbFrustum* __restrict__ frusta,
+                                                               const float4* __restrict__ tris, uint32_t res,
+                                                               float near_m, float far_m, uint32_t* __restrict__ zbuf) {
     const unsigned long long n = min(counts[1], (unsigned long long)cap);
     for (unsigned long long q = blockIdx.x; q < n; q += gridDim.x) {
         const PairFT pr = big[q];
-        const ZbFrustum F = frusta[pr.fix];
+        const ZbFrustum& F = frusta[pr.fix];
+        const float4* v = tris + 3 * (size_t)pr.tri;
         uint32_t* zb = zbuf + (size_t)pr.fix * res * res;
-        ClipPoly P;
-        clip_project(F, tris[3 * (size_t)pr.tri], tris[3 * (size_t)pr.tri + 1], tris[3 * (size_t)pr.tri + 2], P);
-        int x0, x1, y0, y1;
-        poly_bbox(P, (int)res, x0, x1, y0, y1);
-        for (int t = 1; t + 1 < P.n; ++t) {
-            float4 e0, e1, e2, iw;
-            fan_tri(P, t, e0, e1, e2, iw);
-            // 32 x 8 pixels at a time: a warp on a row
-            for (int py = y0 + (int)(threadIdx.x >> 5); py <= y1; py += ZB_THREADS / 32)
-                for (int px = x0 + (int)(threadIdx.x & 31); px <= x1; px += 32)
-                    shade_tri(e0, e1, e2, iw, px + 0.5f, py + 0.5f, F.n, F.f, zb + (size_t)py * res + px);
+        float pu[3], pv[3], iw[3];
+        bool front = true;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            float x, y, w;
+            to_camera(F, v[k].x, v[k].y, v[k].z, x, y, w);
+            front = front && w >= F.n;
+            iw[k] = 1.0f / w;
+            pu[k] = fmaf(F.sx, x * iw[k], F.ox);
+            pv[k] = fmaf(F.sy, y * iw[k], F.oy);
         }
+        if (!front) {
+            draw_rows_clipped(F, v, res, zb);
+            continue;
+        }
+        int x0, x1, y0, y1;
+        pixel_box(fmin3(pu[0], pu[1], pu[2]), fmax3(pu[0], pu[1], pu[2]), fmin3(pv[0], pv[1], pv[2]),
+                  fmax3(pv[0], pv[1], pv[2]), (int)res, x0, x1, y0, y1);
+        draw_rows(canonical_edge(pu[1], pv[1], pu[2], pv[2]), canonical_edge(pu[2], pv[2], pu[0], pv[0]),
+                  canonical_edge(pu[0], pv[0], pu[1], pv[1]), make_float4(iw[0], iw[1], iw[2], 0.f), x0, x1, y0, y1, near_m,
+                  far_m, res, zb);
     }
 }
 
@@ -785,7 +852,8 @@ gm_status render_zbuffers(gm_ctx* ctx, gm_scene* sc, const ZbFrustum* frusta, ui
     const dim3 grid(gm_div_up(sc->n_tris, ZB_THREADS), std::min<uint32_t>(gm_div_up(nfix, ZB_SMEM_FRUSTA), 65535));
     k_zb_draw<<<grid, ZB_THREADS, 0, s>>>(sc->bvh_tris, sc->n_tris, frusta, nfix, res, near_m, far_m, zbuf, big, cap,
                                           counts);
-    k_zb_draw_big<<<(uint32_t)ctx->n_sm * 4, ZB_THREADS, 0, s>>>(counts, big, cap, frusta, sc->bvh_tris, res, zbuf);
+    k_zb_draw_big<<<(uint32_t)ctx->n_sm * 6, ZB_THREADS, 0, s>>>(counts, big, cap, frusta, sc->bvh_tris, res, near_m,
+                                                               far_m, zbuf);
     *launches += 2;
     GM_TRY_CUDA(cudaGetLastError());
     return GM_OK;

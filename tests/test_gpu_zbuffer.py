@@ -335,3 +335,38 @@ def test_full_list_of_large_pairs(env):
     assert out[0][1] == out[1][1] > n * res * res // 64
     # the cones cover about 0.9 m2 of the nearest wall: 27 samples at 30 a m2
     assert np.array_equal(out[0][0], out[1][0]) and (out[0][0] > 0).sum() > 10
+
+
+@pytest.mark.parametrize("res", [16, 33, 96])
+def test_boxes_of_every_size_against_oracle(env, res):
+    """Triangles whose pixel boxes run from under one pixel to the whole window, as squarish, wide and tall boxes (those
+    are drawn mixed with others, one at a time or by a block: the lines lie at 128 and 1024 pixels), some clipped at the
+    near plane: depths against the oracle."""
+    G, pipe, ctx = env
+    rng = np.random.default_rng(res)
+    theta, zb = f32(math.radians(2.0)), oracle.ZBuffer(res=res, near=f32(0.05), far=100.0)
+    half = 4.0 * math.tan(theta) * 2.0      # of the window, 2 m before the eye
+    tri = []
+    for k in range(200):
+        w, h = half * np.exp(rng.uniform(math.log(0.01), math.log(2.0), 2))
+        c = np.array([rng.uniform(-half, half), rng.uniform(-half, half), 2.0 + 0.002 * k])
+        p = c + np.array([[-w, -h, 0], [w, -0.3 * h, 0.1 * w], [-0.2 * w, h, -0.1 * h]])
+        if k % 20 == 0:
+            p[1] = [0.02, -0.03, -0.4]      # behind the eye
+        tri.append(p)
+    v, f = np.array(tri, np.float32).reshape(-1, 3), np.arange(600, dtype=np.uint32).reshape(-1, 3)
+    eye = np.float32([[0, 0, 0], [0.01, -0.02, 0], [-0.03, 0.01, 0.02]])
+    gaze, up = np.float32([[0, 0, 1], [0.01, 0.01, 1], [0, -0.02, 1]]), np.tile(np.float32([0, 1, 0]), (3, 1))
+    sc = G.gm_build_scene(ctx, [(v, f, np.eye(4), 0)])
+    z, _ = G.gm_zbuffer_render(sc, eye, gaze, theta, 4.0, G.zbuffer_params(zb.res, zb.near, zb.far), gaze, up)
+    G.gm_scene_free(sc)
+    world, sure_px = v[f.astype(np.int64)].astype(np.float64), 0
+    for i in range(3):
+        F = oracle.zb_frustum(eye[i], gaze[i], gaze[i], up[i], theta, 4.0, zb.near, zb.far)
+        zo, amb = oracle.zb_render(world, F, res, delta_px=DPX)
+        zg, sure = z[i].astype(np.float64), ~amb
+        assert np.array_equal(np.isinf(zg[sure]), np.isinf(zo[sure]))
+        fin = sure & np.isfinite(zo)
+        assert np.all(np.abs(zg[fin] - zo[fin]) <= 1e-4 * zo[fin])
+        sure_px += int(fin.sum())
+    assert sure_px > 0.5 * 3 * res ** 2
