@@ -79,7 +79,13 @@ struct gm_samples {
     uint32_t* tile_lists = nullptr;
 };
 
-constexpr uint64_t GM_TILE_LIST_MIN = 1u << 16;
+// Smaller sets have too few tiles of 128 samples for 608 blocks: the longest decide. With wide tiles / without,
+// us, per-ray walks in brackets, for a room of 12 triangles with 60k of objects in it: 70k samples x 400
+// fixations 352 / 202 (206), 200k x 1000 448 / 374 (420), 300k x 3000 553 / 519, 500k x 5000 771 / 909, 1.5M x
+// 3000 998 / 1261; a city of 200k triangles: 200k x 1000 291 / 285, 500k x 1000 448 / 483, 1.5M x 3000
+// 1616 / 2091; a sphere of 3000: 130k x 1000 587 / 485, 300k x 3000 2516 / 2302, 500k x 5000 5380 / 5589,
+// 1.5M x 3000 7041 / 8731.
+constexpr uint64_t GM_TILE_LIST_MIN = 3u << 17;
 // Where the list of 32-sample tiles starts in gm_samples::tile_lists.
 __host__ __device__ inline size_t gm_tile_list_fine(uint64_t n) { return 2 + (size_t)((n + 127) / 128); }
 // Whether n samples of which n_wide tiles of 128 lie on few triangles are traced in wide tiles: from half of

@@ -243,7 +243,7 @@ def test_tuning_file_of_other_kernels_is_timed_again(env, tmp_path):
 
 
 def test_sessions_in_wide_tiles(env):
-    """Sessions of 65536 samples and more on few triangles are traced in tiles of 128 samples, as a single call does,
+    """Sessions of 393216 samples and more on few triangles are traced in tiles of 128 samples, as a single call does,
     beside sessions that are not: each map is its single call's, also after the plan is tuned."""
     import math
     G, pipe, ctx = env
@@ -253,7 +253,7 @@ def test_sessions_in_wide_tiles(env):
     floor, ball = (q, np.array([[0, 2, 1], [0, 3, 2]], np.uint32)), M.uv_sphere(40, 80, 0.15, 0.1, 8.0, seed=2)
     above = M.translate(ball[0], (0.5, 0.3, 0.5))
     sess = []
-    for meshes, density in (((floor, (above, ball[1])), [70000.0, 9000.0]), ((ball,), [2000.0]), ((floor,), [66000.0])):
+    for meshes, density in (((floor, (above, ball[1])), [400000.0, 9000.0]), ((ball,), [2000.0]), ((floor,), [394000.0])):
         sc = G.gm_build_scene(ctx, [(v, f, np.eye(4), i) for i, (v, f) in enumerate(meshes)])
         sm = G.gm_sample_surface(sc, density, 4)
         n = 120

@@ -2,7 +2,7 @@
 scenes: both decide every ray with the same arithmetic and add the weights in the same order, so the
 maps are equal bit for bit. Sizes at the edges of a warp tile, of a fill step (512 fixations), of a batch
 and of the ranges of the block sizes (456 tiles, 256 fixations, a quarter as many fixations as tiles);
-sample sets of 65536 samples and more, which have tiles of 128 samples where those lie on few triangles,
+sample sets of 393216 samples and more, which have tiles of 128 samples where those lie on few triangles,
 with such tiles in the majority and without any, near a surface, over the budget, reached by few fixations
 and in a posed scene; trees of one and two triangles; triangles far smaller than the sample spacing (a
 shaft over its budget); an eye close to the surface, whose rays differ in
@@ -61,7 +61,8 @@ def _points(kind, v, f, n, rng):
     ("sphere", 14592, 255, 2.0, False, 1), ("sphere", 14592, 256, 2.0, False, 2), ("sphere", 14624, 256, 2.0, False, 1),
     ("sphere", 32768, 256, 2.0, False, 1), ("sphere", 32769, 256, 2.0, False, 1),
     ("mixed", 65537, 300, 2.0, False, 1), ("mixed", 70001, 300, 3.0, False, 3),
-    ("fine", 2048, 600, 1.0, False, 1), ("fine", 65600, 60, 1.0, False, 1), ("sphere", 3000, 200, 15.0, True, 1), ("sphere", 257, 0, 1.0, False, 2)])
+    ("mixed", 393215, 60, 2.0, False, 1), ("mixed", 393216, 60, 2.0, False, 1), ("mixed", 393301, 60, 3.0, False, 3),
+    ("fine", 2048, 600, 1.0, False, 1), ("fine", 65600, 60, 1.0, False, 1), ("fine", 393300, 20, 1.0, False, 1), ("sphere", 3000, 200, 15.0, True, 1), ("sphere", 257, 0, 1.0, False, 2)])
 def test_shaft_walk_equals_per_ray_walk(env, kind, n, nf, theta, near, windows):
     G, ctx = env
     rng = np.random.default_rng(n + nf)
@@ -110,17 +111,17 @@ def _floor(n, occluder):
 
 
 def test_wide_tile_with_a_ray_in_a_coordinate_plane(env):
-    """Eyes exactly above samples, 1.5 cm over the floor: the ray straight down has no image point on the side of the
+    """Eyes exactly above samples, 6 mm over the floor: the ray straight down has no image point on the side of the
     tile's first ray (0 / 0 there), and what hides it crosses the plane through the eye."""
     G, ctx = env
     rng = np.random.default_rng(5)
-    q = np.array([[0.2, 0.007, 0.2], [0.8, 0.007, 0.2], [0.8, 0.007, 0.8], [0.2, 0.007, 0.8]], np.float32)
-    v, f, xyz, tri = _floor(70000, (q, np.array([[0, 2, 1], [0, 3, 2]], np.uint32)))
+    q = np.array([[0.2, 0.003, 0.2], [0.8, 0.003, 0.2], [0.8, 0.003, 0.8], [0.2, 0.003, 0.8]], np.float32)
+    v, f, xyz, tri = _floor(400000, (q, np.array([[0, 2, 1], [0, 3, 2]], np.uint32)))
     nf = 400
     at = rng.integers(0, len(xyz), nf)
     turn = rng.uniform(0.0, 2.0 * math.pi, nf)
     tilt = math.radians(24.0)
-    eye = xyz[at] + np.float32([0.0, 0.015, 0.0])
+    eye = xyz[at] + np.float32([0.0, 0.006, 0.0])
     gaze = np.stack([math.sin(tilt) * np.cos(turn), np.full(nf, -math.cos(tilt)), math.sin(tilt) * np.sin(turn)], 1)
     fix = [np.ascontiguousarray(eye, np.float32), np.ascontiguousarray(gaze, np.float32),
            rng.uniform(0.1, 0.6, nf).astype(np.float32), np.arange(float(nf))]
@@ -173,14 +174,14 @@ def test_blocks_of_wide_tiles(env, n, nf, theta, windows):
     assert a[1:] == b[1:] and a[2] > 0 and np.array_equal(a[0], b[0])
 
 
-@pytest.mark.parametrize("n,nf", [(7000, 100), (7000, 400), (14592, 300), (20000, 6000), (130000, 60), (70000, 200)])
+@pytest.mark.parametrize("n,nf", [(7000, 100), (7000, 400), (14592, 300), (20000, 6000), (130000, 60), (400000, 50)])
 def test_pair_records_of_every_block_size(env, n, nf):
     """The recorded pairs (blocks of 512, 1024, 1024, 512 and 256 threads; 256 with wide tiles) are the per-ray walk's:
     sample, fixation, visibility and weight."""
     G, ctx = env
     rng = np.random.default_rng(n)
-    v, f = _scene("mixed" if n == 70000 else "sphere")
-    xyz, tri = _points("mixed" if n == 70000 else "sphere", v, f, n, rng)
+    v, f = _scene("mixed" if n == 400000 else "sphere")
+    xyz, tri = _points("mixed" if n == 400000 else "sphere", v, f, n, rng)
     eye = rng.normal(size=(nf, 3))
     eye *= 2.5 / np.linalg.norm(eye, axis=1, keepdims=True)
     at = xyz[rng.integers(0, n, nf)].astype(np.float64)
@@ -211,12 +212,12 @@ def _above(n, rng, lo=0.3, hi=0.6, target=None):
 
 
 def test_wide_tiles_over_the_budget(env):
-    """80k triangles of about 1 mm between the viewers and a floor in wide tiles: shafts run over their budget and
+    """320k triangles of about half a millimetre between the viewers and a floor in wide tiles: shafts run over their budget and
     their four rays a lane walk the tree one by one."""
     G, ctx = env
     rng = np.random.default_rng(8)
-    ball = M.uv_sphere(142, 284, 0.06, 0.05, 30.0, seed=3)
-    v, f, xyz, tri = _floor(70000, (M.translate(ball[0], (0.5, 0.07, 0.5)), ball[1]))
+    ball = M.uv_sphere(284, 568, 0.06, 0.05, 30.0, seed=3)
+    v, f, xyz, tri = _floor(400000, (M.translate(ball[0], (0.5, 0.07, 0.5)), ball[1]))
     fix = [*_above(60, rng, target=(0.52, 0.02, 0.5)), np.arange(60.0)]
     scene = G.gm_build_scene(ctx, [(v, f, np.eye(4), 0)])
     samples = G.gm_samples_from_points(scene, xyz, tri)
@@ -234,7 +235,7 @@ def test_wide_tiles_of_a_posed_scene(env):
     ball, windows = M.uv_sphere(30, 60, 0.12, 0.1, 8.0, seed=2), 3
     scene = G.gm_build_scene(ctx, [(q, np.array([[0, 2, 1], [0, 3, 2]], np.uint32), np.eye(4), 0), (*ball, np.eye(4), 1)],
                              dynamic=True)
-    samples = G.gm_sample_surface(scene, [70000.0, 0.0], 3)
+    samples = G.gm_sample_surface(scene, [400000.0, 0.0], 3)
     poses = np.tile(np.eye(4), (windows, 2, 1, 1))
     for w in range(windows):
         a = 0.1 * w
