@@ -180,16 +180,17 @@ __global__ void __launch_bounds__(NT, MINB) k_accumulate(
     warp_stats_commit(st, counters);
 }
 
-// Whether a set with wide tiles takes blocks of 128 threads: where a wide tile is reached by few fixations, most
-// warps of a larger block wait for its slowest shaft, and twice the tiles in flight help more. The measure is
-// the mean, over SPARSE_TILES tiles of 128 samples spread over the work order, of the fixations that reach the
-// tile (64 at most: a few tiles are reached by all). Probed are lists of up to RS_SMALL fixations over
+// Whether the halves of a block (128 threads each) take a wide tile of their own: where a wide tile is reached by
+// few fixations, most warps of a whole block wait for its slowest shaft, and twice the tiles in flight help more.
+// Tiles of 32 samples on many triangles, the longest ones there, stay the whole block's and come first. The
+// measure is the mean, over SPARSE_TILES tiles of 128 samples spread over the work order, of the fixations that
+// reach the tile (64 at most: a few tiles are reached by all). Probed are lists of up to RS_SMALL fixations over
 // SPARSE_MIN samples or more: with more fixations tiles are not sparse, smaller sets end by their longest tile.
-// Walks in cities of 0.1-0.6M triangles, 1000-1500 fixations, us with 256 / 128 threads (per-ray walks): mean
-// 4: 2429 / 2107 (2260), 5: 1186 / 947 (1121), 8: 2920 / 2573 (2874), 9: 815 / 675 (799), but on four objects
-// of 20k triangles, where the longest tile decides: 6: 932 / 818, 10: 1193 / 1275, 12: 1441 / 1498,
-// 19: 1980 / 2191, 37: 3583 / 4126. (A city at 14: 672 / 583 (634): the line is drawn for the objects.) The probe
-// and a kernel that returns at once take 3 to 9 us.
+// us by whole blocks / by halves (per-ray walks), at a mean of 4: 2518 / 2170 (2308) (a city of 600k triangles,
+// 4M samples, 1000 fixations of 0.5 degrees), 5: 1204 / 959 (1138), 8: 3017 / 2630 (2907), 9: 819 / 680 (802); a room
+// with 60k triangles of objects that seven in ten of 600 fixations look at, 600k samples: 1602 / 1474 (4637).
+// Above, the longest wide tiles decide: 14: 651 / 709 (a city), 20: 1980 / 2191, 40: 3583 / 4126 (four objects of
+// 20k triangles, blocks of 128 threads). The probe and a kernel that returns at once take 3 to 9 us.
 constexpr int SPARSE_TILES = 256;
 constexpr uint32_t SPARSE_SUM = 19 * SPARSE_TILES / 2;
 constexpr uint64_t SPARSE_MIN = 1u << 19;
@@ -223,45 +224,63 @@ __global__ void __launch_bounds__(256) k_sparse_probe(const float4* __restrict__
 
 // The default: the rays of a (tile, fixation) pair traced as one shaft (gm_shaft.cuh). Blocks pull tiles
 // from a device counter (or, static, take their own): all tiles of 32 samples or, LISTS, the sample set's
-// tiles of 128 samples on few triangles and then its other tiles of 32 (gm_samples::tile_lists). For a set
-// with lists several forms are launched and the device knows which has the work; probed: among them the one
-// of 128 threads.
-template <bool DEBUG, bool LISTS, int NT = ACC_THREADS>
+// tiles of 128 samples on few triangles and then its other tiles of 32 (gm_samples::tile_lists); HALVES: first
+// the tiles of 32, then each half of the block wide ones of its own. For a set with lists several forms are
+// launched and the device knows which has the work; probed: HALVES among them. (One kernel of both: 612 bytes of
+// spills instead of 364.)
+template <bool DEBUG, bool LISTS, int NT = ACC_THREADS, bool HALVES = false>
 __global__ void __launch_bounds__(NT, 1024 / NT) k_accumulate_shaft(
     const float4* __restrict__ spos, const uint32_t* __restrict__ sidx, const float4* __restrict__ fix,
     const uint32_t* __restrict__ n_fix_dev, const float4* __restrict__ nodes, const float4* __restrict__ nodes4,
     const float4* __restrict__ tris, AccParams P, uint32_t n_tiles, const uint32_t* __restrict__ lists, bool probed,
     int persistent, float* __restrict__ out, unsigned int* __restrict__ max_bits,
     unsigned long long* __restrict__ counters, int* __restrict__ err, DebugOut dbg) {
-    constexpr size_t B1 = sizeof(ShaftBlock<1, NT>), B4 = sizeof(ShaftBlock<4, NT>);
+    constexpr size_t B1 = sizeof(ShaftBlock<1, NT>), B4 = HALVES ? 2 * sizeof(ShaftBlock<4, 128>) : sizeof(ShaftBlock<4>);
     __shared__ __align__(16) unsigned char fixed[NT > ACC_THREADS ? 16 : LISTS && B4 > B1 ? B4 : B1];
     extern __shared__ __align__(16) unsigned char dynamic[];   // above 48 KB
     unsigned char* smem = NT > ACC_THREADS ? dynamic : fixed;
-    __shared__ uint32_t s_tile;
+    __shared__ uint32_t s_tile[2];
     const uint32_t nf = *n_fix_dev;
     if (lists && gm_wide_tiles_pay(lists[0], P.ns) != LISTS) return;
-    if (LISTS && probed && sparse_tiles(n_fix_dev) != (NT < ACC_THREADS)) return;
-    const uint32_t n_wide = LISTS ? lists[0] : 0u;
-    const uint32_t n = LISTS ? n_wide + lists[1] : n_tiles;
+    if (LISTS && probed && sparse_tiles(n_fix_dev) != HALVES) return;
+    const uint32_t n_wide = LISTS ? lists[0] : 0u, n_fine = LISTS ? lists[1] : n_tiles;
+    const uint32_t n_first = HALVES ? n_fine : n_wide, n = n_wide + n_fine;
     unsigned int* next = reinterpret_cast<unsigned int*>(&counters[6]);
     TileStats st;
     uint32_t k = blockIdx.x;
     for (;;) {
         if (persistent) {
             __syncthreads();
-            if (threadIdx.x == 0) s_tile = atomicAdd(next, 1u);
+            if (threadIdx.x == 0) s_tile[0] = atomicAdd(next, 1u);
             __syncthreads();
-            k = s_tile;
+            k = s_tile[0];
         }
-        if (k >= n) break;
-        if (LISTS && k < n_wide)
-            shaft_tile<DEBUG, 4, NT>(__ldg(&lists[2 + k]), spos, sidx, fix, nf, nodes, nodes4, tris, P, out, max_bits,
-                                 *reinterpret_cast<ShaftBlock<4, NT>*>(smem), &counters[2], dbg, err, st);
+        if (k >= (HALVES ? n_first : n)) break;
+        if (LISTS && !HALVES && k < n_first)
+            shaft_tile<DEBUG, 4>(__ldg(&lists[2 + k]), spos, sidx, fix, nf, nodes, nodes4, tris, P, out, max_bits,
+                                 *reinterpret_cast<ShaftBlock<4>*>(smem), &counters[2], dbg, err, st);
         else
-            shaft_tile<DEBUG, 1, NT>(LISTS ? __ldg(&lists[gm_tile_list_fine(P.ns) + (k - n_wide)]) : k, spos, sidx, fix, nf, nodes,
-                                 nodes4, tris, P, out, max_bits, *reinterpret_cast<ShaftBlock<1, NT>*>(smem), &counters[2],
-                                 dbg, err, st);
+            shaft_tile<DEBUG, 1, NT>(LISTS ? __ldg(&lists[gm_tile_list_fine(P.ns) + (HALVES ? k : k - n_first)]) : k, spos,
+                                     sidx, fix, nf, nodes, nodes4, tris, P, out, max_bits,
+                                     *reinterpret_cast<ShaftBlock<1, NT>*>(smem), &counters[2], dbg, err, st);
         if (!persistent) break;
+    }
+    if constexpr (HALVES) {   // (persistent) the tile that ended the loop is the first half's
+        const int h = threadIdx.x >> 7;
+        auto pull = [&]() {
+            if ((threadIdx.x & 127) == 0) s_tile[h] = atomicAdd(next, 1u);
+            half_sync(h);
+            return s_tile[h];
+        };
+        __syncthreads();   // s_tile[0] has been read
+        if (h == 1) k = pull();
+        while (k < n) {
+            shaft_tile<DEBUG, 4, 128, true>(__ldg(&lists[2 + (k - n_first)]), spos, sidx, fix, nf, nodes, nodes4, tris, P, out,
+                                            max_bits, *(reinterpret_cast<ShaftBlock<4, 128>*>(smem) + h), &counters[2], dbg,
+                                            err, st);
+            half_sync(h);   // the tile's shared memory and s_tile[h] have been read
+            k = pull();
+        }
     }
     warp_stats_commit(st, counters);
 }
@@ -675,7 +694,7 @@ gm_status accumulate_impl(gm_scene* sc, gm_samples* sm, const gm_fixations* fx, 
             if (shaft) {
                 static const int per_sm = blocks_per_sm(k_accumulate_shaft<false, false>, ACC_THREADS);
                 static const int per_sm_lists = blocks_per_sm(k_accumulate_shaft<false, true>, ACC_THREADS);
-                static const int per_sm_128 = blocks_per_sm(k_accumulate_shaft<false, true, 128>, 128);
+                static const int per_sm_halves = blocks_per_sm(k_accumulate_shaft<false, true, ACC_THREADS, true>, ACC_THREADS);
                 const uint32_t* lists = reorder && persistent ? sm->tile_lists : nullptr;
                 const uint32_t tiles = gm_div_up(ns, 32);
                 auto grid = [&](int b) { return persistent ? std::min<uint32_t>((uint32_t)(ctx->n_sm * b), tiles) : tiles; };
@@ -696,21 +715,20 @@ gm_status accumulate_impl(gm_scene* sc, gm_samples* sm, const gm_fixations* fx, 
                     GM_TRY_CUDA(few(debug ? k_accumulate_shaft<true, false, 512> : k_accumulate_shaft<false, false, 512>,
                                     512, sizeof(ShaftBlock<1, 512>)));
                 } else {
-                    auto run = [&](auto kern, int threads, int blocks, bool probed) {
-                        kern<<<grid(blocks), threads, 0, s>>>(spos, sidx, packed, n_valid, sc->nodes, sc->nodes4,
-                                                              sc->bvh_tris, P, tiles, lists, probed, persistent,
-                                                              mp->values, mp->max_bits, mp->counters, ctx->dev_err, dbg);
+                    auto run = [&](auto kern, int blocks, bool probed) {
+                        kern<<<grid(blocks), ACC_THREADS, 0, s>>>(spos, sidx, packed, n_valid, sc->nodes, sc->nodes4,
+                                                                  sc->bvh_tris, P, tiles, lists, probed, persistent,
+                                                                  mp->values, mp->max_bits, mp->counters, ctx->dev_err, dbg);
                     };
                     const bool probed = lists && prep && !debug && P.tile_cull && ns >= SPARSE_MIN;
                     if (probed) {
                         k_sparse_probe<<<SPARSE_TILES, 256, 0, s>>>(spos, P.ns, packed, n_valid, P.tanphi);
-                        run(k_accumulate_shaft<false, true, 128>, 128, per_sm_128, true);
+                        run(k_accumulate_shaft<false, true, ACC_THREADS, true>, per_sm_halves, true);
                         launches += 2;
                     }
-                    run(debug ? k_accumulate_shaft<true, false> : k_accumulate_shaft<false, false>, ACC_THREADS, per_sm, false);
+                    run(debug ? k_accumulate_shaft<true, false> : k_accumulate_shaft<false, false>, per_sm, false);
                     if (lists) {
-                        run(debug ? k_accumulate_shaft<true, true> : k_accumulate_shaft<false, true>, ACC_THREADS,
-                            per_sm_lists, probed);
+                        run(debug ? k_accumulate_shaft<true, true> : k_accumulate_shaft<false, true>, per_sm_lists, probed);
                         launches++;
                     }
                 }

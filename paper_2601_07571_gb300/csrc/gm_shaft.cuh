@@ -586,10 +586,14 @@ __device__ __forceinline__ float4 tile_sphere(float lo[3], float hi[3]) {
                                     (hi[2] - lo[2]) * (hi[2] - lo[2])) * 1.0001f);
 }
 
+// The 128 threads of half h of a block wait for one another (barrier 0 is the block's).
+__device__ __forceinline__ void half_sync(int h) { asm volatile("bar.sync %0, 128;" ::"r"(h + 1) : "memory"); }
+
 // One block, all threads: tile `tile` (32 NS consecutive work-order samples) against fixations [0, nf) of
 // `fix` (packed (e, w), (r^, window), sorted by window). A window's sums are written when the next visible
 // fixation opens another one, or at the end.
-template <bool DEBUG, int NS, int NT = ACC_THREADS>
+// HALF: by the 128 threads of one half of a block (0 or 1), on its own barrier.
+template <bool DEBUG, int NS, int NT = ACC_THREADS, bool HALF = false>
 __device__ __forceinline__ void shaft_tile(const uint32_t tile, const float4* __restrict__ spos,
                                            const uint32_t* __restrict__ sidx, const float4* __restrict__ fix,
                                            const uint32_t nf, const float4* __restrict__ nodes,
@@ -598,8 +602,12 @@ __device__ __forceinline__ void shaft_tile(const uint32_t tile, const float4* __
                                            unsigned int* __restrict__ max_bits, ShaftBlock<NS, NT>& B,
                                            unsigned long long* __restrict__ dbg_cursor, const DebugOut& dbg,
                                            int* __restrict__ err, TileStats& st) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int tid = HALF ? threadIdx.x & (NT - 1) : threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned lt = gm_lanemask_lt();
+    auto sync = [&]() {
+        if constexpr (HALF) half_sync(threadIdx.x / NT);
+        else __syncthreads();
+    };
     const uint32_t j0 = tile * (32u * NS) + lane;
     float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
     uint32_t n_live = 0;   // of this lane
@@ -646,7 +654,7 @@ __device__ __forceinline__ void shaft_tile(const uint32_t tile, const float4* __
                 mine += __popc(reach[r]);
             }
             if (lane == 0) B.pass[warp] = mine;
-            __syncthreads();
+            sync();
             const int n = lane < NT / 32 ? (int)B.pass[lane] : 0;
             int at = cnt + __reduce_add_sync(0xffffffffu, lane < warp ? n : 0);
             cnt += __reduce_add_sync(0xffffffffu, n);
@@ -656,8 +664,8 @@ __device__ __forceinline__ void shaft_tile(const uint32_t tile, const float4* __
                 at += __popc(reach[r]);
             }
             pos += PER * NT;
-            if (threadIdx.x == 0) B.next = 0;
-            __syncthreads();
+            if (tid == 0) B.next = 0;
+            sync();
         }
         if (warp == 0) n_items += cnt;
         // trace the items
@@ -701,7 +709,7 @@ __device__ __forceinline__ void shaft_tile(const uint32_t tile, const float4* __
                 if (lane == 0) B.vis[r][k] = vm;
             }
         }
-        __syncthreads();
+        sync();
         // add the visible weights in list order
         if (warp < NS) {
             const float4 p = NS == 1 ? p0 : B.pos[32 * warp + lane];
@@ -732,7 +740,7 @@ __device__ __forceinline__ void shaft_tile(const uint32_t tile, const float4* __
                 }
             }
         }
-        __syncthreads();
+        sync();
     }
     if (warp < NS) {
         if (cur != 0xffffffffu) flush(cur);
