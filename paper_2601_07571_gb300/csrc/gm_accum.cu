@@ -103,7 +103,8 @@ __global__ void k_fix_pack(FixIn I, const uint32_t* __restrict__ keys, const uin
 // The same for up to RS_SMALL fixations and windows in one block: keys, sort, list, and the map's counters
 // and maxima set to what the accumulation starts from (into an existing map: the tile counter alone, the
 // valid fixations added). Bound by latency: at 100 fixations 7.3 us against 11.9 for the three kernels, and
-// three fills, a copy and two allocations fewer around it; a call with 6656 samples takes 84 us, not 95.
+// three fills, a copy and two allocations fewer around it: a call with 6656 samples took 84 us instead of 95
+// when this came (77 now, by other steps).
 __global__ void __launch_bounds__(1024) k_fix_prep(FixIn I, int bits, bool into, float4* __restrict__ packed,
                                                    uint32_t* __restrict__ orig, uint32_t* __restrict__ n_valid,
                                                    unsigned int* __restrict__ max_bits,
@@ -398,9 +399,6 @@ gm_status n_windows_of(const gm_params* prm, uint64_t* W_out) {
     return GM_OK;
 }
 
-// The accumulation of one fixation set. into == nullptr: a new map (returned in *out) over all
-// windows. into != nullptr: adds the fixations of window `only_window` to that existing map
-// (no normalisation, no stage timing), for dynamic scenes posed window by window.
 // Threads of a shaft kernel's blocks for n_fix fixations. A tile is one block's from beginning to end, so
 // where the GPU has few tiles a block and each sees many fixations, the longest tile sets the time and more
 // warps shorten it; where they see few, a large block mostly waits at the end of its batches. With 256 /
@@ -414,12 +412,15 @@ int shaft_threads(uint64_t tiles, uint64_t n_fix, int n_sm) {
 }
 
 template <typename K>
-int blocks_per_sm(K kern, int nt) {
+int blocks_per_sm(K kern) {
     int b = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, nt, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, ACC_THREADS, 0);
     return b > 0 ? b : 1;
 }
 
+// The accumulation of one fixation set. into == nullptr: a new map (returned in *out) over all
+// windows. into != nullptr: adds the fixations of window `only_window` to that existing map
+// (no normalisation, no stage timing), for dynamic scenes posed window by window.
 gm_status accumulate_impl(gm_scene* sc, gm_samples* sm, const gm_fixations* fx, const gm_params* prm,
                           gm_stream stream, gm_map* into, int64_t only_window, gm_map** out) {
     if (!sc || !sm || !fx || !prm || (!out && !into))
@@ -692,9 +693,9 @@ gm_status accumulate_impl(gm_scene* sc, gm_samples* sm, const gm_fixations* fx, 
                 cudaEventRecord(mp->ev[5], s);
             }
             if (shaft) {
-                static const int per_sm = blocks_per_sm(k_accumulate_shaft<false, false>, ACC_THREADS);
-                static const int per_sm_lists = blocks_per_sm(k_accumulate_shaft<false, true>, ACC_THREADS);
-                static const int per_sm_halves = blocks_per_sm(k_accumulate_shaft<false, true, ACC_THREADS, true>, ACC_THREADS);
+                static const int per_sm = blocks_per_sm(k_accumulate_shaft<false, false>);
+                static const int per_sm_lists = blocks_per_sm(k_accumulate_shaft<false, true>);
+                static const int per_sm_halves = blocks_per_sm(k_accumulate_shaft<false, true, ACC_THREADS, true>);
                 const uint32_t* lists = reorder && persistent ? sm->tile_lists : nullptr;
                 const uint32_t tiles = gm_div_up(ns, 32);
                 auto grid = [&](int b) { return persistent ? std::min<uint32_t>((uint32_t)(ctx->n_sm * b), tiles) : tiles; };

@@ -547,7 +547,7 @@ struct ShaftBlock {
     float4 pos[NS == 1 ? 1 : 32 * NS];   // the tile's samples (NS = 1: in registers)
     uint32_t list[shaft_list(NS, NT)];      // fixation indices
     uint32_t vis[NS][shaft_list(NS, NT)];   // visible samples of each item
-    uint32_t pass[NT / 32];    // passing fixations of each warp's 64 in one fill step
+    uint32_t pass[NT / 32];    // passing fixations of each warp's 32 shaft_per in one fill step
     int next;                   // next item to trace
 };
 

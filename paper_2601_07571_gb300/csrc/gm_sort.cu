@@ -5,8 +5,8 @@
 // Up to RS_SMALL keys: one block sorts them in shared memory, one launch for all digits. More: three
 // kernels per radix pass: per-tile digit histograms, an exclusive scan of every digit's row of the
 // digit-major histogram table (a block per digit), then a stable scatter in which each warp ranks its
-// own run of keys with warp match and its own digit counters, so that a tile synchronises four times
-// rather than three times per 256 keys. Tiles of 2048 keys: at 800k keys they make 390 blocks (196 of
+// own run of keys with warp match and its own digit counters, so that a tile synchronises five times (three
+// of them the scan's) rather than three times per 256 keys. Tiles of 2048 keys: at 800k keys they make 390 blocks (196 of
 // 4096 keys left the 152 SMs at one block each). No spin-waits anywhere.
 // Bound by launches and latency at these sizes (800k 63-bit keys: 19 MB a pass).
 #include <algorithm>
