@@ -46,8 +46,8 @@ SM_MAX_MHZ_NOMINAL = 2070.0
 # one-pass ncu capture of the default bench command (paper scene, default flags and builder).
 # The figure stands only while the sources that shape the kernel and its inputs are the ones it
 # was taken on: their SHA-256 is stored beside it and `traffic` is null on any mismatch.
-ACC_TRAFFIC = {"workload": "paper_scene_800ktri_2Msample_6000fix", "bytes": 302.960896e6,
-               "sources_sha256": "c59521bbaaf6497f4b1adecafce564437f0c6675df823863a8315827be39c6ab"}
+ACC_TRAFFIC = {"workload": "paper_scene_800ktri_2Msample_6000fix", "bytes": 302.185728e6,
+               "sources_sha256": "63d63a89636ccbec83b61402fd34f49de387ae358393ca9337d3c1aa1b877b57"}
 ACC_TRAFFIC_SOURCES = ("paper_2601_07571_gb300/csrc/gm_trace.cuh", "paper_2601_07571_gb300/csrc/gm_accum.cu",
                        "paper_2601_07571_gb300/csrc/gm_shaft.cuh",
                        "paper_2601_07571_gb300/csrc/gm_scene.cu", "paper_2601_07571_gb300/csrc/gm_sampler.cu")
