@@ -227,21 +227,23 @@ def test_wide_tiles_over_the_budget(env):
     assert a[1:] == b[1:] and 0 < a[2] < a[1] and np.array_equal(a[0], b[0])
 
 
-def test_wide_tiles_of_a_posed_scene(env):
-    """A floor in wide tiles, turning, below a ball that moves: every window's map is the per-ray walk's."""
+@pytest.mark.parametrize("density,nf", [(400000.0, 300), (530000.0, 45)])
+def test_wide_tiles_of_a_posed_scene(env, density, nf):
+    """A floor in wide tiles (whole blocks; halves of blocks), turning, below a ball that moves: every window's map is
+    the per-ray walk's."""
     G, ctx = env
     rng = np.random.default_rng(9)
     q = np.array([[0.0, 0.0, 0.0], [1.0, 0.0, 0.0], [1.0, 0.0, 1.0], [0.0, 0.0, 1.0]], np.float32)
     ball, windows = M.uv_sphere(30, 60, 0.12, 0.1, 8.0, seed=2), 3
     scene = G.gm_build_scene(ctx, [(q, np.array([[0, 2, 1], [0, 3, 2]], np.uint32), np.eye(4), 0), (*ball, np.eye(4), 1)],
                              dynamic=True)
-    samples = G.gm_sample_surface(scene, [400000.0, 0.0], 3)
+    samples = G.gm_sample_surface(scene, [density, 0.0], 3)
     poses = np.tile(np.eye(4), (windows, 2, 1, 1))
     for w in range(windows):
         a = 0.1 * w
         poses[w, 0, :3, :3] = [[math.cos(a), 0, math.sin(a)], [0, 1, 0], [-math.sin(a), 0, math.cos(a)]]
         poses[w, 1, :3, 3] = [0.3 + 0.2 * w, 0.2, 0.5]
-    fix = [*_above(300, rng), np.sort(rng.uniform(0, windows, 300))]
+    fix = [*_above(nf, rng), np.sort(rng.uniform(0, windows, nf))]
     prm = dict(t_begin=0.0, t_end=float(windows), window_s=1.0, normalize=False)
     out = []
     for flags in (0, G.GM_F_FIX_L1):
